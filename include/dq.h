@@ -10,12 +10,15 @@
  *   dq_quantize_pack           Q_b[g] of Eq. 5/6, b-bit codes packed (workers)
  *   dq_unpack_dequant_average  "Average" step of Algorithm 1         (server)
  *
- * and two calls that merge neighbouring steps:
+ * and calls that merge neighbouring steps:
  *
  *   dq_norms_quantize_pack     norms and quantizer in one pass over the gradients
  *                              (b_t is known before step t: Algorithm 1 derives
  *                              b_{t+1} from iteration t)
  *   dq_unpack_average_update   the average followed by x <- x - eta * average (Eq. 2)
+ *   dq_quantize_average        quantizer and average in one pass, for a process that holds all
+ *                              workers' gradients
+ *   dq_norms_quantize_average  a whole round of Algorithm 1 in one call, the next b included
  *
  * M workers are M gradient buffers on one GPU: worker m's data is at
  * base + m * stride for every per-worker array.  There is no CPU fallback.
@@ -311,6 +314,37 @@ int dq_norms_quantize_pack_worker(const dq_layout_t* layout, const float* dev_gr
                                   int32_t M, const int32_t* dev_b, uint64_t seed, uint32_t step,
                                   uint32_t first_worker, float* dev_norms, uint32_t* dev_packed,
                                   int64_t packed_stride_words, int32_t* dev_status, void* stream);
+
+/* ------------------ quantizer and average in one pass, Eq. 5 and 6 and "Average"
+ * For a process that holds all M workers' gradients: the codes of a bucket are added to
+ * the average while they are still in registers, so the packed words are written (exactly
+ * as dq_quantize_pack writes them) but not read back.  update = 0: dev_out receives exactly
+ * what dq_unpack_dequant_average computes from those words.  update != 0: dev_out holds the
+ * parameters and becomes dev_out - lr * average, as dq_unpack_average_update does it.
+ * in : dev_grads, dev_norms [M][nb], dev_b (dev_out with update)
+ * out: dev_packed, dev_out fp32 [D32]
+ * Device conditions: those of both calls. */
+int dq_quantize_average(const dq_layout_t* layout, const float* dev_grads, int64_t worker_stride_elems,
+                        int32_t M, const float* dev_norms, const int32_t* dev_b, uint64_t seed, uint32_t step,
+                        uint32_t* dev_packed, int64_t packed_stride_words,
+                        float* dev_out, int32_t update, float lr, int32_t* dev_status, void* stream);
+
+/* A whole round in Algorithm 1's order: norms, codes with the b that dev_b holds, average
+ * (or parameter update), and the b of the next round from this round's norms -- the
+ * results of
+ *   dq_norms_quantize_pack -> dq_unpack_dequant_average (or _update) -> dq_choose_bits,
+ * for every layout (whole-tensor ones included), with the gradients read once where the
+ * bucket length is 32 * 2^k and twice otherwise.  (The sum behind G-bar is fp64 in another
+ * fixed order than dq_choose_bits'.)  dev_b is read and then overwritten with the next
+ * (b, s).  dev_workspace: dq_round_workspace_bytes() bytes of 16-byte aligned device
+ * memory, ZEROED ONCE before its first use and afterwards left to the calls; calls that may
+ * overlap on the GPU need a workspace each. */
+size_t dq_round_workspace_bytes(const dq_layout_t* layout, int32_t M);
+int dq_norms_quantize_average(const dq_layout_t* layout, const float* dev_grads, int64_t worker_stride_elems,
+                              int32_t M, int32_t* dev_b, uint64_t seed, uint32_t step, float* dev_norms,
+                              uint32_t* dev_packed, int64_t packed_stride_words,
+                              float* dev_out, int32_t update, float lr, const dq_rule_t* next_rule,
+                              void* dev_workspace, size_t workspace_bytes, int32_t* dev_status, void* stream);
 
 /* ----------------------------------- Algorithm 1, server side: "Average"
  * dev_out[j] = (1/M) sum_m (code_m - s) * norm_m / s   (Eq. 5 inverted, then

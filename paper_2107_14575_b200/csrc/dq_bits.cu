@@ -1,14 +1,10 @@
-// dq_choose_bits: the bit rule of Eq. 17 evaluated on the device.
-//
-//   G-bar^2 = (1/M) sum over workers and buckets of norm^2        (Lemma 1)
-//   x       = sqrt(T/eps_hat) * alpha^((T-1-t)/2) * G-bar
-//   b       = smallest b in [b_min, b_max] with 2^(b-1) - 1 >= x   (else b_max)
+// dq_choose_bits: the bit rule of Eq. 17 evaluated on the device (dq_rule.cuh).
 //
 // Two small kernels: fixed-size chunks of the norm array are summed in fp64
 // (fixed assignment of elements to threads, fixed tree), then one CTA adds
-// the chunk sums in a fixed order and applies the rule.  The factor
-// sqrt(T/eps_hat) * alpha^((T-1-t)/2) is a host scalar.
+// the chunk sums in a fixed order and applies the rule.
 #include "dq_common.cuh"
+#include "dq_rule.cuh"
 
 #include <cmath>
 #include <mutex>
@@ -21,23 +17,6 @@ namespace {
 constexpr int kThreads = 128;       // threads of the second kernel
 constexpr int kChunk = 8192;        // norms per CTA of the first kernel
 constexpr int kSumThreads = 128;    // threads of the first kernel: 64 norms each, all loads in flight at once
-
-// Sum over the CTA in a fixed order: shuffle tree inside each warp, then the warp sums
-// added in warp order by thread 0.  Returns the total in thread 0.
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double total = 0.0;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 0; w < NT / 32; ++w) total += sh[w];
-    }
-    return total;
-}
 
 __global__ void __launch_bounds__(kSumThreads, 8)
 norm_square_partials(const float* __restrict__ norms, const int64_t n, double* __restrict__ partial)
@@ -67,38 +46,43 @@ norm_square_partials(const float* __restrict__ norms, const int64_t n, double* _
 }
 
 __global__ void __launch_bounds__(kThreads)
-apply_rule(const double* __restrict__ partial, const int npartial, const int M, const double coef,
-           const int b_min, const int b_max, const int fixed_b,
-           int32_t* __restrict__ dev_b, int32_t* __restrict__ status)
+apply_rule(const RuleArgs r, const int npartial, int32_t* __restrict__ dev_b, int32_t* __restrict__ status)
 {
     __shared__ double sh[kThreads / 32];
     grid_dependency_wait();
     double acc = 0.0;
-    for (int i = threadIdx.x; i < npartial; i += kThreads) acc += partial[i];
+    for (int i = threadIdx.x; i < npartial; i += kThreads) acc += r.partial[i];
     const double sum = block_sum<kThreads>(acc, sh);
-    if (threadIdx.x != 0) return;
-
-    int b;
-    if (fixed_b != 0) {
-        b = fixed_b;
-    } else {
-        const double x = coef * sqrt(sum / (double)M);
-        b = b_max;
-        if (isfinite(x)) {
-            for (int c = b_min; c <= b_max; ++c) {
-                if ((double)((1 << (c - 1)) - 1) >= x) { b = c; break; }
-            }
-        } else {
-            atomicOr(status, DQ_STAT_NONFINITE);
-        }
-    }
-    dev_b[0] = b;
-    dev_b[1] = (1 << (b - 1)) - 1;
+    if (threadIdx.x == 0) write_next_bits(r, sum, dev_b, status);
 }
 
 inline int64_t num_chunks(int64_t n) { return (n + kChunk - 1) / kChunk; }
 
 }  // namespace
+
+int dq_check_rule(const dq_rule_t* rule)
+{
+    if (rule->fixed_b < 0 || rule->fixed_b > DQ_MAX_BITS) return DQ_ERR_RANGE;
+    if (rule->b_min < 1 || rule->b_max > DQ_MAX_BITS || rule->b_min > rule->b_max) return DQ_ERR_RANGE;
+    if (rule->fixed_b == 0 &&
+        (rule->T < 1 || rule->t < 0 || rule->t >= rule->T || !(rule->eps_hat > 0.0) || !(rule->alpha > 0.0) ||
+         !std::isfinite(rule->eps_hat) || !std::isfinite(rule->alpha)))
+        return DQ_ERR_RANGE;
+    return DQ_OK;
+}
+
+RuleArgs dq_rule_args(const dq_rule_t* rule, int32_t M)
+{
+    RuleArgs r = {};
+    r.b_min = rule->b_min;
+    r.b_max = rule->b_max;
+    r.fixed_b = rule->fixed_b;
+    r.M = M;
+    if (rule->fixed_b == 0)
+        r.coef = std::sqrt((double)rule->T / rule->eps_hat) *
+                 std::pow(rule->alpha, (double)(rule->T - 1 - rule->t) / 2.0);
+    return r;
+}
 
 extern "C" size_t dq_choose_bits_scratch_bytes(const dq_layout_t* L, int32_t M)
 {
@@ -120,13 +104,7 @@ int check_rule_args(const dq_layout_t* L, const float* dev_norms, int32_t M, con
     if ((reinterpret_cast<uintptr_t>(dev_norms) & 3u) || (reinterpret_cast<uintptr_t>(dev_b) & 3u) ||
         (reinterpret_cast<uintptr_t>(dev_status) & 3u))
         return DQ_ERR_ALIGN;
-    if (rule->fixed_b < 0 || rule->fixed_b > DQ_MAX_BITS) return DQ_ERR_RANGE;
-    if (rule->b_min < 1 || rule->b_max > DQ_MAX_BITS || rule->b_min > rule->b_max) return DQ_ERR_RANGE;
-    if (rule->fixed_b == 0 &&
-        (rule->T < 1 || rule->t < 0 || rule->t >= rule->T || !(rule->eps_hat > 0.0) || !(rule->alpha > 0.0) ||
-         !std::isfinite(rule->eps_hat) || !std::isfinite(rule->alpha)))
-        return DQ_ERR_RANGE;
-    return DQ_OK;
+    return dq_check_rule(rule);
 }
 
 // The two kernels of the rule, with the chunk sums in `partial` (at least num_chunks(M * nb) doubles).
@@ -135,17 +113,14 @@ int launch_rule(const dq_layout_t* L, const float* dev_norms, int32_t M, const d
 {
     const int64_t n = (int64_t)M * L->nb;
     const int64_t chunks = num_chunks(n);
-    double coef = 0.0;
-    if (rule->fixed_b == 0)
-        coef = std::sqrt((double)rule->T / rule->eps_hat) *
-               std::pow(rule->alpha, (double)(rule->T - 1 - rule->t) / 2.0);
+    RuleArgs r = dq_rule_args(rule, M);
+    r.partial = partial;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (rule->fixed_b == 0) {
         dq_launch(norm_square_partials, dim3((unsigned)chunks), dim3(kSumThreads), 0, st, dev_norms, n, partial);
         if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
     }
-    dq_launch(apply_rule, dim3(1), dim3(kThreads), 0, st, partial, rule->fixed_b == 0 ? (int)chunks : 0, M, coef,
-              rule->b_min, rule->b_max, rule->fixed_b, dev_b, dev_status);
+    dq_launch(apply_rule, dim3(1), dim3(kThreads), 0, st, r, rule->fixed_b == 0 ? (int)chunks : 0, dev_b, dev_status);
     if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
     return DQ_OK;
 }

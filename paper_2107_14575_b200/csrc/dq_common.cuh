@@ -113,12 +113,18 @@ inline void dq_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
 // lies inside [base, base + extent) and, if it does not, raises DQ_STAT_INTERNAL instead of storing:
 // the stand-in for a memory checker where none can be run.
 #ifdef DQ_CHECKED
+__device__ __forceinline__ bool dq_store_allowed(const void* p, const int bytes, const void* base, const int64_t extent_bytes,
+                                                 int32_t* status)
+{
+    const int64_t off = reinterpret_cast<const char*>(p) - reinterpret_cast<const char*>(base);
+    if (off >= 0 && off + bytes <= extent_bytes) return true;
+    atomicOr(status, DQ_STAT_INTERNAL);
+    return false;
+}
 template <class T>
 __device__ __forceinline__ void dq_checked_store(T* p, const T& v, const void* base, const int64_t extent_bytes, int32_t* status)
 {
-    const int64_t off = reinterpret_cast<const char*>(p) - reinterpret_cast<const char*>(base);
-    if (off < 0 || off + (int64_t)sizeof(T) > extent_bytes) atomicOr(status, DQ_STAT_INTERNAL);
-    else *p = v;
+    if (dq_store_allowed(p, (int)sizeof(T), base, extent_bytes, status)) *p = v;
 }
 #define DQ_STORE(p, v, base, extent_bytes, status) dq_checked_store((p), (v), (base), (int64_t)(extent_bytes), (status))
 #else

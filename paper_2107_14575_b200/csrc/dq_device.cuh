@@ -8,7 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "dq.h"
+#include "dq_common.cuh"
 
 // Round keys of Philox4x32-10: key + r * (0x9E3779B9, 0xBB67AE85).  They are the
 // same for the whole grid, so the host computes them and they travel as kernel
@@ -163,32 +163,24 @@ __device__ __forceinline__ uint64_t fma_pair(const uint64_t a, const uint64_t b,
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-// Eq. 5/6 for one element.  With x = RZ(g * inv), inv = RZ(s / norm), the element's
-// position on the level grid and v = (2k + 1) / 2^17 its uniform draw (k a 16-bit
-// half of a Philox word), the code is floor(x + v) + s: for either sign the
-// neighbour of x away from zero is taken with probability frac(|x|), Eq. 6.
-//  * Both roundings are toward zero, so |x| <= s whenever |g| <= norm (a bucket's
-//    norm dominates its entries): no clamp, no absolute value, no sign handling.
-//  * HALF selects the low (0) or high (1) 16 bits of w.  The bits
-//    0x3F800040 | k << 7 are the float 1 + v (the constant comes in a register the
-//    compiler cannot fold, see and_or).
-//  * An add rounded toward -inf never crosses an integer downwards, so
-//    floor(fl(x + (1 + v))) is the floor of the exact sum; adding 2^23 + s - 1,
-//    again toward -inf, leaves floor(x + v) + s in the low mantissa bits.  No
-//    conversion instruction.
-// The result carries the code in its low B bits and the exponent bits of 2^23
-// above them; the packer drops everything above bit B-1.
-template <int B, int HALF>
-__device__ __forceinline__ uint32_t encode(const float g, const float inv, const uint32_t w, const uint32_t one_bits)
+__device__ __forceinline__ uint64_t mul_pair_rz(const uint64_t a, const uint64_t b)
 {
-    constexpr int s = (1 << (B - 1)) - 1;
-    const float x = __fmul_rz(g, inv);
-    // k << 7 in place: the high half comes down by a multiply-high (w * 2^23 >> 32 = w >> 9),
-    // which runs on the multiplier and leaves the logic pipe to the generator
-    const uint32_t kbits = HALF ? __umulhi(w, 0x00800000u) : (w << 7);
-    const float one_plus_v = __uint_as_float(and_or(kbits, 0x007FFF80u, one_bits));   // one_bits = 0x3F800040
-    const float t = __fadd_rd(__fadd_rd(x, one_plus_v), 8388608.0f + (float)(s - 1));
-    return __float_as_uint(t);
+    uint64_t r;
+    asm("mul.rz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_pair_rm(const uint64_t a, const uint64_t b)
+{
+    uint64_t r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// the same number in both lanes of a pair
+__host__ __device__ constexpr uint64_t both(const uint32_t bits) { return (uint64_t)bits << 32 | bits; }
+// bits of the float n + 2^p for 0 <= n < 2^p, p <= 23 (n an integer)
+__host__ __device__ constexpr uint32_t float_bits(const uint32_t n, const int p)
+{
+    return (uint32_t)(127 + p) << 23 | n << (23 - p);
 }
 
 // inv = RZ(s / norm), the scale of Eq. 5 rounded toward zero (0 for norm < 2^-100, where the
@@ -210,27 +202,26 @@ __device__ __forceinline__ float inv_scale(const float sf, const float norm)
     return __uint_as_float(__float_as_uint(q) - (e < 0.0f ? 1u : 0u));
 }
 
-// Appends code number E of a group to the group's little-endian bit string.
-// `cur` is a shift register: a funnel shift pushes the B code bits in at the
-// top, so after 32 bits the first code sits at bit 0 and the word is complete.
-// A code that straddles two words finishes the current word with its low bits
-// and seeds the next one with itself at the top; the surplus low bits fall off
-// as that word fills up.  Bits of `code` above B-1 never reach a word.
-template <int B, int E>
-__device__ __forceinline__ void push_code(uint32_t (&acc)[B], uint32_t& cur, const uint32_t code)
+// Appends W bits at position BIT of a group's little-endian bit string of N words.  `cur` is a
+// shift register: a funnel shift pushes the bits in at the top, so after 32 bits the first of them
+// sits at bit 0 and the word is complete.  Bits that straddle two words finish the current word with
+// their low part and seed the next one with themselves at the top; the surplus low bits fall off as
+// that word fills up.  What stands above bit W-1 of `bits` never reaches a word.
+template <int BIT, int W, int N>
+__device__ __forceinline__ void push_bits(uint32_t (&acc)[N], uint32_t& cur, const uint32_t bits)
 {
-    constexpr int bit = E * B;
-    constexpr int w = bit >> 5;
-    constexpr int sh = bit & 31;
-    constexpr int end = sh + B;
+    constexpr int w = BIT >> 5;
+    constexpr int sh = BIT & 31;
+    constexpr int end = sh + W;
     if constexpr (end < 32) {
-        if constexpr (sh == 0) cur = code << (32 - B);
-        else cur = __funnelshift_r(cur, code, B);
+        if constexpr (sh == 0) cur = bits << (32 - W);
+        else cur = __funnelshift_r(cur, bits, W);
     } else if constexpr (end == 32) {
-        acc[w] = __funnelshift_r(cur, code, B);
+        if constexpr (sh == 0) acc[w] = bits;
+        else acc[w] = __funnelshift_r(cur, bits, W);
     } else {
-        acc[w] = __funnelshift_r(cur, code, 32 - sh);
-        cur = code << (32 - B);
+        acc[w] = __funnelshift_r(cur, bits, 32 - sh);
+        cur = bits << (32 - W);
     }
 }
 
@@ -241,7 +232,7 @@ template <int B, int E>
 struct PushSame {
     static __device__ __forceinline__ void run(uint32_t (&acc)[B], uint32_t& cur, const uint32_t code)
     {
-        push_code<B, E>(acc, cur, code);
+        push_bits<E * B, B>(acc, cur, code);
         PushSame<B, E + 1>::run(acc, cur, code);
     }
 };
@@ -256,41 +247,191 @@ __device__ __forceinline__ void zero_group_words(uint32_t (&acc)[B])
     PushSame<B, 0>::run(acc, cur, (1u << (B - 1)) - 1u);
 }
 
-// Stores the B words of one group into the warp's staging area (stride B words
-// between lanes; the widest access the alignment allows keeps bank conflicts low).
-template <int B>
-__device__ __forceinline__ void stage_words(uint32_t* __restrict__ dst, const uint32_t (&acc)[B])
+// ---- Eq. 5/6 for the 32 elements of a group, two at a time ----------------------------------
+// With x = RZ(g * inv), inv = RZ(s / norm), the element's position on the level grid and
+// v = (2k + 1) / 2^17 its uniform draw (k a 16-bit half of a Philox word), the code is
+// floor(x + v) + s: for either sign the neighbour of x away from zero is taken with probability
+// frac(|x|), Eq. 6.
+//  * Both roundings are toward zero, so |x| <= s whenever |g| <= norm (a bucket's norm dominates its
+//    entries): no clamp, no absolute value, no sign handling.
+//  * A byte permute puts k under the upper half of the float 128 + c (c an integer): that float is
+//    K = 128 + c + k / 2^16, one instruction for draw, shift and exponent.
+//  * s <= 63 (b <= 7): with c = s the sum x + K lies in [128, 256), where floats are multiples of
+//    2^-16, and t = RN(x + K) has floor(x + v) + s as its integer part.  Rounding to nearest adds the
+//    half step 2^-17 that K lacks: the integer n is reached if and only if x + k / 2^16 >= n - 2^-17,
+//    a tie at the integer itself included (it goes to the even neighbour, and n is a multiple of 2^16
+//    steps).  The code stands in bits 16..22 of t.
+//  * Larger s: the half step is added first, y = RD(x + 2^-17), then RD(y + K).  An addition rounded
+//    down never crosses a representable number downwards, and the numbers x + 2^-17 is compared with,
+//    n - k / 2^16, are representable where |x| < 128; from there on x itself is a multiple of 2^-16,
+//    and y = x compares with them as x + 2^-17 does.
+//  * RD(t + (1.5 * 2^23 - 128)) drops the fraction: its low bits are the code, and subtracting
+//    1.5 * 2^23 + s leaves the signed level, exactly, for the average.
+// The packed two-lane forms halve the instructions issued (the kernels are bound by issue, not by
+// the lanes): 5.5 per element at b = 4 with its share of the average, against 6 for the code alone in
+// scalar form.
+
+// two Philox halves -> K for elements 2i and 2i + 1
+__device__ __forceinline__ uint64_t draw_pair(const uint32_t w, const uint32_t base)
 {
-    if constexpr (B % 4 == 0) {
+    return pack_pair(__byte_perm(w, base, 0x7610), __byte_perm(w, base, 0x7632));
+}
+// codes of two t's (bits 16..22 of each) as one word, 16 bits apart, everything else zero: the top
+// byte of t, 0x43, is replaced by copies of its sign
+__device__ __forceinline__ uint32_t code_halves(const uint32_t ta, const uint32_t tb)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, 0xF6B2;" : "=r"(r) : "r"(ta), "r"(tb));
+    return r;
+}
+__device__ __forceinline__ void split_pair(const uint64_t v, uint32_t& lo, uint32_t& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
+}
+
+// Appends the codes of elements 8C .. 8C + 7 to the group's words.  t: for b <= 7 the float with the
+// code in bits 16..22; u: the float with the code in its low bits (not formed where t is enough).
+template <int B>
+struct PacksFromT {
+    static constexpr bool value = B <= 4;
+};
+template <int B, int C>
+__device__ __forceinline__ void pack_eight(uint32_t (&words)[B], uint32_t& cur, const uint32_t (&t)[8], const uint32_t (&u)[8])
+{
+    if constexpr (B <= 4) {
+        // halves of q: the codes of elements 0..3 and of 4..7, 4 * B bits each
+        const uint32_t q = (((code_halves(t[3], t[7]) << B) + code_halves(t[2], t[6]) << B) + code_halves(t[1], t[5]) << B) +
+                           code_halves(t[0], t[4]);
+        if constexpr (B == 4) {
+            words[C] = q;
+        } else if constexpr (B == 3) {
+            push_bits<24 * C, 24>(words, cur, (q & 0xFFFu) | ((q >> 4) & 0xFFF000u));
+        } else {
+            if constexpr (C % 2 == 0) cur = q;
+            else words[C / 2] = __byte_perm(cur, q, 0x6420);
+        }
+    } else if constexpr (B == 8) {
+        words[2 * C] = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+        words[2 * C + 1] = __byte_perm(__byte_perm(u[4], u[5], 0x0040), __byte_perm(u[6], u[7], 0x0040), 0x5410);
+    } else if constexpr (B == 16) {
 #pragma unroll
-        for (int i = 0; i < B / 4; ++i)
-            reinterpret_cast<uint4*>(dst)[i] = make_uint4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-    } else if constexpr (B % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < B / 2; ++i)
-            reinterpret_cast<uint2*>(dst)[i] = make_uint2(acc[2 * i], acc[2 * i + 1]);
+        for (int i = 0; i < 4; ++i) words[4 * C + i] = __byte_perm(u[2 * i], u[2 * i + 1], 0x5410);
     } else {
-#pragma unroll
-        for (int i = 0; i < B; ++i) dst[i] = acc[i];
+        push_bits<(8 * C + 0) * B, B>(words, cur, u[0]);
+        push_bits<(8 * C + 1) * B, B>(words, cur, u[1]);
+        push_bits<(8 * C + 2) * B, B>(words, cur, u[2]);
+        push_bits<(8 * C + 3) * B, B>(words, cur, u[3]);
+        push_bits<(8 * C + 4) * B, B>(words, cur, u[4]);
+        push_bits<(8 * C + 5) * B, B>(words, cur, u[5]);
+        push_bits<(8 * C + 6) * B, B>(words, cur, u[6]);
+        push_bits<(8 * C + 7) * B, B>(words, cur, u[7]);
     }
 }
 
-// Encodes elements 8C .. 8C+7 of a group (one Philox block) and appends the codes.
-template <int B, int C>
-__device__ __forceinline__ void encode_block(uint32_t (&acc)[B], uint32_t& cur, const float4 lo, const float4 hi,
-                                             const float inv, const uint32_t q, const uint32_t m,
-                                             const uint32_t step, const PhiloxKeys& keys, const uint32_t ob)
+// Elements 8C .. 8C + 7 (one Philox block); with AVG, level * scale is added to their sums.
+template <int B, int C, bool AVG>
+__device__ __forceinline__ void encode_eight(const uint64_t (&x)[16], const uint64_t inv2, const uint64_t scale2,
+                                             uint64_t (&acc2)[16], uint32_t (&words)[B], uint32_t& cur, const uint32_t q,
+                                             const uint32_t worker, const uint32_t step, const PhiloxKeys& keys)
 {
+    constexpr uint32_t s = (1u << (B - 1)) - 1u;
     uint32_t w[4];
-    philox4x32_10(q, 0u, m, step, keys, w);
-    push_code<B, 8 * C + 0>(acc, cur, encode<B, 0>(lo.x, inv, w[0], ob));
-    push_code<B, 8 * C + 1>(acc, cur, encode<B, 1>(lo.y, inv, w[0], ob));
-    push_code<B, 8 * C + 2>(acc, cur, encode<B, 0>(lo.z, inv, w[1], ob));
-    push_code<B, 8 * C + 3>(acc, cur, encode<B, 1>(lo.w, inv, w[1], ob));
-    push_code<B, 8 * C + 4>(acc, cur, encode<B, 0>(hi.x, inv, w[2], ob));
-    push_code<B, 8 * C + 5>(acc, cur, encode<B, 1>(hi.y, inv, w[2], ob));
-    push_code<B, 8 * C + 6>(acc, cur, encode<B, 0>(hi.z, inv, w[3], ob));
-    push_code<B, 8 * C + 7>(acc, cur, encode<B, 1>(hi.w, inv, w[3], ob));
+    philox4x32_10(q, 0u, worker, step, keys, w);
+    uint32_t t[8], u[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint64_t pos = mul_pair_rz(x[4 * C + i], inv2);
+        uint64_t t2;
+        if constexpr (B <= 7) t2 = add_pair(pos, draw_pair(w[i], float_bits(s, 7)));
+        else t2 = add_pair_rm(add_pair_rm(pos, both(0x37000000u)), draw_pair(w[i], float_bits(0, 7)));     // 2^-17
+        if constexpr (B <= 7) split_pair(t2, t[2 * i], t[2 * i + 1]);
+        if constexpr (AVG || !PacksFromT<B>::value) {
+            // 1.5 * 2^23 + code: t carries 128 + s (b <= 7) or 128
+            constexpr uint32_t kTo = 0x4B400000u - 128u + (B <= 7 ? 0u : s);
+            const uint64_t u2 = add_pair_rm(t2, both(kTo));
+            split_pair(u2, u[2 * i], u[2 * i + 1]);
+            if constexpr (AVG) {
+                const uint64_t level = add_pair(u2, both(0xCB400000u + s));
+                acc2[4 * C + i] = fma_pair(level, scale2, acc2[4 * C + i]);
+            }
+        }
+    }
+    pack_eight<B, C>(words, cur, t, u);
+}
+
+template <int B, bool AVG>
+__device__ __forceinline__ void encode_row(const uint64_t (&x)[16], const uint64_t inv2, const uint64_t scale2,
+                                           uint64_t (&acc2)[16], uint32_t (&words)[B], const uint32_t q0, const uint32_t worker,
+                                           const uint32_t step, const PhiloxKeys& keys)
+{
+    uint32_t cur = 0;
+    encode_eight<B, 0, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 0u, worker, step, keys);
+    encode_eight<B, 1, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 1u, worker, step, keys);
+    encode_eight<B, 2, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 2u, worker, step, keys);
+    encode_eight<B, 3, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 3u, worker, step, keys);
+}
+
+// ---- global memory, 32 bytes at a time ----
+__device__ __forceinline__ void load_wide(const float* p, float (&r)[8])
+{
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void store_wide_bits(void* p, const uint32_t (&r)[8], const void* base, const int64_t extent, int32_t* status)
+{
+#ifdef DQ_CHECKED
+    if (!dq_store_allowed(p, 32, base, extent, status)) return;
+#else
+    (void)base; (void)extent; (void)status;
+#endif
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),
+                 "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void store_wide(float* p, const float (&r)[8], const void* base, const int64_t extent, int32_t* status)
+{
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __float_as_uint(r[i]);
+    store_wide_bits(p, v, base, extent, status);
+}
+
+// Words that leave straight from registers: a lane's B words start on a boundary of their own size
+// (1, 2, 4 words) or are whole 16-byte units, so neighbouring lanes fill whole sectors.  The other
+// widths go through shared memory.
+template <int B>
+struct StoresDirectly {
+    static constexpr bool value = B <= 2 || B % 4 == 0;
+};
+template <int B>
+__device__ __forceinline__ void store_words(uint32_t* dst, const uint32_t (&w)[B], const bool wide, const void* base,
+                                            const int64_t extent, int32_t* status)
+{
+    (void)wide;
+    if constexpr (B == 1) {
+        DQ_STORE(dst, w[0], base, extent, status);
+    } else if constexpr (B == 2) {
+        DQ_STORE(reinterpret_cast<uint2*>(dst), make_uint2(w[0], w[1]), base, extent, status);
+    } else {
+        if constexpr (B % 8 == 0) {
+            if (wide) {                          // 32-byte stores: whole sectors from one lane
+#pragma unroll
+                for (int i = 0; i < B / 8; ++i) {
+                    uint32_t v[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] = w[8 * i + k];
+                    store_wide_bits(dst + 8 * i, v, base, extent, status);
+                }
+                return;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < B / 4; ++i)
+            DQ_STORE(reinterpret_cast<uint4*>(dst) + i, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]), base, extent,
+                     status);
+    }
 }
 
 // Decoding for the average.  A code holds s + sgn * level.  Its B bits are

@@ -1,0 +1,679 @@
+// The quantizer kernels: one pass over the gradients that takes the bucket norms (or reads
+// them), encodes and packs (Eq. 5/6), and -- in the round kernels -- also forms the server's
+// average (Algorithm 1) from the codes while they are still in registers.
+//
+// Modes (where the norms come from):
+//   kWarpBuckets   buckets of 32 * 2^k <= 1024 elements: a warp tile is 1024 / bucket buckets
+//   kTeamBuckets   buckets of 2048 or 4096: a team of 2 or 4 warps of the CTA takes a bucket
+//   kGivenNorms    any bucket length, whole-tensor layouts: norms are read, a tile is 32 groups
+// AVG = false: codes (and norms) of every worker.  AVG = true: a warp keeps its tile of the output
+// while it goes through the M workers, whose words it writes as it goes; the averaged gradient (or
+// the updated parameters) leaves at the end of the tile.
+//
+// Every WARP is a pipeline of its own: two 4 KB stages filled by TMA tensor copies with the 128-byte
+// swizzle.  A lane owns one 128-byte row (32 elements, one group): it takes the row into registers,
+// the stage is refilled at once, and norm, draws, codes and words are formed from the registers.
+// HBM traffic: 4 + b/8 bytes per element and worker, plus 4 (8 with the update) per output element.
+#pragma once
+
+#include "dq_common.cuh"
+#include "dq_device.cuh"
+#include "dq_rule.cuh"
+#include "dq_tma.cuh"
+
+enum RoundMode { kWarpBuckets = 0, kTeamBuckets = 1, kGivenNorms = 2 };
+
+struct RoundArgs {
+    LayoutView v;
+    float* norms;                 // written, or read (kGivenNorms)
+    int32_t* dev_b;               // b of this call; with the rule attached, the next b when the kernel ends
+    uint32_t* packed;
+    int64_t packed_stride;
+    float* out;                   // AVG: averaged gradient, or the parameters (update != 0)
+    int32_t* status;
+    PhiloxKeys keys;
+    uint32_t step;
+    uint32_t worker0;             // worker m of the call draws the uniforms of worker worker0 + m
+    int32_t M;
+    int32_t map_has_worker_dim;   // 0 when all workers read the same buffer (stride 0)
+    int32_t gpb_shift;            // log2(groups per bucket), computed norms only
+    uint32_t div_magic;           // kGivenNorms: groups_per_bucket as multiply-shift, or as a shift if a power of two
+    int32_t div_shift;            //              (>= 0: the shift; < 0: use div_magic with a 33-bit shift)
+    int32_t stream_reads;         // 1: the gradients exceed the L2, read them with the evict-first policy
+    int32_t linf;                 // norm kind
+    int32_t update;               // AVG: out <- out + neg_lr * average instead of out <- average
+    int32_t wide_words;           // packed rows start on 32-byte boundaries: 32-byte stores allowed
+    int32_t wide_out;             // out starts on a 32-byte boundary
+    uint32_t each, extra;         // list entries per warp (or team): `each`, one more for the first `extra` of them
+    float neg_lr;
+    int32_t with_rule;            // AVG: choose the next b from this call's norms (dev_b, in place)
+    RuleArgs rule;
+    WaitLimits wait;
+};
+
+// Launch of one of the six kernels (each in a translation unit of its own).
+template <int MODE, bool AVG>
+int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t tiles, cudaStream_t st);
+
+// Registers: 128 per thread (4 CTAs) hold a row, its 32 sums and the generator's state; without the
+// sums five CTAs fit.
+template <bool AVG>
+struct RoundShape {
+    static constexpr int ctas_per_sm = AVG ? 4 : 5;
+};
+
+constexpr int kRoundThreads = 128;
+constexpr int kRoundWarps = kRoundThreads / 32;
+
+#ifdef DQ_ROUND_KERNELS
+
+namespace {
+
+constexpr int kStages = 2;
+constexpr int kTileBytes = 32 * 128;
+constexpr int kStagingBytes = 15 * 128 + 128;        // 32 * 15 words in the 16-byte phase of the stream, rounded up
+constexpr int kMaxSmemSegs = 1023;
+
+// Dynamic shared memory, addressed only through this symbol so that every access compiles to a
+// shared-memory instruction:
+//   [0, kWarps * kStages * 4 KB)  input tiles, warp-major (1024-byte aligned for the swizzle)
+//   then a staging area per warp for words that do not leave straight from registers, the stage
+//   barriers, the teams' exchange slots, the rule's partial sums, and the tensor table
+extern __shared__ __align__(1024) unsigned char smem[];
+constexpr int kStagingOffset = kRoundWarps * kStages * kTileBytes;
+constexpr int kBarOffset = kStagingOffset + kRoundWarps * kStagingBytes;
+constexpr int kPartOffset = kBarOffset + kRoundWarps * kStages * 8;         // [2 parities][4 warps] of {partial, lost}
+constexpr int kSumOffset = kPartOffset + 2 * kRoundWarps * 8;                // 4 doubles + the last-CTA word
+constexpr int kTblOffset = kSumOffset + kRoundWarps * 8 + 16;
+
+__device__ __forceinline__ uint64_t* stage_bar(int warp, int st)
+{
+    return reinterpret_cast<uint64_t*>(smem + kBarOffset) + warp * kStages + st;
+}
+__device__ __forceinline__ unsigned char* stage_ptr(int warp, int st) { return smem + (warp * kStages + st) * kTileBytes; }
+
+__device__ __forceinline__ uint32_t div_gpb(const RoundArgs& a, uint32_t n)
+{
+    if (a.div_shift >= 0) return n >> a.div_shift;
+    return (uint32_t)(((uint64_t)n * a.div_magic) >> 33);     // exact for n < 2^26, divisor <= 128
+}
+
+// A norm load that stays where it is written (a volatile statement keeps its place among the other
+// volatile statements, the barrier wait among them): the next worker's norm is requested before this
+// one's encoding, not after it.
+__device__ __forceinline__ float load_norm_early(const float* p)
+{
+    float x;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    return x;
+}
+
+__device__ __forceinline__ void load_quad(const uint32_t offset, uint64_t& lo, uint64_t& hi)
+{
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(smem + offset);
+    lo = t.x; hi = t.y;
+}
+
+// What a warp knows about a tile position: where it starts and what this lane's share of it is.
+struct TilePos {
+    int row0;        // first group of the tile
+    int row;         // this lane's row of the tile (its group is row0 + row)
+    int valid;       // elements of that group that count (0: nobody's row)
+    int bucket;      // its bucket
+    int span;        // groups of the tile that get words
+    bool regular;    // every lane owns its own full row
+    bool writes;     // this lane writes the norm of its bucket
+};
+
+// Bucket reductions in the order of dq_bucket_norms: four accumulators over a full row's float4
+// components (one over a tensor's last, partial row, whose tail is zero here), a pairwise join.
+__device__ __forceinline__ float row_sum_squares(const uint64_t (&x)[16], const bool regular, const int valid)
+{
+    uint64_t a01 = 0ull, a23 = 0ull;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        a01 = fma_pair(x[2 * c], x[2 * c], a01);
+        a23 = fma_pair(x[2 * c + 1], x[2 * c + 1], a23);
+    }
+    float a0, a1, a2, a3;
+    unpack_pair(a01, a0, a1);
+    unpack_pair(a23, a2, a3);
+    float sum = (a0 + a1) + (a2 + a3);
+    if (!regular) {
+        float chain = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            float u, w;
+            unpack_pair(x[q], u, w);
+            chain = fmaf(u, u, chain);
+            chain = fmaf(w, w, chain);
+        }
+        if (valid < 32) sum = chain;
+    }
+    return sum;
+}
+__device__ __forceinline__ float row_max(const uint64_t (&x)[16])
+{
+    float m0 = 0.0f, m1 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        float u, w;
+        unpack_pair(x[q], u, w);
+        m0 = max_nan(m0, fabsf(u));
+        m1 = max_nan(m1, fabsf(w));
+    }
+    return max_nan(m0, m1);
+}
+// sum of squares of the row scaled by 2^-e, same order as row_sum_squares
+__device__ __forceinline__ float row_scaled_squares(const uint64_t (&x)[16], const int valid, const int e)
+{
+    const ScaledSquares red{e};
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, chain = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        float u, w;
+        unpack_pair(x[2 * c], u, w);
+        a0 = red.take(a0, u); a1 = red.take(a1, w);
+        chain = red.take(chain, u); chain = red.take(chain, w);
+        unpack_pair(x[2 * c + 1], u, w);
+        a2 = red.take(a2, u); a3 = red.take(a3, w);
+        chain = red.take(chain, u); chain = red.take(chain, w);
+    }
+    return valid < 32 ? chain : (a0 + a1) + (a2 + a3);
+}
+
+// The 128-byte row of sums (or the update of the parameters there), straight from registers: a lane's
+// row is four whole sectors, and it happens once per tile and M workers.
+__device__ __forceinline__ void store_row(const RoundArgs& a, float* dst, const float (&r)[32], const int64_t extent)
+{
+    if (a.wide_out) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float y[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[e] = r[8 * i + e];
+            if (a.update) {
+                float p[8];
+                load_wide(dst + 8 * i, p);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) y[e] = fmaf(a.neg_lr, y[e], p[e]);
+            }
+            store_wide(dst + 8 * i, y, a.out, extent, a.status);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float4 y = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+            if (a.update) {
+                const float4 p = *reinterpret_cast<const float4*>(dst + 4 * i);
+                y = make_float4(fmaf(a.neg_lr, y.x, p.x), fmaf(a.neg_lr, y.y, p.y), fmaf(a.neg_lr, y.z, p.z),
+                                fmaf(a.neg_lr, y.w, p.w));
+            }
+            DQ_STORE(reinterpret_cast<float4*>(dst + 4 * i), y, a.out, extent, a.status);
+        }
+    }
+}
+
+template <int B, int MODE, bool AVG>
+__device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
+{
+    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
+    auto tbl = [&](int i) -> int { return (MODE != kGivenNorms || tbl_in_smem) ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
+    constexpr int s = (1 << (B - 1)) - 1;
+    const float sf = (float)s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n1 = a.v.n_seg + 1;
+    const int M = a.M;
+    const int nb = a.v.nb;
+    const int G = a.v.total_groups;
+    const int gpb = 1 << a.gpb_shift;
+    // warps of the CTA that share a bucket, and this warp's place among them
+    const int T_shift = MODE == kTeamBuckets ? a.gpb_shift - 5 : 0;
+    const int T = 1 << T_shift;
+    const int sub = warp & (T - 1);
+    const int R = MODE == kWarpBuckets ? 32 >> a.gpb_shift : 1;       // buckets per warp tile
+
+    // Tile positions of one worker; a team takes bucket `pos`, each of its warps 1024 elements of it.
+    const int positions = MODE == kWarpBuckets ? (nb + R - 1) / R : (MODE == kTeamBuckets ? nb : (G + 31) / 32);
+    // Contiguous ranges: of positions (AVG: every position goes through all workers), or of the
+    // worker-major list of all tiles.
+    // (each unit -- a warp, or a team -- takes `each` entries, the first `extra` units one more)
+    const uint32_t unit = (blockIdx.x * kRoundWarps + warp) >> T_shift;
+    const int n_pos = (int)(a.each + (unit < a.extra ? 1u : 0u));
+    const int64_t begin = (int64_t)unit * a.each + (unit < a.extra ? unit : a.extra);
+    const int m_first = (AVG || M == 1) ? 0 : (int)(begin / positions);
+    int pos = (int)(begin - (int64_t)m_first * positions);
+    const int items = AVG ? n_pos * M : n_pos;
+
+    // ---- where tiles lie.  c_*: the tensor looked at last (its first bucket or group, first group,
+    //      end of its full buckets, elements); lookups move forward or start over
+    int c_b0 = 0, c_g0 = 0, c_full_end = 0, c_seg = 0;
+    if constexpr (MODE == kWarpBuckets) c_full_end = a.v.n_seg == 1 ? (a.v.seg0_elems >> (a.gpb_shift + 5)) : 0;
+    // last tensor whose first bucket (column 1) or group (column 0) is <= x
+    auto find_seg = [&](int column, int x) -> int {
+        int lo = 0, hi = a.v.n_seg;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (tbl(column * n1 + mid) <= x) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    // first group of the tile at position p, bit 31 set if the tile is regular by its place alone
+    auto first_group = [&](int p) -> uint32_t {
+        if constexpr (MODE == kWarpBuckets) {
+            const int k0 = p * R;
+            if (k0 < c_b0 || k0 + R > c_full_end) {
+                if (a.v.n_seg > 1) {
+                    const int i = find_seg(1, k0);
+                    c_b0 = tbl(n1 + i);
+                    c_g0 = tbl(i);
+                    c_full_end = c_b0 + (tbl(2 * n1 + i) >> (a.gpb_shift + 5));
+                }
+            }
+            return (uint32_t)(c_g0 + ((k0 - c_b0) << a.gpb_shift)) | ((k0 + R <= c_full_end) ? 0x80000000u : 0u);
+        } else if constexpr (MODE == kTeamBuckets) {
+            // one bucket: its first group plus this warp's 32 groups; regular if the warp's 1024 elements exist;
+            // bits 30..: 0 elements are reported by an all-ones value
+            int local = p, n = a.v.seg0_elems, g0 = 0;
+            if (a.v.n_seg > 1) {
+                if (p < tbl(n1 + c_seg) || p >= tbl(n1 + c_seg + 1)) c_seg = find_seg(1, p);
+                local = p - tbl(n1 + c_seg);
+                n = tbl(2 * n1 + c_seg);
+                g0 = tbl(c_seg);
+            }
+            const int left = n - ((local << T_shift) + sub) * 1024;
+            if (left <= 0) return 0x7fffffffu;                   // the bucket ends before this warp's share
+            return (uint32_t)(g0 + ((local << T_shift) + sub) * 32) | (left >= 1024 ? 0x80000000u : 0u);
+        } else {
+            return (uint32_t)(p * 32);
+        }
+    };
+    constexpr uint32_t kNoTile = 0x7fffffffu;
+    auto locate = [&](int p) -> TilePos {
+        TilePos t;
+        t.row = lane; t.valid = 32; t.span = 32; t.bucket = 0; t.writes = false;
+        const uint32_t d = first_group(p);
+        t.row0 = (int)(d & 0x7fffffffu);
+        t.regular = (d >> 31) != 0;
+        if constexpr (MODE == kWarpBuckets) {
+            const int r = lane >> a.gpb_shift, l = lane & (gpb - 1);
+            const int k = p * R + r;
+            t.bucket = k;
+            t.writes = l == 0 && k < nb;
+            if (!t.regular) {
+                // the tile touches the end of a tensor: buckets may be short, rows may be nobody's
+                int first = 0, len = 0;
+                if (k < nb) {
+                    int local = k, n = a.v.seg0_elems, g0 = 0;
+                    if (a.v.n_seg > 1) {
+                        const int i = find_seg(1, k);
+                        local = k - tbl(n1 + i);
+                        n = tbl(2 * n1 + i);
+                        g0 = tbl(i);
+                    }
+                    first = g0 + (local << a.gpb_shift);
+                    const int left = n - local * (gpb * 32);
+                    len = left < gpb * 32 ? left : gpb * 32;
+                }
+                t.row = first - t.row0 + l;
+                const int v = len - l * 32;
+                t.valid = v < 0 ? 0 : (v > 32 ? 32 : v);
+                if (t.valid == 0) t.row = lane;
+                t.span = __reduce_max_sync(0xffffffffu, t.valid > 0 ? t.row + 1 : 0);
+            }
+        } else if constexpr (MODE == kTeamBuckets) {
+            t.bucket = p;
+            t.writes = sub == 0 && lane == 0;
+            if (!t.regular) {
+                if (d == kNoTile) {
+                    t.row0 = -1; t.valid = 0; t.span = 0;
+                } else {
+                    int local = p, n = a.v.seg0_elems;
+                    if (a.v.n_seg > 1) { local = p - tbl(n1 + c_seg); n = tbl(2 * n1 + c_seg); }
+                    const int v = n - ((local << T_shift) + sub) * 1024 - lane * 32;
+                    t.valid = v < 0 ? 0 : (v > 32 ? 32 : v);
+                    t.span = __reduce_max_sync(0xffffffffu, t.valid > 0 ? lane + 1 : 0);
+                }
+            }
+        } else {
+            const int g = t.row0 + lane;
+            t.valid = 0;
+            if (g < G) {
+                int local = g, n = a.v.seg0_elems, b0 = 0;
+                if (a.v.n_seg > 1) {
+                    if (g < tbl(c_seg)) c_seg = 0;
+                    if (c_seg == 0) c_seg = find_seg(0, g);
+                    while (g >= tbl(c_seg + 1)) ++c_seg;
+                    local = g - tbl(c_seg);
+                    b0 = tbl(n1 + c_seg);
+                    n = tbl(2 * n1 + c_seg);
+                }
+                const int k = (int)div_gpb(a, (uint32_t)local);
+                t.bucket = b0 + k;
+                t.writes = local == k * a.v.groups_per_bucket;       // (the lane that accounts for the bucket's norm)
+                const int left = n - local * 32;
+                t.valid = left < 32 ? left : 32;
+            }
+            t.regular = __all_sync(0xffffffffu, t.valid == 32);
+            t.span = (G - t.row0) < 32 ? (G - t.row0) : 32;
+        }
+        return t;
+    };
+
+    // ---- producer side: tiles are fetched in the order they are consumed, two ahead
+    int p_pos = pos, p_m = m_first, p_left = items;
+    uint32_t p_first = items > 0 ? first_group(p_pos) : kNoTile;
+    const uint64_t policy = tma::policy_evict_first();
+    // Copies in flight.  A team's warp has no tile of some buckets, so it counts the copies that landed
+    // in each stage; the others find a stage's parity in the item's number.
+    bool flying0 = false, flying1 = false;
+    uint32_t fills0 = 0, fills1 = 0;
+    auto stage_parity = [&](uint32_t item) -> uint32_t {
+        if constexpr (MODE == kTeamBuckets) return ((item & 1u) ? fills1 : fills0) & 1u;
+        else return (item >> 1) & 1u;
+    };
+    auto seen_to_land = [&](int st) {
+        if constexpr (MODE == kTeamBuckets) {
+            if (st) { ++fills1; flying1 = false; } else { ++fills0; flying0 = false; }
+        }
+    };
+    auto fetch = [&](int st) {
+        if (p_left <= 0) return;
+        --p_left;
+        if (MODE == kTeamBuckets && p_first != kNoTile) { if (st) flying1 = true; else flying0 = true; }
+        if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile)) {
+            const int row0 = (int)(p_first & 0x7fffffffu);
+            uint64_t* bar = stage_bar(warp, st);
+            tma::mbar_expect_tx(bar, kTileBytes);
+            if (a.stream_reads)
+                tma::load_tile_3d_hint(stage_ptr(warp, st), map, bar, 0, row0, a.map_has_worker_dim ? p_m : 0, policy);
+            else
+                tma::load_tile_3d(stage_ptr(warp, st), map, bar, 0, row0, a.map_has_worker_dim ? p_m : 0);
+        }
+        if (AVG) {
+            if (++p_m == M) { p_m = 0; ++p_pos; if (p_left > 0) p_first = first_group(p_pos); }
+        } else {
+            if (++p_pos == positions) { p_pos = 0; ++p_m; }
+            if (p_left > 0) p_first = first_group(p_pos);
+        }
+    };
+#pragma unroll
+    for (int st = 0; st < kStages; ++st) fetch(st);
+
+    const float to_unit = (B == 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
+    uint32_t it = 0;                              // items consumed; item i travels through stage i & 1
+    uint32_t exchanges = 0;
+    bool timed_out = false, bad = false;
+    // (test hook: the warp's first wait counts as lost, and the warp goes straight to what follows a time-out)
+    const bool skip_all = a.wait.lose_first != 0u && items > 0;
+    int m = m_first;
+
+    for (int ip = 0; ip < n_pos && !skip_all; ++ip) {
+        const TilePos t = locate(pos);
+        const bool has_tile = MODE != kTeamBuckets || t.row0 >= 0;
+        // byte offset of the lane's row inside a stage, swizzle phase folded in: chunk c sits at own ^ (c << 4)
+        const uint32_t own = (uint32_t)(t.row * 128 + ((t.row & 7) << 4));
+        const uint32_t q0 = (uint32_t)(t.row0 + t.row) * 4u;
+        uint64_t acc2[16];
+        if constexpr (AVG) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
+        }
+        float norm_next = 0.0f;
+        if constexpr (MODE == kGivenNorms) {
+            if (t.valid > 0) norm_next = load_norm_early(a.norms + (int64_t)m * nb + t.bucket);
+        }
+
+        const int workers = AVG ? M : 1;
+#pragma unroll 1
+        for (int j = 0; j < workers; ++j) {
+            const int mm = AVG ? j : m;
+            const int st = it & 1;
+            bool landed = true;
+            if (has_tile) {
+                // every lane polls the barrier itself; the verdict is made warp-uniform so that the
+                // warp-level synchronisations below are always reached by all lanes or by none
+                landed = __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), stage_parity(it), a.wait));
+                if (landed) seen_to_land(st);
+            }
+            if (MODE != kTeamBuckets && !landed) { timed_out = true; break; }
+
+            // ---- the row, in registers; the stage is free again
+            uint64_t x[16];
+            {
+                const uint32_t base = (uint32_t)((warp * kStages + st) * kTileBytes) + own;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) load_quad(base ^ (uint32_t)(c << 4), x[2 * c], x[2 * c + 1]);
+            }
+            if (!t.regular) {                    // what follows a tensor's end is padding, whatever it holds
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    float u, w;
+                    unpack_pair(x[q], u, w);
+                    x[q] = pack_pair(2 * q < t.valid ? __float_as_uint(u) : 0u, 2 * q + 1 < t.valid ? __float_as_uint(w) : 0u);
+                }
+            }
+            __syncwarp();
+            if (MODE != kTeamBuckets || landed) fetch(st);
+            ++it;
+
+            // ---- norm of the bucket
+            float nrm;
+            bool maybe_zero = true;              // some bucket of the tile may be all zeros
+            if constexpr (MODE == kGivenNorms) {
+                nrm = norm_next;
+                if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(a.norms + (int64_t)(mm + 1) * nb + t.bucket);
+                if (AVG && a.with_rule && t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
+            } else {
+                // combines the lanes (and the team's warps) of a bucket; false if a team mate's wait ran out
+                auto join_lanes = [&](float v, auto op) -> float {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const float other = __shfl_xor_sync(0xffffffffu, v, o);
+                        if (MODE == kTeamBuckets || o < gpb) v = op(v, other);
+                    }
+                    return v;
+                };
+                bool team_lost = false;
+                auto join_team = [&](float v, auto op) -> float {
+                    if constexpr (MODE == kTeamBuckets) {
+                        float2* slots = reinterpret_cast<float2*>(smem + kPartOffset) + (exchanges & 1u) * kRoundWarps;
+                        ++exchanges;
+                        if (lane == 0) slots[warp] = make_float2(v, landed ? 0.0f : 1.0f);
+                        asm volatile("bar.sync %0, %1;" ::"r"(1 + (warp >> T_shift)), "r"(32 << T_shift) : "memory");
+                        const float2* mine = slots + (warp & ~(T - 1));
+                        float r = op(0.0f, mine[0].x), lost = mine[0].y;
+                        for (int i = 1; i < T; ++i) { r = op(r, mine[i].x); lost += mine[i].y; }
+                        team_lost |= lost != 0.0f;
+                        return r;
+                    } else {
+                        return v;
+                    }
+                };
+                auto add = [](float p, float q) { return p + q; };
+                auto larger = [](float p, float q) { return max_nan(p, q); };
+                if (a.linf) {
+                    nrm = join_team(join_lanes(row_max(x), larger), larger);
+                } else {
+                    const float sum = join_team(join_lanes(row_sum_squares(x, t.regular, t.valid), add), add);
+                    nrm = sqrtf(sum);
+                    // Rarely a bucket's sum of squares is out of range (see l2_sum_in_range): all zeros, tiny
+                    // entries, an overflowed square.  Zero buckets are settled by their largest magnitude; the
+                    // others are reduced again with their entries scaled.
+                    maybe_zero = __any_sync(0xffffffffu, !l2_sum_in_range(sum));
+                    if (maybe_zero && !team_lost) {
+                        const float mx = join_team(join_lanes(row_max(x), larger), larger);
+                        float again = mx;
+                        if (__any_sync(0xffffffffu, !l2_sum_in_range(sum) && magnitude_scalable(mx))) {
+                            const int e = scale_exponent(mx);
+                            again = rescaled_l2(mx, join_team(join_lanes(row_scaled_squares(x, t.valid, e), add), add), e);
+                        }
+                        if (!l2_sum_in_range(sum)) nrm = again;
+                    }
+                }
+                if (team_lost) { timed_out = true; break; }
+                if (t.writes) {
+                    DQ_STORE(a.norms + ((int64_t)mm * nb + t.bucket), nrm, a.norms, (int64_t)M * nb * 4, a.status);
+                    bad |= !isfinite(nrm);
+                    if (AVG && a.with_rule) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                }
+            }
+            if (!has_tile) continue;
+
+            // ---- codes of the row against that norm, and the lane's share of the average
+            uint32_t words[B];
+            const float inv = inv_scale(sf, nrm);
+            if constexpr (B == 1) {
+                words[0] = 0u;
+            } else if (maybe_zero && __all_sync(0xffffffffu, nrm == 0.0f)) {
+                // sparse gradients are full of zero buckets: every code is s, whatever the draw, and adds 0 to the average
+                zero_group_words<B>(words);
+            } else {
+                const uint64_t inv2 = pack_pair(__float_as_uint(inv), __float_as_uint(inv));
+                const float scale = nrm * to_unit;
+                const uint64_t scale2 = pack_pair(__float_as_uint(scale), __float_as_uint(scale));
+                encode_row<B, AVG>(x, inv2, scale2, acc2, words, q0, (uint32_t)mm + a.worker0, a.step, a.keys);
+            }
+
+            // ---- words out
+            uint32_t* const row_dst = a.packed + (int64_t)mm * a.packed_stride + (int64_t)t.row0 * B;
+            const int64_t extent = (int64_t)M * a.packed_stride * 4;
+            if constexpr (StoresDirectly<B>::value) {
+                // a lane's words are whole 4-, 8- or 16-byte units of the stream: neighbouring lanes fill sectors
+                if (t.valid > 0)
+                    store_words<B>(row_dst + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
+            } else {
+                uint32_t* out_words = reinterpret_cast<uint32_t*>(smem + kStagingOffset + warp * kStagingBytes);
+                // the staging area keeps the 16-byte phase of the output stream; whole quads move 16 bytes per
+                // lane, the ragged ends word by word
+                const int off = (int)(((int64_t)t.row0 * B) & 3);
+                uint32_t* aligned_dst = row_dst - off;
+                if (t.valid > 0) {
+#pragma unroll
+                    for (int i = 0; i < B; ++i) out_words[off + t.row * B + i] = words[i];
+                }
+                __syncwarp();
+                const int jend = off + t.span * B;
+                const int f0 = off ? 1 : 0, f1 = jend >> 2;          // full quads [f0, f1)
+#pragma unroll
+                for (int i = 0; i < (8 * B + 31) / 32; ++i) {
+                    const int q = lane + 32 * i;
+                    if (q >= f0 && q < f1)
+                        DQ_STORE(reinterpret_cast<uint4*>(aligned_dst) + q, reinterpret_cast<const uint4*>(out_words)[q],
+                                 a.packed, extent, a.status);
+                }
+                if (off | (jend & 3)) {
+                    if (off && lane >= off && lane < 4 && lane < jend)                                        // head
+                        DQ_STORE(aligned_dst + lane, out_words[lane], a.packed, extent, a.status);
+                    int ts = f1 * 4;                                                                          // tail
+                    if (off && ts < 4) ts = 4;
+                    if (lane < jend - ts) DQ_STORE(aligned_dst + (ts + lane), out_words[ts + lane], a.packed, extent, a.status);
+                }
+                __syncwarp();
+            }
+        }
+        if (timed_out) break;
+
+        if constexpr (AVG) {
+            if (t.valid > 0 && has_tile && !(B == 1 && a.update)) {
+                float r[32];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], r[2 * q], r[2 * q + 1]);
+                if (!t.regular) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (e >= t.valid) r[e] = 0.0f;
+                }
+                store_row(a, a.out + ((int64_t)t.row0 + t.row) * 32, r, (int64_t)G * 128);
+            }
+            ++pos;
+        } else {
+            if (++pos == positions) { pos = 0; ++m; }
+        }
+    }
+    if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
+    if (timed_out || skip_all) {
+        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
+        // every copy the warp has issued and not seen land, the one whose wait ran out included, gets the
+        // full limit before the CTA's shared memory is released
+        if constexpr (MODE == kTeamBuckets) {
+            if (flying0) (void)tma::mbar_wait(stage_bar(warp, 0), fills0 & 1u, a.wait);
+            if (flying1) (void)tma::mbar_wait(stage_bar(warp, 1), fills1 & 1u, a.wait);
+        } else {
+            for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
+                (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), stage_parity(i), a.wait);
+        }
+    }
+}
+
+template <int MODE, bool AVG>
+__global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
+round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+{
+    // (nothing up to the wait touches memory that an earlier kernel may still be writing)
+    if (threadIdx.x == 0) {
+        tma::prefetch_tensor_map(&map);
+        for (int i = 0; i < kRoundWarps * kStages; ++i) tma::mbar_init(stage_bar(0, i), 1);
+        tma::fence_barrier_init();
+    }
+    grid_dependency_wait();
+    const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
+    const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
+    if (tbl_in_smem) {
+        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + kTblOffset);
+        for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
+    }
+    __syncthreads();
+    uint32_t trouble = 0;
+    if (tma::smem_addr(smem) & 1023u) trouble = DQ_STAT_INTERNAL;          // the swizzled tiles need a 1024-byte aligned base
+    else if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
+    else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
+    if (trouble) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
+        // nothing is written but the next b, which follows from the norms that are there
+        if (AVG && a.with_rule && blockIdx.x == 0)
+            rule_from_norms<kRoundThreads>(a.rule, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + kSumOffset),
+                                           a.dev_b, a.status);
+        return;
+    }
+
+    double square_sum = 0.0;
+    switch (b) {
+#define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG>(a, &map, tbl_in_smem, square_sum); break;
+#ifdef DQ_ONLY_B
+        DQ_CASE(DQ_ONLY_B)
+#else
+        DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
+        DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
+#endif
+#undef DQ_CASE
+        default: break;
+    }
+    if (AVG && a.with_rule)
+        rule_from_partials<kRoundThreads>(a.rule, square_sum, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, a.status);
+}
+
+}  // namespace
+
+template <int MODE, bool AVG>
+int dq_launch_round(const RoundArgs& args, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+{
+    RoundArgs a = args;
+    const auto kernel = round_kernel<MODE, AVG>;
+    size_t smem_need = (size_t)kTblOffset;
+    if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return DQ_ERR_CUDA;
+    }
+    // units of work per CTA: warps, or teams
+    const int units = MODE == kTeamBuckets ? kRoundWarps >> (a.gpb_shift - 5) : kRoundWarps;
+    int64_t blocks = (int64_t)dq_sm_count() * RoundShape<AVG>::ctas_per_sm;
+    if (blocks * units > entries) blocks = (entries + units - 1) / units;
+    a.each = (uint32_t)(entries / (blocks * units));
+    a.extra = (uint32_t)(entries - (int64_t)a.each * blocks * units);
+    dq_launch(kernel, dim3((unsigned)blocks), dim3(kRoundThreads), smem_need, st, a, map);
+    return cudaGetLastError() == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+}
+
+#endif  // DQ_ROUND_KERNELS

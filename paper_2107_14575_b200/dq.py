@@ -28,7 +28,7 @@ SYMBOLS = [
     "dq_bucket_norms", "dq_tensor_norms_scratch_bytes", "dq_tensor_norms", "dq_choose_bits_scratch_bytes", "dq_choose_bits",
     "dq_choose_bits_noalloc_max_norms", "dq_choose_bits_noalloc",
     "dq_quantize_pack", "dq_quantize_pack_worker", "dq_norms_quantize_pack", "dq_norms_quantize_pack_worker", "dq_unpack_dequant_average",
-    "dq_unpack_average_update", "dq_status_string", "dq_debug_set_wait_limits",
+    "dq_unpack_average_update", "dq_quantize_average", "dq_round_workspace_bytes", "dq_norms_quantize_average", "dq_status_string", "dq_debug_set_wait_limits",
 ]
 
 
@@ -121,6 +121,13 @@ def lib():
         L.dq_unpack_dequant_average.argtypes = [vp, vp, i64, vp, i32, vp, vp, vp, vp]
         L.dq_unpack_average_update.restype = C.c_int
         L.dq_unpack_average_update.argtypes = [vp, vp, i64, vp, i32, vp, C.c_float, vp, vp, vp]
+        L.dq_quantize_average.restype = C.c_int
+        L.dq_quantize_average.argtypes = [vp, vp, i64, i32, vp, vp, u64, u32, vp, i64, vp, i32, C.c_float, vp, vp]
+        L.dq_round_workspace_bytes.restype = sz
+        L.dq_round_workspace_bytes.argtypes = [vp, i32]
+        L.dq_norms_quantize_average.restype = C.c_int
+        L.dq_norms_quantize_average.argtypes = [vp, vp, i64, i32, vp, u64, u32, vp, vp, i64, vp, i32, C.c_float,
+                                                C.POINTER(Rule), vp, sz, vp, vp]
         L.dq_status_string.restype = C.c_char_p
         L.dq_status_string.argtypes = [C.c_int]
         L.dq_debug_set_wait_limits.restype = None
@@ -318,3 +325,32 @@ def unpack_average_update(layout: Layout, packed, packed_stride_words: int, norm
     _check(lib().dq_unpack_average_update(layout.handle, _ptr(packed), int(packed_stride_words), _ptr(norms),
                                           int(M), _ptr(dev_b), float(lr), _ptr(params), _ptr(status),
                                           _stream(stream)), "dq_unpack_average_update")
+
+
+def quantize_average(layout: Layout, grads, worker_stride_elems: int, M: int, norms, dev_b, seed: int, step: int,
+                     packed, packed_stride_words: int, out, status, lr: Optional[float] = None, stream=None) -> None:
+    """Codes for the given norms and the average of all workers in one pass (``dq_quantize_average``);
+    with ``lr`` the average is applied to the parameters in ``out`` instead of stored there."""
+    _check(lib().dq_quantize_average(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
+                                     _ptr(dev_b), int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(packed),
+                                     int(packed_stride_words), _ptr(out), 0 if lr is None else 1,
+                                     0.0 if lr is None else float(lr), _ptr(status), _stream(stream)),
+           "dq_quantize_average")
+
+
+def round_workspace_bytes(layout: Layout, M: int) -> int:
+    return int(lib().dq_round_workspace_bytes(layout.handle, int(M)))
+
+
+def norms_quantize_average(layout: Layout, grads, worker_stride_elems: int, M: int, dev_b, seed: int, step: int, norms,
+                           packed, packed_stride_words: int, out, next_rule: Rule, workspace, workspace_bytes: int, status,
+                           lr: Optional[float] = None, stream=None) -> None:
+    """A whole round in Algorithm 1's order (``dq_norms_quantize_average``): ``dev_b`` holds this round's b and then
+    the next one; with ``lr`` the average is applied to the parameters in ``out`` instead of stored there.
+    ``workspace`` is zeroed once by its owner."""
+    _check(lib().dq_norms_quantize_average(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(dev_b),
+                                           int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(norms), _ptr(packed),
+                                           int(packed_stride_words), _ptr(out), 0 if lr is None else 1,
+                                           0.0 if lr is None else float(lr), C.byref(next_rule), _ptr(workspace),
+                                           int(workspace_bytes), _ptr(status), _stream(stream)),
+           "dq_norms_quantize_average")

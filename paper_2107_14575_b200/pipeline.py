@@ -40,6 +40,9 @@ class Round:
         self.norm_scratch_bytes = dq.tensor_norms_scratch_bytes(L, M)
         self.norm_scratch = (torch.empty(self.norm_scratch_bytes, dtype=torch.uint8, device=self.device)
                              if self.norm_scratch_bytes else None)
+        # of the one-call round: zeroed once, kept in order by the calls
+        self._ws_bytes = dq.round_workspace_bytes(L, M)
+        self._ws = torch.zeros(self._ws_bytes, dtype=torch.uint8, device=self.device)
         self._host_in = None
         self._host_out = None
         self._dev_in = None
@@ -88,8 +91,8 @@ class Round:
         """Whole round on device gradients; returns the averaged gradient [D32] (device)."""
         self.norms_(grads)
         self.bits_(rule)
-        self.quantize_(grads, seed, step)
-        self.average_()
+        dq.quantize_average(self.layout, grads, self.stride, self.M, self.norms, self.dev_b, seed, step, self.packed,
+                            self.packed_stride, self.out, self.status)
         return self.out
 
     # below this many norms the bit rule takes a few microseconds and the hand-over between two
@@ -115,6 +118,12 @@ class Round:
         update of Eq. 2, ``params <- params - lr * average``, in the same kernel; ``out`` is
         then not written and ``params`` is returned.
         """
+        if events is None:
+            dq.norms_quantize_average(self.layout, grads, self.stride, self.M, self.dev_b, seed, step, self.norms, self.packed,
+                                      self.packed_stride, self.out if params is None else params, next_rule, self._ws,
+                                      self._ws_bytes, self.status, None if params is None else lr)
+            return self.out if params is None else params
+
         def server_step():
             if params is None:
                 self.average_()

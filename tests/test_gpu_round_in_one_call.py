@@ -1,0 +1,116 @@
+"""``dq_norms_quantize_average`` and ``dq_quantize_average`` against the calls they merge.
+
+Words, norms and the average (or the updated parameters) of the one-pass kernels equal those of
+dq_norms_quantize_pack / dq_bucket_norms / dq_tensor_norms, dq_quantize_pack and
+dq_unpack_dequant_average / dq_unpack_average_update bit for bit: same operations, same order over
+the workers.  The next b is the rule's (threshold search on sums that differ by 1e-15).
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+SEED = 0x0DD_5EED_71
+# tensors shorter than a bucket, on and beside the edges of groups and warp tiles, an empty one
+RAGGED = [70, 1, 1023, 1024, 1025, 0, 4097, 31, 2048, 3 * 4096 + 77, 32, 9000]
+
+
+@pytest.fixture(scope="module")
+def G(dqlib):
+    if not torch.cuda.is_available():
+        pytest.fail("the gpu tests need a CUDA device")
+    import gpu_util
+    return gpu_util
+
+
+def _grads(ref, segs, M, seed):
+    """Normal values of very different scales, a tensor of zeros, a bucket of tiny entries, NaN in the padding."""
+    rng = np.random.default_rng(seed)
+    g = np.full((M, ref.D32), np.nan, np.float32)
+    for i, (o, n) in enumerate(zip(ref.offsets, segs)):
+        g[:, o: o + n] = rng.standard_normal((M, n)).astype(np.float32) * np.float32(10.0 ** (i % 5 - 2))
+    if len(segs) > 8:
+        g[:, ref.offsets[8]: ref.offsets[8] + segs[8]] = 0.0
+        g[0, ref.offsets[4]: ref.offsets[4] + segs[4]] *= np.float32(1e-30)
+    return g
+
+
+CASES = [(RAGGED, 512, 3, 4), (RAGGED, 32, 2, 7), (RAGGED, 1024, 5, 3), (RAGGED, 2048, 3, 5), (RAGGED, 4096, 2, 8),
+         (RAGGED, 96, 2, 6), (RAGGED, 0, 3, 4), ([1 << 18], 512, 4, 2), ([70001], 128, 1, 16), ([1], 4096, 2, 4),
+         ([33] * 1100, 64, 2, 12), ([300000], 2048, 33, 4)] + [(RAGGED, 256, 2, b) for b in range(1, 17)]
+
+
+@pytest.mark.parametrize("segs,bucket,M,b", CASES)
+def test_one_call_equals_the_calls_it_merges(G, segs, bucket, M, b):
+    dq = G.dq
+    for norm in ((dq.NORM_L2, dq.NORM_LINF) if b in (4, 5) else (dq.NORM_L2,)):
+        r = G.GpuRound(segs, bucket, M, norm=norm, packed_stride=None)
+        ref = oracle.Layout(segs, bucket if bucket else oracle.whole_tensor_bucket(segs))
+        g = _grads(ref, segs, M, 17 * M + b)
+        r.set_grads(g)
+        r.set_b(b)
+        rule = dq.Rule.dynamic(10, 3, 0.37 * 10 * max(1e-30, float(np.nansum(g.astype(np.float64) ** 2)) / M) / 400.0, 0.9)
+        # the separate calls
+        norms = r.norms().copy()
+        packed = r.quantize(SEED, 5, fill=-1).copy()
+        avg = r.average(fill=1.0).copy()
+        x0 = np.linspace(-1, 1, r.lay.D32, dtype=np.float32)
+        upd = r.update(0.125, x0).copy()
+        want_b = r.bits(rule)
+        # one call with the norms given, one with everything; the average and the update; two runs in a row
+        nbytes = dq.round_workspace_bytes(r.lay, M)
+        ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+        for whole in (False, True, True):
+            for lr, want in ((None, avg), (0.125, upd)):
+                r.set_b(b)
+                r.g_packed.view.fill_(-1)
+                r.g_out.view.copy_(torch.from_numpy(x0))
+                if whole:
+                    r.g_norms.view.fill_(-1.0)
+                    dq.norms_quantize_average(r.lay, r.grads, r.stride, M, r.g_b.view, SEED, 5, r.g_norms.view, r.g_packed.view,
+                                              r.pstride, r.g_out.view, rule, ws, nbytes, r.status, lr=lr)
+                    assert tuple(r.g_b.view.cpu().tolist()) == want_b
+                else:
+                    dq.quantize_average(r.lay, r.grads, r.stride, M, r.g_norms.view, r.g_b.view, SEED, 5, r.g_packed.view,
+                                        r.pstride, r.g_out.view, r.status, lr=lr)
+                np.testing.assert_array_equal(r.g_norms.view.cpu().numpy().reshape(M, -1), norms)
+                np.testing.assert_array_equal(r.g_packed.view.cpu().numpy().view(np.uint32).reshape(M, -1), packed)
+                np.testing.assert_array_equal(r.g_out.view.cpu().numpy(), want)
+        assert r.read_status() == 0 and r.guards_intact()
+        nw = ref.packed_words(b)
+        np.testing.assert_array_equal(packed[:, :nw], oracle.quantize_pack(ref, np.nan_to_num(g), norms, b, SEED, 5))
+
+
+def test_lost_first_wait_and_bad_bits(G):
+    """A lost wait raises DQ_STAT_WAIT and nothing else; a b outside 1..16 writes no output but still gets its successor."""
+    dq = G.dq
+    for bucket in (512, 4096, 96):
+        r = G.GpuRound(RAGGED, bucket, 3)
+        ref = oracle.Layout(RAGGED, bucket)
+        r.set_grads(np.nan_to_num(_grads(ref, RAGGED, 3, 1)))
+        nbytes = dq.round_workspace_bytes(r.lay, 3)
+        ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+
+        def call():
+            dq.norms_quantize_average(r.lay, r.grads, r.stride, 3, r.g_b.view, SEED, 0, r.g_norms.view, r.g_packed.view, r.pstride,
+                                      r.g_out.view, dq.Rule.fixed(6), ws, nbytes, r.status)
+            torch.cuda.synchronize()
+        r.set_b(4)
+        try:
+            dq.debug_set_wait_limits(50_000_000, True)
+            call()
+        finally:
+            dq.debug_set_wait_limits()
+        assert r.read_status() == dq.STAT_WAIT and r.guards_intact()
+        r.clear_status()
+        r.g_packed.view.fill_(-7)
+        r.set_b(17)
+        call()
+        assert r.read_status() == dq.STAT_BAD_BITS and bool((r.g_packed.view == -7).all())
+        assert r.g_b.view.tolist() == [6, 31]
+        r.clear_status()
+        call()
+        assert r.read_status() == 0 and r.guards_intact() and not bool((r.g_packed.view == -7).all())
