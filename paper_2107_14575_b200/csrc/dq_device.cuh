@@ -190,16 +190,28 @@ __host__ __device__ constexpr uint32_t float_bits(const uint32_t n, const int p)
 // before its rounding, i.e. to one of the two floats that enclose s / norm; the sign of the
 // exactly rounded residual s - q * norm then tells which, and the upper one steps down an ulp.
 // Norms above 2^125, whose reciprocal estimate would be flushed to zero, take the library route.
-__device__ __forceinline__ float inv_scale(const float sf, const float norm)
+__device__ __forceinline__ float inv_scale_normal(const float sf, const float norm)      // 2^-100 <= norm <= 2^125
 {
-    if (!(norm >= 0x1p-100f)) return 0.0f;
-    if (norm > 0x1p125f) return __fdiv_rz(sf, norm);
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(norm));
     float q = __fmul_rn(sf, r);
     q = __fmaf_rn(__fmaf_rn(-q, norm, sf), r, q);
     const float e = __fmaf_rn(-q, norm, sf);
     return __uint_as_float(__float_as_uint(q) - (e < 0.0f ? 1u : 0u));
+}
+__device__ __forceinline__ float inv_scale(const float sf, const float norm)
+{
+    if (!(norm >= 0x1p-100f)) return 0.0f;
+    if (norm > 0x1p125f) return __fdiv_rz(sf, norm);
+    return inv_scale_normal(sf, norm);
+}
+// the correctly rounded square root, for a result that counts only where the argument is in range
+// (see l2_sum_in_range): the flushing form has no subnormal arguments to take care of
+__device__ __forceinline__ float sqrt_normal(const float x)
+{
+    float r;
+    asm("sqrt.rn.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // Appends W bits at position BIT of a group's little-endian bit string of N words.  `cur` is a
@@ -330,17 +342,18 @@ __device__ __forceinline__ void pack_eight(uint32_t (&words)[B], uint32_t& cur, 
 
 // Elements 8C .. 8C + 7 (one Philox block); with AVG, level * scale is added to their sums.
 template <int B, int C, bool AVG>
-__device__ __forceinline__ void encode_eight(const uint64_t (&x)[16], const uint64_t inv2, const uint64_t scale2,
+__device__ __forceinline__ void encode_eight(const ulonglong2 lo, const ulonglong2 hi, const uint64_t inv2, const uint64_t scale2,
                                              uint64_t (&acc2)[16], uint32_t (&words)[B], uint32_t& cur, const uint32_t q,
                                              const uint32_t worker, const uint32_t step, const PhiloxKeys& keys)
 {
     constexpr uint32_t s = (1u << (B - 1)) - 1u;
     uint32_t w[4];
     philox4x32_10(q, 0u, worker, step, keys, w);
+    const uint64_t x[4] = {lo.x, lo.y, hi.x, hi.y};
     uint32_t t[8], u[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint64_t pos = mul_pair_rz(x[4 * C + i], inv2);
+        const uint64_t pos = mul_pair_rz(x[i], inv2);
         uint64_t t2;
         if constexpr (B <= 7) t2 = add_pair(pos, draw_pair(w[i], float_bits(s, 7)));
         else t2 = add_pair_rm(add_pair_rm(pos, both(0x37000000u)), draw_pair(w[i], float_bits(0, 7)));     // 2^-17
@@ -359,16 +372,17 @@ __device__ __forceinline__ void encode_eight(const uint64_t (&x)[16], const uint
     pack_eight<B, C>(words, cur, t, u);
 }
 
-template <int B, bool AVG>
-__device__ __forceinline__ void encode_row(const uint64_t (&x)[16], const uint64_t inv2, const uint64_t scale2,
+// A whole group; quad(c) gives elements 4c .. 4c + 3.
+template <int B, bool AVG, class Quads>
+__device__ __forceinline__ void encode_row(const Quads& quad, const uint64_t inv2, const uint64_t scale2,
                                            uint64_t (&acc2)[16], uint32_t (&words)[B], const uint32_t q0, const uint32_t worker,
                                            const uint32_t step, const PhiloxKeys& keys)
 {
     uint32_t cur = 0;
-    encode_eight<B, 0, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 0u, worker, step, keys);
-    encode_eight<B, 1, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 1u, worker, step, keys);
-    encode_eight<B, 2, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 2u, worker, step, keys);
-    encode_eight<B, 3, AVG>(x, inv2, scale2, acc2, words, cur, q0 + 3u, worker, step, keys);
+    encode_eight<B, 0, AVG>(quad(0), quad(1), inv2, scale2, acc2, words, cur, q0 + 0u, worker, step, keys);
+    encode_eight<B, 1, AVG>(quad(2), quad(3), inv2, scale2, acc2, words, cur, q0 + 1u, worker, step, keys);
+    encode_eight<B, 2, AVG>(quad(4), quad(5), inv2, scale2, acc2, words, cur, q0 + 2u, worker, step, keys);
+    encode_eight<B, 3, AVG>(quad(6), quad(7), inv2, scale2, acc2, words, cur, q0 + 3u, worker, step, keys);
 }
 
 // ---- global memory, 32 bytes at a time ----

@@ -11,8 +11,9 @@
 // the updated parameters) leaves at the end of the tile.
 //
 // Every WARP is a pipeline of its own: two 4 KB stages filled by TMA tensor copies with the 128-byte
-// swizzle.  A lane owns one 128-byte row (32 elements, one group): it takes the row into registers,
-// the stage is refilled at once, and norm, draws, codes and words are formed from the registers.
+// swizzle.  A lane owns one 128-byte row (32 elements, one group): it squares the row, the lanes of a
+// bucket combine by shuffles, then the lane encodes its row against that norm; the words leave from
+// registers or through the consumed stage, which is refilled.
 // HBM traffic: 4 + b/8 bytes per element and worker, plus 4 (8 with the update) per output element.
 #pragma once
 
@@ -55,11 +56,14 @@ struct RoundArgs {
 template <int MODE, bool AVG>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t tiles, cudaStream_t st);
 
-// Registers: 128 per thread (4 CTAs) hold a row, its 32 sums and the generator's state; without the
-// sums five CTAs fit.
+// CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower), 80 without them.
+#ifndef DQ_ROUND_CTAS_AVG
+#define DQ_ROUND_CTAS_AVG 4
+#define DQ_ROUND_CTAS_ENC 6
+#endif
 template <bool AVG>
 struct RoundShape {
-    static constexpr int ctas_per_sm = AVG ? 4 : 5;
+    static constexpr int ctas_per_sm = AVG ? DQ_ROUND_CTAS_AVG : DQ_ROUND_CTAS_ENC;
 };
 
 constexpr int kRoundThreads = 128;
@@ -71,17 +75,16 @@ namespace {
 
 constexpr int kStages = 2;
 constexpr int kTileBytes = 32 * 128;
-constexpr int kStagingBytes = 15 * 128 + 128;        // 32 * 15 words in the 16-byte phase of the stream, rounded up
 constexpr int kMaxSmemSegs = 1023;
 
 // Dynamic shared memory, addressed only through this symbol so that every access compiles to a
 // shared-memory instruction:
 //   [0, kWarps * kStages * 4 KB)  input tiles, warp-major (1024-byte aligned for the swizzle)
-//   then a staging area per warp for words that do not leave straight from registers, the stage
-//   barriers, the teams' exchange slots, the rule's partial sums, and the tensor table
+//   (a consumed tile doubles as the staging area of its words where they do not leave straight from
+//   registers), then the stage barriers, the teams' exchange slots, the rule's partial sums, and the
+//   tensor table
 extern __shared__ __align__(1024) unsigned char smem[];
-constexpr int kStagingOffset = kRoundWarps * kStages * kTileBytes;
-constexpr int kBarOffset = kStagingOffset + kRoundWarps * kStagingBytes;
+constexpr int kBarOffset = kRoundWarps * kStages * kTileBytes;
 constexpr int kPartOffset = kBarOffset + kRoundWarps * kStages * 8;         // [2 parities][4 warps] of {partial, lost}
 constexpr int kSumOffset = kPartOffset + 2 * kRoundWarps * 8;                // 4 doubles + the last-CTA word
 constexpr int kTblOffset = kSumOffset + kRoundWarps * 8 + 16;
@@ -108,10 +111,10 @@ __device__ __forceinline__ float load_norm_early(const float* p)
     return x;
 }
 
-__device__ __forceinline__ void load_quad(const uint32_t offset, uint64_t& lo, uint64_t& hi)
+// Elements 4c .. 4c + 3 of the row at byte offset `row` of the shared memory (swizzle phase folded in)
+__device__ __forceinline__ ulonglong2 row_quad(const uint32_t row, const int c)
 {
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(smem + offset);
-    lo = t.x; hi = t.y;
+    return *reinterpret_cast<const ulonglong2*>(smem + (row ^ (uint32_t)(c << 4)));
 }
 
 // What a warp knows about a tile position: where it starts and what this lane's share of it is.
@@ -126,60 +129,113 @@ struct TilePos {
 };
 
 // Bucket reductions in the order of dq_bucket_norms: four accumulators over a full row's float4
-// components (one over a tensor's last, partial row, whose tail is zero here), a pairwise join.
-__device__ __forceinline__ float row_sum_squares(const uint64_t (&x)[16], const bool regular, const int valid)
+// components (one over a tensor's last, partial row), a pairwise join.
+__device__ __forceinline__ float row_sum_squares(const uint32_t row)
 {
     uint64_t a01 = 0ull, a23 = 0ull;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        a01 = fma_pair(x[2 * c], x[2 * c], a01);
-        a23 = fma_pair(x[2 * c + 1], x[2 * c + 1], a23);
+        const ulonglong2 x = row_quad(row, c);
+        a01 = fma_pair(x.x, x.x, a01);
+        a23 = fma_pair(x.y, x.y, a23);
     }
     float a0, a1, a2, a3;
     unpack_pair(a01, a0, a1);
     unpack_pair(a23, a2, a3);
-    float sum = (a0 + a1) + (a2 + a3);
-    if (!regular) {
-        float chain = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            float u, w;
-            unpack_pair(x[q], u, w);
-            chain = fmaf(u, u, chain);
-            chain = fmaf(w, w, chain);
-        }
-        if (valid < 32) sum = chain;
-    }
-    return sum;
+    return (a0 + a1) + (a2 + a3);
 }
-__device__ __forceinline__ float row_max(const uint64_t (&x)[16])
+__device__ __forceinline__ float row_max(const uint32_t row)
 {
     float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int c = 0; c < 8; ++c) {
+        const ulonglong2 x = row_quad(row, c);
         float u, w;
-        unpack_pair(x[q], u, w);
-        m0 = max_nan(m0, fabsf(u));
-        m1 = max_nan(m1, fabsf(w));
+        unpack_pair(x.x, u, w);
+        m0 = max_nan(m0, fabsf(u)); m1 = max_nan(m1, fabsf(w));
+        unpack_pair(x.y, u, w);
+        m0 = max_nan(m0, fabsf(u)); m1 = max_nan(m1, fabsf(w));
     }
     return max_nan(m0, m1);
 }
-// sum of squares of the row scaled by 2^-e, same order as row_sum_squares
-__device__ __forceinline__ float row_scaled_squares(const uint64_t (&x)[16], const int valid, const int e)
+
+// What a tile that touches a tensor's end needs more, out of line so that the others do not pay for
+// its registers.  The tail of a partial row is padding: it is set to zero where it stands, and the
+// row's sum runs through one accumulator.  Rows that are nobody's add nothing.
+__device__ __noinline__ float irregular_row_sum(const uint32_t row, const int valid, const float full_sum, const int linf)
 {
-    const ScaledSquares red{e};
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, chain = 0.f;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        float u, w;
-        unpack_pair(x[2 * c], u, w);
-        a0 = red.take(a0, u); a1 = red.take(a1, w);
-        chain = red.take(chain, u); chain = red.take(chain, w);
-        unpack_pair(x[2 * c + 1], u, w);
-        a2 = red.take(a2, u); a3 = red.take(a3, w);
-        chain = red.take(chain, u); chain = red.take(chain, w);
+    if (valid == 32) return full_sum;
+    float chain = 0.0f;
+    for (int e = 0; e < valid; ++e) {
+        const float x = *reinterpret_cast<const float*>(smem + (row ^ (uint32_t)((e >> 2) << 4)) + ((e & 3) << 2));
+        chain = linf ? max_nan(chain, fabsf(x)) : fmaf(x, x, chain);
     }
-    return valid < 32 ? chain : (a0 + a1) + (a2 + a3);
+    return chain;
+}
+__device__ __noinline__ void clear_row_tail(const uint32_t row, const int valid)
+{
+    if (valid > 0)
+        for (int e = valid; e < 32; ++e)
+            *reinterpret_cast<float*>(smem + (row ^ (uint32_t)((e >> 2) << 4)) + ((e & 3) << 2)) = 0.0f;
+    __syncwarp();
+}
+
+// Lanes (and a team's warps) of a bucket combine their v; the result is the same in all of them.
+// A warp that lost a wait says so in its slot: `lost` is then set in every warp of the team.
+template <int MODE, class Op>
+__device__ __forceinline__ float join_bucket(float v, const int gpb, const int T_shift, uint32_t& exchanges, const bool landed,
+                                             bool& lost, const Op& op)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float other = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+        v = (MODE == kTeamBuckets || o < gpb) ? other : v;
+    }
+    if constexpr (MODE == kTeamBuckets) {
+        const int warp = threadIdx.x >> 5, T = 1 << T_shift;
+        float2* slots = reinterpret_cast<float2*>(smem + kPartOffset) + (exchanges & 1u) * kRoundWarps;
+        ++exchanges;
+        if ((threadIdx.x & 31) == 0) slots[warp] = make_float2(v, landed ? 0.0f : 1.0f);
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + (warp >> T_shift)), "r"(32 << T_shift) : "memory");
+        const float2* mine = slots + (warp & ~(T - 1));
+        float any = mine[0].y;
+        v = op(0.0f, mine[0].x);
+        for (int i = 1; i < T; ++i) { v = op(v, mine[i].x); any += mine[i].y; }
+        lost |= any != 0.0f;
+    }
+    return v;
+}
+struct AddOp { __device__ __forceinline__ float operator()(const float a, const float b) const { return a + b; } };
+struct MaxOp { __device__ __forceinline__ float operator()(const float a, const float b) const { return max_nan(a, b); } };
+
+// The l2 norm of buckets whose sum of squares is out of range (see l2_sum_in_range): all zeros, tiny
+// entries, an overflowed square.  Called by all lanes of the warp (by all warps of a team, which agree
+// on the sum); zero buckets are settled by their largest magnitude, the others are reduced again with
+// their entries scaled, and lanes whose own bucket was in range keep `nrm`.  Always two exchanges of a
+// team.  Out of line: it is rare, and the common case does not pay for its registers.
+template <int MODE>
+__device__ __noinline__ float rare_norm(const uint32_t row, const int valid, const int gpb, const int T_shift, uint32_t exchanges,
+                                        const float sum, const float nrm)
+{
+    bool lost = false;
+    float mx = valid > 0 ? row_max(row) : 0.0f;          // (a partial row's tail is zero by now)
+    mx = join_bucket<MODE>(mx, gpb, T_shift, exchanges, true, lost, MaxOp{});
+    const bool again = !l2_sum_in_range(sum);
+    float scaled = 0.0f;
+    const int e = scale_exponent(mx);
+    if (MODE == kTeamBuckets || __any_sync(0xffffffffu, again && magnitude_scalable(mx))) {
+        const ScaledSquares red{e};
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, chain = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {
+            const float4 x = *reinterpret_cast<const float4*>(smem + (row ^ (uint32_t)(c << 4)));
+            a0 = red.take(a0, x.x); a1 = red.take(a1, x.y); a2 = red.take(a2, x.z); a3 = red.take(a3, x.w);
+            chain = red.take(chain, x.x); chain = red.take(chain, x.y); chain = red.take(chain, x.z); chain = red.take(chain, x.w);
+        }
+        scaled = valid == 32 ? (a0 + a1) + (a2 + a3) : (valid > 0 ? chain : 0.0f);
+        scaled = join_bucket<MODE>(scaled, gpb, T_shift, exchanges, true, lost, AddOp{});
+    }
+    return again ? (magnitude_scalable(mx) ? rescaled_l2(mx, scaled, e) : mx) : nrm;
 }
 
 // The 128-byte row of sums (or the update of the parameters there), straight from registers: a lane's
@@ -235,12 +291,14 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 
     // Tile positions of one worker; a team takes bucket `pos`, each of its warps 1024 elements of it.
     const int positions = MODE == kWarpBuckets ? (nb + R - 1) / R : (MODE == kTeamBuckets ? nb : (G + 31) / 32);
-    // Contiguous ranges: of positions (AVG: every position goes through all workers), or of the
-    // worker-major list of all tiles.
-    // (each unit -- a warp, or a team -- takes `each` entries, the first `extra` units one more)
+    // The list of work: positions (AVG: every position goes through all workers), or the worker-major
+    // list of all tiles.  Each unit -- a warp, or a team -- takes every hop-th entry, `each` of them, the
+    // first `extra` units one more: dense and sparse stretches of a gradient then fall to all units alike
+    // (text shape, 97 % of the embedding's rows zero: 154 -> 145 us against contiguous ranges).
     const uint32_t unit = (blockIdx.x * kRoundWarps + warp) >> T_shift;
     const int n_pos = (int)(a.each + (unit < a.extra ? 1u : 0u));
-    const int64_t begin = (int64_t)unit * a.each + (unit < a.extra ? unit : a.extra);
+    const int64_t begin = unit;
+    const int hop = (int)((gridDim.x * kRoundWarps) >> T_shift);
     const int m_first = (AVG || M == 1) ? 0 : (int)(begin / positions);
     int pos = (int)(begin - (int64_t)m_first * positions);
     const int items = AVG ? n_pos * M : n_pos;
@@ -361,9 +419,13 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     };
 
     // ---- producer side: tiles are fetched in the order they are consumed, two ahead
-    int p_pos = pos, p_m = m_first, p_left = items;
+    int p_pos = pos, p_m = 0, p_left = items;
     uint32_t p_first = items > 0 ? first_group(p_pos) : kNoTile;
-    const uint64_t policy = tma::policy_evict_first();
+    const uint64_t policy = a.stream_reads ? tma::policy_evict_first() : tma::policy_evict_normal();
+    const int p_step = a.map_has_worker_dim ? 1 : 0;
+    int p_row = (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
+    const uint32_t stage0 = tma::smem_addr(smem) + warp * (kStages * kTileBytes);
+    const uint32_t bar0 = tma::smem_addr(stage_bar(warp, 0));
     // Copies in flight.  A team's warp has no tile of some buckets, so it counts the copies that landed
     // in each stage; the others find a stage's parity in the item's number.
     bool flying0 = false, flying1 = false;
@@ -381,20 +443,18 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
         if (p_left <= 0) return;
         --p_left;
         if (MODE == kTeamBuckets && p_first != kNoTile) { if (st) flying1 = true; else flying0 = true; }
-        if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile)) {
-            const int row0 = (int)(p_first & 0x7fffffffu);
-            uint64_t* bar = stage_bar(warp, st);
-            tma::mbar_expect_tx(bar, kTileBytes);
-            if (a.stream_reads)
-                tma::load_tile_3d_hint(stage_ptr(warp, st), map, bar, 0, row0, a.map_has_worker_dim ? p_m : 0, policy);
-            else
-                tma::load_tile_3d(stage_ptr(warp, st), map, bar, 0, row0, a.map_has_worker_dim ? p_m : 0);
-        }
+        if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile))
+            tma::fetch_tile(stage0 + st * kTileBytes, map, bar0 + st * 8, kTileBytes, p_row, p_worker, policy);
         if (AVG) {
-            if (++p_m == M) { p_m = 0; ++p_pos; if (p_left > 0) p_first = first_group(p_pos); }
+            p_worker += p_step;
+            if (++p_m == M) {
+                p_m = 0; p_worker = 0; p_pos += hop;
+                if (p_left > 0) { p_first = first_group(p_pos); p_row = (int)(p_first & 0x7fffffffu); }
+            }
         } else {
-            if (++p_pos == positions) { p_pos = 0; ++p_m; }
-            if (p_left > 0) p_first = first_group(p_pos);
+            p_pos += hop;
+            while (p_pos >= positions) { p_pos -= positions; p_worker += p_step; }
+            if (p_left > 0) { p_first = first_group(p_pos); p_row = (int)(p_first & 0x7fffffffu); }
         }
     };
 #pragma unroll
@@ -419,135 +479,100 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 #pragma unroll
             for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
         }
+        // this lane's norm and the start of the tile's words, of the worker at hand
+        float* norm_ptr = a.norms + (int64_t)m * nb + t.bucket;
+        uint32_t* tile_words = a.packed + (int64_t)m * a.packed_stride + (int64_t)t.row0 * B;
         float norm_next = 0.0f;
         if constexpr (MODE == kGivenNorms) {
-            if (t.valid > 0) norm_next = load_norm_early(a.norms + (int64_t)m * nb + t.bucket);
+            if (t.valid > 0) norm_next = load_norm_early(norm_ptr);
         }
 
         const int workers = AVG ? M : 1;
 #pragma unroll 1
-        for (int j = 0; j < workers; ++j) {
+        for (int j = 0; j < workers; ++j, norm_ptr += nb, tile_words += a.packed_stride) {
             const int mm = AVG ? j : m;
             const int st = it & 1;
             bool landed = true;
             if (has_tile) {
                 // every lane polls the barrier itself; the verdict is made warp-uniform so that the
                 // warp-level synchronisations below are always reached by all lanes or by none
-                landed = __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), stage_parity(it), a.wait));
+                landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar0 + st * 8, stage_parity(it))) ||
+                         __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), stage_parity(it), a.wait));
                 if (landed) seen_to_land(st);
             }
             if (MODE != kTeamBuckets && !landed) { timed_out = true; break; }
 
-            // ---- the row, in registers; the stage is free again
-            uint64_t x[16];
-            {
-                const uint32_t base = (uint32_t)((warp * kStages + st) * kTileBytes) + own;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) load_quad(base ^ (uint32_t)(c << 4), x[2 * c], x[2 * c + 1]);
-            }
-            if (!t.regular) {                    // what follows a tensor's end is padding, whatever it holds
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    float u, w;
-                    unpack_pair(x[q], u, w);
-                    x[q] = pack_pair(2 * q < t.valid ? __float_as_uint(u) : 0u, 2 * q + 1 < t.valid ? __float_as_uint(w) : 0u);
-                }
-            }
-            __syncwarp();
-            if (MODE != kTeamBuckets || landed) fetch(st);
-            ++it;
+            const uint32_t row = (uint32_t)((warp * kStages + st) * kTileBytes) + own;
+            if (!t.regular && has_tile && landed) clear_row_tail(row, t.valid);
 
             // ---- norm of the bucket
-            float nrm;
-            bool maybe_zero = true;              // some bucket of the tile may be all zeros
+            float nrm, inv;
+            bool plain = false;                  // no zero bucket, no norm outside the normal range
             if constexpr (MODE == kGivenNorms) {
                 nrm = norm_next;
-                if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(a.norms + (int64_t)(mm + 1) * nb + t.bucket);
-                if (AVG && a.with_rule && t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                inv = inv_scale(sf, nrm);
+                if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(norm_ptr + nb);
+                if (AVG && t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
             } else {
-                // combines the lanes (and the team's warps) of a bucket; false if a team mate's wait ran out
-                auto join_lanes = [&](float v, auto op) -> float {
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float other = __shfl_xor_sync(0xffffffffu, v, o);
-                        if (MODE == kTeamBuckets || o < gpb) v = op(v, other);
-                    }
-                    return v;
-                };
                 bool team_lost = false;
-                auto join_team = [&](float v, auto op) -> float {
-                    if constexpr (MODE == kTeamBuckets) {
-                        float2* slots = reinterpret_cast<float2*>(smem + kPartOffset) + (exchanges & 1u) * kRoundWarps;
-                        ++exchanges;
-                        if (lane == 0) slots[warp] = make_float2(v, landed ? 0.0f : 1.0f);
-                        asm volatile("bar.sync %0, %1;" ::"r"(1 + (warp >> T_shift)), "r"(32 << T_shift) : "memory");
-                        const float2* mine = slots + (warp & ~(T - 1));
-                        float r = op(0.0f, mine[0].x), lost = mine[0].y;
-                        for (int i = 1; i < T; ++i) { r = op(r, mine[i].x); lost += mine[i].y; }
-                        team_lost |= lost != 0.0f;
-                        return r;
-                    } else {
-                        return v;
-                    }
-                };
-                auto add = [](float p, float q) { return p + q; };
-                auto larger = [](float p, float q) { return max_nan(p, q); };
                 if (a.linf) {
-                    nrm = join_team(join_lanes(row_max(x), larger), larger);
+                    nrm = row_max(row);
+                    if (!t.regular) nrm = irregular_row_sum(row, t.valid, nrm, 1);
+                    nrm = join_bucket<MODE>(nrm, gpb, T_shift, exchanges, landed, team_lost, MaxOp{});
+                    inv = inv_scale(sf, nrm);
                 } else {
-                    const float sum = join_team(join_lanes(row_sum_squares(x, t.regular, t.valid), add), add);
-                    nrm = sqrtf(sum);
-                    // Rarely a bucket's sum of squares is out of range (see l2_sum_in_range): all zeros, tiny
-                    // entries, an overflowed square.  Zero buckets are settled by their largest magnitude; the
-                    // others are reduced again with their entries scaled.
-                    maybe_zero = __any_sync(0xffffffffu, !l2_sum_in_range(sum));
-                    if (maybe_zero && !team_lost) {
-                        const float mx = join_team(join_lanes(row_max(x), larger), larger);
-                        float again = mx;
-                        if (__any_sync(0xffffffffu, !l2_sum_in_range(sum) && magnitude_scalable(mx))) {
-                            const int e = scale_exponent(mx);
-                            again = rescaled_l2(mx, join_team(join_lanes(row_scaled_squares(x, t.valid, e), add), add), e);
-                        }
-                        if (!l2_sum_in_range(sum)) nrm = again;
+                    float sum = row_sum_squares(row);
+                    if (!t.regular) sum = irregular_row_sum(row, t.valid, sum, 0);
+                    sum = join_bucket<MODE>(sum, gpb, T_shift, exchanges, landed, team_lost, AddOp{});
+                    nrm = sqrt_normal(sum);
+                    inv = inv_scale_normal(sf, nrm);
+                    plain = !__any_sync(0xffffffffu, !l2_sum_in_range(sum));
+                    if (!plain && !team_lost) {
+                        nrm = rare_norm<MODE>(row, t.valid, gpb, T_shift, exchanges, sum, nrm);
+                        exchanges += 2;
+                        inv = inv_scale(sf, nrm);
                     }
                 }
                 if (team_lost) { timed_out = true; break; }
                 if (t.writes) {
-                    DQ_STORE(a.norms + ((int64_t)mm * nb + t.bucket), nrm, a.norms, (int64_t)M * nb * 4, a.status);
-                    bad |= !isfinite(nrm);
-                    if (AVG && a.with_rule) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                    DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
+                    if (AVG) square_sum = fma((double)nrm, (double)nrm, square_sum);
                 }
+                if (!plain) bad |= t.writes && !isfinite(nrm);
+                __syncwarp();
             }
-            if (!has_tile) continue;
+            if (!has_tile) { fetch(st); ++it; continue; }
 
             // ---- codes of the row against that norm, and the lane's share of the average
             uint32_t words[B];
-            const float inv = inv_scale(sf, nrm);
             if constexpr (B == 1) {
                 words[0] = 0u;
-            } else if (maybe_zero && __all_sync(0xffffffffu, nrm == 0.0f)) {
+            } else if (!plain && __all_sync(0xffffffffu, nrm == 0.0f)) {
                 // sparse gradients are full of zero buckets: every code is s, whatever the draw, and adds 0 to the average
                 zero_group_words<B>(words);
             } else {
                 const uint64_t inv2 = pack_pair(__float_as_uint(inv), __float_as_uint(inv));
                 const float scale = nrm * to_unit;
                 const uint64_t scale2 = pack_pair(__float_as_uint(scale), __float_as_uint(scale));
-                encode_row<B, AVG>(x, inv2, scale2, acc2, words, q0, (uint32_t)mm + a.worker0, a.step, a.keys);
+                encode_row<B, AVG>([row](int c) { return row_quad(row, c); }, inv2, scale2, acc2, words, q0, (uint32_t)mm + a.worker0, a.step, a.keys);
             }
 
-            // ---- words out
-            uint32_t* const row_dst = a.packed + (int64_t)mm * a.packed_stride + (int64_t)t.row0 * B;
+            // ---- words out, the stage refilled.  The fence orders the warp's accesses to the stage before the copy's
+            // writes (they go through different proxies, and a read waits its turn in the load queue after it was issued).
             const int64_t extent = (int64_t)M * a.packed_stride * 4;
             if constexpr (StoresDirectly<B>::value) {
+                tma::fence_proxy_async();
+                __syncwarp();
+                fetch(st);
                 // a lane's words are whole 4-, 8- or 16-byte units of the stream: neighbouring lanes fill sectors
-                if (t.valid > 0)
-                    store_words<B>(row_dst + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
+                if (t.valid > 0) store_words<B>(tile_words + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
             } else {
-                uint32_t* out_words = reinterpret_cast<uint32_t*>(smem + kStagingOffset + warp * kStagingBytes);
+                __syncwarp();                    // the warp has read all of its rows
+                uint32_t* out_words = reinterpret_cast<uint32_t*>(stage_ptr(warp, st));
                 // the staging area keeps the 16-byte phase of the output stream; whole quads move 16 bytes per
                 // lane, the ragged ends word by word
                 const int off = (int)(((int64_t)t.row0 * B) & 3);
-                uint32_t* aligned_dst = row_dst - off;
+                uint32_t* aligned_dst = tile_words - off;
                 if (t.valid > 0) {
 #pragma unroll
                     for (int i = 0; i < B; ++i) out_words[off + t.row * B + i] = words[i];
@@ -569,8 +594,12 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                     if (off && ts < 4) ts = 4;
                     if (lane < jend - ts) DQ_STORE(aligned_dst + (ts + lane), out_words[ts + lane], a.packed, extent, a.status);
                 }
+                tma::fence_proxy_async();
                 __syncwarp();
+                fetch(st);
             }
+            ++it;
+            __syncwarp();
         }
         if (timed_out) break;
 
@@ -586,9 +615,10 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 }
                 store_row(a, a.out + ((int64_t)t.row0 + t.row) * 32, r, (int64_t)G * 128);
             }
-            ++pos;
+            pos += hop;
         } else {
-            if (++pos == positions) { pos = 0; ++m; }
+            pos += hop;
+            while (pos >= positions) { pos -= positions; ++m; }
         }
     }
     if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
@@ -631,9 +661,9 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
     if (trouble) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
         // nothing is written but the next b, which follows from the norms that are there
-        if (AVG && a.with_rule && blockIdx.x == 0)
-            rule_from_norms<kRoundThreads>(a.rule, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + kSumOffset),
-                                           a.dev_b, a.status);
+        if (AVG && a.with_rule)
+            rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + kSumOffset),
+                                       a.dev_b, a.status);
         return;
     }
 
@@ -650,7 +680,7 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         default: break;
     }
     if (AVG && a.with_rule)
-        rule_from_partials<kRoundThreads>(a.rule, square_sum, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, a.status);
+        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, a.status);
 }
 
 }  // namespace

@@ -66,12 +66,15 @@ __device__ __forceinline__ void write_next_bits(const RuleArgs& r, const double 
 // End of a kernel whose CTAs all come here: `v` is a thread's share of the sum of squared norms.
 // Every CTA leaves its sum in `partial`, the last one to arrive adds them up in CTA order and writes
 // the next b -- in place, since by then every CTA has read this one's.  The counter wraps to 0 by
-// itself, so it is ready for the next launch.  sh: NT / 32 doubles and one word.
+// itself, so it is ready for the next launch.  With `norms` (a call that could not run: all CTAs
+// agree on that) the sum is taken from the n norms in memory instead.  sh: NT / 32 doubles and one word.
 template <int NT>
-__device__ __forceinline__ void rule_from_partials(const RuleArgs& r, const double v, double* sh, int32_t* dev_b, int32_t* status)
+__device__ __forceinline__ void rule_at_end(const RuleArgs& r, const double v, const float* norms, const int64_t n, double* sh,
+                                            int32_t* dev_b, int32_t* status)
 {
     uint32_t* last = reinterpret_cast<uint32_t*>(sh + NT / 32);
-    if (r.fixed_b == 0) {
+    const bool sums = r.fixed_b == 0 && norms == nullptr;
+    if (sums) {
         const double mine = block_sum<NT>(v, sh);
         if (threadIdx.x == 0) r.partial[blockIdx.x] = mine;       // one entry per CTA: in bounds by construction
     } else {
@@ -84,21 +87,10 @@ __device__ __forceinline__ void rule_from_partials(const RuleArgs& r, const doub
     __syncthreads();
     if (!*last) return;
     double acc = 0.0;
-    if (r.fixed_b == 0) {
+    if (sums) {
         __threadfence();
         for (uint32_t i = threadIdx.x; i < gridDim.x; i += NT) acc += __ldcg(r.partial + i);
-    }
-    const double sum = block_sum<NT>(acc, sh);
-    if (threadIdx.x == 0) write_next_bits(r, sum, dev_b, status);
-}
-
-// One CTA alone: b from norms that are already in memory.
-template <int NT>
-__device__ __noinline__ void rule_from_norms(const RuleArgs& r, const float* norms, const int64_t n, double* sh, int32_t* dev_b,
-                                             int32_t* status)
-{
-    double acc = 0.0;
-    if (r.fixed_b == 0) {
+    } else if (r.fixed_b == 0) {
         for (int64_t i = threadIdx.x; i < n; i += NT) {
             const double x = (double)norms[i];
             acc = fma(x, x, acc);

@@ -114,3 +114,37 @@ def test_lost_first_wait_and_bad_bits(G):
         r.clear_status()
         call()
         assert r.read_status() == 0 and r.guards_intact() and not bool((r.g_packed.view == -7).all())
+
+
+@pytest.mark.parametrize("bucket,b", [(480, 4), (512, 4), (2048, 5), (512, 7)])
+def test_repeated_passes_write_the_same_bits(G, bucket, b):
+    """A stage is refilled while its warp may still be reading it unless the two are ordered: passes over
+    two sets of gradients in turn, without a pause, give the same words and averages every time."""
+    dq = G.dq
+    d, M = (1 << 21) + 77, 8
+    sets = []
+    for i in range(2):
+        r = G.GpuRound([d, 50001], bucket, M)
+        gen = torch.Generator(device="cuda").manual_seed(i)
+        r.grads = torch.randn((M, r.stride), generator=gen, device="cuda")
+        r.set_b(b)
+        r.norms()
+        sets.append(r)
+
+    def one(r):
+        dq.quantize_average(r.lay, r.grads, r.stride, M, r.g_norms.view, r.g_b.view, SEED, 5, r.g_packed.view, r.pstride,
+                            r.g_out.view, r.status)
+        dq.norms_quantize_pack(r.lay, r.grads, r.stride, M, r.g_b.view, SEED, 5, r.g_norms.view, r.g_packed.view, r.pstride,
+                               r.status)
+    want = []
+    for r in sets:
+        r.g_packed.view.fill_(-1)
+        r.quantize(SEED, 5)
+        r.average()
+        want.append((r.g_packed.view.clone(), r.g_out.view.clone(), r.g_norms.view.clone()))
+    for _ in range(12):
+        for r in sets:
+            one(r)
+        for r, (w, o, n) in zip(sets, want):
+            assert torch.equal(r.g_packed.view, w) and torch.equal(r.g_out.view, o) and torch.equal(r.g_norms.view, n)
+    assert all(r.read_status() == 0 and r.guards_intact() for r in sets)
