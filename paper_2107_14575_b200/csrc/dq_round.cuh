@@ -40,7 +40,7 @@ struct RoundArgs {
     int32_t gpb_shift;            // log2(groups per bucket), computed norms only
     uint32_t div_magic;           // kGivenNorms: groups_per_bucket as multiply-shift, or as a shift if a power of two
     int32_t div_shift;            //              (>= 0: the shift; < 0: use div_magic with a 33-bit shift)
-    int32_t stream_reads;         // 1: the gradients exceed the L2, read them with the evict-first policy
+    int32_t stream_reads;         // 1: more than 64 MB of gradients (see the L2 policy of the reads)
     int32_t linf;                 // norm kind
     int32_t update;               // AVG: out <- out + neg_lr * average instead of out <- average
     int32_t wide_words;           // packed rows start on 32-byte boundaries: 32-byte stores allowed
@@ -421,7 +421,12 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     // ---- producer side: tiles are fetched in the order they are consumed, two ahead
     int p_pos = pos, p_m = 0, p_left = items;
     uint32_t p_first = items > 0 ? first_group(p_pos) : kNoTile;
-    const uint64_t policy = a.stream_reads ? tma::policy_evict_first() : tma::policy_evict_normal();
+    // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
+    // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
+    // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
+    // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
+    // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).
+    const uint64_t policy = (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal();
     const int p_step = a.map_has_worker_dim ? 1 : 0;
     int p_row = (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
     const uint32_t stage0 = tma::smem_addr(smem) + warp * (kStages * kTileBytes);
