@@ -61,6 +61,13 @@ __device__ __forceinline__ float max_nan(const float a, const float b)
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
 }
+// largest magnitude of three, by one instruction
+__device__ __forceinline__ float max_magnitude(const float a, const float b, const float c)
+{
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 template <int P>
 __device__ __forceinline__ float take(const float acc, const float x)
 {
@@ -199,6 +206,7 @@ __device__ __forceinline__ float inv_scale_normal(const float sf, const float no
     const float e = __fmaf_rn(-q, norm, sf);
     return __uint_as_float(__float_as_uint(q) - (e < 0.0f ? 1u : 0u));
 }
+__device__ __forceinline__ bool norm_is_plain(const float norm) { return norm >= 0x1p-100f && norm <= 0x1p125f; }
 __device__ __forceinline__ float inv_scale(const float sf, const float norm)
 {
     if (!(norm >= 0x1p-100f)) return 0.0f;

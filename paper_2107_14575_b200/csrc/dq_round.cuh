@@ -152,9 +152,9 @@ __device__ __forceinline__ float row_max(const uint32_t row)
         const ulonglong2 x = row_quad(row, c);
         float u, w;
         unpack_pair(x.x, u, w);
-        m0 = max_nan(m0, fabsf(u)); m1 = max_nan(m1, fabsf(w));
+        m0 = max_magnitude(m0, u, w);
         unpack_pair(x.y, u, w);
-        m0 = max_nan(m0, fabsf(u)); m1 = max_nan(m1, fabsf(w));
+        m1 = max_magnitude(m1, u, w);
     }
     return max_nan(m0, m1);
 }
@@ -303,56 +303,61 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     int pos = (int)(begin - (int64_t)m_first * positions);
     const int items = AVG ? n_pos * M : n_pos;
 
-    // ---- where tiles lie.  c_*: the tensor looked at last (its first bucket or group, first group,
-    //      end of its full buckets, elements); lookups move forward or start over
-    int c_b0 = 0, c_g0 = 0, c_full_end = 0, c_seg = 0;
-    if constexpr (MODE == kWarpBuckets) c_full_end = a.v.n_seg == 1 ? (a.v.seg0_elems >> (a.gpb_shift + 5)) : 0;
-    // last tensor whose first bucket (column 1) or group (column 0) is <= x
+    // ---- where tiles lie.  Codes alone: a position is worked out once, when the producer moves there, and the
+    //      consumer finds the answer in a queue.  AVG: twice, the second time from the cached tensor as a rule.
+    // last tensor whose first bucket (column 1) or group (column 0) is <= x; x and the answer are the
+    // warp's: 32 entries are looked at together, so that 1023 tensors take two steps and not ten
     auto find_seg = [&](int column, int x) -> int {
-        int lo = 0, hi = a.v.n_seg;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (tbl(column * n1 + mid) <= x) lo = mid; else hi = mid;
-        }
+        int lo = 0, len = a.v.n_seg, stride;
+        do {
+            stride = (len + 31) >> 5;
+            const int at = lane * stride;
+            const uint32_t below = __ballot_sync(0xffffffffu, at < len && tbl(column * n1 + lo + at) <= x);
+            const int skip = (__popc(below) - 1) * stride;
+            lo += skip;
+            len = len - skip < stride ? len - skip : stride;
+        } while (stride > 1);
         return lo;
     };
-    // first group of the tile at position p, bit 31 set if the tile is regular by its place alone
-    auto first_group = [&](int p) -> uint32_t {
-        if constexpr (MODE == kWarpBuckets) {
-            const int k0 = p * R;
-            if (k0 < c_b0 || k0 + R > c_full_end) {
-                if (a.v.n_seg > 1) {
-                    const int i = find_seg(1, k0);
-                    c_b0 = tbl(n1 + i);
-                    c_g0 = tbl(i);
-                    c_full_end = c_b0 + (tbl(2 * n1 + i) >> (a.gpb_shift + 5));
-                }
-            }
-            return (uint32_t)(c_g0 + ((k0 - c_b0) << a.gpb_shift)) | ((k0 + R <= c_full_end) ? 0x80000000u : 0u);
-        } else if constexpr (MODE == kTeamBuckets) {
-            // one bucket: its first group plus this warp's 32 groups; regular if the warp's 1024 elements exist;
-            // bits 30..: 0 elements are reported by an all-ones value
-            int local = p, n = a.v.seg0_elems, g0 = 0;
-            if (a.v.n_seg > 1) {
-                if (p < tbl(n1 + c_seg) || p >= tbl(n1 + c_seg + 1)) c_seg = find_seg(1, p);
-                local = p - tbl(n1 + c_seg);
-                n = tbl(2 * n1 + c_seg);
-                g0 = tbl(c_seg);
-            }
-            const int left = n - ((local << T_shift) + sub) * 1024;
-            if (left <= 0) return 0x7fffffffu;                   // the bucket ends before this warp's share
-            return (uint32_t)(g0 + ((local << T_shift) + sub) * 32) | (left >= 1024 ? 0x80000000u : 0u);
-        } else {
-            return (uint32_t)(p * 32);
-        }
+    // the same for an x of each lane's own, from tensor `from` on
+    auto walk_seg = [&](int column, int from, int x) -> int {
+        while (x >= tbl(column * n1 + from + 1)) ++from;
+        return from;
     };
     constexpr uint32_t kNoTile = 0x7fffffffu;
-    auto locate = [&](int p) -> TilePos {
+    // kWarpBuckets, kTeamBuckets: first group of the warp's tile at position p, bit 31 set if every lane owns
+    // a full row of it; kNoTile if a team's bucket ends before this warp's share.  kGivenNorms: the tensor of
+    // the tile's first group.  c_*: the tensor looked at last.
+    int c_b0 = 0, c_g0 = 0, c_n = a.v.seg0_elems, c_end = a.v.n_seg == 1 ? 0x7fffffff : 0;
+    auto describe = [&](int p) -> uint32_t {
+        const int k0 = MODE == kGivenNorms ? p * 32 : p * R;
+        if constexpr (MODE == kGivenNorms) {
+            return a.v.n_seg == 1 ? 0u : (uint32_t)find_seg(0, k0);
+        } else {
+            if (k0 < c_b0 || k0 >= c_end) {
+                const int i = find_seg(1, k0);
+                c_b0 = tbl(n1 + i);
+                c_end = tbl(n1 + i + 1);
+                c_g0 = tbl(i);
+                c_n = tbl(2 * n1 + i);
+            }
+            const int local = k0 - c_b0;
+            if constexpr (MODE == kWarpBuckets) {
+                const int full = c_n >> (a.gpb_shift + 5);
+                return (uint32_t)(c_g0 + (local << a.gpb_shift)) | (local + R <= full ? 0x80000000u : 0u);
+            } else {
+                const int share = (local << T_shift) + sub;              // 1024-element pieces of the tensor before it
+                const int left = c_n - share * 1024;
+                if (left <= 0) return kNoTile;
+                return (uint32_t)(c_g0 + share * 32) | (left >= 1024 ? 0x80000000u : 0u);
+            }
+        }
+    };
+    auto locate = [&](int p, uint32_t desc) -> TilePos {
         TilePos t;
-        t.row = lane; t.valid = 32; t.span = 32; t.bucket = 0; t.writes = false;
-        const uint32_t d = first_group(p);
-        t.row0 = (int)(d & 0x7fffffffu);
-        t.regular = (d >> 31) != 0;
+        t.row = lane; t.valid = 32; t.span = 32; t.bucket = p; t.writes = false;
+        t.row0 = MODE == kGivenNorms ? p * 32 : (int)(desc & 0x7fffffffu);
+        t.regular = (desc >> 31) != 0;
         if constexpr (MODE == kWarpBuckets) {
             const int r = lane >> a.gpb_shift, l = lane & (gpb - 1);
             const int k = p * R + r;
@@ -361,10 +366,11 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             if (!t.regular) {
                 // the tile touches the end of a tensor: buckets may be short, rows may be nobody's
                 int first = 0, len = 0;
+                const int seg0 = a.v.n_seg > 1 ? find_seg(1, p * R) : 0;
                 if (k < nb) {
                     int local = k, n = a.v.seg0_elems, g0 = 0;
                     if (a.v.n_seg > 1) {
-                        const int i = find_seg(1, k);
+                        const int i = walk_seg(1, seg0, k);
                         local = k - tbl(n1 + i);
                         n = tbl(2 * n1 + i);
                         g0 = tbl(i);
@@ -380,14 +386,17 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 t.span = __reduce_max_sync(0xffffffffu, t.valid > 0 ? t.row + 1 : 0);
             }
         } else if constexpr (MODE == kTeamBuckets) {
-            t.bucket = p;
             t.writes = sub == 0 && lane == 0;
             if (!t.regular) {
-                if (d == kNoTile) {
+                if (desc == kNoTile) {
                     t.row0 = -1; t.valid = 0; t.span = 0;
                 } else {
                     int local = p, n = a.v.seg0_elems;
-                    if (a.v.n_seg > 1) { local = p - tbl(n1 + c_seg); n = tbl(2 * n1 + c_seg); }
+                    if (a.v.n_seg > 1) {
+                        const int i = find_seg(1, p);
+                        local = p - tbl(n1 + i);
+                        n = tbl(2 * n1 + i);
+                    }
                     const int v = n - ((local << T_shift) + sub) * 1024 - lane * 32;
                     t.valid = v < 0 ? 0 : (v > 32 ? 32 : v);
                     t.span = __reduce_max_sync(0xffffffffu, t.valid > 0 ? lane + 1 : 0);
@@ -399,12 +408,10 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             if (g < G) {
                 int local = g, n = a.v.seg0_elems, b0 = 0;
                 if (a.v.n_seg > 1) {
-                    if (g < tbl(c_seg)) c_seg = 0;
-                    if (c_seg == 0) c_seg = find_seg(0, g);
-                    while (g >= tbl(c_seg + 1)) ++c_seg;
-                    local = g - tbl(c_seg);
-                    b0 = tbl(n1 + c_seg);
-                    n = tbl(2 * n1 + c_seg);
+                    const int i = walk_seg(0, (int)desc, g);
+                    local = g - tbl(i);
+                    b0 = tbl(n1 + i);
+                    n = tbl(2 * n1 + i);
                 }
                 const int k = (int)div_gpb(a, (uint32_t)local);
                 t.bucket = b0 + k;
@@ -420,7 +427,10 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 
     // ---- producer side: tiles are fetched in the order they are consumed, two ahead
     int p_pos = pos, p_m = 0, p_left = items;
-    uint32_t p_first = items > 0 ? first_group(p_pos) : kNoTile;
+    uint32_t p_first = items > 0 ? describe(p_pos) : kNoTile;
+    // !AVG: descriptions of the positions fetched and not done with, the consumer's and at most two more
+    uint32_t queue0 = 0, queue1 = 0, queue2 = 0;
+    int queued = 0;
     // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
     // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
     // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
@@ -428,7 +438,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).
     const uint64_t policy = (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal();
     const int p_step = a.map_has_worker_dim ? 1 : 0;
-    int p_row = (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
+    int p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
     const uint32_t stage0 = tma::smem_addr(smem) + warp * (kStages * kTileBytes);
     const uint32_t bar0 = tma::smem_addr(stage_bar(warp, 0));
     // Copies in flight.  A team's warp has no tile of some buckets, so it counts the copies that landed
@@ -444,9 +454,19 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             if (st) { ++fills1; flying1 = false; } else { ++fills0; flying0 = false; }
         }
     };
+    auto move_producer = [&]() {
+        p_first = describe(p_pos);
+        p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu);
+    };
     auto fetch = [&](int st) {
         if (p_left <= 0) return;
         --p_left;
+        if (!AVG) {
+            if (queued == 0) queue0 = p_first;
+            else if (queued == 1) queue1 = p_first;
+            else queue2 = p_first;
+            ++queued;
+        }
         if (MODE == kTeamBuckets && p_first != kNoTile) { if (st) flying1 = true; else flying0 = true; }
         if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile))
             tma::fetch_tile(stage0 + st * kTileBytes, map, bar0 + st * 8, kTileBytes, p_row, p_worker, policy);
@@ -454,12 +474,12 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             p_worker += p_step;
             if (++p_m == M) {
                 p_m = 0; p_worker = 0; p_pos += hop;
-                if (p_left > 0) { p_first = first_group(p_pos); p_row = (int)(p_first & 0x7fffffffu); }
+                if (p_left > 0) move_producer();
             }
         } else {
             p_pos += hop;
             while (p_pos >= positions) { p_pos -= positions; p_worker += p_step; }
-            if (p_left > 0) { p_first = first_group(p_pos); p_row = (int)(p_first & 0x7fffffffu); }
+            if (p_left > 0) move_producer();
         }
     };
 #pragma unroll
@@ -474,7 +494,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     int m = m_first;
 
     for (int ip = 0; ip < n_pos && !skip_all; ++ip) {
-        const TilePos t = locate(pos);
+        const TilePos t = locate(pos, AVG ? describe(pos) : queue0);
         const bool has_tile = MODE != kTeamBuckets || t.row0 >= 0;
         // byte offset of the lane's row inside a stage, swizzle phase folded in: chunk c sits at own ^ (c << 4)
         const uint32_t own = (uint32_t)(t.row * 128 + ((t.row & 7) << 4));
@@ -515,7 +535,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             bool plain = false;                  // no zero bucket, no norm outside the normal range
             if constexpr (MODE == kGivenNorms) {
                 nrm = norm_next;
-                inv = inv_scale(sf, nrm);
+                inv = inv_scale_normal(sf, nrm);
+                plain = !__any_sync(0xffffffffu, !norm_is_plain(nrm));
+                if (!plain) inv = inv_scale(sf, nrm);
                 if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(norm_ptr + nb);
                 if (AVG && t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
             } else {
@@ -524,7 +546,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                     nrm = row_max(row);
                     if (!t.regular) nrm = irregular_row_sum(row, t.valid, nrm, 1);
                     nrm = join_bucket<MODE>(nrm, gpb, T_shift, exchanges, landed, team_lost, MaxOp{});
-                    inv = inv_scale(sf, nrm);
+                    inv = inv_scale_normal(sf, nrm);
+                    plain = !__any_sync(0xffffffffu, !norm_is_plain(nrm));
+                    if (!plain) inv = inv_scale(sf, nrm);
                 } else {
                     float sum = row_sum_squares(row);
                     if (!t.regular) sum = irregular_row_sum(row, t.valid, sum, 0);
@@ -625,6 +649,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             pos += hop;
             while (pos >= positions) { pos -= positions; ++m; }
         }
+        if (!AVG) { queue0 = queue1; queue1 = queue2; --queued; }
     }
     if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
     if (timed_out || skip_all) {

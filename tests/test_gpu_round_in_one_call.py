@@ -148,3 +148,32 @@ def test_repeated_passes_write_the_same_bits(G, bucket, b):
         for r, (w, o, n) in zip(sets, want):
             assert torch.equal(r.g_packed.view, w) and torch.equal(r.g_out.view, o) and torch.equal(r.g_norms.view, n)
     assert all(r.read_status() == 0 and r.guards_intact() for r in sets)
+
+
+@pytest.mark.parametrize("n_seg", [2, 31, 32, 33, 64, 500, 1023, 1100])
+@pytest.mark.parametrize("bucket", [32, 512, 2048, 96])
+def test_many_tensors_of_every_size(G, n_seg, bucket):
+    """The warp-wide search of the tensor table (32 entries a step; 1023 tensors in shared memory, more from
+    global memory): tables around its step sizes, empty tensors among them."""
+    rng = np.random.default_rng(n_seg * 7 + bucket)
+    segs = [int(x) for x in rng.choice([0, 1, 31, 33, 500, 2049, 5000], size=n_seg)]
+    segs[0], segs[-1] = 4097, 70
+    M, b = 2, 3
+    ref = oracle.Layout(segs, bucket)
+    g = np.zeros((M, ref.D32), np.float32)
+    for o, n in zip(ref.offsets, segs):
+        g[:, o: o + n] = rng.standard_normal((M, n)).astype(np.float32)
+    r = G.GpuRound(segs, bucket, M)
+    r.set_grads(g)
+    r.set_b(b)
+    norms, packed = r.norms_quantize(SEED, 1, fill=-1)
+    nw = ref.packed_words(b)
+    np.testing.assert_allclose(norms, oracle.bucket_norms(ref, g), rtol=1e-6)
+    np.testing.assert_array_equal(packed[:, :nw], oracle.quantize_pack(ref, g, norms, b, SEED, 1))
+    avg = r.average(fill=1.0).copy()
+    r.g_packed.view.fill_(-1)
+    G.dq.quantize_average(r.lay, r.grads, r.stride, M, r.g_norms.view, r.g_b.view, SEED, 1, r.g_packed.view, r.pstride,
+                          r.g_out.view, r.status)
+    np.testing.assert_array_equal(r.g_packed.view.cpu().numpy().view(np.uint32).reshape(M, -1), packed)
+    np.testing.assert_array_equal(r.g_out.view.cpu().numpy(), avg)
+    assert r.read_status() == 0 and r.guards_intact()
