@@ -56,10 +56,12 @@ struct RoundArgs {
 template <int MODE, bool AVG>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t tiles, cudaStream_t st);
 
-// CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower), 80 without them.
+// CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower); 102 without them
+// (codes of 2^24 elements, b = 6: 17.4 us with five CTAs, 18.1 with six of 80 registers, 18.7 with four; buckets of
+// 4096, M = 16, b = 5: 251, 256 and 254 us).
 #ifndef DQ_ROUND_CTAS_AVG
 #define DQ_ROUND_CTAS_AVG 4
-#define DQ_ROUND_CTAS_ENC 6
+#define DQ_ROUND_CTAS_ENC 5
 #endif
 template <bool AVG>
 struct RoundShape {
@@ -196,7 +198,10 @@ __device__ __forceinline__ float join_bucket(float v, const int gpb, const int T
         float2* slots = reinterpret_cast<float2*>(smem + kPartOffset) + (exchanges & 1u) * kRoundWarps;
         ++exchanges;
         if ((threadIdx.x & 31) == 0) slots[warp] = make_float2(v, landed ? 0.0f : 1.0f);
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + (warp >> T_shift)), "r"(32 << T_shift) : "memory");
+        // (numbers the assembler sees: a number from a register reserves all sixteen barriers for the CTA, and
+        // only four such CTAs fit an SM)
+        if (warp >> T_shift) asm volatile("bar.sync 2, %0;" ::"r"(32 << T_shift) : "memory");
+        else asm volatile("bar.sync 1, %0;" ::"r"(32 << T_shift) : "memory");
         const float2* mine = slots + (warp & ~(T - 1));
         float any = mine[0].y;
         v = op(0.0f, mine[0].x);
