@@ -2,7 +2,8 @@
 
 Usage: ``python -m paper_2107_14575_b200.build [--force] [--verbose] [--checked]``
 Objects go to ``paper_2107_14575_b200/_build``; the shared library sits next
-to the Python binding so that it travels with the source tree.
+to the Python binding so that it travels with the source tree, and so does ``_dqcall.so``, the
+binding's calls as a CPython extension (gcc).
 
 ``--checked`` builds ``libdq_checked.so`` instead (objects in ``_build_checked``): the same
 sources with ``-DDQ_CHECKED``, under which every store of a kernel to global memory checks that
@@ -15,6 +16,7 @@ import concurrent.futures as cf
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -38,16 +40,37 @@ def _nvcc() -> str:
 
 def _deps_mtime() -> float:
     paths = [os.path.join(ROOT, "include", "dq.h")]
-    paths += [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    paths += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".c")]
     return max(os.path.getmtime(p) for p in paths)
 
 
 LIB_CHECKED = os.path.join(PKG, "libdq_checked.so")
 
 
+# the binding's calls (csrc/dq_py.c), a CPython extension next to the library
+CALLS = os.path.join(PKG, "_dqcall.so")
+
+
+def build_calls(force: bool = False) -> str:
+    src = os.path.join(CSRC, "dq_py.c")
+    newest = max(os.path.getmtime(src), os.path.getmtime(os.path.join(ROOT, "include", "dq.h")))
+    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= newest:
+        return CALLS
+    tmp = CALLS + ".tmp.%d" % os.getpid()
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+           "-I", os.path.join(ROOT, "include"), src, "-o", tmp]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("gcc failed on dq_py.c")
+    os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
     LIB = LIB_CHECKED if checked else globals()["LIB"]
     OBJ = globals()["OBJ"] + ("_checked" if checked else "")
+    build_calls(force)
     newest = _deps_mtime()
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB

@@ -1,0 +1,159 @@
+/* The Python binding's calls of a step, as vector-call functions.
+ *
+ * Bound by host work: a round's one call has 18 arguments, which ctypes converts in 5 us and a Python
+ * wrapper prepares in as much again (one core of the host), longer than a small round takes on the GPU.
+ * Here an argument costs some tens of nanoseconds.  Arguments are integers, or objects with a data_ptr()
+ * method (device addresses), or None (NULL); the answer is the C call's status.  No state is kept but the
+ * addresses of the library's entry points, which bind() receives from the Python side, so that any build
+ * of the library can stand behind them. */
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <stdint.h>
+
+#include "dq.h"
+
+static PyObject* g_data_ptr; /* the string "data_ptr" */
+
+/* Integer value or device address of an argument; 0 on success. */
+static int to_u64(PyObject* o, uint64_t* v)
+{
+    PyObject* n;
+    if (PyLong_CheckExact(o)) {
+        *v = PyLong_AsUnsignedLongLongMask(o);
+        return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
+    }
+    if (o == Py_None) {
+        *v = 0;
+        return 0;
+    }
+    n = PyObject_VectorcallMethod(g_data_ptr, &o, 1 | PY_VECTORCALL_ARGUMENTS_OFFSET, NULL);
+    if (!n) {
+        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return -1;
+        PyErr_Clear();
+        n = PyNumber_Long(o); /* numpy integers and other numbers */
+        if (!n) return -1;
+    }
+    *v = PyLong_AsUnsignedLongLongMask(n);
+    Py_DECREF(n);
+    return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
+}
+
+/* The rule travels as a ctypes structure of dq_rule_t's layout. */
+static int to_rule(PyObject* o, dq_rule_t* r)
+{
+    Py_buffer b;
+    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) return -1;
+    if (b.len != (Py_ssize_t)sizeof(dq_rule_t)) {
+        PyBuffer_Release(&b);
+        PyErr_SetString(PyExc_TypeError, "a dq.Rule is wanted");
+        return -1;
+    }
+    *r = *(const dq_rule_t*)b.buf;
+    PyBuffer_Release(&b);
+    return 0;
+}
+
+enum { MAX_ARGS = 18 };
+
+/* All arguments as integers, except number `rule` (a dq_rule_t) and number `real` (a float); -1: none. */
+static int convert(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, int rule, int real, uint64_t* v, dq_rule_t* r, float* f)
+{
+    Py_ssize_t i;
+    if (n != want) {
+        PyErr_Format(PyExc_TypeError, "%zd arguments are wanted, got %zd", want, n);
+        return -1;
+    }
+    for (i = 0; i < n; ++i) {
+        if (i == rule) {
+            if (to_rule(args[i], r) != 0) return -1;
+        } else if (i == real) {
+            const double d = PyFloat_AsDouble(args[i]);
+            if (d == -1.0 && PyErr_Occurred()) return -1;
+            *f = (float)d;
+        } else if (to_u64(args[i], &v[i]) != 0) {
+            return -1;
+        }
+    }
+    return 0;
+}
+
+#define P(i) ((void*)(uintptr_t)v[i])
+#define I64(i) ((int64_t)v[i])
+#define I32(i) ((int32_t)v[i])
+#define U32(i) ((uint32_t)v[i])
+
+#define ENTRY(name, want, rule, real, call)                                                         \
+    static __typeof__(&dq_##name) p_##name;                                                         \
+    static PyObject* py_##name(PyObject* self, PyObject* const* args, Py_ssize_t n)                 \
+    {                                                                                               \
+        uint64_t v[MAX_ARGS];                                                                       \
+        dq_rule_t r;                                                                                \
+        float f = 0.0f;                                                                             \
+        int rc;                                                                                     \
+        (void)self; (void)f; (void)r;                                                               \
+        if (convert(args, n, want, rule, real, v, &r, &f) != 0) return NULL;                        \
+        Py_BEGIN_ALLOW_THREADS                                                                      \
+        rc = p_##name call;                                                                         \
+        Py_END_ALLOW_THREADS                                                                        \
+        return PyLong_FromLong(rc);                                                                 \
+    }
+
+ENTRY(bucket_norms, 7, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), P(6)))
+ENTRY(tensor_norms, 9, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), (size_t)v[6], P(7), P(8)))
+ENTRY(choose_bits, 9, 3, -1, (P(0), P(1), I32(2), &r, P(4), P(5), (size_t)v[6], P(7), P(8)))
+ENTRY(quantize_pack, 12, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), P(11)))
+ENTRY(quantize_pack_worker, 13, -1, -1,
+      (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), U32(8), P(9), I64(10), P(11), P(12)))
+ENTRY(norms_quantize_pack, 12, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), P(7), P(8), I64(9), P(10), P(11)))
+ENTRY(norms_quantize_pack_worker, 13, -1, -1,
+      (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), U32(7), P(8), P(9), I64(10), P(11), P(12)))
+ENTRY(unpack_dequant_average, 9, -1, -1, (P(0), P(1), I64(2), P(3), I32(4), P(5), P(6), P(7), P(8)))
+ENTRY(unpack_average_update, 10, -1, 6, (P(0), P(1), I64(2), P(3), I32(4), P(5), f, P(7), P(8), P(9)))
+ENTRY(quantize_average, 15, -1, 12,
+      (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), I32(11), f, P(13), P(14)))
+ENTRY(norms_quantize_average, 18, 13, 12,
+      (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), P(7), P(8), I64(9), P(10), I32(11), f, &r, P(14), (size_t)v[15], P(16), P(17)))
+
+#define EACH(X)                                                                                     \
+    X(bucket_norms) X(tensor_norms) X(choose_bits) X(quantize_pack) X(quantize_pack_worker)         \
+    X(norms_quantize_pack) X(norms_quantize_pack_worker) X(unpack_dequant_average)                  \
+    X(unpack_average_update) X(quantize_average) X(norms_quantize_average)
+
+/* bind({"dq_...": address}): the entry points of the library that was loaded. */
+static PyObject* py_bind(PyObject* self, PyObject* dict)
+{
+    (void)self;
+    if (!PyDict_Check(dict)) {
+        PyErr_SetString(PyExc_TypeError, "a dict of addresses is wanted");
+        return NULL;
+    }
+#define X(name)                                                                                     \
+    {                                                                                               \
+        PyObject* o = PyDict_GetItemString(dict, "dq_" #name);                                      \
+        uint64_t a = 0;                                                                             \
+        if (!o || to_u64(o, &a) != 0 || !a) {                                                       \
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_KeyError, "dq_" #name);                    \
+            return NULL;                                                                            \
+        }                                                                                           \
+        p_##name = (__typeof__(p_##name))(uintptr_t)a;                                              \
+    }
+    EACH(X)
+#undef X
+    Py_RETURN_NONE;
+}
+
+static PyMethodDef methods[] = {
+    {"bind", py_bind, METH_O, NULL},
+#define X(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL},
+    EACH(X)
+#undef X
+    {NULL, NULL, 0, NULL}};
+
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_dqcall", NULL, -1, methods, NULL, NULL, NULL, NULL};
+
+PyMODINIT_FUNC PyInit__dqcall(void)
+{
+    g_data_ptr = PyUnicode_InternFromString("data_ptr");
+    if (!g_data_ptr) return NULL;
+    return PyModule_Create(&module);
+}

@@ -1,6 +1,7 @@
-"""Thin ctypes binding of the C-ABI CUDA library (``include/dq.h``).
+"""Thin binding of the C-ABI CUDA library (``include/dq.h``).
 
-Argument marshalling only: every step of the path runs in the library's
+Argument marshalling only: ctypes for the calls a program makes once, a small
+CPython extension (``csrc/dq_py.c``) for the calls of a step.  Every step of the path runs in the library's
 kernels.  Tensors are torch CUDA tensors (device memory and streams are
 torch's); the functions have the names and the argument order of the C calls.
 There is no fallback: a missing ``libdq.so`` raises.
@@ -53,11 +54,12 @@ class Rule(C.Structure):
 
 
 _lib = None
+_calls = None
 
 
 def lib():
     """Loads ``libdq.so`` (built by ``python -m paper_2107_14575_b200.build``)."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -132,8 +134,22 @@ def lib():
         L.dq_status_string.argtypes = [C.c_int]
         L.dq_debug_set_wait_limits.restype = None
         L.dq_debug_set_wait_limits.argtypes = [u64, i32]
+        try:
+            from . import _dqcall
+        except ImportError as e:
+            raise RuntimeError("the binding's _dqcall.so is missing: build it with "
+                               "`python -m paper_2107_14575_b200.build`") from e
+        _dqcall.bind({n: C.cast(getattr(L, n), vp).value for n in SYMBOLS})
+        _calls = _dqcall
         _lib = L
     return _lib
+
+
+def _step():
+    """The calls of a step (``_dqcall``), with the library behind them loaded."""
+    if _lib is None:
+        lib()
+    return _calls
 
 
 def status_string(code: int) -> str:
@@ -146,7 +162,7 @@ def debug_set_wait_limits(limit_ns: int = 0, lose_first_wait: bool = False) -> N
 
 
 def _check(rc: int, where: str) -> None:
-    if rc != OK:
+    if rc:
         raise DQError(rc, where)
 
 
@@ -159,10 +175,18 @@ def _ptr(t) -> int:
     return t.data_ptr()
 
 
+_raw_stream = None
+
+
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream() builds an object (1.5 us); its two C calls take a tenth of that
+        global _raw_stream
+        if _raw_stream is None:
+            import torch
+            torch.cuda.current_stream()            # initialises CUDA
+            _raw_stream = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        return _raw_stream[0](_raw_stream[1]())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -186,6 +210,7 @@ class Layout:
             _check(lib().dq_layout_create_ex(arr, len(seg_elems), int(bucket), int(norm), C.byref(h)),
                    "dq_layout_create_ex")
         self._h = h
+        self._address = h.value
         self.bucket = int(bucket)
         self.norm = int(lib().dq_layout_norm(h))
         self.whole_tensor = bool(lib().dq_layout_whole_tensor(h))
@@ -246,8 +271,8 @@ class Layout:
 
 
 def bucket_norms(layout: Layout, grads, worker_stride_elems: int, M: int, norms, status, stream=None) -> None:
-    _check(lib().dq_bucket_norms(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
-                                 _ptr(status), _stream(stream)), "dq_bucket_norms")
+    _check(_step().bucket_norms(layout._address, grads, worker_stride_elems, M, norms, status, _stream(stream)),
+           "dq_bucket_norms")
 
 
 def tensor_norms_scratch_bytes(layout: Layout, M: int) -> int:
@@ -257,8 +282,8 @@ def tensor_norms_scratch_bytes(layout: Layout, M: int) -> int:
 def tensor_norms(layout: Layout, grads, worker_stride_elems: int, M: int, norms, scratch, scratch_bytes: int, status,
                  stream=None) -> None:
     """One norm per tensor of a whole-tensor layout (``dq_tensor_norms``)."""
-    _check(lib().dq_tensor_norms(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
-                                 _ptr(scratch), int(scratch_bytes), _ptr(status), _stream(stream)), "dq_tensor_norms")
+    _check(_step().tensor_norms(layout._address, grads, worker_stride_elems, M, norms, scratch, scratch_bytes,
+                                status, _stream(stream)), "dq_tensor_norms")
 
 
 def choose_bits_scratch_bytes(layout: Layout, M: int) -> int:
@@ -267,8 +292,8 @@ def choose_bits_scratch_bytes(layout: Layout, M: int) -> int:
 
 def choose_bits(layout: Layout, norms, M: int, rule: Rule, dev_b, scratch, scratch_bytes: int, status,
                 stream=None) -> None:
-    _check(lib().dq_choose_bits(layout.handle, _ptr(norms), int(M), C.byref(rule), _ptr(dev_b), _ptr(scratch),
-                                int(scratch_bytes), _ptr(status), _stream(stream)), "dq_choose_bits")
+    _check(_step().choose_bits(layout._address, norms, M, rule, dev_b, scratch, scratch_bytes, status, _stream(stream)),
+           "dq_choose_bits")
 
 
 def choose_bits_noalloc(layout: Layout, norms, M: int, rule: Rule, dev_b, status, stream=None) -> None:
@@ -281,61 +306,51 @@ def choose_bits_noalloc(layout: Layout, norms, M: int, rule: Rule, dev_b, status
 
 def quantize_pack(layout: Layout, grads, worker_stride_elems: int, M: int, norms, dev_b, seed: int, step: int,
                   packed, packed_stride_words: int, status, stream=None) -> None:
-    _check(lib().dq_quantize_pack(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
-                                  _ptr(dev_b), int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(packed),
-                                  int(packed_stride_words), _ptr(status), _stream(stream)), "dq_quantize_pack")
+    _check(_step().quantize_pack(layout._address, grads, worker_stride_elems, M, norms, dev_b, seed, step, packed,
+                                 packed_stride_words, status, _stream(stream)), "dq_quantize_pack")
 
 
 def quantize_pack_worker(layout: Layout, grads, worker_stride_elems: int, M: int, norms, dev_b, seed: int, step: int,
                          first_worker: int, packed, packed_stride_words: int, status, stream=None) -> None:
-    _check(lib().dq_quantize_pack_worker(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
-                                         _ptr(dev_b), int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF,
-                                         int(first_worker) & 0xFFFFFFFF, _ptr(packed), int(packed_stride_words),
-                                         _ptr(status), _stream(stream)), "dq_quantize_pack_worker")
+    _check(_step().quantize_pack_worker(layout._address, grads, worker_stride_elems, M, norms, dev_b, seed, step,
+                                        first_worker, packed, packed_stride_words, status, _stream(stream)),
+           "dq_quantize_pack_worker")
 
 
 def norms_quantize_pack_worker(layout: Layout, grads, worker_stride_elems: int, M: int, dev_b, seed: int, step: int,
                                first_worker: int, norms, packed, packed_stride_words: int, status,
                                stream=None) -> None:
-    _check(lib().dq_norms_quantize_pack_worker(layout.handle, _ptr(grads), int(worker_stride_elems), int(M),
-                                               _ptr(dev_b), int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF,
-                                               int(first_worker) & 0xFFFFFFFF, _ptr(norms), _ptr(packed),
-                                               int(packed_stride_words), _ptr(status), _stream(stream)),
-           "dq_norms_quantize_pack_worker")
+    _check(_step().norms_quantize_pack_worker(layout._address, grads, worker_stride_elems, M, dev_b, seed, step,
+                                              first_worker, norms, packed, packed_stride_words, status,
+                                              _stream(stream)), "dq_norms_quantize_pack_worker")
 
 
 def norms_quantize_pack(layout: Layout, grads, worker_stride_elems: int, M: int, dev_b, seed: int, step: int,
                         norms, packed, packed_stride_words: int, status, stream=None) -> None:
-    _check(lib().dq_norms_quantize_pack(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(dev_b),
-                                        int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(norms), _ptr(packed),
-                                        int(packed_stride_words), _ptr(status), _stream(stream)),
-           "dq_norms_quantize_pack")
+    _check(_step().norms_quantize_pack(layout._address, grads, worker_stride_elems, M, dev_b, seed, step, norms,
+                                       packed, packed_stride_words, status, _stream(stream)), "dq_norms_quantize_pack")
 
 
 def unpack_dequant_average(layout: Layout, packed, packed_stride_words: int, norms, M: int, dev_b, out, status,
                            stream=None) -> None:
-    _check(lib().dq_unpack_dequant_average(layout.handle, _ptr(packed), int(packed_stride_words), _ptr(norms),
-                                           int(M), _ptr(dev_b), _ptr(out), _ptr(status), _stream(stream)),
-           "dq_unpack_dequant_average")
+    _check(_step().unpack_dequant_average(layout._address, packed, packed_stride_words, norms, M, dev_b, out, status,
+                                          _stream(stream)), "dq_unpack_dequant_average")
 
 
 def unpack_average_update(layout: Layout, packed, packed_stride_words: int, norms, M: int, dev_b, lr: float, params,
                           status, stream=None) -> None:
     """``params <- params - lr * average`` (Eq. 2), the average formed on the fly."""
-    _check(lib().dq_unpack_average_update(layout.handle, _ptr(packed), int(packed_stride_words), _ptr(norms),
-                                          int(M), _ptr(dev_b), float(lr), _ptr(params), _ptr(status),
-                                          _stream(stream)), "dq_unpack_average_update")
+    _check(_step().unpack_average_update(layout._address, packed, packed_stride_words, norms, M, dev_b, lr, params,
+                                         status, _stream(stream)), "dq_unpack_average_update")
 
 
 def quantize_average(layout: Layout, grads, worker_stride_elems: int, M: int, norms, dev_b, seed: int, step: int,
                      packed, packed_stride_words: int, out, status, lr: Optional[float] = None, stream=None) -> None:
     """Codes for the given norms and the average of all workers in one pass (``dq_quantize_average``);
     with ``lr`` the average is applied to the parameters in ``out`` instead of stored there."""
-    _check(lib().dq_quantize_average(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(norms),
-                                     _ptr(dev_b), int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(packed),
-                                     int(packed_stride_words), _ptr(out), 0 if lr is None else 1,
-                                     0.0 if lr is None else float(lr), _ptr(status), _stream(stream)),
-           "dq_quantize_average")
+    _check(_step().quantize_average(layout._address, grads, worker_stride_elems, M, norms, dev_b, seed, step, packed,
+                                    packed_stride_words, out, 0 if lr is None else 1, 0.0 if lr is None else lr,
+                                    status, _stream(stream)), "dq_quantize_average")
 
 
 def round_workspace_bytes(layout: Layout, M: int) -> int:
@@ -348,9 +363,7 @@ def norms_quantize_average(layout: Layout, grads, worker_stride_elems: int, M: i
     """A whole round in Algorithm 1's order (``dq_norms_quantize_average``): ``dev_b`` holds this round's b and then
     the next one; with ``lr`` the average is applied to the parameters in ``out`` instead of stored there.
     ``workspace`` is zeroed once by its owner."""
-    _check(lib().dq_norms_quantize_average(layout.handle, _ptr(grads), int(worker_stride_elems), int(M), _ptr(dev_b),
-                                           int(seed) & (2 ** 64 - 1), int(step) & 0xFFFFFFFF, _ptr(norms), _ptr(packed),
-                                           int(packed_stride_words), _ptr(out), 0 if lr is None else 1,
-                                           0.0 if lr is None else float(lr), C.byref(next_rule), _ptr(workspace),
-                                           int(workspace_bytes), _ptr(status), _stream(stream)),
-           "dq_norms_quantize_average")
+    _check(_step().norms_quantize_average(layout._address, grads, worker_stride_elems, M, dev_b, seed, step, norms,
+                                          packed, packed_stride_words, out, 0 if lr is None else 1,
+                                          0.0 if lr is None else lr, next_rule, workspace, workspace_bytes, status,
+                                          _stream(stream)), "dq_norms_quantize_average")
