@@ -76,16 +76,43 @@ bool norms_inside(const dq_layout_t* L)
     return !L->whole_tensor && power_of_two((uint32_t)(L->bucket / 32)) && L->n_seg <= kMaxTableSegs;
 }
 
+// Tile positions of a worker, and how many warps (or teams) go through them at a time.
+int64_t positions(const RoundArgs& a, const dq_layout_t* L, bool given)
+{
+    if (given) return (a.v.total_groups + 31) / 32;
+    if (a.gpb_shift > 5) return L->nb;
+    const int64_t R = 32 >> a.gpb_shift;
+    return (L->nb + R - 1) / R;
+}
+
 template <bool AVG>
 int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, bool given, cudaStream_t st)
 {
-    const int64_t per = AVG ? 1 : a.M;                       // list entries per tile position
-    if (given) return dq_launch_round<kGivenNorms, AVG>(a, map, L->n_seg, per * ((a.v.total_groups + 31) / 32), st);
-    if (a.gpb_shift <= 5) {
-        const int64_t R = 32 >> a.gpb_shift;
-        return dq_launch_round<kWarpBuckets, AVG>(a, map, L->n_seg, per * ((L->nb + R - 1) / R), st);
-    }
-    return dq_launch_round<kTeamBuckets, AVG>(a, map, L->n_seg, per * L->nb, st);
+    const int64_t entries = positions(a, L, given) * (AVG ? 1 : a.M);
+    if (given) return dq_launch_round<kGivenNorms, AVG>(a, map, L->n_seg, entries, st);
+    if (a.gpb_shift <= 5) return dq_launch_round<kWarpBuckets, AVG>(a, map, L->n_seg, entries, st);
+    return dq_launch_round<kTeamBuckets, AVG>(a, map, L->n_seg, entries, st);
+}
+
+// One pass for codes and average, or codes (all workers' tiles side by side) and then the average from
+// the words?  In one pass a warp takes a position through all M workers, one after the other: P positions
+// on U warps are `full` turns of M tiles and a last turn in which only a fraction f of the warps has work.
+// Two kernels spread the M * P tiles evenly, but cost a launch and read the words back.  Per worker, a
+// turn's tile takes 1.8 us when the SMs are nearly empty (1.2 with given norms) and 0.9 more when they are
+// full; two kernels take 2.6 us times the turns' share, and 7.5 us for the second launch; a full turn is
+// 0.4 us cheaper in one pass (0.7 with given norms).  So the last turn decides.  Measured on one B200, b = 5, bucket 512, one
+// pass / two kernels (us): 70k elements M = 4 14.5 / 13.2, M = 32 80 / 20; 600k M = 4 12.6 / 14.2, M = 8
+// 20.4 / 19.2, M = 32 66 / 35; 1.5M M = 8 24.9 / 26.0, M = 32 82 / 64; 3M M = 8 36.5 / 39.3, M = 32
+// 123 / 114; 6M M = 32 210 / 217; bucket 480: 600k M = 8 21.6 / 22.9, M = 32 66 / 55.
+bool one_pass(const RoundArgs& a, const dq_layout_t* L, bool given)
+{
+    int64_t units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
+    if (!given && a.gpb_shift > 5) units >>= a.gpb_shift - 5;
+    const int64_t p = positions(a, L, given);
+    const int64_t full = p / units;
+    const double f = (double)(p - full * units) / (double)units;
+    if (a.M == 1 || f == 0.0) return true;                       // no worker to wait for, or no idle warp
+    return a.M * ((given ? 1.2 : 1.8) - 1.7 * f - (given ? 0.7 : 0.4) * (double)full) <= 7.5;
 }
 
 }  // namespace
@@ -165,9 +192,22 @@ void fill_average(RoundArgs& a, float* dev_out, int32_t update, float lr)
     a.wide_out = reinterpret_cast<uintptr_t>(dev_out) % 32 == 0 ? 1 : 0;
 }
 
-// Workspace of the attached rule: the arrival counter (0 between calls), then a sum per CTA.
+// Workspace of the attached rule: the arrival counter (0 between calls) and this call's b, then a sum per CTA.
 constexpr size_t kCounterBytes = 256;
-size_t rule_workspace_bytes() { return kCounterBytes + (size_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * sizeof(double); }
+constexpr size_t kThisBOffset = 128;
+size_t rule_workspace_bytes()
+{
+    constexpr int ctas = RoundShape<true>::ctas_per_sm > RoundShape<false>::ctas_per_sm ? RoundShape<true>::ctas_per_sm
+                                                                                       : RoundShape<false>::ctas_per_sm;
+    return kCounterBytes + (size_t)dq_sm_count() * ctas * sizeof(double);
+}
+
+int average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t packed_stride_words, const float* dev_norms, int32_t M,
+            const int32_t* dev_b, float* dev_out, int32_t update, float lr, int32_t* dev_status, void* stream)
+{
+    return update ? dq_unpack_average_update(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, lr, dev_out, dev_status, stream)
+                  : dq_unpack_dequant_average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, dev_out, dev_status, stream);
+}
 
 }  // namespace
 
@@ -184,6 +224,11 @@ extern "C" int dq_quantize_average(const dq_layout_t* L, const float* dev_grads,
     if (!fill_args(a, map, L, dev_grads, worker_stride_elems, M, dev_norms, dev_b, seed, step, 0u, dev_packed,
                    packed_stride_words, dev_status))
         return DQ_ERR_CUDA;
+    if (!one_pass(a, L, true)) {
+        rc = launch<false>(a, map, L, true, static_cast<cudaStream_t>(stream));
+        if (rc != DQ_OK) return rc;
+        return average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, dev_out, update, lr, dev_status, stream);
+    }
     fill_average(a, dev_out, update, lr);
     return launch<true>(a, map, L, true, static_cast<cudaStream_t>(stream));
 }
@@ -227,10 +272,17 @@ extern "C" int dq_norms_quantize_average(const dq_layout_t* L, const float* dev_
     if (!fill_args(a, map, L, dev_grads, worker_stride_elems, M, dev_norms, dev_b, seed, step, 0u, dev_packed,
                    packed_stride_words, dev_status))
         return DQ_ERR_CUDA;
-    fill_average(a, dev_out, update, lr);
     a.with_rule = 1;
     a.rule = dq_rule_args(next_rule, M);
     a.rule.arrivals = reinterpret_cast<uint32_t*>(ws);
     a.rule.partial = reinterpret_cast<double*>(ws + kCounterBytes);
+    if (!one_pass(a, L, given)) {
+        // the next b is chosen at the end of the first kernel, which leaves its own for the second
+        a.rule.this_b = reinterpret_cast<int32_t*>(ws + kThisBOffset);
+        rc = launch<false>(a, map, L, given, static_cast<cudaStream_t>(stream));
+        if (rc != DQ_OK) return rc;
+        return average(L, dev_packed, packed_stride_words, dev_norms, M, a.rule.this_b, dev_out, update, lr, dev_status, stream);
+    }
+    fill_average(a, dev_out, update, lr);
     return launch<true>(a, map, L, given, static_cast<cudaStream_t>(stream));
 }

@@ -47,7 +47,7 @@ struct RoundArgs {
     int32_t wide_out;             // out starts on a 32-byte boundary
     uint32_t each, extra;         // list entries per warp (or team): `each`, one more for the first `extra` of them
     float neg_lr;
-    int32_t with_rule;            // AVG: choose the next b from this call's norms (dev_b, in place)
+    int32_t with_rule;            // choose the next b from this call's norms (dev_b, in place)
     RuleArgs rule;
     WaitLimits wait;
 };
@@ -544,7 +544,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 plain = !__any_sync(0xffffffffu, !norm_is_plain(nrm));
                 if (!plain) inv = inv_scale(sf, nrm);
                 if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(norm_ptr + nb);
-                if (AVG && t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                if (t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
             } else {
                 bool team_lost = false;
                 if (a.linf) {
@@ -570,7 +570,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 if (team_lost) { timed_out = true; break; }
                 if (t.writes) {
                     DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
-                    if (AVG) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                    square_sum = fma((double)nrm, (double)nrm, square_sum);
                 }
                 if (!plain) bad |= t.writes && !isfinite(nrm);
                 __syncwarp();
@@ -696,9 +696,9 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
     if (trouble) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
         // nothing is written but the next b, which follows from the norms that are there
-        if (AVG && a.with_rule)
+        if (a.with_rule)
             rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + kSumOffset),
-                                       a.dev_b, a.status);
+                                       a.dev_b, b, a.status);
         return;
     }
 
@@ -714,8 +714,8 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 #undef DQ_CASE
         default: break;
     }
-    if (AVG && a.with_rule)
-        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, a.status);
+    if (a.with_rule)
+        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, b, a.status);
 }
 
 }  // namespace

@@ -17,6 +17,7 @@ struct RuleArgs {
     int32_t M;
     double* partial;              // one sum per CTA
     uint32_t* arrivals;           // CTAs that have written theirs; 0 between launches
+    int32_t* this_b;              // where the call's own b is kept for the kernel that follows, or null
 };
 
 // Host: the rule's argument check and its coefficient (dq_bits.cu).
@@ -67,10 +68,11 @@ __device__ __forceinline__ void write_next_bits(const RuleArgs& r, const double 
 // Every CTA leaves its sum in `partial`, the last one to arrive adds them up in CTA order and writes
 // the next b -- in place, since by then every CTA has read this one's.  The counter wraps to 0 by
 // itself, so it is ready for the next launch.  With `norms` (a call that could not run: all CTAs
-// agree on that) the sum is taken from the n norms in memory instead.  sh: NT / 32 doubles and one word.
+// agree on that) the sum is taken from the n norms in memory instead.  b: this call's.  sh: NT / 32
+// doubles and one word.
 template <int NT>
 __device__ __forceinline__ void rule_at_end(const RuleArgs& r, const double v, const float* norms, const int64_t n, double* sh,
-                                            int32_t* dev_b, int32_t* status)
+                                            int32_t* dev_b, const int b, int32_t* status)
 {
     uint32_t* last = reinterpret_cast<uint32_t*>(sh + NT / 32);
     const bool sums = r.fixed_b == 0 && norms == nullptr;
@@ -97,7 +99,10 @@ __device__ __forceinline__ void rule_at_end(const RuleArgs& r, const double v, c
         }
     }
     const double sum = block_sum<NT>(acc, sh);
-    if (threadIdx.x == 0) write_next_bits(r, sum, dev_b, status);
+    if (threadIdx.x == 0) {
+        if (r.this_b) *r.this_b = b;
+        write_next_bits(r, sum, dev_b, status);
+    }
 }
 
 #endif  // __CUDACC__

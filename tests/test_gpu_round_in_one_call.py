@@ -40,7 +40,8 @@ def _grads(ref, segs, M, seed):
 
 CASES = [(RAGGED, 512, 3, 4), (RAGGED, 32, 2, 7), (RAGGED, 1024, 5, 3), (RAGGED, 2048, 3, 5), (RAGGED, 4096, 2, 8),
          (RAGGED, 96, 2, 6), (RAGGED, 0, 3, 4), ([1 << 18], 512, 4, 2), ([70001], 128, 1, 16), ([1], 4096, 2, 4),
-         ([33] * 1100, 64, 2, 12), ([300000], 2048, 33, 4)] + [(RAGGED, 256, 2, b) for b in range(1, 17)]
+         ([33] * 1100, 64, 2, 12), ([300000], 2048, 33, 4), (RAGGED, 512, 24, 5), (RAGGED, 4096, 24, 4), (RAGGED, 0, 24, 7), (RAGGED, 480, 24, 3),
+         ([3 << 20], 512, 8, 4)] + [(RAGGED, 256, 2, b) for b in range(1, 17)]
 
 
 @pytest.mark.parametrize("segs,bucket,M,b", CASES)
@@ -87,15 +88,15 @@ def test_one_call_equals_the_calls_it_merges(G, segs, bucket, M, b):
 def test_lost_first_wait_and_bad_bits(G):
     """A lost wait raises DQ_STAT_WAIT and nothing else; a b outside 1..16 writes no output but still gets its successor."""
     dq = G.dq
-    for bucket in (512, 4096, 96):
-        r = G.GpuRound(RAGGED, bucket, 3)
+    for bucket, M in ((512, 3), (4096, 3), (96, 3), (512, 40), (4096, 40), (96, 40)):        # one kernel; codes, then average
+        r = G.GpuRound(RAGGED, bucket, M)
         ref = oracle.Layout(RAGGED, bucket)
-        r.set_grads(np.nan_to_num(_grads(ref, RAGGED, 3, 1)))
-        nbytes = dq.round_workspace_bytes(r.lay, 3)
+        r.set_grads(np.nan_to_num(_grads(ref, RAGGED, M, 1)))
+        nbytes = dq.round_workspace_bytes(r.lay, M)
         ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
 
         def call():
-            dq.norms_quantize_average(r.lay, r.grads, r.stride, 3, r.g_b.view, SEED, 0, r.g_norms.view, r.g_packed.view, r.pstride,
+            dq.norms_quantize_average(r.lay, r.grads, r.stride, M, r.g_b.view, SEED, 0, r.g_norms.view, r.g_packed.view, r.pstride,
                                       r.g_out.view, dq.Rule.fixed(6), ws, nbytes, r.status)
             torch.cuda.synchronize()
         r.set_b(4)
