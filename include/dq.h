@@ -217,6 +217,16 @@ int dq_choose_bits(const dq_layout_t* layout, const float* dev_norms, int32_t M,
                    int32_t* dev_b, void* dev_scratch, size_t scratch_bytes,
                    int32_t* dev_status, void* stream);
 
+/* ------------------------------------- norms and bit rule in one call, Eq. 5 and 17
+ * dq_bucket_norms (dq_tensor_norms for a whole-tensor layout) followed by dq_choose_bits on
+ * its norms; where the bucket length is 32 * 2^k one kernel does both.  (The sum behind
+ * G-bar is fp64 in another fixed order than dq_choose_bits'.)  dev_workspace: as for
+ * dq_norms_quantize_average. */
+size_t dq_round_workspace_bytes(const dq_layout_t* layout, int32_t M);
+int dq_norms_choose_bits(const dq_layout_t* layout, const float* dev_grads, int64_t worker_stride_elems,
+                         int32_t M, float* dev_norms, const dq_rule_t* rule, int32_t* dev_b,
+                         void* dev_workspace, size_t workspace_bytes, int32_t* dev_status, void* stream);
+
 /* ------------------------------------------- bit rule without any allocation
  * (The paper has no counterpart: this entry point exists for the library's
  * users, not for the method.)
@@ -339,7 +349,6 @@ int dq_quantize_average(const dq_layout_t* layout, const float* dev_grads, int64
  * (b, s).  dev_workspace: dq_round_workspace_bytes() bytes of 16-byte aligned device
  * memory, ZEROED ONCE before its first use and afterwards left to the calls; calls that may
  * overlap on the GPU need a workspace each. */
-size_t dq_round_workspace_bytes(const dq_layout_t* layout, int32_t M);
 int dq_norms_quantize_average(const dq_layout_t* layout, const float* dev_grads, int64_t worker_stride_elems,
                               int32_t M, int32_t* dev_b, uint64_t seed, uint32_t step, float* dev_norms,
                               uint32_t* dev_packed, int64_t packed_stride_words,

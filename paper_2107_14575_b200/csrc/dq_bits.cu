@@ -2,7 +2,8 @@
 //
 // Two small kernels: fixed-size chunks of the norm array are summed in fp64
 // (fixed assignment of elements to threads, fixed tree), then one CTA adds
-// the chunk sums in a fixed order and applies the rule.
+// the chunk sums in a fixed order and applies the rule.  Where one chunk holds all norms the first
+// kernel applies the rule itself.
 #include "dq_common.cuh"
 #include "dq_rule.cuh"
 
@@ -19,7 +20,8 @@ constexpr int kChunk = 8192;        // norms per CTA of the first kernel
 constexpr int kSumThreads = 128;    // threads of the first kernel: 64 norms each, all loads in flight at once
 
 __global__ void __launch_bounds__(kSumThreads, 8)
-norm_square_partials(const float* __restrict__ norms, const int64_t n, double* __restrict__ partial)
+norm_square_partials(const float* __restrict__ norms, const int64_t n, double* __restrict__ partial, const RuleArgs r,
+                     int32_t* __restrict__ dev_b, int32_t* __restrict__ status)
 {
     __shared__ double sh[kSumThreads / 32];
     grid_dependency_wait();
@@ -42,7 +44,9 @@ norm_square_partials(const float* __restrict__ norms, const int64_t n, double* _
         }
     }
     const double s = block_sum<kSumThreads>(a0 + a1, sh);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;       // one entry per CTA of the grid: in bounds by construction
+    if (threadIdx.x != 0) return;
+    if (gridDim.x == 1) write_next_bits(r, s, dev_b, status);
+    else partial[blockIdx.x] = s;       // one entry per CTA of the grid: in bounds by construction
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -117,8 +121,9 @@ int launch_rule(const dq_layout_t* L, const float* dev_norms, int32_t M, const d
     r.partial = partial;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (rule->fixed_b == 0) {
-        dq_launch(norm_square_partials, dim3((unsigned)chunks), dim3(kSumThreads), 0, st, dev_norms, n, partial);
+        dq_launch(norm_square_partials, dim3((unsigned)chunks), dim3(kSumThreads), 0, st, dev_norms, n, partial, r, dev_b, dev_status);
         if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
+        if (chunks == 1) return DQ_OK;
     }
     dq_launch(apply_rule, dim3(1), dim3(kThreads), 0, st, r, rule->fixed_b == 0 ? (int)chunks : 0, dev_b, dev_status);
     if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;

@@ -2,15 +2,57 @@
 // ||g||_p of Eq. 5 applied per bucket; p = 2, or p = infinity for layouts created
 // with DQ_NORM_LINF), and dq_tensor_norms: one norm per tensor.
 //
-// One team of LANES threads (8, 16 or a full warp, by bucket size) owns a
-// bucket: 128-bit coalesced loads, four independent fp32 accumulators per
+// Bucket lengths of 32 * 2^k are taken by the norm kernels of dq_round.cuh (the pipelines of the
+// quantizer without the codes), the others by the kernels below.  There, one team of LANES threads
+// (8, 16 or a full warp, by bucket size) owns a bucket: 128-bit coalesced loads, four independent fp32 accumulators per
 // lane, a shuffle reduction inside the team.  A warp takes runs of consecutive
 // buckets of one worker (blockIdx.y), so the tensor a bucket belongs to is
 // searched once per run and then followed; neighbouring warps read neighbouring
 // memory.  HBM-bound: 4 bytes read per element, 4/bucket bytes written.
 #include "dq_common.cuh"
 #include "dq_device.cuh"
-#include "dq_tma.cuh"
+#include "dq_round.cuh"
+
+bool dq_norms_inside(const dq_layout_t* L)
+{
+    const uint32_t gpb = (uint32_t)(L->bucket / 32);
+    return !L->whole_tensor && (gpb & (gpb - 1)) == 0;
+}
+
+int64_t dq_tile_positions(const RoundArgs& a, bool given)
+{
+    if (given) return (a.v.total_groups + 31) / 32;
+    if (a.gpb_shift > 5) return a.v.nb;
+    const int64_t R = 32 >> a.gpb_shift;
+    return (a.v.nb + R - 1) / R;
+}
+
+bool dq_fill_round(RoundArgs& a, CUtensorMap& map, const dq_layout_t* L, const LayoutView& v, const float* dev_grads,
+                   int64_t worker_stride_elems, int32_t M, int32_t* dev_status)
+{
+    a = RoundArgs{};
+    a.v = v;
+    a.status = dev_status;
+    a.M = M;
+    a.linf = L->norm == DQ_NORM_LINF ? 1 : 0;
+    a.wait = dq_wait_limits();
+    a.stream_reads = ((int64_t)M * L->padded * 4 > (int64_t(64) << 20)) ? 1 : 0;
+    const bool worker_dim = (M > 1 && worker_stride_elems != 0);
+    a.map_has_worker_dim = worker_dim ? 1 : 0;
+    const uint32_t gpb = (uint32_t)v.groups_per_bucket;
+    a.div_shift = -1;
+    a.div_magic = (uint32_t)(((uint64_t(1) << 33) + gpb - 1) / gpb);
+    if ((gpb & (gpb - 1)) == 0) {
+        a.div_shift = 0;
+        while ((1u << a.div_shift) < gpb) ++a.div_shift;
+        a.gpb_shift = a.div_shift;
+    }
+    // tensor map over the gradients, [worker][group][32 floats], box = one warp tile of 32 groups
+    const uint64_t dims[3] = {32, (uint64_t)v.total_groups, worker_dim ? (uint64_t)M : 1};
+    const uint64_t strides[2] = {128, worker_dim ? (uint64_t)worker_stride_elems * 4 : (uint64_t)L->padded * 4};
+    const uint32_t box[3] = {32, 32, 1};
+    return dq_encode_tensor_map(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, dev_grads, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
 
 namespace {
 
@@ -255,211 +297,6 @@ bucket_norms_warp_kernel(const LayoutView v, const float* __restrict__ grads, co
     if (bad) atomicOr(status, DQ_STAT_NONFINITE);
 }
 
-// Bulk-copy variant for bucket sizes that are 32 times a power of two (every size in
-// common use).  Persistent CTAs each take a contiguous range of tiles of
-// R = 4096 / bucket consecutive buckets of one worker; in the padded layout such
-// a run is one contiguous span of at most 128 groups, fetched by a single TMA
-// tensor copy into a ring of swizzled shared-memory stages, so the bytes in
-// flight are set by the ring and not by how many loads the warps manage to
-// issue.  Thread t of a tile owns group (t % gpb) of bucket (t / gpb): it squares
-// its 128-byte row, the gpb threads of a bucket combine by shuffles (and through
-// shared memory when a bucket spans several warps).
-constexpr int kTmaThreads = 128;
-constexpr int kTmaStages = 4;
-constexpr int kTmaTileBytes = kTmaThreads * 128;
-constexpr int kTmaMaxSmemSegs = 1023;
-
-extern __shared__ __align__(1024) unsigned char smem[];
-constexpr int kPartOffset = kTmaStages * kTmaTileBytes;          // 4 floats: per-warp partial results
-constexpr int kAbortOffset = kPartOffset + 16;                   // set by a thread whose wait ran out
-constexpr int kBarOffset = kPartOffset + 32;
-constexpr int kTblOffset = kBarOffset + kTmaStages * 8;
-
-__device__ __forceinline__ uint64_t* full_bar(int st) { return reinterpret_cast<uint64_t*>(smem + kBarOffset) + st; }
-
-struct NormsArgs {
-    LayoutView v;
-    const float* grads;
-    float* norms;
-    int32_t* status;
-    int32_t M;
-    int32_t map_has_worker_dim;
-    int32_t gpb_shift;           // log2(groups per bucket)
-    WaitLimits wait;
-};
-
-template <int P>
-__global__ void __launch_bounds__(kTmaThreads)
-bucket_norms_tma_kernel(const __grid_constant__ NormsArgs a, const __grid_constant__ CUtensorMap map)
-{
-    grid_dependency_wait();
-    const int tid = threadIdx.x;
-    if (tma::smem_addr(smem) & 1023u) {
-        if (tid == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
-        return;
-    }
-    const int n1 = a.v.n_seg + 1;
-    const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kTmaMaxSmemSegs;
-    int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + kTblOffset);
-    if (tbl_in_smem)
-        for (int i = tid; i < 3 * n1; i += kTmaThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kAbortOffset);
-    if (tid == 0) {
-        tma::prefetch_tensor_map(&map);
-#pragma unroll
-        for (int st = 0; st < kTmaStages; ++st) tma::mbar_init(full_bar(st), 1);
-        tma::fence_barrier_init();
-        *abort_flag = 0;
-    }
-    __syncthreads();
-    auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
-
-    const int gpb = 1 << a.gpb_shift;
-    const int R = kTmaThreads >> a.gpb_shift;                   // buckets per tile
-    const int nb = a.v.nb;
-    const int tiles_per_worker = (nb + R - 1) / R;
-    const int total_tiles = a.M * tiles_per_worker;
-    const int bsz = gpb * 32;
-    // every CTA takes one contiguous range of the worker-major tile list
-    const int tile_begin = (int)((int64_t)blockIdx.x * total_tiles / gridDim.x);
-    const int tile_end = (int)((int64_t)(blockIdx.x + 1) * total_tiles / gridDim.x);
-
-    // first group and valid elements of bucket k; `seg` is a walking hint (buckets only move forward)
-    auto locate = [&](int k, int& seg, int& first_group, int& len) {
-        int local, n, g0;
-        if (a.v.n_seg == 1) {
-            local = k; n = a.v.seg0_elems; g0 = 0;
-        } else {
-            while (k >= tbl(n1 + seg + 1)) ++seg;
-            local = k - tbl(n1 + seg);
-            n = tbl(2 * n1 + seg);
-            g0 = tbl(seg);
-        }
-        first_group = g0 + (local << a.gpb_shift);
-        const int left = n - local * bsz;
-        len = left < bsz ? left : bsz;
-    };
-    auto advance = [&](int& mm, int& rr) {
-        if (++rr == tiles_per_worker) { rr = 0; ++mm; }
-    };
-
-    int m = tile_begin / tiles_per_worker, kt = tile_begin - m * tiles_per_worker;
-    int pm = m, pkt = kt, ptile = tile_begin, pseg = 0, pseg_m = m;
-    auto issue = [&](int st) {
-        if (pm != pseg_m) { pseg = 0; pseg_m = pm; }
-        int row0, len0;
-        locate(pkt * R, pseg, row0, len0);
-        tma::mbar_expect_tx(full_bar(st), kTmaTileBytes);
-        tma::load_tile_3d(smem + st * kTmaTileBytes, &map, full_bar(st), 0, row0, a.map_has_worker_dim ? pm : 0);
-    };
-#pragma unroll
-    for (int st = 0; st < kTmaStages; ++st) {
-        if (ptile < tile_end && tid == 0) issue(st);
-        ++ptile;
-        advance(pm, pkt);
-    }
-
-    const int r = tid >> a.gpb_shift;            // bucket of the tile this thread works on
-    const int l = tid & (gpb - 1);               // its group inside that bucket
-    const int lane = tid & 31, warp = tid >> 5;
-    float* part = reinterpret_cast<float*>(smem + kPartOffset);
-    int seg = 0, seg0 = 0, seg_m = -1;
-    int it = 0;
-    bool timed_out = false, bad = false;
-    for (int tile = tile_begin; tile < tile_end; ++tile, ++it, advance(m, kt)) {
-        const int st = it % kTmaStages;
-        if (m != seg_m) { seg = 0; seg0 = 0; seg_m = m; }
-        const int k0 = kt * R;
-        const int k = k0 + r;
-        int row0, len0, first = 0, len = 0;
-        locate(k0, seg0, row0, len0);
-        if (k < nb) locate(k, seg, first, len);
-        const int row = first - row0 + l;        // this thread's row of the tile
-        int valid = len - l * 32;                // elements of its group that count
-        valid = valid < 0 ? 0 : (valid > 32 ? 32 : valid);
-
-        // A thread whose wait runs out says so in shared memory and goes on (what it reads from the
-        // stage is then arbitrary, and unused): every thread reaches the barriers below, after which all
-        // of them see the flag and leave together.
-        bool landed = tma::mbar_wait(full_bar(st), (it / kTmaStages) & 1, a.wait);
-        if (it == 0 && a.wait.lose_first != 0u) landed = false;      // test hook: the first wait counts as lost
-        if (!landed) *abort_flag = 1;
-
-        // One reduction of the tile: the gpb threads of a bucket combine inside a warp by shuffles and
-        // across the warps of a bucket through shared memory; the result counts in the threads with l == 0
-        // (in all threads of the bucket when it lies inside one warp).
-        const unsigned char* base = smem + st * kTmaTileBytes;
-        auto tile_reduce = [&](const auto& red) -> float {
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            if (valid > 0) {
-                if (valid == 32) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float4 x = *reinterpret_cast<const float4*>(base + tma::swizzle128(row, c));
-                        a0 = red.take(a0, x.x); a1 = red.take(a1, x.y); a2 = red.take(a2, x.z); a3 = red.take(a3, x.w);
-                    }
-                } else {                             // last group of a tensor: what follows is padding
-                    for (int e = 0; e < valid; ++e) {
-                        const float x = *reinterpret_cast<const float*>(base + tma::swizzle128(row, e >> 2) + ((e & 3) << 2));
-                        a0 = red.take(a0, x);
-                    }
-                }
-            }
-            float v = red.join(red.join(a0, a1), red.join(a2, a3));
-            const int w = gpb < 32 ? gpb : 32;
-            for (int o = w >> 1; o > 0; o >>= 1) v = red.join(v, __shfl_xor_sync(0xffffffffu, v, o));
-            if (gpb > 32) {
-                if (lane == 0) part[warp] = v;
-                __syncthreads();
-                if (l == 0) {
-                    v = 0.f;
-                    for (int i = 0; i < (gpb >> 5); ++i) v = red.join(v, part[(tid >> 5) + i]);
-                }
-            }
-            return v;
-        };
-        const float sum = tile_reduce(typename FamilyReduction<P>::type{});
-        float nrm = finish<P>(sum);
-        const bool writes = (l == 0 && k < nb);
-        const bool out_of_range = (P == DQ_NORM_L2) && writes && !l2_sum_in_range(sum);
-        // after this barrier everyone is done with the stage and with part[]
-        if (__syncthreads_or(out_of_range || !landed)) {
-            if (*abort_flag) { timed_out = true; break; }
-            if constexpr (P == DQ_NORM_L2) {
-                // some bucket of the tile needs the rescaled reduction (see l2_sum_in_range): the whole
-                // CTA takes it, the buckets that were in range keep their norm
-                float mx = tile_reduce(MaxMagnitude{});
-                if (gpb > 32) {                  // the bucket's largest magnitude, for all of its threads
-                    __syncthreads();
-                    if (l == 0) part[warp] = mx;
-                    __syncthreads();
-                    mx = part[(tid >> a.gpb_shift) << (a.gpb_shift - 5)];
-                    __syncthreads();
-                }
-                const int e = scale_exponent(mx);
-                const float scaled = tile_reduce(ScaledSquares{e});
-                if (out_of_range) nrm = rescaled_l2(mx, scaled, e);
-                __syncthreads();
-            }
-        }
-        if (writes) {
-            DQ_STORE(a.norms + ((int64_t)m * nb + k), nrm, a.norms, (int64_t)a.M * a.v.nb * 4, a.status);
-            bad |= !isfinite(nrm);
-        }
-        if (ptile < tile_end && tid == 0) issue(st);
-        ++ptile;
-        advance(pm, pkt);
-    }
-    if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
-    if (timed_out) {
-        if (tid == 0) atomicOr(a.status, DQ_STAT_WAIT);
-        // every copy already issued, the one whose wait ran out included, gets the full limit to land
-        // before the CTA's shared memory is released
-        for (int j = it; j < it + kTmaStages; ++j)
-            if (tile_begin + j < tile_end) (void)tma::mbar_wait(full_bar(j % kTmaStages), (j / kTmaStages) & 1, a.wait);
-    }
-}
-
 // Second step of dq_tensor_norms: block (tensor, worker) joins the norms of the tensor's pieces in
 // a fixed order -- thread t takes pieces t, t + 256, ..., then a tree over the block -- and writes
 // the tensor's norm.  l2: the squares of the piece norms are exact in fp64 and cannot leave its
@@ -518,43 +355,17 @@ tensor_norms_join_kernel(const int32_t n_seg, const int32_t* __restrict__ piece0
     if (!isfinite(nrm)) atomicOr(status, DQ_STAT_NONFINITE);
 }
 
-// Launch of the bulk-copy kernel over view `v` (groups per bucket a power of two, at most 128).
-template <int P>
-int launch_tma(const dq_layout_t* L, const LayoutView& v, const float* dev_grads, int64_t worker_stride_elems, int32_t M,
-               float* dev_out, int32_t* dev_status, cudaStream_t st)
+// Norms of the buckets of view `v` (32 * 2^k elements, up to 4096).
+int launch_norms(const dq_layout_t* L, const LayoutView& v, const float* dev_grads, int64_t worker_stride_elems, int32_t M,
+                 float* dev_out, int32_t* dev_status, cudaStream_t st)
 {
-    const uint32_t gpb = (uint32_t)v.groups_per_bucket;
-    NormsArgs a;
-    a.v = v;
-    a.grads = dev_grads;
-    a.norms = dev_out;
-    a.status = dev_status;
-    a.M = M;
-    a.gpb_shift = 0;
-    while ((1u << a.gpb_shift) < gpb) ++a.gpb_shift;
-    a.wait = dq_wait_limits();
-    const bool worker_dim = (M > 1 && worker_stride_elems != 0);
-    a.map_has_worker_dim = worker_dim ? 1 : 0;
+    RoundArgs a;
     CUtensorMap map;
-    const uint64_t dims[3] = {32, (uint64_t)v.total_groups, worker_dim ? (uint64_t)M : 1};
-    const uint64_t strides[2] = {128, worker_dim ? (uint64_t)worker_stride_elems * 4 : (uint64_t)L->padded * 4};
-    const uint32_t box[3] = {32, (uint32_t)kTmaThreads, 1};
-    if (!dq_encode_tensor_map(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, dev_grads, dims, strides, box,
-                              CU_TENSOR_MAP_SWIZZLE_128B))
-        return DQ_ERR_CUDA;
-    size_t smem_need = (size_t)kTblOffset;
-    if (L->n_seg > 1 && L->n_seg <= kTmaMaxSmemSegs) smem_need += (size_t)3 * (L->n_seg + 1) * 4;
-    if (cudaFuncSetAttribute(bucket_norms_tma_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return DQ_ERR_CUDA;
-    }
-    const int R = kTmaThreads >> a.gpb_shift;
-    const int64_t tiles = (int64_t)M * ((v.nb + R - 1) / R);
-    int64_t blocks = (int64_t)dq_sm_count() * 3;    // three 65 KB CTAs per SM
-    if (blocks > tiles) blocks = tiles;
-    dq_launch(bucket_norms_tma_kernel<P>, dim3((unsigned)blocks), dim3(kTmaThreads), smem_need, st, a, map);
-    if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
-    return DQ_OK;
+    if (!dq_fill_round(a, map, L, v, dev_grads, worker_stride_elems, M, dev_status)) return DQ_ERR_CUDA;
+    a.norms = dev_out;
+    const int64_t entries = dq_tile_positions(a, false) * M;
+    return a.gpb_shift <= 5 ? dq_launch_norms<kWarpBuckets>(a, map, L->n_seg, entries, st)
+                            : dq_launch_norms<kTeamBuckets>(a, map, L->n_seg, entries, st);
 }
 
 // other bucket sizes: plain-load kernels
@@ -608,13 +419,8 @@ extern "C" int dq_bucket_norms(const dq_layout_t* L, const float* dev_grads, int
 
     const LayoutView v = make_view(L);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const uint32_t gpb = (uint32_t)v.groups_per_bucket;
     const bool linf = (L->norm == DQ_NORM_LINF);
-    if ((gpb & (gpb - 1)) == 0) {
-        // bucket = 32 * 2^k: bulk-copy kernel
-        return linf ? launch_tma<DQ_NORM_LINF>(L, v, dev_grads, worker_stride_elems, M, dev_norms, dev_status, st)
-                    : launch_tma<DQ_NORM_L2>(L, v, dev_grads, worker_stride_elems, M, dev_norms, dev_status, st);
-    }
+    if (dq_norms_inside(L)) return launch_norms(L, v, dev_grads, worker_stride_elems, M, dev_norms, dev_status, st);
     return linf ? launch_plain<DQ_NORM_LINF>(L, v, dev_grads, worker_stride_elems, M, dev_norms, dev_status, st)
                 : launch_plain<DQ_NORM_L2>(L, v, dev_grads, worker_stride_elems, M, dev_norms, dev_status, st);
 }
@@ -640,8 +446,7 @@ extern "C" int dq_tensor_norms(const dq_layout_t* L, const float* dev_grads, int
     float* partial = static_cast<float*>(dev_scratch);
     const LayoutView pv = make_piece_view(L);
     const bool linf = (L->norm == DQ_NORM_LINF);
-    const int r1 = linf ? launch_tma<DQ_NORM_LINF>(L, pv, dev_grads, worker_stride_elems, M, partial, dev_status, st)
-                        : launch_tma<DQ_NORM_L2>(L, pv, dev_grads, worker_stride_elems, M, partial, dev_status, st);
+    const int r1 = launch_norms(L, pv, dev_grads, worker_stride_elems, M, partial, dev_status, st);
     if (r1 != DQ_OK) return r1;
     const int32_t n1 = L->n_seg + 1;
     const int32_t* piece0 = L->n_seg > 1 ? L->dev_table + 4 * n1 : nullptr;

@@ -109,6 +109,7 @@ ENTRY(norms_quantize_pack_worker, 13, -1, -1,
       (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), U32(7), P(8), P(9), I64(10), P(11), P(12)))
 ENTRY(unpack_dequant_average, 9, -1, -1, (P(0), P(1), I64(2), P(3), I32(4), P(5), P(6), P(7), P(8)))
 ENTRY(unpack_average_update, 10, -1, 6, (P(0), P(1), I64(2), P(3), I32(4), P(5), f, P(7), P(8), P(9)))
+ENTRY(norms_choose_bits, 11, 5, -1, (P(0), P(1), I64(2), I32(3), P(4), &r, P(6), P(7), (size_t)v[8], P(9), P(10)))
 ENTRY(quantize_average, 15, -1, 12,
       (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), I32(11), f, P(13), P(14)))
 ENTRY(norms_quantize_average, 18, 13, 12,
@@ -117,7 +118,7 @@ ENTRY(norms_quantize_average, 18, 13, 12,
 #define EACH(X)                                                                                     \
     X(bucket_norms) X(tensor_norms) X(choose_bits) X(quantize_pack) X(quantize_pack_worker)         \
     X(norms_quantize_pack) X(norms_quantize_pack_worker) X(unpack_dequant_average)                  \
-    X(unpack_average_update) X(quantize_average) X(norms_quantize_average)
+    X(unpack_average_update) X(norms_choose_bits) X(quantize_average) X(norms_quantize_average)
 
 /* bind({"dq_...": address}): the entry points of the library that was loaded. */
 static PyObject* py_bind(PyObject* self, PyObject* dict)

@@ -6,7 +6,7 @@
 //   kWarpBuckets   buckets of 32 * 2^k <= 1024 elements: a warp tile is 1024 / bucket buckets
 //   kTeamBuckets   buckets of 2048 or 4096: a team of 2 or 4 warps of the CTA takes a bucket
 //   kGivenNorms    any bucket length, whole-tensor layouts: norms are read, a tile is 32 groups
-// AVG = false: codes (and norms) of every worker.  AVG = true: a warp keeps its tile of the output
+// B = 0: norms alone.  AVG = false: codes (and norms) of every worker.  AVG = true: a warp keeps its tile of the output
 // while it goes through the M workers, whose words it writes as it goes; the averaged gradient (or
 // the updated parameters) leaves at the end of the tile.
 //
@@ -52,7 +52,10 @@ struct RoundArgs {
     WaitLimits wait;
 };
 
-// Launch of one of the six kernels (each in a translation unit of its own).
+// Launch of one of the kernels (each in a translation unit of its own): norms alone, or codes with or
+// without the average.  `entries`: length of the list of work (see round_tiles).
+template <int MODE>
+int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 template <int MODE, bool AVG>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t tiles, cudaStream_t st);
 
@@ -70,6 +73,15 @@ struct RoundShape {
 
 constexpr int kRoundThreads = 128;
 constexpr int kRoundWarps = kRoundThreads / 32;
+constexpr int kRoundMaxCtasPerSm = 6;            // of any of the kernels (the rule's workspace has a sum per CTA)
+
+// Host, dq_norms.cu: geometry, gradients and tensor map of a launch over view `v` (not the norms, b, words, draws).
+bool dq_fill_round(RoundArgs& a, CUtensorMap& map, const dq_layout_t* L, const LayoutView& v, const float* dev_grads,
+                   int64_t worker_stride_elems, int32_t M, int32_t* dev_status);
+// Whether the kernels take the norms of a layout's buckets themselves.
+bool dq_norms_inside(const dq_layout_t* L);
+// Positions of a worker's tiles; given: those of kGivenNorms.
+int64_t dq_tile_positions(const RoundArgs& a, bool given);
 
 #ifdef DQ_ROUND_KERNELS
 
@@ -279,8 +291,8 @@ template <int B, int MODE, bool AVG>
 __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
 {
     const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
-    auto tbl = [&](int i) -> int { return (MODE != kGivenNorms || tbl_in_smem) ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
-    constexpr int s = (1 << (B - 1)) - 1;
+    auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
+    constexpr int s = B > 0 ? (1 << (B > 0 ? B - 1 : 0)) - 1 : 0;
     const float sf = (float)s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n1 = a.v.n_seg + 1;
@@ -490,7 +502,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 #pragma unroll
     for (int st = 0; st < kStages; ++st) fetch(st);
 
-    const float to_unit = (B == 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
+    const float to_unit = (B <= 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
     uint32_t it = 0;                              // items consumed; item i travels through stage i & 1
     uint32_t exchanges = 0;
     bool timed_out = false, bad = false;
@@ -576,9 +588,16 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 __syncwarp();
             }
             if (!has_tile) { fetch(st); ++it; continue; }
+            if constexpr (B == 0) {              // norms alone: the row has been read (see the refill below)
+                tma::fence_proxy_async();
+                __syncwarp();
+                fetch(st);
+                ++it;
+                __syncwarp();
+            } else {
 
             // ---- codes of the row against that norm, and the lane's share of the average
-            uint32_t words[B];
+            uint32_t words[B > 0 ? B : 1];
             if constexpr (B == 1) {
                 words[0] = 0u;
             } else if (!plain && __all_sync(0xffffffffu, nrm == 0.0f)) {
@@ -634,6 +653,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             }
             ++it;
             __syncwarp();
+            }
         }
         if (timed_out) break;
 
@@ -671,9 +691,8 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     }
 }
 
-template <int MODE, bool AVG>
-__global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
-round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+// Barriers, tensor table (true if it is in shared memory), and the wait for the kernel before.
+__device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& map)
 {
     // (nothing up to the wait touches memory that an earlier kernel may still be writing)
     if (threadIdx.x == 0) {
@@ -682,13 +701,40 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         tma::fence_barrier_init();
     }
     grid_dependency_wait();
-    const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
     const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
     if (tbl_in_smem) {
         int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + kTblOffset);
         for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
     }
     __syncthreads();
+    return tbl_in_smem;
+}
+
+// Norms alone.  Bound by HBM, 4 bytes read per element.  Against a CTA-wide ring of 16 KB tiles with a barrier
+// per tile (three CTAs of 128 threads per SM): ResNet-18 shape M = 8 72 -> 57 us (6.3 TB/s), VGG-16 shape M = 16,
+// bucket 2048, 191 -> 150, text shape with its zero rows 407 -> 103, pieces of whole tensors 84 -> 60.
+constexpr int kNormCtasPerSm = 6;
+template <int MODE>
+__global__ void __launch_bounds__(kRoundThreads, kNormCtasPerSm)
+norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+{
+    const bool tbl_in_smem = set_up(a, map);
+    if (tma::smem_addr(smem) & 1023u) {          // the swizzled tiles need a 1024-byte aligned base
+        if (threadIdx.x == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
+        return;
+    }
+    double square_sum = 0.0;
+    round_tiles<0, MODE, false>(a, &map, tbl_in_smem, square_sum);
+    if (a.with_rule)
+        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, 0, a.status);
+}
+
+template <int MODE, bool AVG>
+__global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
+round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+{
+    const bool tbl_in_smem = set_up(a, map);
+    const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
     uint32_t trouble = 0;
     if (tma::smem_addr(smem) & 1023u) trouble = DQ_STAT_INTERNAL;          // the swizzled tiles need a 1024-byte aligned base
     else if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
@@ -718,13 +764,11 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, b, a.status);
 }
 
-}  // namespace
 
-template <int MODE, bool AVG>
-int dq_launch_round(const RoundArgs& args, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+template <int MODE>
+int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, RoundArgs a, const CUtensorMap& map, int n_seg,
+                      int64_t entries, cudaStream_t st)
 {
-    RoundArgs a = args;
-    const auto kernel = round_kernel<MODE, AVG>;
     size_t smem_need = (size_t)kTblOffset;
     if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
@@ -733,12 +777,25 @@ int dq_launch_round(const RoundArgs& args, const CUtensorMap& map, int n_seg, in
     }
     // units of work per CTA: warps, or teams
     const int units = MODE == kTeamBuckets ? kRoundWarps >> (a.gpb_shift - 5) : kRoundWarps;
-    int64_t blocks = (int64_t)dq_sm_count() * RoundShape<AVG>::ctas_per_sm;
+    int64_t blocks = (int64_t)dq_sm_count() * ctas_per_sm;
     if (blocks * units > entries) blocks = (entries + units - 1) / units;
     a.each = (uint32_t)(entries / (blocks * units));
     a.extra = (uint32_t)(entries - (int64_t)a.each * blocks * units);
     dq_launch(kernel, dim3((unsigned)blocks), dim3(kRoundThreads), smem_need, st, a, map);
     return cudaGetLastError() == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+}
+
+}  // namespace
+
+template <int MODE>
+int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+{
+    return launch_persistent<MODE>(norms_kernel<MODE>, kNormCtasPerSm, a, map, n_seg, entries, st);
+}
+template <int MODE, bool AVG>
+int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+{
+    return launch_persistent<MODE>(round_kernel<MODE, AVG>, RoundShape<AVG>::ctas_per_sm, a, map, n_seg, entries, st);
 }
 
 #endif  // DQ_ROUND_KERNELS

@@ -1,0 +1,6 @@
+// The norm kernels of dq_round.cuh.
+#define DQ_ROUND_KERNELS
+#include "dq_round.cuh"
+
+template int dq_launch_norms<kWarpBuckets>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_norms<kTeamBuckets>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);

@@ -29,7 +29,7 @@ SYMBOLS = [
     "dq_bucket_norms", "dq_tensor_norms_scratch_bytes", "dq_tensor_norms", "dq_choose_bits_scratch_bytes", "dq_choose_bits",
     "dq_choose_bits_noalloc_max_norms", "dq_choose_bits_noalloc",
     "dq_quantize_pack", "dq_quantize_pack_worker", "dq_norms_quantize_pack", "dq_norms_quantize_pack_worker", "dq_unpack_dequant_average",
-    "dq_unpack_average_update", "dq_quantize_average", "dq_round_workspace_bytes", "dq_norms_quantize_average", "dq_status_string", "dq_debug_set_wait_limits",
+    "dq_unpack_average_update", "dq_norms_choose_bits", "dq_quantize_average", "dq_round_workspace_bytes", "dq_norms_quantize_average", "dq_status_string", "dq_debug_set_wait_limits",
 ]
 
 
@@ -123,6 +123,8 @@ def lib():
         L.dq_unpack_dequant_average.argtypes = [vp, vp, i64, vp, i32, vp, vp, vp, vp]
         L.dq_unpack_average_update.restype = C.c_int
         L.dq_unpack_average_update.argtypes = [vp, vp, i64, vp, i32, vp, C.c_float, vp, vp, vp]
+        L.dq_norms_choose_bits.restype = C.c_int
+        L.dq_norms_choose_bits.argtypes = [vp, vp, i64, i32, vp, C.POINTER(Rule), vp, vp, sz, vp, vp]
         L.dq_quantize_average.restype = C.c_int
         L.dq_quantize_average.argtypes = [vp, vp, i64, i32, vp, vp, u64, u32, vp, i64, vp, i32, C.c_float, vp, vp]
         L.dq_round_workspace_bytes.restype = sz
@@ -351,6 +353,13 @@ def quantize_average(layout: Layout, grads, worker_stride_elems: int, M: int, no
     _check(_step().quantize_average(layout._address, grads, worker_stride_elems, M, norms, dev_b, seed, step, packed,
                                     packed_stride_words, out, 0 if lr is None else 1, 0.0 if lr is None else lr,
                                     status, _stream(stream)), "dq_quantize_average")
+
+
+def norms_choose_bits(layout: Layout, grads, worker_stride_elems: int, M: int, norms, rule: Rule, dev_b, workspace,
+                      workspace_bytes: int, status, stream=None) -> None:
+    """Norms and the b they give in one call (``dq_norms_choose_bits``); ``workspace`` as for a whole round."""
+    _check(_step().norms_choose_bits(layout._address, grads, worker_stride_elems, M, norms, rule, dev_b, workspace,
+                                     workspace_bytes, status, _stream(stream)), "dq_norms_choose_bits")
 
 
 def round_workspace_bytes(layout: Layout, M: int) -> int:

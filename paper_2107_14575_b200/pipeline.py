@@ -89,8 +89,8 @@ class Round:
 
     def step(self, grads, rule: dq.Rule, seed: int, step: int) -> torch.Tensor:
         """Whole round on device gradients; returns the averaged gradient [D32] (device)."""
-        self.norms_(grads)
-        self.bits_(rule)
+        dq.norms_choose_bits(self.layout, grads, self.stride, self.M, self.norms, rule, self.dev_b, self._ws,
+                             self._ws_bytes, self.status)
         dq.quantize_average(self.layout, grads, self.stride, self.M, self.norms, self.dev_b, seed, step, self.packed,
                             self.packed_stride, self.out, self.status)
         return self.out

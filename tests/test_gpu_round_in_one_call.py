@@ -178,3 +178,27 @@ def test_many_tensors_of_every_size(G, n_seg, bucket):
     np.testing.assert_array_equal(r.g_packed.view.cpu().numpy().view(np.uint32).reshape(M, -1), packed)
     np.testing.assert_array_equal(r.g_out.view.cpu().numpy(), avg)
     assert r.read_status() == 0 and r.guards_intact()
+
+
+@pytest.mark.parametrize("segs,bucket,M", [(RAGGED, 512, 3), (RAGGED, 4096, 2), (RAGGED, 96, 3), (RAGGED, 0, 3), ([5], 32, 1),
+                                           ([1 << 20], 128, 4), ([33] * 1100, 64, 2)])
+def test_norms_and_rule_in_one_call(G, segs, bucket, M):
+    """dq_norms_choose_bits writes the norms of the separate calls and the b of dq_choose_bits, twice in a row."""
+    dq = G.dq
+    r = G.GpuRound(segs, bucket, M)
+    ref = oracle.Layout(segs, bucket if bucket else oracle.whole_tensor_bucket(segs))
+    r.set_grads(_grads(ref, segs, M, 3))
+    norms = r.norms().copy()
+    nbytes = dq.round_workspace_bytes(r.lay, M)
+    ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+    # x half a level away from every s(b): the two fp64 sums are taken in different orders and differ by up to
+    # n * 2^-53, about 1e-12 of x, so that an x on a threshold could fall on either side
+    for x in (2.5, 100.5):
+        rule = dq.Rule.dynamic(10, 0, 10 * float((norms.astype(np.float64) ** 2).sum()) / M / x ** 2, 1.0)
+        want = r.bits(rule)
+        r.g_norms.view.fill_(-1.0)
+        r.set_b(1)
+        dq.norms_choose_bits(r.lay, r.grads, r.stride, M, r.g_norms.view, rule, r.g_b.view, ws, nbytes, r.status)
+        np.testing.assert_array_equal(r.g_norms.view.cpu().numpy().reshape(M, -1), norms)
+        assert tuple(r.g_b.view.cpu().tolist()) == want
+    assert r.read_status() == 0 and r.guards_intact()
