@@ -25,8 +25,10 @@ OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdq.so")
 
 SOURCES = ["dq_layout.cu", "dq_tma.cu", "dq_norms.cu", "dq_bits.cu", "dq_quantize.cu", "dq_unpack.cu",
-           "dq_round_warp_encode.cu", "dq_round_warp_average.cu", "dq_round_team_encode.cu", "dq_round_team_average.cu",
-           "dq_round_given_encode.cu", "dq_round_given_average.cu", "dq_round_norms.cu"]
+           "dq_round_warp_encode.cu", "dq_round_warp_encode_linf.cu", "dq_round_warp_average.cu",
+           "dq_round_warp_average_linf.cu", "dq_round_team_encode.cu", "dq_round_team_encode_linf.cu",
+           "dq_round_team_average.cu", "dq_round_team_average_linf.cu", "dq_round_given_encode.cu",
+           "dq_round_given_average.cu", "dq_round_norms.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 

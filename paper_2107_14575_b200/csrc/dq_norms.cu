@@ -27,6 +27,16 @@ int64_t dq_tile_positions(const RoundArgs& a, bool given)
     return (a.v.nb + R - 1) / R;
 }
 
+int dq_norms_of_buckets(const RoundArgs& a, const CUtensorMap& map, int n_seg, cudaStream_t st)
+{
+    const int64_t entries = dq_tile_positions(a, false) * a.M;
+    if (a.gpb_shift <= 5)
+        return a.linf ? dq_launch_norms<kWarpBuckets, true>(a, map, n_seg, entries, st)
+                      : dq_launch_norms<kWarpBuckets, false>(a, map, n_seg, entries, st);
+    return a.linf ? dq_launch_norms<kTeamBuckets, true>(a, map, n_seg, entries, st)
+                  : dq_launch_norms<kTeamBuckets, false>(a, map, n_seg, entries, st);
+}
+
 bool dq_fill_round(RoundArgs& a, CUtensorMap& map, const dq_layout_t* L, const LayoutView& v, const float* dev_grads,
                    int64_t worker_stride_elems, int32_t M, int32_t* dev_status)
 {
@@ -363,9 +373,7 @@ int launch_norms(const dq_layout_t* L, const LayoutView& v, const float* dev_gra
     CUtensorMap map;
     if (!dq_fill_round(a, map, L, v, dev_grads, worker_stride_elems, M, dev_status)) return DQ_ERR_CUDA;
     a.norms = dev_out;
-    const int64_t entries = dq_tile_positions(a, false) * M;
-    return a.gpb_shift <= 5 ? dq_launch_norms<kWarpBuckets>(a, map, L->n_seg, entries, st)
-                            : dq_launch_norms<kTeamBuckets>(a, map, L->n_seg, entries, st);
+    return dq_norms_of_buckets(a, map, L->n_seg, st);
 }
 
 // other bucket sizes: plain-load kernels

@@ -50,9 +50,12 @@ template <bool AVG>
 int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, bool given, cudaStream_t st)
 {
     const int64_t entries = dq_tile_positions(a, given) * (AVG ? 1 : a.M);
-    if (given) return dq_launch_round<kGivenNorms, AVG>(a, map, L->n_seg, entries, st);
-    if (a.gpb_shift <= 5) return dq_launch_round<kWarpBuckets, AVG>(a, map, L->n_seg, entries, st);
-    return dq_launch_round<kTeamBuckets, AVG>(a, map, L->n_seg, entries, st);
+    if (given) return dq_launch_round<kGivenNorms, AVG, false>(a, map, L->n_seg, entries, st);
+    if (a.gpb_shift <= 5)
+        return a.linf ? dq_launch_round<kWarpBuckets, AVG, true>(a, map, L->n_seg, entries, st)
+                      : dq_launch_round<kWarpBuckets, AVG, false>(a, map, L->n_seg, entries, st);
+    return a.linf ? dq_launch_round<kTeamBuckets, AVG, true>(a, map, L->n_seg, entries, st)
+                  : dq_launch_round<kTeamBuckets, AVG, false>(a, map, L->n_seg, entries, st);
 }
 
 // One pass for codes and average, or codes (all workers' tiles side by side) and then the average from
@@ -202,9 +205,7 @@ extern "C" int dq_norms_choose_bits(const dq_layout_t* L, const float* dev_grads
         a.norms = dev_norms;
         a.dev_b = dev_b;
         attach_rule(a, rule, M, ws);
-        const int64_t entries = dq_tile_positions(a, false) * M;
-        return a.gpb_shift <= 5 ? dq_launch_norms<kWarpBuckets>(a, map, L->n_seg, entries, static_cast<cudaStream_t>(stream))
-                                : dq_launch_norms<kTeamBuckets>(a, map, L->n_seg, entries, static_cast<cudaStream_t>(stream));
+        return dq_norms_of_buckets(a, map, L->n_seg, static_cast<cudaStream_t>(stream));
     }
     char* scratch = ws + rule_workspace_bytes();
     const size_t choose = dq_choose_bits_scratch_bytes(L, M);

@@ -41,7 +41,7 @@ struct RoundArgs {
     uint32_t div_magic;           // kGivenNorms: groups_per_bucket as multiply-shift, or as a shift if a power of two
     int32_t div_shift;            //              (>= 0: the shift; < 0: use div_magic with a 33-bit shift)
     int32_t stream_reads;         // 1: more than 64 MB of gradients (see the L2 policy of the reads)
-    int32_t linf;                 // norm kind
+    int32_t linf;                 // norm kind (host: which kernel)
     int32_t update;               // AVG: out <- out + neg_lr * average instead of out <- average
     int32_t wide_words;           // packed rows start on 32-byte boundaries: 32-byte stores allowed
     int32_t wide_out;             // out starts on a 32-byte boundary
@@ -54,10 +54,10 @@ struct RoundArgs {
 
 // Launch of one of the kernels (each in a translation unit of its own): norms alone, or codes with or
 // without the average.  `entries`: length of the list of work (see round_tiles).
-template <int MODE>
+template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
-template <int MODE, bool AVG>
-int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t tiles, cudaStream_t st);
+template <int MODE, bool AVG, bool LINF>
+int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 
 // CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower); 102 without them
 // (codes of 2^24 elements, b = 6: 17.4 us with five CTAs, 18.1 with six of 80 registers, 18.7 with four; buckets of
@@ -80,6 +80,8 @@ bool dq_fill_round(RoundArgs& a, CUtensorMap& map, const dq_layout_t* L, const L
                    int64_t worker_stride_elems, int32_t M, int32_t* dev_status);
 // Whether the kernels take the norms of a layout's buckets themselves.
 bool dq_norms_inside(const dq_layout_t* L);
+// The norm kernel over the buckets `a` describes.
+int dq_norms_of_buckets(const RoundArgs& a, const CUtensorMap& map, int n_seg, cudaStream_t st);
 // Positions of a worker's tiles; given: those of kGivenNorms.
 int64_t dq_tile_positions(const RoundArgs& a, bool given);
 
@@ -87,25 +89,28 @@ int64_t dq_tile_positions(const RoundArgs& a, bool given);
 
 namespace {
 
-constexpr int kStages = 2;
 constexpr int kTileBytes = 32 * 128;
 constexpr int kMaxSmemSegs = 1023;
+
+constexpr int kStages = 2;                          // per warp: a tile being encoded and one on its way
 
 // Dynamic shared memory, addressed only through this symbol so that every access compiles to a
 // shared-memory instruction:
 //   [0, kWarps * kStages * 4 KB)  input tiles, warp-major (1024-byte aligned for the swizzle)
 //   (a consumed tile doubles as the staging area of its words where they do not leave straight from
-//   registers), then the stage barriers, the teams' exchange slots, the rule's partial sums, and the
-//   tensor table
+//   registers), then the stage barriers, the teams' exchange slots ([2 parities][4 warps] of {partial,
+//   lost}), the rule's partial sums and its last-CTA word, and the tensor table
 extern __shared__ __align__(1024) unsigned char smem[];
-constexpr int kBarOffset = kRoundWarps * kStages * kTileBytes;
-constexpr int kPartOffset = kBarOffset + kRoundWarps * kStages * 8;         // [2 parities][4 warps] of {partial, lost}
-constexpr int kSumOffset = kPartOffset + 2 * kRoundWarps * 8;                // 4 doubles + the last-CTA word
-constexpr int kTblOffset = kSumOffset + kRoundWarps * 8 + 16;
+struct SmemMap {
+    static constexpr int bars = kRoundWarps * kStages * kTileBytes;
+    static constexpr int slots = bars + kRoundWarps * kStages * 8;
+    static constexpr int sums = slots + 2 * kRoundWarps * 8;
+    static constexpr int table = sums + kRoundWarps * 8 + 16;
+};
 
 __device__ __forceinline__ uint64_t* stage_bar(int warp, int st)
 {
-    return reinterpret_cast<uint64_t*>(smem + kBarOffset) + warp * kStages + st;
+    return reinterpret_cast<uint64_t*>(smem + SmemMap::bars) + warp * kStages + st;
 }
 __device__ __forceinline__ unsigned char* stage_ptr(int warp, int st) { return smem + (warp * kStages + st) * kTileBytes; }
 
@@ -194,20 +199,26 @@ __device__ __noinline__ void clear_row_tail(const uint32_t row, const int valid)
     __syncwarp();
 }
 
-// Lanes (and a team's warps) of a bucket combine their v; the result is the same in all of them.
-// A warp that lost a wait says so in its slot: `lost` is then set in every warp of the team.
+// The lanes of a bucket combine their v; the result is the same in all of them.
 template <int MODE, class Op>
-__device__ __forceinline__ float join_bucket(float v, const int gpb, const int T_shift, uint32_t& exchanges, const bool landed,
-                                             bool& lost, const Op& op)
+__device__ __forceinline__ float join_lanes(float v, const int gpb, const Op& op)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const float other = op(v, __shfl_xor_sync(0xffffffffu, v, o));
-        v = (MODE == kTeamBuckets || o < gpb) ? other : v;
+        const float other = __shfl_xor_sync(0xffffffffu, v, o);
+        if (MODE == kTeamBuckets || o < gpb) v = op(v, other);
     }
+    return v;
+}
+// ... and so do the warps of a team.  A warp that lost a wait says so in its slot: `lost` is then set in
+// every warp of the team.  slots: float2[2][kRoundWarps], the exchanges of even and of odd number.
+template <int MODE, class Op>
+__device__ __forceinline__ float join_team(float v, float2* slots, const int T_shift, uint32_t& exchanges, const bool landed,
+                                           bool& lost, const Op& op)
+{
     if constexpr (MODE == kTeamBuckets) {
         const int warp = threadIdx.x >> 5, T = 1 << T_shift;
-        float2* slots = reinterpret_cast<float2*>(smem + kPartOffset) + (exchanges & 1u) * kRoundWarps;
+        slots += (exchanges & 1u) * kRoundWarps;
         ++exchanges;
         if ((threadIdx.x & 31) == 0) slots[warp] = make_float2(v, landed ? 0.0f : 1.0f);
         // (numbers the assembler sees: a number from a register reserves all sixteen barriers for the CTA, and
@@ -224,6 +235,8 @@ __device__ __forceinline__ float join_bucket(float v, const int gpb, const int T
 }
 struct AddOp { __device__ __forceinline__ float operator()(const float a, const float b) const { return a + b; } };
 struct MaxOp { __device__ __forceinline__ float operator()(const float a, const float b) const { return max_nan(a, b); } };
+template <bool LINF> struct JoinOp { using type = AddOp; };
+template <> struct JoinOp<true> { using type = MaxOp; };
 
 // The l2 norm of buckets whose sum of squares is out of range (see l2_sum_in_range): all zeros, tiny
 // entries, an overflowed square.  Called by all lanes of the warp (by all warps of a team, which agree
@@ -231,12 +244,12 @@ struct MaxOp { __device__ __forceinline__ float operator()(const float a, const 
 // their entries scaled, and lanes whose own bucket was in range keep `nrm`.  Always two exchanges of a
 // team.  Out of line: it is rare, and the common case does not pay for its registers.
 template <int MODE>
-__device__ __noinline__ float rare_norm(const uint32_t row, const int valid, const int gpb, const int T_shift, uint32_t exchanges,
-                                        const float sum, const float nrm)
+__device__ __noinline__ float rare_norm(const uint32_t row, const int valid, const int gpb, float2* slots, const int T_shift,
+                                        uint32_t exchanges, const float sum, const float nrm)
 {
     bool lost = false;
     float mx = valid > 0 ? row_max(row) : 0.0f;          // (a partial row's tail is zero by now)
-    mx = join_bucket<MODE>(mx, gpb, T_shift, exchanges, true, lost, MaxOp{});
+    mx = join_team<MODE>(join_lanes<MODE>(mx, gpb, MaxOp{}), slots, T_shift, exchanges, true, lost, MaxOp{});
     const bool again = !l2_sum_in_range(sum);
     float scaled = 0.0f;
     const int e = scale_exponent(mx);
@@ -250,7 +263,7 @@ __device__ __noinline__ float rare_norm(const uint32_t row, const int valid, con
             chain = red.take(chain, x.x); chain = red.take(chain, x.y); chain = red.take(chain, x.z); chain = red.take(chain, x.w);
         }
         scaled = valid == 32 ? (a0 + a1) + (a2 + a3) : (valid > 0 ? chain : 0.0f);
-        scaled = join_bucket<MODE>(scaled, gpb, T_shift, exchanges, true, lost, AddOp{});
+        scaled = join_team<MODE>(join_lanes<MODE>(scaled, gpb, AddOp{}), slots, T_shift, exchanges, true, lost, AddOp{});
     }
     return again ? (magnitude_scalable(mx) ? rescaled_l2(mx, scaled, e) : mx) : nrm;
 }
@@ -287,10 +300,12 @@ __device__ __forceinline__ void store_row(const RoundArgs& a, float* dst, const 
     }
 }
 
-template <int B, int MODE, bool AVG>
+template <int B, int MODE, bool AVG, bool LINF>
 __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
 {
-    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
+    using Join = typename JoinOp<LINF>::type;
+    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + SmemMap::table);
+    float2* slots = reinterpret_cast<float2*>(smem + SmemMap::slots);
     auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
     constexpr int s = B > 0 ? (1 << (B > 0 ? B - 1 : 0)) - 1 : 0;
     const float sf = (float)s;
@@ -458,19 +473,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     int p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
     const uint32_t stage0 = tma::smem_addr(smem) + warp * (kStages * kTileBytes);
     const uint32_t bar0 = tma::smem_addr(stage_bar(warp, 0));
-    // Copies in flight.  A team's warp has no tile of some buckets, so it counts the copies that landed
-    // in each stage; the others find a stage's parity in the item's number.
-    bool flying0 = false, flying1 = false;
-    uint32_t fills0 = 0, fills1 = 0;
-    auto stage_parity = [&](uint32_t item) -> uint32_t {
-        if constexpr (MODE == kTeamBuckets) return ((item & 1u) ? fills1 : fills0) & 1u;
-        else return (item >> 1) & 1u;
-    };
-    auto seen_to_land = [&](int st) {
-        if constexpr (MODE == kTeamBuckets) {
-            if (st) { ++fills1; flying1 = false; } else { ++fills0; flying0 = false; }
-        }
-    };
+    // A team's warp has no tile of some buckets, so it keeps the parity of each stage's next copy and which
+    // copies are on their way, a bit each; the others find the parity by counting.
+    uint32_t parities = 0, flying = 0;
     auto move_producer = [&]() {
         p_first = describe(p_pos);
         p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu);
@@ -484,7 +489,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             else queue2 = p_first;
             ++queued;
         }
-        if (MODE == kTeamBuckets && p_first != kNoTile) { if (st) flying1 = true; else flying0 = true; }
+        if (MODE == kTeamBuckets && p_first != kNoTile) flying |= 1u << st;
         if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile))
             tma::fetch_tile(stage0 + st * kTileBytes, map, bar0 + st * 8, kTileBytes, p_row, p_worker, policy);
         if (AVG) {
@@ -509,6 +514,15 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     // (test hook: the warp's first wait counts as lost, and the warp goes straight to what follows a time-out)
     const bool skip_all = a.wait.lose_first != 0u && items > 0;
     int m = m_first;
+    // Every lane polls the barrier itself; the verdict is made warp-uniform so that the warp-level
+    // synchronisations are always reached by all lanes or by none.
+    auto wait_for = [&](int stage) -> bool {
+        const uint32_t par = MODE == kTeamBuckets ? (parities >> stage) & 1u : (it >> 1) & 1u;
+        const bool landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar0 + stage * 8, par)) ||
+                            __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, stage), par, a.wait));
+        if (MODE == kTeamBuckets && landed) { parities ^= 1u << stage; flying &= ~(1u << stage); }
+        return landed;
+    };
 
     for (int ip = 0; ip < n_pos && !skip_all; ++ip) {
         const TilePos t = locate(pos, AVG ? describe(pos) : queue0);
@@ -529,27 +543,47 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             if (t.valid > 0) norm_next = load_norm_early(norm_ptr);
         }
 
+        // The norm of a tile: the lane's share from its row, ...
+        auto row_share = [&](uint32_t row) -> float {
+            float v = LINF ? row_max(row) : row_sum_squares(row);
+            if (!t.regular) v = irregular_row_sum(row, t.valid, v, LINF ? 1 : 0);
+            return v;
+        };
+        // ... the norm and its scale from the bucket's sum (or maximum) `v`, ...
+        float nrm = 0.0f, inv = 0.0f;
+        bool plain = false;                      // no zero bucket, no norm outside the normal range
+        auto scale_of = [&](float v) {
+            nrm = LINF ? v : sqrt_normal(v);
+            inv = inv_scale_normal(sf, nrm);
+        };
+        // ... and what remains: the buckets out of range, and the norm written.  Rarely a bucket's sum of squares
+        // is out of range (see l2_sum_in_range): all zeros, tiny entries, an overflowed square.
+        auto settle = [&](float v, uint32_t row, float* dst) {
+            plain = !__any_sync(0xffffffffu, LINF ? !norm_is_plain(v) : !l2_sum_in_range(v));
+            if (!plain) {
+                if constexpr (!LINF) {
+                    nrm = rare_norm<MODE>(row, t.valid, gpb, slots, T_shift, exchanges, v, nrm);
+                    exchanges += 2;
+                }
+                inv = inv_scale(sf, nrm);
+                bad |= t.writes && !isfinite(nrm);
+            }
+            if (t.writes) {
+                DQ_STORE(dst, nrm, a.norms, (int64_t)M * nb * 4, a.status);
+                square_sum = fma((double)nrm, (double)nrm, square_sum);
+            }
+            __syncwarp();
+        };
+
         const int workers = AVG ? M : 1;
 #pragma unroll 1
         for (int j = 0; j < workers; ++j, norm_ptr += nb, tile_words += a.packed_stride) {
             const int mm = AVG ? j : m;
-            const int st = it & 1;
-            bool landed = true;
-            if (has_tile) {
-                // every lane polls the barrier itself; the verdict is made warp-uniform so that the
-                // warp-level synchronisations below are always reached by all lanes or by none
-                landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar0 + st * 8, stage_parity(it))) ||
-                         __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), stage_parity(it), a.wait));
-                if (landed) seen_to_land(st);
-            }
-            if (MODE != kTeamBuckets && !landed) { timed_out = true; break; }
-
+            const int st = (int)(it & 1u);
             const uint32_t row = (uint32_t)((warp * kStages + st) * kTileBytes) + own;
+            const bool landed = !has_tile || wait_for(st);
+            if (MODE != kTeamBuckets && !landed) { timed_out = true; break; }
             if (!t.regular && has_tile && landed) clear_row_tail(row, t.valid);
-
-            // ---- norm of the bucket
-            float nrm, inv;
-            bool plain = false;                  // no zero bucket, no norm outside the normal range
             if constexpr (MODE == kGivenNorms) {
                 nrm = norm_next;
                 inv = inv_scale_normal(sf, nrm);
@@ -558,102 +592,79 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 if (AVG && j + 1 < workers && t.valid > 0) norm_next = load_norm_early(norm_ptr + nb);
                 if (t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
             } else {
-                bool team_lost = false;
-                if (a.linf) {
-                    nrm = row_max(row);
-                    if (!t.regular) nrm = irregular_row_sum(row, t.valid, nrm, 1);
-                    nrm = join_bucket<MODE>(nrm, gpb, T_shift, exchanges, landed, team_lost, MaxOp{});
-                    inv = inv_scale_normal(sf, nrm);
-                    plain = !__any_sync(0xffffffffu, !norm_is_plain(nrm));
-                    if (!plain) inv = inv_scale(sf, nrm);
-                } else {
-                    float sum = row_sum_squares(row);
-                    if (!t.regular) sum = irregular_row_sum(row, t.valid, sum, 0);
-                    sum = join_bucket<MODE>(sum, gpb, T_shift, exchanges, landed, team_lost, AddOp{});
-                    nrm = sqrt_normal(sum);
-                    inv = inv_scale_normal(sf, nrm);
-                    plain = !__any_sync(0xffffffffu, !l2_sum_in_range(sum));
-                    if (!plain && !team_lost) {
-                        nrm = rare_norm<MODE>(row, t.valid, gpb, T_shift, exchanges, sum, nrm);
-                        exchanges += 2;
-                        inv = inv_scale(sf, nrm);
-                    }
-                }
-                if (team_lost) { timed_out = true; break; }
-                if (t.writes) {
-                    DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
-                    square_sum = fma((double)nrm, (double)nrm, square_sum);
-                }
-                if (!plain) bad |= t.writes && !isfinite(nrm);
-                __syncwarp();
+                bool lost = false;
+                const float v = join_team<MODE>(join_lanes<MODE>(row_share(row), gpb, Join{}), slots, T_shift, exchanges, landed,
+                                                lost, Join{});
+                if (lost) { timed_out = true; break; }
+                scale_of(v);
+                settle(v, row, norm_ptr);
             }
-            if (!has_tile) { fetch(st); ++it; continue; }
-            if constexpr (B == 0) {              // norms alone: the row has been read (see the refill below)
+            if (!has_tile) {
+                fetch(st);
+            } else if constexpr (B == 0) {       // norms alone: the row has been read (see the refill below)
                 tma::fence_proxy_async();
                 __syncwarp();
                 fetch(st);
-                ++it;
-                __syncwarp();
             } else {
-
-            // ---- codes of the row against that norm, and the lane's share of the average
-            uint32_t words[B > 0 ? B : 1];
-            if constexpr (B == 1) {
-                words[0] = 0u;
-            } else if (!plain && __all_sync(0xffffffffu, nrm == 0.0f)) {
-                // sparse gradients are full of zero buckets: every code is s, whatever the draw, and adds 0 to the average
-                zero_group_words<B>(words);
-            } else {
-                const uint64_t inv2 = pack_pair(__float_as_uint(inv), __float_as_uint(inv));
+                // ---- codes of the row against that norm, and the lane's share of the average
+                uint32_t words[B];
                 const float scale = nrm * to_unit;
+                const uint64_t inv2 = pack_pair(__float_as_uint(inv), __float_as_uint(inv));
                 const uint64_t scale2 = pack_pair(__float_as_uint(scale), __float_as_uint(scale));
-                encode_row<B, AVG>([row](int c) { return row_quad(row, c); }, inv2, scale2, acc2, words, q0, (uint32_t)mm + a.worker0, a.step, a.keys);
-            }
+                if constexpr (B == 1) {
+                    words[0] = 0u;
+                } else if (!plain && __all_sync(0xffffffffu, nrm == 0.0f)) {
+                    // sparse gradients are full of zero buckets: every code is s, whatever the draw, and adds 0 to the average
+                    zero_group_words<B>(words);
+                } else {
+                    encode_row<B, AVG>([row](int c) { return row_quad(row, c); }, inv2, scale2, acc2, words, q0,
+                                       (uint32_t)mm + a.worker0, a.step, a.keys);
+                }
 
-            // ---- words out, the stage refilled.  The fence orders the warp's accesses to the stage before the copy's
-            // writes (they go through different proxies, and a read waits its turn in the load queue after it was issued).
-            const int64_t extent = (int64_t)M * a.packed_stride * 4;
-            if constexpr (StoresDirectly<B>::value) {
-                tma::fence_proxy_async();
-                __syncwarp();
-                fetch(st);
-                // a lane's words are whole 4-, 8- or 16-byte units of the stream: neighbouring lanes fill sectors
-                if (t.valid > 0) store_words<B>(tile_words + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
-            } else {
-                __syncwarp();                    // the warp has read all of its rows
-                uint32_t* out_words = reinterpret_cast<uint32_t*>(stage_ptr(warp, st));
-                // the staging area keeps the 16-byte phase of the output stream; whole quads move 16 bytes per
-                // lane, the ragged ends word by word
-                const int off = (int)(((int64_t)t.row0 * B) & 3);
-                uint32_t* aligned_dst = tile_words - off;
-                if (t.valid > 0) {
+                // ---- words out, the stage refilled.  The fence orders the warp's accesses to the stage before the copy's
+                // writes (they go through different proxies, and a read waits its turn in the load queue after it was issued).
+                const int64_t extent = (int64_t)M * a.packed_stride * 4;
+                if constexpr (StoresDirectly<B>::value) {
+                    tma::fence_proxy_async();
+                    __syncwarp();
+                    fetch(st);
+                    // a lane's words are whole 4-, 8- or 16-byte units of the stream: neighbouring lanes fill sectors
+                    if (t.valid > 0) store_words<B>(tile_words + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
+                } else {
+                    __syncwarp();                // the warp has read all of its rows
+                    uint32_t* out_words = reinterpret_cast<uint32_t*>(stage_ptr(warp, st));
+                    // the staging area keeps the 16-byte phase of the output stream; whole quads move 16 bytes per
+                    // lane, the ragged ends word by word
+                    const int off = (int)(((int64_t)t.row0 * B) & 3);
+                    uint32_t* aligned_dst = tile_words - off;
+                    if (t.valid > 0) {
 #pragma unroll
-                    for (int i = 0; i < B; ++i) out_words[off + t.row * B + i] = words[i];
-                }
-                __syncwarp();
-                const int jend = off + t.span * B;
-                const int f0 = off ? 1 : 0, f1 = jend >> 2;          // full quads [f0, f1)
+                        for (int i = 0; i < B; ++i) out_words[off + t.row * B + i] = words[i];
+                    }
+                    __syncwarp();
+                    const int jend = off + t.span * B;
+                    const int f0 = off ? 1 : 0, f1 = jend >> 2;          // full quads [f0, f1)
 #pragma unroll
-                for (int i = 0; i < (8 * B + 31) / 32; ++i) {
-                    const int q = lane + 32 * i;
-                    if (q >= f0 && q < f1)
-                        DQ_STORE(reinterpret_cast<uint4*>(aligned_dst) + q, reinterpret_cast<const uint4*>(out_words)[q],
-                                 a.packed, extent, a.status);
+                    for (int i = 0; i < (8 * B + 31) / 32; ++i) {
+                        const int q = lane + 32 * i;
+                        if (q >= f0 && q < f1)
+                            DQ_STORE(reinterpret_cast<uint4*>(aligned_dst) + q, reinterpret_cast<const uint4*>(out_words)[q],
+                                     a.packed, extent, a.status);
+                    }
+                    if (off | (jend & 3)) {
+                        if (off && lane >= off && lane < 4 && lane < jend)                                        // head
+                            DQ_STORE(aligned_dst + lane, out_words[lane], a.packed, extent, a.status);
+                        int ts = f1 * 4;                                                                          // tail
+                        if (off && ts < 4) ts = 4;
+                        if (lane < jend - ts) DQ_STORE(aligned_dst + (ts + lane), out_words[ts + lane], a.packed, extent, a.status);
+                    }
+                    tma::fence_proxy_async();
+                    __syncwarp();
+                    fetch(st);
                 }
-                if (off | (jend & 3)) {
-                    if (off && lane >= off && lane < 4 && lane < jend)                                        // head
-                        DQ_STORE(aligned_dst + lane, out_words[lane], a.packed, extent, a.status);
-                    int ts = f1 * 4;                                                                          // tail
-                    if (off && ts < 4) ts = 4;
-                    if (lane < jend - ts) DQ_STORE(aligned_dst + (ts + lane), out_words[ts + lane], a.packed, extent, a.status);
-                }
-                tma::fence_proxy_async();
                 __syncwarp();
-                fetch(st);
             }
             ++it;
-            __syncwarp();
-            }
         }
         if (timed_out) break;
 
@@ -673,8 +684,8 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
         } else {
             pos += hop;
             while (pos >= positions) { pos -= positions; ++m; }
+            queue0 = queue1; queue1 = queue2; --queued;
         }
-        if (!AVG) { queue0 = queue1; queue1 = queue2; --queued; }
     }
     if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
     if (timed_out || skip_all) {
@@ -682,11 +693,11 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
         // every copy the warp has issued and not seen land, the one whose wait ran out included, gets the
         // full limit before the CTA's shared memory is released
         if constexpr (MODE == kTeamBuckets) {
-            if (flying0) (void)tma::mbar_wait(stage_bar(warp, 0), fills0 & 1u, a.wait);
-            if (flying1) (void)tma::mbar_wait(stage_bar(warp, 1), fills1 & 1u, a.wait);
+            for (int i = 0; i < kStages; ++i)
+                if ((flying >> i) & 1u) (void)tma::mbar_wait(stage_bar(warp, i), (parities >> i) & 1u, a.wait);
         } else {
             for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
-                (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), stage_parity(i), a.wait);
+                (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
         }
     }
 }
@@ -703,7 +714,7 @@ __device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& ma
     grid_dependency_wait();
     const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
     if (tbl_in_smem) {
-        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + kTblOffset);
+        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + SmemMap::table);
         for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
     }
     __syncthreads();
@@ -714,7 +725,7 @@ __device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& ma
 // per tile (three CTAs of 128 threads per SM): ResNet-18 shape M = 8 72 -> 57 us (6.3 TB/s), VGG-16 shape M = 16,
 // bucket 2048, 191 -> 150, text shape with its zero rows 407 -> 103, pieces of whole tensors 84 -> 60.
 constexpr int kNormCtasPerSm = 6;
-template <int MODE>
+template <int MODE, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, kNormCtasPerSm)
 norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
@@ -724,12 +735,12 @@ norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         return;
     }
     double square_sum = 0.0;
-    round_tiles<0, MODE, false>(a, &map, tbl_in_smem, square_sum);
+    round_tiles<0, MODE, false, LINF>(a, &map, tbl_in_smem, square_sum);
     if (a.with_rule)
-        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, 0, a.status);
+        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + SmemMap::sums), a.dev_b, 0, a.status);
 }
 
-template <int MODE, bool AVG>
+template <int MODE, bool AVG, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
 round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
@@ -743,14 +754,14 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
         // nothing is written but the next b, which follows from the norms that are there
         if (a.with_rule)
-            rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + kSumOffset),
+            rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + SmemMap::sums),
                                        a.dev_b, b, a.status);
         return;
     }
 
     double square_sum = 0.0;
     switch (b) {
-#define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG>(a, &map, tbl_in_smem, square_sum); break;
+#define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG, LINF>(a, &map, tbl_in_smem, square_sum); break;
 #ifdef DQ_ONLY_B
         DQ_CASE(DQ_ONLY_B)
 #else
@@ -761,7 +772,7 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         default: break;
     }
     if (a.with_rule)
-        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + kSumOffset), a.dev_b, b, a.status);
+        rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + SmemMap::sums), a.dev_b, b, a.status);
 }
 
 
@@ -769,7 +780,7 @@ template <int MODE>
 int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, RoundArgs a, const CUtensorMap& map, int n_seg,
                       int64_t entries, cudaStream_t st)
 {
-    size_t smem_need = (size_t)kTblOffset;
+    size_t smem_need = (size_t)SmemMap::table;
     if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -787,15 +798,16 @@ int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, R
 
 }  // namespace
 
-template <int MODE>
+template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<MODE>(norms_kernel<MODE>, kNormCtasPerSm, a, map, n_seg, entries, st);
+    return launch_persistent<MODE>(norms_kernel<MODE, LINF>, kNormCtasPerSm, a, map, n_seg, entries, st);
 }
-template <int MODE, bool AVG>
+template <int MODE, bool AVG, bool LINF>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<MODE>(round_kernel<MODE, AVG>, RoundShape<AVG>::ctas_per_sm, a, map, n_seg, entries, st);
+    return launch_persistent<MODE>(round_kernel<MODE, AVG, LINF>, RoundShape<AVG>::ctas_per_sm, a, map,
+                                                               n_seg, entries, st);
 }
 
 #endif  // DQ_ROUND_KERNELS

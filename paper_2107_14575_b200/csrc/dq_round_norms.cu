@@ -2,5 +2,7 @@
 #define DQ_ROUND_KERNELS
 #include "dq_round.cuh"
 
-template int dq_launch_norms<kWarpBuckets>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
-template int dq_launch_norms<kTeamBuckets>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_norms<kWarpBuckets, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_norms<kWarpBuckets, true>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_norms<kTeamBuckets, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_norms<kTeamBuckets, true>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);

@@ -1,5 +1,5 @@
-// The quantize-and-average kernel of dq_round.cuh for buckets of 2048 and 4096 elements.
+// The quantize-and-average kernel of dq_round.cuh for buckets of 2048 and 4096 elements, l2 norms.
 #define DQ_ROUND_KERNELS
 #include "dq_round.cuh"
 
-template int dq_launch_round<kTeamBuckets, true>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_round<kTeamBuckets, true, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);

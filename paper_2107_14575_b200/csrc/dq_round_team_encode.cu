@@ -1,5 +1,5 @@
-// The quantizer kernel of dq_round.cuh for buckets of 2048 and 4096 elements.
+// The quantizer kernel of dq_round.cuh for buckets of 2048 and 4096 elements, l2 norms.
 #define DQ_ROUND_KERNELS
 #include "dq_round.cuh"
 
-template int dq_launch_round<kTeamBuckets, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_round<kTeamBuckets, false, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);

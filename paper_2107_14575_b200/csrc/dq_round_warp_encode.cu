@@ -1,5 +1,5 @@
-// The quantizer kernel of dq_round.cuh for buckets of up to 1024 elements.
+// The quantizer kernel of dq_round.cuh for buckets of up to 1024 elements, l2 norms.
 #define DQ_ROUND_KERNELS
 #include "dq_round.cuh"
 
-template int dq_launch_round<kWarpBuckets, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_round<kWarpBuckets, false, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
