@@ -420,22 +420,27 @@ __device__ __forceinline__ void store_wide(float* p, const float (&r)[8], const 
     store_wide_bits(p, v, base, extent, status);
 }
 
-// Words that leave straight from registers: a lane's B words start on a boundary of their own size
-// (1, 2, 4 words) or are whole 16-byte units, so neighbouring lanes fill whole sectors.  The other
-// widths go through shared memory.
+// Words that leave straight from registers, by 4-, 8-, 16- or 32-byte stores: a tile's words are one
+// contiguous span, the L2 puts partial sectors together, and staging them in shared memory costs some
+// sixty instructions a tile.  From nine words on the scattered stores cost more.  Measured, staged / straight
+// (us): 2^24 elements M = 32, b = 3 510 / 492, b = 5 515 / 502, b = 6 520 / 510, b = 7 551 / 536, b = 11
+// 570 / 597, b = 14 598 / 617, b = 15 613 / 979.  (One bulk copy of the staged words instead of 16-byte
+// stores by all lanes: 2 % slower than those.)
 template <int B>
 struct StoresDirectly {
-    static constexpr bool value = B <= 2 || B % 4 == 0;
+    static constexpr bool value = B <= 8 || B % 4 == 0;
 };
 template <int B>
 __device__ __forceinline__ void store_words(uint32_t* dst, const uint32_t (&w)[B], const bool wide, const void* base,
                                             const int64_t extent, int32_t* status)
 {
     (void)wide;
-    if constexpr (B == 1) {
-        DQ_STORE(dst, w[0], base, extent, status);
-    } else if constexpr (B == 2) {
-        DQ_STORE(reinterpret_cast<uint2*>(dst), make_uint2(w[0], w[1]), base, extent, status);
+    if constexpr (B % 2 != 0) {
+#pragma unroll
+        for (int i = 0; i < B; ++i) DQ_STORE(dst + i, w[i], base, extent, status);
+    } else if constexpr (B % 4 != 0) {
+#pragma unroll
+        for (int i = 0; i < B / 2; ++i) DQ_STORE(reinterpret_cast<uint2*>(dst) + i, make_uint2(w[2 * i], w[2 * i + 1]), base, extent, status);
     } else {
         if constexpr (B % 8 == 0) {
             if (wide) {                          // 32-byte stores: whole sectors from one lane

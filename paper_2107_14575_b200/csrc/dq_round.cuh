@@ -628,7 +628,6 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                     tma::fence_proxy_async();
                     __syncwarp();
                     fetch(st);
-                    // a lane's words are whole 4-, 8- or 16-byte units of the stream: neighbouring lanes fill sectors
                     if (t.valid > 0) store_words<B>(tile_words + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
                 } else {
                     __syncwarp();                // the warp has read all of its rows
