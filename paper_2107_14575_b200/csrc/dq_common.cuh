@@ -143,6 +143,24 @@ __device__ __forceinline__ int last_not_above(const int32_t* __restrict__ starts
     return lo;
 }
 
+// The same for the warp together (x and the answer are the warp's): 32 entries are looked at a step, so
+// that 1023 tensors take two steps and not ten.  start(i) is entry i.
+template <class Start>
+__device__ __forceinline__ int last_not_above_by_warp(const int x, const int n, const Start& start)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = n, stride;
+    do {
+        stride = (len + 31) >> 5;
+        const int at = lane * stride;
+        const uint32_t below = __ballot_sync(0xffffffffu, at < len && start(lo + at) <= x);
+        const int skip = (__popc(below) - 1) * stride;
+        lo += skip;
+        len = len - skip < stride ? len - skip : stride;
+    } while (stride > 1);
+    return lo;
+}
+
 // Bucket and number of valid elements of group g (32 padded elements).
 __device__ __forceinline__ void group_info(const LayoutView& v, int g, int& bucket, int& valid)
 {

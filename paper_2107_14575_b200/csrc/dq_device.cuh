@@ -420,6 +420,39 @@ __device__ __forceinline__ void store_wide(float* p, const float (&r)[8], const 
     store_wide_bits(p, v, base, extent, status);
 }
 
+// The 128-byte row of sums (or the update of the parameters there), straight from registers: a lane's
+// row is four whole sectors, and it happens once per tile and M workers.
+__device__ __forceinline__ void store_row(float* dst, const float (&r)[32], const bool update, const float neg_lr, const bool wide,
+                                          const void* base, const int64_t extent, int32_t* status)
+{
+    if (wide) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float y[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[e] = r[8 * i + e];
+            if (update) {
+                float p[8];
+                load_wide(dst + 8 * i, p);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) y[e] = fmaf(neg_lr, y[e], p[e]);
+            }
+            store_wide(dst + 8 * i, y, base, extent, status);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float4 y = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+            if (update) {
+                const float4 p = *reinterpret_cast<const float4*>(dst + 4 * i);
+                y = make_float4(fmaf(neg_lr, y.x, p.x), fmaf(neg_lr, y.y, p.y), fmaf(neg_lr, y.z, p.z),
+                                fmaf(neg_lr, y.w, p.w));
+            }
+            DQ_STORE(reinterpret_cast<float4*>(dst + 4 * i), y, base, extent, status);
+        }
+    }
+}
+
 // Words that leave straight from registers, by 4-, 8-, 16- or 32-byte stores: a tile's words are one
 // contiguous span, the L2 puts partial sectors together, and staging them in shared memory costs some
 // sixty instructions a tile.  From nine words on the scattered stores cost more.  Measured, staged / straight

@@ -268,38 +268,6 @@ __device__ __noinline__ float rare_norm(const uint32_t row, const int valid, con
     return again ? (magnitude_scalable(mx) ? rescaled_l2(mx, scaled, e) : mx) : nrm;
 }
 
-// The 128-byte row of sums (or the update of the parameters there), straight from registers: a lane's
-// row is four whole sectors, and it happens once per tile and M workers.
-__device__ __forceinline__ void store_row(const RoundArgs& a, float* dst, const float (&r)[32], const int64_t extent)
-{
-    if (a.wide_out) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float y[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) y[e] = r[8 * i + e];
-            if (a.update) {
-                float p[8];
-                load_wide(dst + 8 * i, p);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) y[e] = fmaf(a.neg_lr, y[e], p[e]);
-            }
-            store_wide(dst + 8 * i, y, a.out, extent, a.status);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float4 y = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-            if (a.update) {
-                const float4 p = *reinterpret_cast<const float4*>(dst + 4 * i);
-                y = make_float4(fmaf(a.neg_lr, y.x, p.x), fmaf(a.neg_lr, y.y, p.y), fmaf(a.neg_lr, y.z, p.z),
-                                fmaf(a.neg_lr, y.w, p.w));
-            }
-            DQ_STORE(reinterpret_cast<float4*>(dst + 4 * i), y, a.out, extent, a.status);
-        }
-    }
-}
-
 template <int B, int MODE, bool AVG, bool LINF>
 __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
 {
@@ -337,19 +305,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 
     // ---- where tiles lie.  Codes alone: a position is worked out once, when the producer moves there, and the
     //      consumer finds the answer in a queue.  AVG: twice, the second time from the cached tensor as a rule.
-    // last tensor whose first bucket (column 1) or group (column 0) is <= x; x and the answer are the
-    // warp's: 32 entries are looked at together, so that 1023 tensors take two steps and not ten
+    // last tensor whose first bucket (column 1) or group (column 0) is <= x
     auto find_seg = [&](int column, int x) -> int {
-        int lo = 0, len = a.v.n_seg, stride;
-        do {
-            stride = (len + 31) >> 5;
-            const int at = lane * stride;
-            const uint32_t below = __ballot_sync(0xffffffffu, at < len && tbl(column * n1 + lo + at) <= x);
-            const int skip = (__popc(below) - 1) * stride;
-            lo += skip;
-            len = len - skip < stride ? len - skip : stride;
-        } while (stride > 1);
-        return lo;
+        return last_not_above_by_warp(x, a.v.n_seg, [&](int i) { return tbl(column * n1 + i); });
     };
     // the same for an x of each lane's own, from tensor `from` on
     auto walk_seg = [&](int column, int from, int x) -> int {
@@ -677,7 +635,8 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                     for (int e = 0; e < 32; ++e)
                         if (e >= t.valid) r[e] = 0.0f;
                 }
-                store_row(a, a.out + ((int64_t)t.row0 + t.row) * 32, r, (int64_t)G * 128);
+                store_row(a.out + ((int64_t)t.row0 + t.row) * 32, r, a.update != 0, a.neg_lr, a.wide_out != 0, a.out, (int64_t)G * 128,
+                          a.status);
             }
             pos += hop;
         } else {

@@ -2,90 +2,52 @@
 // packed codes: out_j = (1/M) sum_m (code_m - s) * norm_m / s  (Eq. 5 inverted;
 // a code holds s + sgn * level).
 //
-// Persistent CTAs each take a contiguous range of tiles of 128 groups (one
-// group = 32 padded elements = one thread, which keeps its 32 fp32 sums in
-// registers).  The M workers' words of a tile are fetched in chunks of a few
-// workers by linear bulk copies (TMA) into a ring of shared-memory stages, so
-// the copies of the next chunks overlap the decoding of the current one.  A
-// fifth warp does nothing but issue those copies: a bulk copy holds its issuing
-// thread until the copy engine accepts it, about a microsecond per tile when the
-// SM's four CTAs queue there at once, and nobody waits for that warp.  A
-// code is decoded where it stands in its word (mask under the exponent of 2^23,
-// subtract 2^23 + s: see decode_code) and accumulated with one FMA; the power
-// of two its position carries is removed once per element after the last
-// worker.  The 128 x 32 results of a tile go through a swizzled shared-memory
-// tile and leave with one bulk tensor store.
-// HBM traffic per output element: M*b/8 bytes read, 4 written.
+// Every WARP is a pipeline of its own.  It takes tiles of 32 groups (one group = 32 padded elements =
+// one lane, which keeps its 32 fp32 sums in registers) through the M workers, up to eight workers
+// at a time: their words of the tile are as many linear bulk copies, one per lane, into one of two
+// 4 KB stages, so that the copies of the next workers travel while these are decoded.  The norms of the
+// next workers are requested before the wait.  A code is decoded where it stands in its word (mask under
+// the exponent of 2^23, subtract 2^23 + s: see decode_code) and accumulated with one FMA; the power of two
+// its position carries is removed once per element after the last worker.  The 32 rows of sums go through a
+// swizzled 4 KB tile of the warp and leave with one bulk tensor store (straight from registers, 32 bytes a
+// lane, every store touched 32 lines: one worker, 2^25 elements, b = 4 37 us against 30).
+// HBM traffic per output element: M*b/8 bytes read, 4 written.  Bound by the logic pipe for small b
+// (one half-rate operation per code), by HBM from b = 8 on.  AVERAGE_FIGURES
 //
-// dq_unpack_average_update is the same kernel with the parameter update of
-// Algorithm 1 as its epilogue, x <- x - eta * average: the tile of x is fetched into
-// the output tile by a bulk tensor load while the codes are decoded, updated in place
-// and stored back; the averaged gradient itself never reaches memory (M*b/8 + 4 bytes
-// read and 4 written per element).
+// dq_unpack_average_update ends with the parameter update of Algorithm 1 instead, x <- x - eta * average;
+// the averaged gradient itself never reaches memory (M*b/8 + 4 bytes read and 4 written per element).
 #include "dq_common.cuh"
 #include "dq_device.cuh"
 #include "dq_tma.cuh"
 
 namespace {
 
-constexpr int kThreads = 128;                 // groups per tile = consumer threads (warps 0..3)
-constexpr int kBlock = kThreads + 32;         // plus the warp that issues the copies
+constexpr int kThreads = 128;
+constexpr int kWarps = kThreads / 32;
+constexpr int kCtasPerSm = 4;
 constexpr int kStages = 2;
-constexpr int kStageWords = 4096;             // 16 KB per stage
+constexpr int kStageBytes = 4096;
 constexpr int kMaxChunk = 8;                  // workers per stage at most
 constexpr int kMaxSmemSegs = 1023;
 
-// Dynamic shared memory, addressed only through this symbol so that every access
-// compiles to a shared-memory instruction:
-//   [0, 16 KB)                 output tile, 128-byte swizzle (1024-byte aligned)
-//   then kStages * 16 KB of input stages, 8 * 128 scales, the stage barriers, the tensor table
+// Dynamic shared memory, addressed only through this symbol so that every access compiles to a
+// shared-memory instruction: the warps' output tiles (1024-byte aligned for the swizzle), their stages,
+// the barriers of stages and of the tiles of x, the tensor table.
 extern __shared__ __align__(1024) unsigned char smem[];
-constexpr int kOutBytes = kThreads * 128;
-constexpr int kStageOffset = kOutBytes;
-constexpr int kScaleOffset = kStageOffset + kStages * kStageWords * 4;            // [kMaxChunk][kThreads] floats
-// barriers: kStages "stage filled" (copies landed), kStages "stage drained" (one arrival per
-// consumer warp), then the one of the x tile
-constexpr int kBarOffset = kScaleOffset + kMaxChunk * kThreads * 4;
-// one word that says "a wait ran out": written by whoever notices, read by the copy warp (so that it
-// stops issuing) and fed into the consumers' barrier reductions
-constexpr int kAbortOffset = kBarOffset + (2 * kStages + 1) * 8;
-constexpr int kTblOffset = kAbortOffset + 8;
+constexpr int kOutBytes = 32 * 128;
+constexpr int kStageOffset = kWarps * kOutBytes;
+constexpr int kBarOffset = kStageOffset + kWarps * kStages * kStageBytes;
+constexpr int kTblOffset = kBarOffset + kWarps * (kStages + 1) * 8;
 
-__device__ __forceinline__ uint64_t* full_bar(int st) { return reinterpret_cast<uint64_t*>(smem + kBarOffset) + st; }
-__device__ __forceinline__ uint64_t* empty_bar(int st) { return reinterpret_cast<uint64_t*>(smem + kBarOffset) + kStages + st; }
-__device__ __forceinline__ uint64_t* x_bar() { return reinterpret_cast<uint64_t*>(smem + kBarOffset) + 2 * kStages; }
-__device__ __forceinline__ volatile int* abort_flag() { return reinterpret_cast<volatile int*>(smem + kAbortOffset); }
-// barrier among the consumer warps only (the copy warp runs ahead on its own)
-__device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
-// The same barrier with an OR over the consumers' predicates: every consumer gets the same answer,
-// so a decision to leave taken from it is taken by all of them or by none.
-__device__ __forceinline__ bool consumer_sync_or(const bool pred)
+__device__ __forceinline__ uint64_t* stage_bar(int warp, int st)
 {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "bar.red.or.pred p, 1, %2, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)pred), "n"(kThreads)
-        : "memory");
-    return r != 0;
+    return reinterpret_cast<uint64_t*>(smem + kBarOffset) + warp * kStages + st;
 }
-// Wait of the copy warp for a drained stage: as mbar_wait, but it also gives up when the
-// consumers have said that they are leaving.
-__device__ __forceinline__ bool wait_unless_aborted(uint64_t* bar, const uint32_t parity, const WaitLimits& lim)
+__device__ __forceinline__ uint32_t* stage_words(int warp, int st)
 {
-    if (tma::mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = tma::global_timer_ns();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 64; ++i)
-            if (tma::mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag() != 0 || tma::global_timer_ns() - t0 > lim.ns) return false;
-    }
+    return reinterpret_cast<uint32_t*>(smem + kStageOffset + (warp * kStages + st) * kStageBytes);
 }
-__device__ __forceinline__ uint32_t* stage_words(int st) { return reinterpret_cast<uint32_t*>(smem + kStageOffset) + st * kStageWords; }
+__device__ __forceinline__ uint64_t* x_bar(int warp) { return stage_bar(kWarps, 0) + warp; }
 
 struct AverageArgs {
     LayoutView v;
@@ -99,7 +61,9 @@ struct AverageArgs {
     uint32_t div_magic;
     int32_t div_shift;
     uint32_t magic;               // 0x4B000000, kept out of the compiler's sight (see and_or)
-    float neg_lr;                 // -eta of the parameter update (update kernel only)
+    int32_t update;               // out <- out + neg_lr * average instead of out <- average
+    uint32_t each, extra;         // tiles per warp: `each`, one more for the first `extra` of them
+    float neg_lr;                 // -eta of the parameter update
     WaitLimits wait;
 };
 
@@ -119,10 +83,10 @@ __device__ __forceinline__ float load_norm_early(const float* p)
     return x;
 }
 
-// workers per stage: as many as fit 16 KB with 128 groups of B words each, at most kMaxChunk
+// workers per stage: as many as fit with 32 groups of B words each, at most kMaxChunk
 template <int B>
 struct ChunkOf {
-    static constexpr int fit = kStageWords / (kThreads * B);
+    static constexpr int fit = kStageBytes / (128 * B);
     static constexpr int value = fit < 1 ? 1 : (fit > kMaxChunk ? kMaxChunk : fit);
 };
 
@@ -195,93 +159,36 @@ struct Normalise<B, 32> {
     static __device__ __forceinline__ void run(float (&)[32]) {}
 };
 
-// Issues the bulk copies of one pipeline unit: workers [m0, m0 + mc) of the tile at row0.
 template <int B>
-__device__ __forceinline__ void issue_unit(const AverageArgs& a, int st, int row0, int m0, int mc)
-{
-    int rows = a.v.total_groups - row0;
-    rows = rows > kThreads ? kThreads : rows;
-    const uint32_t bytes = ((uint32_t)(rows * B * 4) + 15u) & ~15u;   // the stream's stride is a multiple of 16 bytes
-    tma::mbar_expect_tx(full_bar(st), bytes * (uint32_t)mc);
-    for (int j = 0; j < mc; ++j)
-        tma::load_bulk(stage_words(st) + j * (kThreads * B),
-                       a.packed + (int64_t)(m0 + j) * a.packed_stride + (int64_t)row0 * B, bytes, full_bar(st));
-}
-
-// UPDATE = false: out = average.  UPDATE = true: out holds the parameters x and becomes x - eta * average.
-template <int B, bool UPDATE>
 __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtensorMap* out_map, const bool tbl_in_smem)
 {
     constexpr int s = (1 << (B - 1)) - 1;
     constexpr int MC = ChunkOf<B>::value;
     const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
     auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
-    const int tid = threadIdx.x;
-    const int G = a.v.total_groups;
-    const int M = a.M;
-    const int total_tiles = (G + kThreads - 1) / kThreads;
-    const int nchunk = (M + MC - 1) / MC;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = a.v.total_groups, M = a.M, nb = a.v.nb;
     const int n1 = a.v.n_seg + 1;
+    const int nchunk = (M + MC - 1) / MC;
     const float unit = (B == 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);      // 1 / (s * M)
-    // this thread's column of the [kMaxChunk][kThreads] scale buffer (only this thread touches it)
-    float* my_scales = reinterpret_cast<float*>(smem + kScaleOffset) + tid;
     const uint32_t magic = a.magic;
 
-    // every CTA takes one contiguous range of tiles; its pipeline units are (tile, chunk) pairs
-    const int tile_begin = (int)((int64_t)blockIdx.x * total_tiles / gridDim.x);
-    const int tile_end = (int)((int64_t)(blockIdx.x + 1) * total_tiles / gridDim.x);
-    const int my_units = (B == 1) ? 0 : (tile_end - tile_begin) * nchunk;
-    if (tid >= kThreads) {
-        // the copy warp: unit u goes into stage u % kStages as soon as the consumers have drained
-        // what was there (unit u - kStages)
-        if (tid == kThreads) {
-            int issued = 0;
-            for (int u = 0; u < my_units; ++u) {
-                const int st = u % kStages;
-                if (u >= kStages && !wait_unless_aborted(empty_bar(st), (uint32_t)(u / kStages - 1) & 1u, a.wait)) {
-                    if (*abort_flag() == 0) {            // nobody drained the stage in time
-                        atomicOr(a.status, DQ_STAT_WAIT);
-                        *abort_flag() = 1;
-                    }
-                    break;
-                }
-                const int tile = tile_begin + u / nchunk;
-                const int m0 = (u % nchunk) * MC;
-                issue_unit<B>(a, st, tile * kThreads, m0, (M - m0) < MC ? (M - m0) : MC);
-                issued = u + 1;
-            }
-            // Whoever issues copies sees them land: the last copy into each stage is the only one the
-            // consumers may not have waited for (when they left early), and the CTA's shared memory
-            // must not be released under a copy in flight.
-            for (int u = issued > kStages ? issued - kStages : 0; u < issued; ++u)
-                if (!tma::mbar_wait(full_bar(u % kStages), (uint32_t)(u / kStages) & 1u, a.wait))
-                    atomicOr(a.status, DQ_STAT_WAIT);
-        }
-        return;
-    }
+    // every warp takes every hop-th tile, `each` of them, the first `extra` warps one more
+    const uint32_t id = blockIdx.x * kWarps + warp;
+    const int hop = (int)(gridDim.x * kWarps);
+    const int n_tiles = (int)(a.each + (id < a.extra ? 1u : 0u));
+    const int items = (B == 1) ? 0 : n_tiles * nchunk;
 
-    // Bucket and valid elements of this thread's group in a tile.  The first lookup of a CTA
-    // is a binary search, later ones walk on from the previous tile's tensor.
-    int seg = 0;
-    bool seg_known = false;
-    auto lookup = [&](int tile, int& bucket, int& valid) {
-        const int g = tile * kThreads + tid;
+    // bucket and valid elements of this lane's group in a tile (valid 0: the group lies beyond the layout)
+    auto locate = [&](int tile, int& bucket, int& valid) {
+        const int g = tile * 32 + lane;
+        int seg = 0;
+        if (a.v.n_seg > 1) seg = last_not_above_by_warp(tile * 32, a.v.n_seg, tbl);
         bucket = 0;
-        valid = 0;                                 // 0: the group lies beyond the layout
+        valid = 0;
         if (g >= G) return;
-        int local, n, b0;
-        if (a.v.n_seg == 1) {
-            local = g; n = a.v.seg0_elems; b0 = 0;
-        } else {
-            if (!seg_known) {
-                int lo = 0, hi = a.v.n_seg;
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (tbl(mid) <= g) lo = mid; else hi = mid;
-                }
-                seg = lo;
-                seg_known = true;
-            }
+        int local = g, n = a.v.seg0_elems, b0 = 0;
+        if (a.v.n_seg > 1) {
             while (g >= tbl(seg + 1)) ++seg;
             local = g - tbl(seg);
             b0 = tbl(n1 + seg);
@@ -292,134 +199,102 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
         valid = left < 32 ? left : 32;
     };
 
-    if constexpr (B == 1) {
-        // s = 0: every value is 0, and an update by 0 leaves x as it is
-        if constexpr (!UPDATE) {
-            for (int tile = tile_begin; tile < tile_end; ++tile) {
-                if (tid == 0) tma::store_wait_read();
-                consumer_sync();
+    // ---- producer side: item = (tile, chunk of workers), fetched two ahead of the consumer
+    int p_tile = (int)id, p_m0 = 0, p_left = items;
+    auto fetch = [&](int st) {
+        if (p_left <= 0) return;
+        --p_left;
+        const int rows = (G - p_tile * 32) < 32 ? (G - p_tile * 32) : 32;
+        const uint32_t bytes = ((uint32_t)(rows * B * 4) + 15u) & ~15u;      // the stream's stride is a multiple of 16 bytes
+        const int mc = (M - p_m0) < MC ? (M - p_m0) : MC;
+        if (lane == 0) tma::mbar_expect_tx(stage_bar(warp, st), bytes * (uint32_t)mc);
+        if (lane < mc)
+            tma::load_bulk(stage_words(warp, st) + lane * (32 * B),
+                           a.packed + (int64_t)(p_m0 + lane) * a.packed_stride + (int64_t)p_tile * (32 * B), bytes, stage_bar(warp, st));
+        p_m0 += MC;
+        if (p_m0 >= M) { p_m0 = 0; p_tile += hop; }
+    };
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<float4*>(smem + tma::swizzle128(tid, c)) = make_float4(0.f, 0.f, 0.f, 0.f);
-                tma::fence_proxy_async();
-                consumer_sync();
-                if (tid == 0) {
-                    tma::store_tile_2d(out_map, smem, 0, tile * kThreads);
-                    tma::store_commit();
-                }
-            }
-            if (tid == 0) tma::store_wait_read();
-        }
-        return;
-    } else {
-        // Software pipeline over the units: while unit u is decoded, the norms of unit u + 1 (one
-        // per worker of the chunk, for this thread's bucket) are already on their way in registers.
-        // Nothing touches them before the decode is done -- the first use of a loaded value is
-        // where the warp would wait for it -- and only then do they become scales
-        // (norm * 1/(s M)) in the scale buffer.
-        int bucket, valid, nbucket = 0, nvalid = 0;
-        lookup(tile_begin, bucket, valid);
-        float nxt[MC];
-        {
-            const int mc0 = M < MC ? M : MC;
-            const float* nrm = a.norms + bucket;
-#pragma unroll
-            for (int j = 0; j < MC; ++j)
-                nxt[j] = (j < mc0 && valid > 0 && my_units > 0) ? __ldg(nrm + (int64_t)j * a.v.nb) : 0.0f;
-#pragma unroll
-            for (int j = 0; j < MC; ++j) my_scales[j * kThreads] = nxt[j] * unit;
-        }
+    for (int st = 0; st < kStages; ++st) fetch(st);
 
-        // A warp whose wait for a stage ran out raises the flag, decodes no more and releases no more
-        // stages; it walks on to the barrier at the tile's end, where all consumers learn of it together
-        // and leave.  (Warps that were still waiting for later stages run into their own limit first.)
+    int tile = (int)id, bucket, valid;
+    locate(tile < (G + 31) / 32 ? tile : 0, bucket, valid);
+    float scale[MC], nxt[MC];
+    auto request_norms = [&](int m0, int bk, int vl) {
+        const float* p = a.norms + (int64_t)m0 * nb + bk;
+#pragma unroll
+        for (int j = 0; j < MC; ++j, p += nb) nxt[j] = (m0 + j < M && vl > 0) ? load_norm_early(p) : 0.0f;
+    };
+    if (items > 0) request_norms(0, bucket, valid);
+
+    unsigned char* out_tile = smem + warp * kOutBytes;
+    uint32_t it = 0;
+    bool timed_out = false;
+    uint32_t x_parity = 0;                        // of the tile of x at hand
+    // (test hook: the warp's first wait counts as lost, and the warp goes straight to what follows a time-out)
+    const bool skip_all = a.wait.lose_first != 0u && items > 0;
+    for (int k = 0; k < n_tiles && !skip_all; ++k) {
         uint64_t acc2[16];
-        float acc[32];
-        // (test hook: every warp's first wait counts as lost, so the warps start out that way)
-        bool timed_out = false, warp_out = a.wait.lose_first != 0u, x_pending = false;
-        if (warp_out) *abort_flag() = 1;
-        int u = 0;
-        int tiles_done = 0;
-        for (int tile = tile_begin; tile < tile_end; ++tile) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
-            for (int c = 0; c < nchunk; ++c, ++u) {
-                const int m0 = c * MC;
-                const int mc = (M - m0) < MC ? (M - m0) : MC;
-
-                // next unit: same tile and the next chunk of workers, or the first chunk of the next tile
-                const bool last_chunk = (c == nchunk - 1);
-                const bool has_next = (u + 1 < my_units);
-                int nm0 = m0 + MC;
-                if (last_chunk) {
-                    nm0 = 0;
-                    if (has_next) lookup(tile + 1, nbucket, nvalid);
-                } else {
-                    nbucket = bucket;
-                    nvalid = valid;
-                }
-                {
-                    const int nmc = (M - nm0) < MC ? (M - nm0) : MC;
-                    const float* nrm = a.norms + (int64_t)nm0 * a.v.nb + nbucket;
-#pragma unroll
-                    for (int j = 0; j < MC; ++j)
-                        nxt[j] = (has_next && j < nmc && nvalid > 0) ? load_norm_early(nrm + (int64_t)j * a.v.nb) : 0.0f;
-                }
-
-                if constexpr (UPDATE) {
-                    // the tile of x travels into the output tile while the codes are decoded; the
-                    // previous tile's store must have drained it first
-                    if (c == 0) {
-                        if (tid == 0) {
-                            tma::store_wait_read();
-                            tma::mbar_expect_tx(x_bar(), kOutBytes);
-                            tma::load_tile_2d(smem, out_map, x_bar(), 0, tile * kThreads);
-                        }
-                        x_pending = true;
-                    }
-                }
-                const int st = u % kStages;
-                if (!warp_out &&
-                    !__all_sync(0xffffffffu, tma::mbar_wait(full_bar(st), (u / kStages) & 1, a.wait))) {
-                    warp_out = true;
-                    *abort_flag() = 1;
-                }
-                if (!warp_out) {
-                    const uint32_t* base = stage_words(st) + tid * B;
-                    if (mc == MC) {              // a full unit: no loop
-#pragma unroll
-                        for (int j = 0; j < MC; ++j) {
-                            uint32_t wd[B], hi[B];
-                            load_words<B>(base + j * (kThreads * B), wd);
-                            UpperHalves<B, 0>::run(base + j * (kThreads * B), hi);
-                            const uint32_t sc = __float_as_uint(my_scales[j * kThreads]);
-                            AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
-                        }
-                    } else {
+        for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
+        int nbucket = bucket, nvalid = valid;
+        // the tile before must have left the warp's output tile; the tile of x travels while the codes are decoded
+        x_parity = (uint32_t)k & 1u;
+        if (B > 1 && a.update && lane == 0) {
+            tma::store_wait_read();
+            tma::mbar_expect_tx(x_bar(warp), kOutBytes);
+            tma::load_tile_2d(out_tile, out_map, x_bar(warp), 0, tile * 32);
+        }
+        if constexpr (B > 1) {
 #pragma unroll 1
-                        for (int j = 0; j < mc; ++j) {
-                            uint32_t wd[B], hi[B];
-                            load_words<B>(base + j * (kThreads * B), wd);
-                            UpperHalves<B, 0>::run(base + j * (kThreads * B), hi);
-                            const uint32_t sc = __float_as_uint(my_scales[j * kThreads]);
-                            AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
-                        }
+            for (int m0 = 0; m0 < M; m0 += MC, ++it) {
+                const int st = (int)(it & 1u);
+                // the norms of the chunk after this one travel during the wait and the decoding
+#pragma unroll
+                for (int j = 0; j < MC; ++j) scale[j] = nxt[j] * unit;
+                if (m0 + MC < M) {
+                    request_norms(m0 + MC, bucket, valid);
+                } else if (k + 1 < n_tiles) {
+                    locate(tile + hop, nbucket, nvalid);
+                    request_norms(0, nbucket, nvalid);
+                }
+                // every lane polls the barrier itself; the verdict is made warp-uniform
+                if (!__all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), (it >> 1) & 1u, a.wait))) {
+                    timed_out = true;
+                    break;
+                }
+                const uint32_t* base = stage_words(warp, st) + lane * B;
+                if (m0 + MC <= M) {              // a full stage: no loop
+#pragma unroll
+                    for (int j = 0; j < MC; ++j) {
+                        uint32_t wd[B], hi[B];
+                        load_words<B>(base + j * (32 * B), wd);
+                        UpperHalves<B, 0>::run(base + j * (32 * B), hi);
+                        const uint32_t sc = __float_as_uint(scale[j]);
+                        AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < MC - 1; ++j) {
+                        if (m0 + j >= M) break;
+                        uint32_t wd[B], hi[B];
+                        load_words<B>(base + j * (32 * B), wd);
+                        UpperHalves<B, 0>::run(base + j * (32 * B), hi);
+                        const uint32_t sc = __float_as_uint(scale[j]);
+                        AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
                     }
                 }
-#pragma unroll
-                for (int j = 0; j < MC; ++j) my_scales[j * kThreads] = nxt[j] * unit;
-
-                // this warp is done with the stage: once all four have said so the copy warp refills it
-                // (a warp whose wait ran out says nothing: the stage's copy may still be on its way, and the
-                // copy warp, which watches the flag, issues no more)
+                // the warp's reads of the stage come before the copies that refill it (another proxy)
+                tma::fence_proxy_async();
                 __syncwarp();
-                if ((tid & 31) == 0 && !warp_out) tma::mbar_arrive(empty_bar(st));
+                fetch(st);
+                __syncwarp();
             }
-            // the previous tile's bulk store must have drained the output tile before it is rewritten below
-            if constexpr (!UPDATE) {
-                if (tid == 0) tma::store_wait_read();
-            }
-            if (consumer_sync_or(warp_out || *abort_flag() != 0)) { timed_out = true; break; }
+            if (timed_out) break;
+        }
+        // (B = 1: s = 0, every value is 0, and an update by 0 leaves x as it is)
+        if (!(B == 1 && a.update)) {
+            float acc[32];
 #pragma unroll
             for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], acc[2 * q], acc[2 * q + 1]);
             Normalise<B, 0>::run(acc);
@@ -428,83 +303,71 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
                 for (int e = 0; e < 32; ++e)
                     if (e >= valid) acc[e] = 0.0f;
             }
-            // own row of the swizzled output tile (conflict-free), then one bulk tensor store per tile
-            bool x_landed = true;
-            if constexpr (UPDATE) {
-                x_landed = tma::mbar_wait(x_bar(), (uint32_t)tiles_done & 1u, a.wait);
-                if (x_landed) {
-                    const float neg_lr = a.neg_lr;
+            if (a.update) {
+                // nothing is stored from a tile whose parameters did not arrive
+                if (!__all_sync(0xffffffffu, tma::mbar_wait(x_bar(warp), x_parity, a.wait))) {
+                    timed_out = true;
+                    break;
+                }
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float4* p = reinterpret_cast<float4*>(smem + tma::swizzle128(tid, c));
-                        const float4 x = *p;
-                        *p = make_float4(fmaf(neg_lr, acc[4 * c], x.x), fmaf(neg_lr, acc[4 * c + 1], x.y),
-                                         fmaf(neg_lr, acc[4 * c + 2], x.z), fmaf(neg_lr, acc[4 * c + 3], x.w));
-                    }
+                for (int c = 0; c < 8; ++c) {
+                    float4* p = reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c));
+                    const float4 x = *p;
+                    *p = make_float4(fmaf(a.neg_lr, acc[4 * c], x.x), fmaf(a.neg_lr, acc[4 * c + 1], x.y),
+                                     fmaf(a.neg_lr, acc[4 * c + 2], x.z), fmaf(a.neg_lr, acc[4 * c + 3], x.w));
                 }
             } else {
+                if (lane == 0) tma::store_wait_read();
+                __syncwarp();
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<float4*>(smem + tma::swizzle128(tid, c)) =
+                    *reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c)) =
                         make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
             }
             tma::fence_proxy_async();
-            if constexpr (UPDATE) {
-                // nothing is stored from a tile whose parameters did not arrive
-                if (consumer_sync_or(!x_landed)) { timed_out = true; break; }
-                x_pending = false;
-            } else {
-                consumer_sync();
-            }
-            if (tid == 0) {
-                tma::store_tile_2d(out_map, smem, 0, tile * kThreads);
+            __syncwarp();
+            if (lane == 0) {
+                tma::store_tile_2d(out_map, out_tile, 0, tile * 32);          // (rows outside the layout are clipped)
                 tma::store_commit();
             }
-            bucket = nbucket;
-            valid = nvalid;
-            ++tiles_done;
         }
-
-        if (tid == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
-        if (timed_out) {
-            // The copy warp stops issuing and sees its own copies land; the consumers' only copy is the
-            // tile of x, which gets the full limit before the shared memory is released.
-            *abort_flag() = 1;
-            if (tid == 0) atomicOr(a.status, DQ_STAT_WAIT);
-            if constexpr (UPDATE) {
-                if (x_pending) (void)tma::mbar_wait(x_bar(), (uint32_t)tiles_done & 1u, a.wait);
-            }
-        }
+        tile += hop;
+        if (B == 1 && k + 1 < n_tiles) locate(tile, nbucket, nvalid);
+        bucket = nbucket;
+        valid = nvalid;
+    }
+    if (lane == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
+    if (timed_out || skip_all) {
+        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
+        // every copy the warp has issued and not seen land, the one whose wait ran out included, gets the
+        // full limit before the CTA's shared memory is released
+        for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
+            (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
+        if (B > 1 && a.update && !skip_all) (void)tma::mbar_wait(x_bar(warp), x_parity, a.wait);
     }
 }
 
-template <bool UPDATE>
-__global__ void __launch_bounds__(kBlock, 4)
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
 unpack_average_kernel(const __grid_constant__ AverageArgs a, const __grid_constant__ CUtensorMap out_map)
 {
+    // (nothing up to the wait touches memory that an earlier kernel may still be writing)
+    if (threadIdx.x == 0) {
+        tma::prefetch_tensor_map(&out_map);
+        for (int i = 0; i < kWarps * (kStages + 1); ++i) tma::mbar_init(stage_bar(0, i), 1);
+        tma::fence_barrier_init();
+    }
     grid_dependency_wait();
     const int b = __ldg(a.dev_b);       // issued first, looked at after the set-up below so that the loads overlap
-    if (tma::smem_addr(smem) & 1023u) {           // the swizzled tile needs a 1024-byte aligned base
-        if (threadIdx.x == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
-        return;
-    }
     const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
     if (tbl_in_smem) {
         int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + kTblOffset);
-        for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kBlock) tbl_s[i] = __ldg(a.v.seg_group0 + i);
-    }
-    if (threadIdx.x == 0) {
-        tma::prefetch_tensor_map(&out_map);
-#pragma unroll
-        for (int st = 0; st < kStages; ++st) {
-            tma::mbar_init(full_bar(st), 1);
-            tma::mbar_init(empty_bar(st), kThreads / 32);
-        }
-        tma::mbar_init(x_bar(), 1);
-        tma::fence_barrier_init();
-        *abort_flag() = 0;
+        for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
     }
     __syncthreads();
+    if (tma::smem_addr(smem) & 1023u) {           // the swizzled tiles need a 1024-byte aligned base
+        if (threadIdx.x == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
+        return;
+    }
     if (b < 1 || b > DQ_MAX_BITS) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, DQ_STAT_BAD_BITS);
         return;
@@ -515,7 +378,7 @@ unpack_average_kernel(const __grid_constant__ AverageArgs a, const __grid_consta
     }
 
     switch (b) {
-#define DQ_CASE(BB) case BB: average_tiles<BB, UPDATE>(a, &out_map, tbl_in_smem); break;
+#define DQ_CASE(BB) case BB: average_tiles<BB>(a, &out_map, tbl_in_smem); break;
         DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
         DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
 #undef DQ_CASE
@@ -523,18 +386,10 @@ unpack_average_kernel(const __grid_constant__ AverageArgs a, const __grid_consta
     }
 }
 
-size_t smem_bytes(int n_seg)
-{
-    size_t n = (size_t)kTblOffset;
-    if (n_seg > 1 && n_seg <= kMaxSmemSegs) n += (size_t)3 * (n_seg + 1) * 4;
-    return n;
-}
-
-// Checks, tensor map and launch shared by the two entry points; `dev_out` is the averaged
-// gradient (update = false) or the parameters, read and written (update = true).
-template <bool UPDATE>
+// Checks and launch shared by the two entry points; `dev_out` is the averaged gradient, or the
+// parameters, read and written (update).
 int launch_average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t packed_stride_words, const float* dev_norms,
-                   int32_t M, const int32_t* dev_b, float lr, float* dev_out, int32_t* dev_status, void* stream)
+                   int32_t M, const int32_t* dev_b, bool update, float lr, float* dev_out, int32_t* dev_status, void* stream)
 {
     const int rc = dq_check_common(L, M);
     if (rc != DQ_OK) return rc;
@@ -544,9 +399,9 @@ int launch_average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t pac
         (reinterpret_cast<uintptr_t>(dev_status) & 3u))
         return DQ_ERR_ALIGN;
     if (packed_stride_words < L->padded / 32) return DQ_ERR_RANGE;
-    if (UPDATE && !(lr == lr && lr - lr == 0.0f)) return DQ_ERR_RANGE;      // eta must be finite
+    if (update && !(lr == lr && lr - lr == 0.0f)) return DQ_ERR_RANGE;      // eta must be finite
 
-    AverageArgs a;
+    AverageArgs a = {};
     a.v = make_view(L);
     a.packed = dev_packed;
     a.packed_stride = packed_stride_words;
@@ -556,6 +411,7 @@ int launch_average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t pac
     a.status = dev_status;
     a.M = M;
     a.magic = 0x4B000000u;
+    a.update = update ? 1 : 0;
     a.neg_lr = -lr;
     a.wait = dq_wait_limits();
     const uint32_t gpb = (uint32_t)a.v.groups_per_bucket;
@@ -568,27 +424,27 @@ int launch_average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t pac
         a.div_magic = (uint32_t)(((uint64_t(1) << 33) + gpb - 1) / gpb);
     }
 
-    // tensor map over the output: [group][32 floats], box = one tile of 128 groups, 128-byte swizzle
+    // tensor map over the output: [group][32 floats], box = one warp tile of 32 groups, 128-byte swizzle
     CUtensorMap out_map;
     const uint64_t dims[2] = {32, (uint64_t)a.v.total_groups};
     const uint64_t strides[1] = {128};
-    const uint32_t box[2] = {32, (uint32_t)kThreads};
-    if (!dq_encode_tensor_map(&out_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, dev_out, dims, strides, box,
-                              CU_TENSOR_MAP_SWIZZLE_128B))
+    const uint32_t box[2] = {32, 32};
+    if (!dq_encode_tensor_map(&out_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, dev_out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
         return DQ_ERR_CUDA;
 
-    const size_t smem_need = smem_bytes(L->n_seg);
-    if (cudaFuncSetAttribute(unpack_average_kernel<UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
+    size_t smem_need = (size_t)kTblOffset;
+    if (L->n_seg > 1 && L->n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (L->n_seg + 1) * 4;
+    if (cudaFuncSetAttribute(unpack_average_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
         (void)cudaGetLastError();
         return DQ_ERR_CUDA;
     }
-    const int64_t tiles = ((int64_t)a.v.total_groups + kThreads - 1) / kThreads;
-    int64_t blocks = (int64_t)dq_sm_count() * 4;       // four 53 KB CTAs per SM
-    if (blocks > tiles) blocks = tiles;
-    dq_launch(unpack_average_kernel<UPDATE>, dim3((unsigned)blocks), dim3(kBlock), smem_need, static_cast<cudaStream_t>(stream), a,
-              out_map);
-    if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
-    return DQ_OK;
+    const int64_t tiles = ((int64_t)a.v.total_groups + 31) / 32;
+    int64_t blocks = (int64_t)dq_sm_count() * kCtasPerSm;
+    if (blocks * kWarps > tiles) blocks = (tiles + kWarps - 1) / kWarps;
+    a.each = (uint32_t)(tiles / (blocks * kWarps));
+    a.extra = (uint32_t)(tiles - (int64_t)a.each * blocks * kWarps);
+    dq_launch(unpack_average_kernel, dim3((unsigned)blocks), dim3(kThreads), smem_need, static_cast<cudaStream_t>(stream), a, out_map);
+    return cudaGetLastError() == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
 }  // namespace
@@ -597,8 +453,7 @@ extern "C" int dq_unpack_dequant_average(const dq_layout_t* L, const uint32_t* d
                                          int64_t packed_stride_words, const float* dev_norms, int32_t M,
                                          const int32_t* dev_b, float* dev_out, int32_t* dev_status, void* stream)
 {
-    return launch_average<false>(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, 0.0f, dev_out, dev_status,
-                                 stream);
+    return launch_average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, false, 0.0f, dev_out, dev_status, stream);
 }
 
 extern "C" int dq_unpack_average_update(const dq_layout_t* L, const uint32_t* dev_packed,
@@ -606,6 +461,5 @@ extern "C" int dq_unpack_average_update(const dq_layout_t* L, const uint32_t* de
                                         const int32_t* dev_b, float lr, float* dev_params, int32_t* dev_status,
                                         void* stream)
 {
-    return launch_average<true>(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, lr, dev_params, dev_status,
-                                stream);
+    return launch_average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, true, lr, dev_params, dev_status, stream);
 }
