@@ -63,12 +63,10 @@ def _peaks():
 
 # Sources whose text decides what each timed call moves through DRAM and how many instructions
 # it issues: a counter capture stays valid only while their digest is the one stored beside it.
+_ROUND = ["dq_round.cuh", "dq_device.cuh", "dq_rule.cuh", "dq_tma.cuh", "dq_common.cuh"]
 KERNEL_SOURCES = {
-    "norms_quantize_pack": ["dq_fused.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"],
-    "quantize_pack": ["dq_quantize.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"],
-    "bucket_norms": ["dq_norms.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"],
+    "round": _ROUND, "norms_quantize_pack": _ROUND, "quantize_pack": _ROUND, "bucket_norms": _ROUND,
     "unpack_dequant_average": ["dq_unpack.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"],
-    "choose_bits": ["dq_bits.cu", "dq_common.cuh"],
 }
 
 
@@ -480,9 +478,6 @@ def run_cuda(args) -> dict:
         rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
     torch.cuda.synchronize()
     assert rnd.read_status() == 0, "device status %d" % rnd.read_status()
-    nev = 5
-    ev_stride = max(1, K // 12)
-    ev = {i: [torch.cuda.Event(enable_timing=True) for _ in range(nev)] for i in range(0, K, ev_stride)}
     start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     if world > 1:
         dist.barrier()
@@ -491,7 +486,7 @@ def run_cuda(args) -> dict:
     start.record()
     h0 = time.perf_counter()
     for i in range(K):
-        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None), events=ev.get(i))
+        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
     end.record()
     host_submit_ms = (time.perf_counter() - h0) * 1e3 / K
     torch.cuda.synchronize()
@@ -499,27 +494,31 @@ def run_cuda(args) -> dict:
     ms_total = replicas.max_over_ranks(start.elapsed_time(end), dev)
     assert rnd.read_status() == 0 and rnd.bits() == HEADLINE_B
     sm_mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz")
-    spans = {"norms_quantize_pack": (0, 1), "unpack_dequant_average": (1, 2), "choose_bits": (3, 4)}
-    step_ms = {n: sum(e[p].elapsed_time(e[q]) for e in ev.values()) / len(ev) for n, (p, q) in spans.items()}
+    # the step's one kernel by itself: a launch between its own pair of events
+    n_ev = max(3, min(K, 12))
+    ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(n_ev)]
+    for i, (e0, e1) in enumerate(ev):
+        e0.record()
+        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
+        e1.record()
+    torch.cuda.synchronize()
+    step_ms = {"round": sum(e0.elapsed_time(e1) for e0, e1 in ev) / n_ev}
     alg_bytes = {
         "bucket_norms": lambda b: 4.0 * elems,
         "quantize_pack": lambda b: (4.0 + b / 8.0) * elems,
         "norms_quantize_pack": lambda b: (4.0 + b / 8.0) * elems,
         "unpack_dequant_average": lambda b: (M * b / 8.0 + 4.0) * D32,
+        # every gradient read, every word written, the average written
+        "round": lambda b: (4.0 + b / 8.0) * elems + 4.0 * D32,
     }
     # units of the instruction model: 32-element groups a launch processes (per worker for the
     # quantizers; for the average a group of M x 32 codes)
     units = {"bucket_norms": groups, "quantize_pack": groups, "norms_quantize_pack": groups,
-             "unpack_dequant_average": D32 // 32}
-    kernels = {n: _bound(n, HEADLINE_B, alg_bytes[n](HEADLINE_B), units[n], step_ms[n], peak, sm_count, sm_mhz)
-               for n in ("norms_quantize_pack", "unpack_dequant_average")}
-    path_ms = sum(step_ms[n] for n in kernels)
-    for n in kernels:
-        kernels[n]["share"] = round(step_ms[n] / path_ms, 4)
-    kernels["choose_bits"] = {"ms": round(step_ms["choose_bits"], 5), "share": None,
-                              "runs_beside": "unpack_dequant_average (second stream)" if not args.no_overlap else None,
-                              "algorithmic_bytes": 4.0 * M * L.nb}
-    dominant = max(("norms_quantize_pack", "unpack_dequant_average"), key=lambda n: step_ms[n])
+             "unpack_dequant_average": D32 // 32, "round": groups}
+    kernels = {"round": _bound("round", HEADLINE_B, alg_bytes["round"](HEADLINE_B), units["round"], step_ms["round"], peak,
+                               sm_count, sm_mhz)}
+    kernels["round"]["share"] = 1.0
+    dominant = "round"
     dk = kernels[dominant]
     cnt = _counters(dominant)
     traffic = _interp((cnt or {}).get("dram_bytes_per_group"), HEADLINE_B)
@@ -529,8 +528,8 @@ def run_cuda(args) -> dict:
                 "algorithmic_bytes_per_launch": dk["algorithmic_bytes"], "frac_of_nominal_8tbs": dk["frac_of_8tbs"],
                 "hbm": {"achieved_gbs": dk["achieved_gbs"], "frac_of_measured": dk["frac_of_measured"]},
                 "kernels": kernels,
-                "timing": "CUDA events on the launching stream around each call of every %d-th timed step (%d samples)"
-                          % (ev_stride, len(ev))}
+                "timing": "CUDA events on the launching stream around single steps, after the timed region (%d samples)"
+                          % len(ev)}
     if dk["bound"] == "alu":
         # the instruction roof binds: report against it (lane instructions per second; peak = SMs x 128 lanes x
         # sampled SM clock), the HBM figures stay beside it under "hbm"
@@ -541,23 +540,21 @@ def run_cuda(args) -> dict:
                          "peak_source": "SMs x 4 schedulers x 32 lanes x sampled SM clock (one warp instruction per "
                                         "scheduler and cycle); instructions per group from profiles/counters.json"})
 
-    # ---- the same step with the parameter update of Eq. 2 applied by the averaging kernel (x <- x - eta * average)
+    # ---- the same step with the parameter update of Eq. 2 in it (x <- x - eta * average)
     with_update = None
     if not args.no_per_b:
         x = torch.zeros(D32, dtype=torch.float32, device=dev)
-        evu = [[torch.cuda.Event(enable_timing=True) for _ in range(nev)] for _ in range(min(K, 8))]
         for i in range(W):
             rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, params=x, lr=1e-3)
         torch.cuda.synchronize()
         su, eu = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         su.record()
         for i in range(K):
-            rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, params=x, lr=1e-3,
-                           events=evu[i] if i < len(evu) else None)
+            rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, params=x, lr=1e-3)
         eu.record()
         torch.cuda.synchronize()
         assert rnd.read_status() == 0 and rnd.bits() == HEADLINE_B
-        t_u = sum(e[1].elapsed_time(e[2]) for e in evu) / len(evu)
+        t_u = timer.train(lambda i: rnd.update_(x, 1e-3), K)
         bytes_u = (M * HEADLINE_B / 8.0 + 8.0) * D32            # the words of M workers, x read and written
         with_update = {"ms_per_step": round(su.elapsed_time(eu) / K, 5),
                        "value": round(4.0 * M * d * K / (su.elapsed_time(eu) * 1e-3) / 1e9, 1),
@@ -624,15 +621,14 @@ def run_cuda(args) -> dict:
         "ms_per_step": ms_total / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD,
-                   "order": "Algorithm 1: norms+quantize+pack in one pass with b_t, average, b_{t+1} from this step's norms"
-                            + ("" if args.no_overlap else " (bit rule on a second stream beside the average)"),
+                   "order": "Algorithm 1: norms, quantize+pack with b_t, average, and b_{t+1} from this step's norms, in one kernel",
                    "l2": "inputs larger than L2 (%d MB of gradients per step)" % ((4 * elems) >> 20),
                    "per_b": "b in %s: trains of %d launches and %d single event-bracketed launches per kernel"
                             % (list(PER_B), K, n_single),
                    "size_sweep": "M=1 at d=2^24..2^30 and buckets 128/4096 at d=2^26, M=32, b in %s: trains of %d launches, "
                                  "buffers rotated where one set would fit in the L2" % (list(SWEEP_B), K),
                    "multi_gpu": "independent replicas, no collective" if world > 1 else "single GPU"},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": 4 * K, "roofline": roofline,
+        "clocks": clocks, "e2e": e2e, "gpu_launches": K, "roofline": roofline,
         "per_b": per_b, "bucket_norms": _bound("bucket_norms", 0, 4.0 * elems, groups, norms_ms, peak, sm_count, sm_mhz),
         # what the workers would put on the wire per step (Eq. 7: d * b bits per worker, plus the fp32 norms)
         "wire": {"bytes_per_step": M * (d * HEADLINE_B / 8.0 + 4.0 * L.nb), "fp32_bytes_per_step": 4.0 * M * d,

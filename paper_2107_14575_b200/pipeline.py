@@ -1,9 +1,9 @@
 """One DQ-SGD communication round on one GPU: buffers plus the library calls.
 
 ``Round`` owns the device buffers (torch tensors) of a fixed layout and worker
-count and issues norms -> bit rule -> quantize+pack -> unpack+average on the
-current stream, or, in the order of Algorithm 1, norms+quantize+pack -> average
-with the next bit width chosen on a second stream meanwhile.  It adds no
+count and issues norms + bit rule -> quantize+pack + average on the
+current stream, or, in the order of Algorithm 1, norms, quantize+pack, average and the
+next bit width in one call.  It adds no
 arithmetic of its own: every step is a kernel of the C-ABI library.
 """
 from __future__ import annotations
@@ -95,8 +95,8 @@ class Round:
                             self.packed_stride, self.out, self.status)
         return self.out
 
-    # below this many norms the bit rule takes a few microseconds and the hand-over between two
-    # streams costs more than running it behind the average on the same stream
+    # of the separate calls: below this many norms the bit rule takes a few microseconds and the hand-over
+    # between two streams costs more than running it behind the average on the same stream
     OVERLAP_MIN_NORMS = 1 << 20
 
     def step_fused(self, grads, next_rule: dq.Rule, seed: int, step: int, overlap: Optional[bool] = None,
@@ -106,13 +106,12 @@ class Round:
         this round's norms.  ``dev_b`` must hold a b (a first call to ``bits_`` with the
         initial b_0 does that); on return it holds the next one.
 
-        With ``overlap`` the bit rule runs on a second stream next to the average: it needs
-        only the norms, and writes the other (b, s) slot.  The current stream waits for it
-        before it goes on.  ``overlap=None`` decides by size: a second stream for
-        ``OVERLAP_MIN_NORMS`` norms or more, one stream below (measured on the ResNet-18
-        shape, 175k norms: 102.5 us per step on one stream, 104.2 us with two; at 4.2M
-        norms the second stream hides 85 us of bit rule).  ``events`` = (e0, e1, e2, s0, s1) are recorded around the three
-        calls (e* on the current stream, s* around the bit rule on its own stream).
+        The round is one call of the library (``dq_norms_quantize_average``), which writes the next
+        (b, s) over this one's when it ends.  With ``events`` = (e0, e1, e2, s0, s1) it is the three
+        separate calls instead, with the events recorded around them (e* on the current stream, s*
+        around the bit rule): ``overlap`` then puts the bit rule on a second stream next to the average
+        (it needs only the norms, and writes the other (b, s) slot); ``overlap=None`` decides by size,
+        ``OVERLAP_MIN_NORMS``.
 
         With ``params`` (fp32 [D32] in the padded layout) the server step also applies the
         update of Eq. 2, ``params <- params - lr * average``, in the same kernel; ``out`` is

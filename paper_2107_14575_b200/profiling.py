@@ -29,11 +29,13 @@ import sys
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 
+_ROUND = ["dq_round.cuh", "dq_device.cuh", "dq_rule.cuh", "dq_tma.cuh", "dq_common.cuh"]
 KERNELS = {
     # key -> (substring of the kernel's name in a capture, source files that decide its counters)
-    "norms_quantize_pack": ("norms_quantize_pack_", ["dq_fused.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"]),
-    "quantize_pack": ("quantize_pack_kernel", ["dq_quantize.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"]),
-    "bucket_norms": ("bucket_norms_", ["dq_norms.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"]),
+    "round": ("round_kernel", _ROUND),
+    "norms_quantize_pack": ("round_kernel", _ROUND),
+    "quantize_pack": ("round_kernel", _ROUND),
+    "bucket_norms": ("norms_kernel", _ROUND),
     "unpack_dequant_average": ("unpack_average_kernel", ["dq_unpack.cu", "dq_device.cuh", "dq_tma.cuh", "dq_common.cuh"]),
 }
 
@@ -52,6 +54,8 @@ def algorithmic_bytes(key: str, d32: int, M: int, b: int) -> float:
         return 4.0 * M * d32
     if key in ("quantize_pack", "norms_quantize_pack"):
         return (4.0 + b / 8.0) * M * d32
+    if key == "round":
+        return (4.0 + b / 8.0) * M * d32 + 4.0 * d32
     return (M * b / 8.0 + 4.0) * d32
 
 
@@ -76,7 +80,8 @@ def cmd_run(a) -> None:
     g = torch.randn((a.M, rnd.layout.D32), generator=gen, device="cuda")
     rnd.bits_(dq.Rule.fixed(a.b))
     rnd.norms_quantize_(g, 2107, 0)                  # norms and words for the kernels that read them
-    fn = {"norms_quantize_pack": lambda i: rnd.norms_quantize_(g, 2107, i),
+    fn = {"round": lambda i: rnd.step_fused(g, dq.Rule.fixed(a.b), 2107, i),
+          "norms_quantize_pack": lambda i: rnd.norms_quantize_(g, 2107, i),
           "quantize_pack": lambda i: rnd.quantize_(g, 2107, i),
           "bucket_norms": lambda i: rnd.norms_(g),
           "unpack_dequant_average": lambda i: rnd.average_()}[a.kernel]
@@ -174,7 +179,7 @@ def cmd_summarize(a) -> None:
            "(min..max where they differ)." % len(sel), "", "| figure | value |", "|---|---|"] + lines + [""]
     out.append("Algorithmic bytes per launch: %.1f MB (%s)." % (alg / 1e6, {
         "bucket_norms": "4 B x M x d read", "quantize_pack": "(4 + b/8) B x M x d",
-        "norms_quantize_pack": "(4 + b/8) B x M x d", "unpack_dequant_average": "(M b/8 + 4) B x d"}[a.kernel]))
+        "norms_quantize_pack": "(4 + b/8) B x M x d", "round": "(4 + b/8) B x M x d + 4 B x d", "unpack_dequant_average": "(M b/8 + 4) B x d"}[a.kernel]))
     if traffic is not None:
         out.append("DRAM traffic per launch (read + write): %.1f MB (%.2f x algorithmic; ncu flushes the caches before "
                    "each replayed launch, and output lines still dirty in L2 at the kernel's end are not counted)."
@@ -252,8 +257,8 @@ def cmd_table(a) -> None:
     if line.get("with_parameter_update"):
         u = line["with_parameter_update"]
         k = u["unpack_average_update"]
-        print("\nThe headline step with the parameter update of Eq. 2 applied by the averaging kernel: %.3f ms per step "
-              "(%.0f GB/s of gradient); the update kernel %.3f ms = %.0f GB/s of its algorithmic bytes "
+        print("\nThe headline step with the parameter update of Eq. 2 applied in the round's kernel: %.3f ms per step "
+              "(%.0f GB/s of gradient); the update kernel by itself %.3f ms = %.0f GB/s of its algorithmic bytes "
               "((M b/8 + 8) B per element), %.3f of the copy bandwidth." % (u["ms_per_step"], u["value"], k["ms"],
                                                                           k["achieved_gbs"], k["frac_of_measured"]))
     if line.get("size_sweep"):
@@ -300,8 +305,8 @@ def cmd_launches(a) -> None:
         t = float(r[vi].replace(",", "")) * {"ns": 1e-3, "us": 1.0, "ms": 1e3}[r[ui]]
         n, tot = per.get(name, (0, 0.0))
         per[name] = (n + 1, tot + t)
-    library = ("norms_quantize_pack", "quantize_pack_kernel", "bucket_norms", "unpack_average_kernel", "tensor_norms_join",
-               "norm_square_partials", "apply_rule")
+    library = ("round_kernel", "norms_kernel", "bucket_norms", "unpack_average_kernel", "tensor_norms_join", "norm_square_partials",
+               "apply_rule")
     ours = {k: v for k, v in per.items() if any(k.startswith(p) for p in library)}
     total_ours = sum(t for _, t in ours.values())
     total_all = sum(t for _, t in per.values())
