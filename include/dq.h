@@ -219,7 +219,7 @@ int dq_choose_bits(const dq_layout_t* layout, const float* dev_norms, int32_t M,
 
 /* ------------------------------------- norms and bit rule in one call, Eq. 5 and 17
  * dq_bucket_norms (dq_tensor_norms for a whole-tensor layout) followed by dq_choose_bits on
- * its norms; where the bucket length is 32 * 2^k one kernel does both.  (The sum behind
+ * its norms; one kernel does both for bucket lengths up to 1024, 2048 and 4096.  (The sum behind
  * G-bar is fp64 in another fixed order than dq_choose_bits'.)  dev_workspace: as for
  * dq_norms_quantize_average. */
 size_t dq_round_workspace_bytes(const dq_layout_t* layout, int32_t M);
@@ -343,8 +343,8 @@ int dq_quantize_average(const dq_layout_t* layout, const float* dev_grads, int64
  * (or parameter update), and the b of the next round from this round's norms -- the
  * results of
  *   dq_norms_quantize_pack -> dq_unpack_dequant_average (or _update) -> dq_choose_bits,
- * for every layout (whole-tensor ones included), with the gradients read once where the
- * bucket length is 32 * 2^k and twice otherwise.  (The sum behind G-bar is fp64 in another
+ * for every layout (whole-tensor ones included), with the gradients read once for bucket
+ * lengths up to 1024, 2048 and 4096, and twice otherwise.  (The sum behind G-bar is fp64 in another
  * fixed order than dq_choose_bits'.)  dev_b is read and then overwritten with the next
  * (b, s).  dev_workspace: dq_round_workspace_bytes() bytes of 16-byte aligned device
  * memory, ZEROED ONCE before its first use and afterwards left to the calls; calls that may

@@ -2,13 +2,11 @@
 // ||g||_p of Eq. 5 applied per bucket; p = 2, or p = infinity for layouts created
 // with DQ_NORM_LINF), and dq_tensor_norms: one norm per tensor.
 //
-// Bucket lengths of 32 * 2^k are taken by the norm kernels of dq_round.cuh (the pipelines of the
-// quantizer without the codes), the others by the kernels below.  There, one team of LANES threads
-// (8, 16 or a full warp, by bucket size) owns a bucket: 128-bit coalesced loads, four independent fp32 accumulators per
-// lane, a shuffle reduction inside the team.  A warp takes runs of consecutive
-// buckets of one worker (blockIdx.y), so the tensor a bucket belongs to is
-// searched once per run and then followed; neighbouring warps read neighbouring
-// memory.  HBM-bound: 4 bytes read per element, 4/bucket bytes written.
+// Bucket lengths of up to 1024 elements, 2048 and 4096 are taken by the norm kernels of dq_round.cuh (the
+// pipelines of the quantizer without the codes), the others by the kernel below: 128-bit coalesced
+// loads, four independent fp32 accumulators per lane, a warp per run of consecutive buckets of one
+// worker (blockIdx.y), so that the tensor a bucket belongs to is searched once per run and then followed.
+// HBM-bound: 4 bytes read per element, 4/bucket bytes written.
 #include "dq_common.cuh"
 #include "dq_device.cuh"
 #include "dq_round.cuh"
@@ -16,20 +14,23 @@
 bool dq_norms_inside(const dq_layout_t* L)
 {
     const uint32_t gpb = (uint32_t)(L->bucket / 32);
-    return !L->whole_tensor && (gpb & (gpb - 1)) == 0;
+    return !L->whole_tensor && ((gpb & (gpb - 1)) == 0 || gpb < 32);
 }
 
 int64_t dq_tile_positions(const RoundArgs& a, bool given)
 {
     if (given) return (a.v.total_groups + 31) / 32;
-    if (a.gpb_shift > 5) return a.v.nb;
-    const int64_t R = 32 >> a.gpb_shift;
+    if (a.div_shift >= 0 && a.gpb_shift > 5) return a.v.nb;
+    const int64_t R = 32 / a.v.groups_per_bucket;
     return (a.v.nb + R - 1) / R;
 }
 
 int dq_norms_of_buckets(const RoundArgs& a, const CUtensorMap& map, int n_seg, cudaStream_t st)
 {
     const int64_t entries = dq_tile_positions(a, false) * a.M;
+    if (a.div_shift < 0)
+        return a.linf ? dq_launch_norms<kOddBuckets, true>(a, map, n_seg, entries, st)
+                      : dq_launch_norms<kOddBuckets, false>(a, map, n_seg, entries, st);
     if (a.gpb_shift <= 5)
         return a.linf ? dq_launch_norms<kWarpBuckets, true>(a, map, n_seg, entries, st)
                       : dq_launch_norms<kWarpBuckets, false>(a, map, n_seg, entries, st);
@@ -70,113 +71,25 @@ constexpr int kThreads = 256;
 constexpr int kRun = 8;            // bucket rows a warp handles per run
 
 // l2 norm of a bucket whose fp32 sum of squares is out of range (see l2_sum_in_range), read
-// again with plain loads by its team of LANES lanes: largest magnitude first, then the squares of
+// again with plain loads by the warp: largest magnitude first, then the squares of
 // the scaled entries.  Called by all lanes of the warp; out of line, it is rarely needed.
-template <int LANES>
 __device__ __noinline__ float rescaled_norm_global(const float* __restrict__ g, const int len, const int lane)
 {
     const MaxMagnitude mag;
     float mx = 0.f;
-    for (int i = lane; i < len; i += LANES) mx = mag.take(mx, __ldg(g + i));
+    for (int i = lane; i < len; i += 32) mx = mag.take(mx, __ldg(g + i));
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) mx = mag.join(mx, __shfl_xor_sync(0xffffffffu, mx, o, LANES));
+    for (int o = 16; o > 0; o >>= 1) mx = mag.join(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const int e = scale_exponent(mx);
     const ScaledSquares sq{e};
     float ss = 0.f;
-    for (int i = lane; i < len; i += LANES) ss = sq.take(ss, __ldg(g + i));
+    for (int i = lane; i < len; i += 32) ss = sq.take(ss, __ldg(g + i));
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) ss = sq.join(ss, __shfl_xor_sync(0xffffffffu, ss, o, LANES));
+    for (int o = 16; o > 0; o >>= 1) ss = sq.join(ss, __shfl_xor_sync(0xffffffffu, ss, o));
     return rescaled_l2(mx, ss, e);
 }
 
-template <int LANES, int P>
-__global__ void __launch_bounds__(kThreads)
-bucket_norms_kernel(const LayoutView v, const float* __restrict__ grads, const int64_t worker_stride,
-                    float* __restrict__ norms, int32_t* __restrict__ status)
-{
-    grid_dependency_wait();
-    constexpr int kTeamsPerWarp = 32 / LANES;
-    constexpr int kChunk = kRun * kTeamsPerWarp;          // buckets per run
-    const int lane = threadIdx.x % LANES;
-    const int team = (threadIdx.x % 32) / LANES;
-    const int m = blockIdx.y;
-    const float* gw = grads + (int64_t)m * worker_stride;
-    float* nw = norms + (int64_t)m * v.nb;
-    const int warps_total = gridDim.x * (kThreads / 32);
-    const int nchunks = (v.nb + kChunk - 1) / kChunk;
-    const int bsz = v.groups_per_bucket * 32;
-    bool bad = false;
-
-    // Every lane of a warp runs the same number of iterations of both loops, so
-    // the full-mask shuffles are safe; a team past the end works on an empty bucket.
-    for (int chunk = blockIdx.x * (kThreads / 32) + threadIdx.x / 32; chunk < nchunks; chunk += warps_total) {
-        int k = chunk * kChunk + team;
-        int seg = 0;
-        if (v.n_seg > 1) seg = last_not_above(v.seg_bucket0, v.n_seg, k < v.nb ? k : v.nb - 1);
-#pragma unroll 1
-        for (int r = 0; r < kRun; ++r, k += kTeamsPerWarp) {
-            const bool active = k < v.nb;
-            int len = 0;
-            int64_t start = 0;
-            if (active) {
-                int local, n, g0;
-                if (v.n_seg == 1) {
-                    local = k; n = v.seg0_elems; g0 = 0;
-                } else {
-                    while (k >= __ldg(v.seg_bucket0 + seg + 1)) ++seg;     // buckets only move forward
-                    local = k - __ldg(v.seg_bucket0 + seg);
-                    n = __ldg(v.seg_elems + seg);
-                    g0 = __ldg(v.seg_group0 + seg);
-                }
-                start = (int64_t)g0 * 32 + (int64_t)local * bsz;
-                const int left = n - local * bsz;
-                len = left < bsz ? left : bsz;
-            }
-            const float* g = gw + start;                                   // 128-byte aligned
-            const float4* g4 = reinterpret_cast<const float4*>(g);
-            const int n4 = len >> 2;
-
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            int i = lane;
-#pragma unroll 1
-            for (; i + 3 * LANES < n4; i += 4 * LANES) {
-                const float4 x0 = __ldg(g4 + i);
-                const float4 x1 = __ldg(g4 + i + LANES);
-                const float4 x2 = __ldg(g4 + i + 2 * LANES);
-                const float4 x3 = __ldg(g4 + i + 3 * LANES);
-                a0 = take<P>(a0, x0.x); a1 = take<P>(a1, x0.y); a2 = take<P>(a2, x0.z); a3 = take<P>(a3, x0.w);
-                a0 = take<P>(a0, x1.x); a1 = take<P>(a1, x1.y); a2 = take<P>(a2, x1.z); a3 = take<P>(a3, x1.w);
-                a0 = take<P>(a0, x2.x); a1 = take<P>(a1, x2.y); a2 = take<P>(a2, x2.z); a3 = take<P>(a3, x2.w);
-                a0 = take<P>(a0, x3.x); a1 = take<P>(a1, x3.y); a2 = take<P>(a2, x3.z); a3 = take<P>(a3, x3.w);
-            }
-            for (; i < n4; i += LANES) {
-                const float4 x = __ldg(g4 + i);
-                a0 = take<P>(a0, x.x); a1 = take<P>(a1, x.y); a2 = take<P>(a2, x.z); a3 = take<P>(a3, x.w);
-            }
-            if (lane < (len & 3)) {                       // ragged tail of the tensor's last bucket
-                const float x = __ldg(g + n4 * 4 + lane);
-                a0 = take<P>(a0, x);
-            }
-            float sum = join<P>(join<P>(a0, a1), join<P>(a2, a3));
-#pragma unroll
-            for (int o = LANES / 2; o > 0; o >>= 1) sum = join<P>(sum, __shfl_xor_sync(0xffffffffu, sum, o, LANES));
-            float nrm = finish<P>(sum);
-            if constexpr (P == DQ_NORM_L2) {
-                if (__any_sync(0xffffffffu, active && !l2_sum_in_range(sum))) {
-                    const float again = rescaled_norm_global<LANES>(g, len, lane);
-                    if (!l2_sum_in_range(sum)) nrm = again;
-                }
-            }
-            if (lane == 0 && active) {
-                DQ_STORE(nw + k, nrm, norms, (int64_t)gridDim.y * v.nb * 4, status);
-                bad |= !isfinite(nrm);
-            }
-        }
-    }
-    if (bad) atomicOr(status, DQ_STAT_NONFINITE);
-}
-
-// Full-warp variant for buckets of at least 128 elements.  A warp takes a run of
+// A warp takes a run of
 // eight consecutive buckets: it first works out where each of them lies (so
 // that table lookups never sit between a load and its use), then streams the
 // eight buckets with independent accumulators, and finally reduces the eight
@@ -293,7 +206,7 @@ bucket_norms_warp_kernel(const LayoutView v, const float* __restrict__ grads, co
 #pragma unroll
                 for (int r = 0; r < kRun; ++r) {
                     if ((need >> r) & 1u) {
-                        const float again = rescaled_norm_global<32>(gw + (int64_t)first[r] * 4, len[r], lane);
+                        const float again = rescaled_norm_global(gw + (int64_t)first[r] * 4, len[r], lane);
                         if (lane == r) nrm = again;
                     }
                 }
@@ -365,7 +278,7 @@ tensor_norms_join_kernel(const int32_t n_seg, const int32_t* __restrict__ piece0
     if (!isfinite(nrm)) atomicOr(status, DQ_STAT_NONFINITE);
 }
 
-// Norms of the buckets of view `v` (32 * 2^k elements, up to 4096).
+// Norms of the buckets of view `v` (see dq_norms_inside).
 int launch_norms(const dq_layout_t* L, const LayoutView& v, const float* dev_grads, int64_t worker_stride_elems, int32_t M,
                  float* dev_out, int32_t* dev_status, cudaStream_t st)
 {
@@ -376,13 +289,12 @@ int launch_norms(const dq_layout_t* L, const LayoutView& v, const float* dev_gra
     return dq_norms_of_buckets(a, map, L->n_seg, st);
 }
 
-// other bucket sizes: plain-load kernels
+// other bucket sizes: the plain-load kernel
 template <int P>
 int launch_plain(const dq_layout_t* L, const LayoutView& v, const float* dev_grads, int64_t worker_stride_elems, int32_t M,
                  float* dev_norms, int32_t* dev_status, cudaStream_t st)
 {
-    const int lanes = L->bucket >= 128 ? 32 : (L->bucket >= 64 ? 16 : 8);
-    const int64_t chunk = (int64_t)kRun * (32 / lanes);
+    const int64_t chunk = kRun;
     const int64_t nchunks = (L->nb + chunk - 1) / chunk;
     int64_t bx = (nchunks + kThreads / 32 - 1) / (kThreads / 32);
     // about 8 resident CTAs of 256 threads per SM over all workers
@@ -391,14 +303,8 @@ int launch_plain(const dq_layout_t* L, const LayoutView& v, const float* dev_gra
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
     const dim3 grid((unsigned)bx, (unsigned)M);
-    if (lanes == 32) {
-        const size_t smem = (L->n_seg > 1 && (size_t)3 * (L->n_seg + 1) * 4 <= 12 * 1024) ? (size_t)3 * (L->n_seg + 1) * 4 : 0;
-        dq_launch(bucket_norms_warp_kernel<P>, grid, dim3(kThreads), smem, st, v, dev_grads, worker_stride_elems, dev_norms, dev_status);
-    }
-    else if (lanes == 16)
-        dq_launch(bucket_norms_kernel<16, P>, grid, dim3(kThreads), 0, st, v, dev_grads, worker_stride_elems, dev_norms, dev_status);
-    else
-        dq_launch(bucket_norms_kernel<8, P>, grid, dim3(kThreads), 0, st, v, dev_grads, worker_stride_elems, dev_norms, dev_status);
+    const size_t smem = (L->n_seg > 1 && (size_t)3 * (L->n_seg + 1) * 4 <= 12 * 1024) ? (size_t)3 * (L->n_seg + 1) * 4 : 0;
+    dq_launch(bucket_norms_warp_kernel<P>, grid, dim3(kThreads), smem, st, v, dev_grads, worker_stride_elems, dev_norms, dev_status);
     if (cudaGetLastError() != cudaSuccess) return DQ_ERR_CUDA;
     return DQ_OK;
 }

@@ -51,6 +51,9 @@ int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, boo
 {
     const int64_t entries = dq_tile_positions(a, given) * (AVG ? 1 : a.M);
     if (given) return dq_launch_round<kGivenNorms, AVG, false>(a, map, L->n_seg, entries, st);
+    if (a.div_shift < 0)
+        return a.linf ? dq_launch_round<kOddBuckets, AVG, true>(a, map, L->n_seg, entries, st)
+                      : dq_launch_round<kOddBuckets, AVG, false>(a, map, L->n_seg, entries, st);
     if (a.gpb_shift <= 5)
         return a.linf ? dq_launch_round<kWarpBuckets, AVG, true>(a, map, L->n_seg, entries, st)
                       : dq_launch_round<kWarpBuckets, AVG, false>(a, map, L->n_seg, entries, st);
@@ -71,7 +74,7 @@ int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, boo
 bool one_pass(const RoundArgs& a, bool given)
 {
     int64_t units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
-    if (!given && a.gpb_shift > 5) units >>= a.gpb_shift - 5;
+    if (!given && a.div_shift >= 0 && a.gpb_shift > 5) units >>= a.gpb_shift - 5;
     const int64_t p = dq_tile_positions(a, given);
     const int64_t full = p / units;
     const double f = (double)(p - full * units) / (double)units;

@@ -4,6 +4,7 @@
 //
 // Modes (where the norms come from):
 //   kWarpBuckets   buckets of 32 * 2^k <= 1024 elements: a warp tile is 1024 / bucket buckets
+//   kOddBuckets    other buckets of up to 992 elements: a warp tile is as many buckets as 32 groups hold
 //   kTeamBuckets   buckets of 2048 or 4096: a team of 2 or 4 warps of the CTA takes a bucket
 //   kGivenNorms    any bucket length, whole-tensor layouts: norms are read, a tile is 32 groups
 // B = 0: norms alone.  AVG = false: codes (and norms) of every worker.  AVG = true: a warp keeps its tile of the output
@@ -22,7 +23,7 @@
 #include "dq_rule.cuh"
 #include "dq_tma.cuh"
 
-enum RoundMode { kWarpBuckets = 0, kTeamBuckets = 1, kGivenNorms = 2 };
+enum RoundMode { kWarpBuckets = 0, kTeamBuckets = 1, kGivenNorms = 2, kOddBuckets = 3 };
 
 struct RoundArgs {
     LayoutView v;
@@ -37,8 +38,8 @@ struct RoundArgs {
     uint32_t worker0;             // worker m of the call draws the uniforms of worker worker0 + m
     int32_t M;
     int32_t map_has_worker_dim;   // 0 when all workers read the same buffer (stride 0)
-    int32_t gpb_shift;            // log2(groups per bucket), computed norms only
-    uint32_t div_magic;           // kGivenNorms: groups_per_bucket as multiply-shift, or as a shift if a power of two
+    int32_t gpb_shift;            // log2(groups per bucket) (kWarpBuckets, kTeamBuckets)
+    uint32_t div_magic;           // groups_per_bucket as multiply-shift, or as a shift if a power of two
     int32_t div_shift;            //              (>= 0: the shift; < 0: use div_magic with a 33-bit shift)
     int32_t stream_reads;         // 1: more than 64 MB of gradients (see the L2 policy of the reads)
     int32_t linf;                 // norm kind (host: which kernel)
@@ -143,6 +144,7 @@ struct TilePos {
     int valid;       // elements of that group that count (0: nobody's row)
     int bucket;      // its bucket
     int span;        // groups of the tile that get words
+    int len;         // kOddBuckets: elements of this lane's bucket
     bool regular;    // every lane owns its own full row
     bool writes;     // this lane writes the norm of its bucket
 };
@@ -238,6 +240,83 @@ struct MaxOp { __device__ __forceinline__ float operator()(const float a, const 
 template <bool LINF> struct JoinOp { using type = AddOp; };
 template <> struct JoinOp<true> { using type = MaxOp; };
 
+// kOddBuckets: the bucket sums (maxima) of a tile, in the order of the kernel that took such buckets before.
+// The warp goes through the buckets one by one -- half warps two by two for buckets of 96 --, lane i taking
+// the bucket's float4s i, i + 32, ...; a lane gets the result of its own bucket, r (1 if it has none).
+// stage: byte offset of the tile; the buckets' first rows and lengths are with the lanes r * gpb.
+__device__ __forceinline__ float4 stage_float4(const uint32_t stage, const int first, const int i)
+{
+    const int row = first + (i >> 3);
+    return *reinterpret_cast<const float4*>(smem + stage + tma::swizzle128(row, i & 7));
+}
+__device__ __forceinline__ float stage_float(const uint32_t stage, const int first, const int e)
+{
+    const int row = first + (e >> 5);
+    return *reinterpret_cast<const float*>(smem + stage + tma::swizzle128(row, (e >> 2) & 7) + ((e & 3) << 2));
+}
+template <int P>
+__device__ __forceinline__ float odd_share(const uint32_t stage, const int first, const int len, const int lane, const int lanes)
+{
+    const int n4 = len >> 2;
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    for (int i = lane; i < n4; i += lanes) {
+        const float4 x = stage_float4(stage, first, i);
+        a0 = take<P>(a0, x.x); a1 = take<P>(a1, x.y); a2 = take<P>(a2, x.z); a3 = take<P>(a3, x.w);
+    }
+    if (lane < (len & 3)) a0 = take<P>(a0, stage_float(stage, first, n4 * 4 + lane));
+    return join<P>(join<P>(a0, a1), join<P>(a2, a3));
+}
+template <bool LINF>
+__device__ __forceinline__ float odd_bucket_sums(const uint32_t stage, const int row, const int len, const int gpb, const int R, const int r)
+{
+    constexpr int P = LINF ? DQ_NORM_LINF : DQ_NORM_L2;
+    const int lane = threadIdx.x & 31;
+    float mine = 1.0f;
+    if (gpb >= 4) {
+        for (int k = 0; k < R; ++k) {
+            const int first = __shfl_sync(0xffffffffu, row, k * gpb), n = __shfl_sync(0xffffffffu, len, k * gpb);
+            float v = odd_share<P>(stage, first, n, lane, 32);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) v = join<P>(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (r == k) mine = v;
+        }
+    } else {                                     // 96 elements: R = 10, an even number
+        for (int k = 0; k < R; k += 2) {
+            const int src = (k + (lane >> 4)) * gpb;
+            const int first = __shfl_sync(0xffffffffu, row, src), n = __shfl_sync(0xffffffffu, len, src);
+            float v = odd_share<P>(stage, first, n, lane & 15, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) v = join<P>(v, __shfl_xor_sync(0xffffffffu, v, o));
+            const float lo = __shfl_sync(0xffffffffu, v, 0), hi = __shfl_sync(0xffffffffu, v, 16);
+            if (r == k) mine = lo;
+            if (r == k + 1) mine = hi;
+        }
+    }
+    return mine;
+}
+// ... and the norms of those out of range, as rare_norm has them.
+__device__ __noinline__ float rare_norm_odd(const uint32_t stage, const int row, const int len, const int gpb, const int R, const int r,
+                                            const float sum, const float nrm)
+{
+    const int lane = threadIdx.x & 31, lanes = gpb >= 4 ? 32 : 16;
+    float mine = nrm;
+    for (int k = 0; k < R; ++k) {
+        const int first = __shfl_sync(0xffffffffu, row, k * gpb), n = __shfl_sync(0xffffffffu, len, k * gpb);
+        const MaxMagnitude mag;
+        float mx = 0.f, ss = 0.f;
+        if (lane < lanes)
+            for (int i = lane; i < n; i += lanes) mx = mag.take(mx, stage_float(stage, first, i));
+        for (int o = 16; o > 0; o >>= 1) mx = mag.join(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const int e = scale_exponent(mx);
+        const ScaledSquares sq{e};
+        if (lane < lanes)
+            for (int i = lane; i < n; i += lanes) ss = sq.take(ss, stage_float(stage, first, i));
+        for (int o = 16; o > 0; o >>= 1) ss = sq.join(ss, __shfl_xor_sync(0xffffffffu, ss, o));
+        if (r == k && !l2_sum_in_range(sum)) mine = rescaled_l2(mx, ss, e);
+    }
+    return mine;
+}
+
 // The l2 norm of buckets whose sum of squares is out of range (see l2_sum_in_range): all zeros, tiny
 // entries, an overflowed square.  Called by all lanes of the warp (by all warps of a team, which agree
 // on the sum); zero buckets are settled by their largest magnitude, the others are reduced again with
@@ -282,15 +361,19 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     const int M = a.M;
     const int nb = a.v.nb;
     const int G = a.v.total_groups;
-    const int gpb = 1 << a.gpb_shift;
+    constexpr bool ODD = MODE == kOddBuckets;
+    constexpr bool TILES = MODE == kWarpBuckets || ODD;               // tiles of whole buckets
+    const int gpb = ODD ? a.v.groups_per_bucket : 1 << a.gpb_shift;
     // warps of the CTA that share a bucket, and this warp's place among them
     const int T_shift = MODE == kTeamBuckets ? a.gpb_shift - 5 : 0;
     const int T = 1 << T_shift;
     const int sub = warp & (T - 1);
-    const int R = MODE == kWarpBuckets ? 32 >> a.gpb_shift : 1;       // buckets per warp tile
+    const int R = ODD ? 32 / gpb : (MODE == kWarpBuckets ? 32 >> a.gpb_shift : 1);       // buckets per warp tile
+    // of a regular tile: the lane's bucket and its group in there (kOddBuckets: the last lanes may have none, r >= R)
+    const int r = ODD ? lane / gpb : lane >> a.gpb_shift, l = lane - (ODD ? r * gpb : r << a.gpb_shift);
 
     // Tile positions of one worker; a team takes bucket `pos`, each of its warps 1024 elements of it.
-    const int positions = MODE == kWarpBuckets ? (nb + R - 1) / R : (MODE == kTeamBuckets ? nb : (G + 31) / 32);
+    const int positions = TILES ? (nb + R - 1) / R : (MODE == kTeamBuckets ? nb : (G + 31) / 32);
     // The list of work: positions (AVG: every position goes through all workers), or the worker-major
     // list of all tiles.  Each unit -- a warp, or a team -- takes every hop-th entry, `each` of them, the
     // first `extra` units one more: dense and sparse stretches of a gradient then fall to all units alike
@@ -319,6 +402,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     // a full row of it; kNoTile if a team's bucket ends before this warp's share.  kGivenNorms: the tensor of
     // the tile's first group.  c_*: the tensor looked at last.
     int c_b0 = 0, c_g0 = 0, c_n = a.v.seg0_elems, c_end = a.v.n_seg == 1 ? 0x7fffffff : 0;
+    int c_full = ODD ? (int)div_gpb(a, (uint32_t)c_n >> 5) : c_n >> (a.gpb_shift + 5);        // its full buckets
     auto describe = [&](int p) -> uint32_t {
         const int k0 = MODE == kGivenNorms ? p * 32 : p * R;
         if constexpr (MODE == kGivenNorms) {
@@ -330,11 +414,11 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 c_end = tbl(n1 + i + 1);
                 c_g0 = tbl(i);
                 c_n = tbl(2 * n1 + i);
+                c_full = ODD ? (int)div_gpb(a, (uint32_t)c_n >> 5) : c_n >> (a.gpb_shift + 5);
             }
             const int local = k0 - c_b0;
-            if constexpr (MODE == kWarpBuckets) {
-                const int full = c_n >> (a.gpb_shift + 5);
-                return (uint32_t)(c_g0 + (local << a.gpb_shift)) | (local + R <= full ? 0x80000000u : 0u);
+            if constexpr (TILES) {
+                return (uint32_t)(c_g0 + (ODD ? local * gpb : local << a.gpb_shift)) | (local + R <= c_full ? 0x80000000u : 0u);
             } else {
                 const int share = (local << T_shift) + sub;              // 1024-element pieces of the tensor before it
                 const int left = c_n - share * 1024;
@@ -348,16 +432,21 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
         t.row = lane; t.valid = 32; t.span = 32; t.bucket = p; t.writes = false;
         t.row0 = MODE == kGivenNorms ? p * 32 : (int)(desc & 0x7fffffffu);
         t.regular = (desc >> 31) != 0;
-        if constexpr (MODE == kWarpBuckets) {
-            const int r = lane >> a.gpb_shift, l = lane & (gpb - 1);
+        t.len = gpb * 32;
+        if constexpr (TILES) {
             const int k = p * R + r;
+            const bool mine = k < nb && (!ODD || r < R);
             t.bucket = k;
-            t.writes = l == 0 && k < nb;
+            t.writes = l == 0 && mine;
+            if (ODD) {
+                t.valid = r < R ? 32 : 0;
+                t.span = R * gpb;
+            }
             if (!t.regular) {
                 // the tile touches the end of a tensor: buckets may be short, rows may be nobody's
                 int first = 0, len = 0;
                 const int seg0 = a.v.n_seg > 1 ? find_seg(1, p * R) : 0;
-                if (k < nb) {
+                if (mine) {
                     int local = k, n = a.v.seg0_elems, g0 = 0;
                     if (a.v.n_seg > 1) {
                         const int i = walk_seg(1, seg0, k);
@@ -365,14 +454,15 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                         n = tbl(2 * n1 + i);
                         g0 = tbl(i);
                     }
-                    first = g0 + (local << a.gpb_shift);
+                    first = g0 + (ODD ? local * gpb : local << a.gpb_shift);
                     const int left = n - local * (gpb * 32);
                     len = left < gpb * 32 ? left : gpb * 32;
                 }
                 t.row = first - t.row0 + l;
                 const int v = len - l * 32;
                 t.valid = v < 0 ? 0 : (v > 32 ? 32 : v);
-                if (t.valid == 0) t.row = lane;
+                t.len = len;
+                if (t.valid == 0 && !(ODD && l == 0 && mine)) t.row = lane;
                 t.span = __reduce_max_sync(0xffffffffu, t.valid > 0 ? t.row + 1 : 0);
             }
         } else if constexpr (MODE == kTeamBuckets) {
@@ -520,8 +610,12 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             plain = !__any_sync(0xffffffffu, LINF ? !norm_is_plain(v) : !l2_sum_in_range(v));
             if (!plain) {
                 if constexpr (!LINF) {
-                    nrm = rare_norm<MODE>(row, t.valid, gpb, slots, T_shift, exchanges, v, nrm);
-                    exchanges += 2;
+                    if constexpr (ODD) {
+                        nrm = rare_norm_odd(row - own, t.row, t.len, gpb, R, r, v, nrm);
+                    } else {
+                        nrm = rare_norm<MODE>(row, t.valid, gpb, slots, T_shift, exchanges, v, nrm);
+                        exchanges += 2;
+                    }
                 }
                 inv = inv_scale(sf, nrm);
                 bad |= t.writes && !isfinite(nrm);
@@ -551,7 +645,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 if (t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
             } else {
                 bool lost = false;
-                const float v = join_team<MODE>(join_lanes<MODE>(row_share(row), gpb, Join{}), slots, T_shift, exchanges, landed,
+                float v;
+                if constexpr (ODD) v = odd_bucket_sums<LINF>(row - own, t.row, t.len, gpb, R, r);
+                else v = join_team<MODE>(join_lanes<MODE>(row_share(row), gpb, Join{}), slots, T_shift, exchanges, landed,
                                                 lost, Join{});
                 if (lost) { timed_out = true; break; }
                 scale_of(v);

@@ -39,7 +39,9 @@ def _grads(ref, segs, M, seed):
 
 
 CASES = [(RAGGED, 512, 3, 4), (RAGGED, 32, 2, 7), (RAGGED, 1024, 5, 3), (RAGGED, 2048, 3, 5), (RAGGED, 4096, 2, 8),
-         (RAGGED, 96, 2, 6), (RAGGED, 0, 3, 4), ([1 << 18], 512, 4, 2), ([70001], 128, 1, 16), ([1], 4096, 2, 4),
+         (RAGGED, 96, 2, 6), (RAGGED, 0, 3, 4),
+         (RAGGED, 96, 3, 4), (RAGGED, 160, 2, 5), (RAGGED, 480, 3, 4), (RAGGED, 992, 2, 7), (RAGGED, 1056, 2, 4), ([100001], 96, 5, 3),
+         ([1 << 18], 512, 4, 2), ([70001], 128, 1, 16), ([1], 4096, 2, 4),
          ([33] * 1100, 64, 2, 12), ([300000], 2048, 33, 4), (RAGGED, 512, 24, 5), (RAGGED, 4096, 24, 4), (RAGGED, 0, 24, 7), (RAGGED, 480, 24, 3),
          ([3 << 20], 512, 8, 4)] + [(RAGGED, 256, 2, b) for b in range(1, 17)]
 
