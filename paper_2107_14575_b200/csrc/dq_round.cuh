@@ -16,6 +16,11 @@
 // bucket combine by shuffles, then the lane encodes its row against that norm; the words leave from
 // registers or through the consumed stage, which is refilled.
 // HBM traffic: 4 + b/8 bytes per element and worker, plus 4 (8 with the update) per output element.
+// What bounds it: per tile of a worker a warp issues some 530 instructions at b = 4 (290 of them the codes,
+// their draws and the sums; 65 are the wide multiplies of the generator, four cycles of the multiplier
+// each), 65 % of the issue slots' and 70 % of the multiplier's time, beside loads that alone take 0.9 of
+// the measured copy bandwidth.  Measured: 2^26 elements M = 32 b = 4 1.89 ms (5.2 TB/s; separate
+// quantizer and average 2.29), ResNet-18 shape M = 8 92 us (4.9), VGG-16 shape M = 16 b = 5 with update 260 us.
 #pragma once
 
 #include "dq_common.cuh"

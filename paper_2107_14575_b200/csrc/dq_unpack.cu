@@ -12,7 +12,10 @@
 // swizzled 4 KB tile of the warp and leave with one bulk tensor store (straight from registers, 32 bytes a
 // lane, every store touched 32 lines: one worker, 2^25 elements, b = 4 37 us against 30).
 // HBM traffic per output element: M*b/8 bytes read, 4 written.  Bound by the logic pipe for small b
-// (one half-rate operation per code), by HBM from b = 8 on.  AVERAGE_FIGURES
+// (one half-rate operation per code) and the issue of about 100 instructions per lane, worker and group,
+// by HBM from b = 8 on.  Measured, d = 8.4M, M = 16: b = 4 23.8 us (4.2 TB/s), b = 8 30.2 us (5.6), b = 16
+// 51.7 us (5.8); one worker, 2^25 elements, b = 4 26.9 us (5.6).  (Codes taken two at a time as fp16 pairs,
+// for half the logic operations, and widened by mixed-precision adds: 9 % slower at b = 4.)
 //
 // dq_unpack_average_update ends with the parameter update of Algorithm 1 instead, x <- x - eta * average;
 // the averaged gradient itself never reaches memory (M*b/8 + 4 bytes read and 4 written per element).
