@@ -13,7 +13,7 @@
 // lane, every store touched 32 lines: one worker, 2^25 elements, b = 4 37 us against 30).
 // HBM traffic per output element: M*b/8 bytes read, 4 written.  Bound by the logic pipe for small b
 // (one half-rate operation per code) and the issue of about 100 instructions per lane, worker and group,
-// by HBM from b = 8 on.  Measured, d = 8.4M, M = 16: b = 4 23.8 us (4.2 TB/s), b = 8 30.2 us (5.6), b = 16
+// by HBM from b = 8 on.  For many workers and b <= 4 the words go straight into registers (below).  Measured, d = 8.4M, M = 16: b = 4 23.8 us (4.2 TB/s), b = 8 30.2 us (5.6), b = 16
 // 51.7 us (5.8); one worker, 2^25 elements, b = 4 26.9 us (5.6).  (Codes taken two at a time as fp16 pairs,
 // for half the logic operations, and widened by mixed-precision adds: 9 % slower at b = 4.)
 //
@@ -162,16 +162,210 @@ struct Normalise<B, 32> {
     static __device__ __forceinline__ void run(float (&)[32]) {}
 };
 
+// The end of a tile: the powers of two removed, padding zeroed, the rows through the warp's output tile.
+// False if the tile of x did not arrive.
+template <int B>
+__device__ __forceinline__ bool finish_tile(const AverageArgs& a, const CUtensorMap* out_map, unsigned char* out_tile,
+                                            const uint64_t (&acc2)[16], const int tile, const int valid, uint64_t* xbar,
+                                            const uint32_t x_parity)
+{
+    const int lane = threadIdx.x & 31;
+    // (B = 1: s = 0, every value is 0, and an update by 0 leaves x as it is)
+    if (!(B == 1 && a.update)) {
+        float acc[32];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], acc[2 * q], acc[2 * q + 1]);
+        Normalise<B, 0>::run(acc);
+        if (valid < 32) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+                if (e >= valid) acc[e] = 0.0f;
+        }
+        if (a.update) {
+            // nothing is stored from a tile whose parameters did not arrive
+            if (!__all_sync(0xffffffffu, tma::mbar_wait(xbar, x_parity, a.wait))) return false;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float4* p = reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c));
+                const float4 x = *p;
+                *p = make_float4(fmaf(a.neg_lr, acc[4 * c], x.x), fmaf(a.neg_lr, acc[4 * c + 1], x.y),
+                                 fmaf(a.neg_lr, acc[4 * c + 2], x.z), fmaf(a.neg_lr, acc[4 * c + 3], x.w));
+            }
+        } else {
+            if (lane == 0) tma::store_wait_read();
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                *reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c)) =
+                    make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+        }
+        tma::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            tma::store_tile_2d(out_map, out_tile, 0, tile * 32);          // (rows outside the layout are clipped)
+            tma::store_commit();
+        }
+    }
+    return true;
+}
+// The start of a tile of the update: the tile before must have left the warp's output tile; the tile of x
+// travels while the codes are decoded.
+__device__ __forceinline__ void request_x(const CUtensorMap* out_map, unsigned char* out_tile, const int tile, uint64_t* xbar)
+{
+    tma::store_wait_read();
+    tma::mbar_expect_tx(xbar, kOutBytes);
+    tma::load_tile_2d(out_tile, out_map, xbar, 0, tile * 32);
+}
+// Bucket and valid elements of this lane's group in a tile (valid 0: the group lies beyond the layout).
+__device__ __forceinline__ void locate_group(const AverageArgs& a, const bool tbl_in_smem, const int tile, int& bucket, int& valid)
+{
+    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
+    auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
+    const int n1 = a.v.n_seg + 1;
+    const int g = tile * 32 + (threadIdx.x & 31);
+    int seg = 0;
+    if (a.v.n_seg > 1) seg = last_not_above_by_warp(tile * 32, a.v.n_seg, tbl);
+    bucket = 0;
+    valid = 0;
+    if (g >= a.v.total_groups) return;
+    int local = g, n = a.v.seg0_elems, b0 = 0;
+    if (a.v.n_seg > 1) {
+        while (g >= tbl(seg + 1)) ++seg;
+        local = g - tbl(seg);
+        b0 = tbl(n1 + seg);
+        n = tbl(2 * n1 + seg);
+    }
+    bucket = b0 + (int)div_gpb(a, (uint32_t)local);
+    const int left = n - local * 32;
+    valid = left < 32 ? left : 32;
+}
+
+// ---- b = 2, 3, 4 and 20 workers or more: words straight into registers --------------------------
+// A lane's words of a worker are one to three loads that neighbouring lanes coalesce.  Up to eight workers'
+// words and norms wait in registers; as soon as one has been decoded, its registers are the target of
+// the load for the worker eight further on (of the next tile, when this one's are through), so nothing is
+// moved, staged or waited for.  Pays where tiles are long: staged / direct (us), 2^24 elements M = 32 b = 2
+// 73.7 / 65.4, b = 3 78.3 / 72.0, b = 4 78.5 / 75.8, VGG-16 shape M = 24 b = 4 55.8 / 55.2; d = 8.4M M = 16
+// b = 4 23.9 / 24.4, 2^24 elements M = 4 19.6 / 22.3.
+template <int B>
+struct DirectWords {
+    static constexpr bool value = B >= 2 && B <= 4;
+    static constexpr int workers = 8;
+    static constexpr int min_workers = 20;
+};
+template <int B>
+__device__ __forceinline__ void request_words(const uint32_t* p, uint32_t (&w)[B])
+{
+    if constexpr (B == 4) {
+        asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
+    } else if constexpr (B == 2) {
+        asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
+    } else {
+#pragma unroll
+        for (int i = 0; i < B; ++i) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[i]) : "l"(p + i));
+    }
+}
+template <int B>
+__device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const CUtensorMap* out_map, const bool tbl_in_smem)
+{
+    constexpr int s = (1 << (B - 1)) - 1;
+    constexpr int MC = DirectWords<B>::workers;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = a.v.total_groups, M = a.M, nb = a.v.nb;
+    const float unit = __fdiv_rn(1.0f, (float)s * (float)M);      // 1 / (s * M)
+    const uint32_t magic = a.magic;
+    const uint32_t id = blockIdx.x * kWarps + warp;
+    const int hop = (int)(gridDim.x * kWarps);
+    const int n_tiles = (int)(a.each + (id < a.extra ? 1u : 0u));
+    if (n_tiles == 0) return;
+    if (a.wait.lose_first != 0u) {               // (test hook; there is no copy in flight yet)
+        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
+        return;
+    }
+    unsigned char* out_tile = smem + warp * kOutBytes;
+
+    int tile = (int)id, bucket, valid;
+    locate_group(a, tbl_in_smem, tile, bucket, valid);
+    // words and norm of worker m for this lane's group of a tile (a group beyond the layout reads the last one)
+    auto words_of = [&](int tl, int m) -> const uint32_t* {
+        const int g = tl * 32 + lane;
+        return a.packed + (int64_t)m * a.packed_stride + (int64_t)(g < G ? g : G - 1) * B;
+    };
+    uint32_t wd[MC][B];
+    float nrm[MC];
+    {
+        const uint32_t* p = words_of(tile, 0);
+        const float* q = a.norms + bucket;
+#pragma unroll
+        for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
+            if (j < M) {
+                request_words<B>(p, wd[j]);
+                nrm[j] = load_norm_early(q);
+            }
+        }
+    }
+    auto decode = [&](uint64_t (&acc2)[16], const uint32_t (&w)[B], const float norm) {
+        uint32_t hi[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) hi[i] = w[i] >> 16;
+        const uint32_t sc = __float_as_uint(norm * unit);
+        AccumulateAll<B, 0>::run(acc2, w, hi, pack_pair(sc, sc), magic);
+    };
+    for (int k = 0; k < n_tiles; ++k) {
+        uint64_t acc2[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
+        int nbucket = bucket, nvalid = valid;
+        if (a.update && lane == 0) request_x(out_map, out_tile, tile, x_bar(warp));
+#pragma unroll 1
+        for (int m0 = 0; m0 < M; m0 += MC) {
+            // the workers eight further on: of this tile, or the first ones of the next
+            const bool same = m0 + MC < M;
+            if (!same && k + 1 < n_tiles) locate_group(a, tbl_in_smem, tile + hop, nbucket, nvalid);
+            const int first = same ? m0 + MC : 0;
+            const int more = same ? M - first : (k + 1 < n_tiles ? M : 0);        // workers that are there to be requested
+            const uint32_t* p = words_of(same ? tile : tile + hop, first);
+            const float* q = a.norms + (int64_t)first * nb + (same ? bucket : nbucket);
+            if (m0 + MC <= M && more >= MC) {
+#pragma unroll
+                for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
+                    decode(acc2, wd[j], nrm[j]);
+                    request_words<B>(p, wd[j]);
+                    nrm[j] = load_norm_early(q);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
+                    if (m0 + j < M) decode(acc2, wd[j], nrm[j]);
+                    if (j < more) {
+                        request_words<B>(p, wd[j]);
+                        nrm[j] = load_norm_early(q);
+                    }
+                }
+            }
+        }
+        if (!finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), (uint32_t)k & 1u)) {
+            if (lane == 0) {
+                atomicOr(a.status, DQ_STAT_WAIT);
+                tma::store_wait_read();
+            }
+            (void)tma::mbar_wait(x_bar(warp), (uint32_t)k & 1u, a.wait);       // the copy must not outlive the shared memory
+            return;
+        }
+        tile += hop;
+        bucket = nbucket;
+        valid = nvalid;
+    }
+    if (lane == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
+}
+
 template <int B>
 __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtensorMap* out_map, const bool tbl_in_smem)
 {
     constexpr int s = (1 << (B - 1)) - 1;
     constexpr int MC = ChunkOf<B>::value;
-    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + kTblOffset);
-    auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int G = a.v.total_groups, M = a.M, nb = a.v.nb;
-    const int n1 = a.v.n_seg + 1;
     const int nchunk = (M + MC - 1) / MC;
     const float unit = (B == 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);      // 1 / (s * M)
     const uint32_t magic = a.magic;
@@ -182,25 +376,7 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
     const int n_tiles = (int)(a.each + (id < a.extra ? 1u : 0u));
     const int items = (B == 1) ? 0 : n_tiles * nchunk;
 
-    // bucket and valid elements of this lane's group in a tile (valid 0: the group lies beyond the layout)
-    auto locate = [&](int tile, int& bucket, int& valid) {
-        const int g = tile * 32 + lane;
-        int seg = 0;
-        if (a.v.n_seg > 1) seg = last_not_above_by_warp(tile * 32, a.v.n_seg, tbl);
-        bucket = 0;
-        valid = 0;
-        if (g >= G) return;
-        int local = g, n = a.v.seg0_elems, b0 = 0;
-        if (a.v.n_seg > 1) {
-            while (g >= tbl(seg + 1)) ++seg;
-            local = g - tbl(seg);
-            b0 = tbl(n1 + seg);
-            n = tbl(2 * n1 + seg);
-        }
-        bucket = b0 + (int)div_gpb(a, (uint32_t)local);
-        const int left = n - local * 32;
-        valid = left < 32 ? left : 32;
-    };
+    auto locate = [&](int tl, int& bk, int& vl) { locate_group(a, tbl_in_smem, tl, bk, vl); };
 
     // ---- producer side: item = (tile, chunk of workers), fetched two ahead of the consumer
     int p_tile = (int)id, p_m0 = 0, p_left = items;
@@ -223,12 +399,17 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
     int tile = (int)id, bucket, valid;
     locate(tile < (G + 31) / 32 ? tile : 0, bucket, valid);
     float scale[MC], nxt[MC];
-    auto request_norms = [&](int m0, int bk, int vl) {
+    auto request_norms = [&](int m0, int bk) {
         const float* p = a.norms + (int64_t)m0 * nb + bk;
+        if (m0 + MC <= M) {
 #pragma unroll
-        for (int j = 0; j < MC; ++j, p += nb) nxt[j] = (m0 + j < M && vl > 0) ? load_norm_early(p) : 0.0f;
+            for (int j = 0; j < MC; ++j) nxt[j] = load_norm_early(p + (int64_t)j * nb);
+        } else {
+#pragma unroll
+            for (int j = 0; j < MC; ++j) nxt[j] = m0 + j < M ? load_norm_early(p + (int64_t)j * nb) : 0.0f;
+        }
     };
-    if (items > 0) request_norms(0, bucket, valid);
+    if (items > 0) request_norms(0, bucket);
 
     unsigned char* out_tile = smem + warp * kOutBytes;
     uint32_t it = 0;
@@ -241,13 +422,8 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
 #pragma unroll
         for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
         int nbucket = bucket, nvalid = valid;
-        // the tile before must have left the warp's output tile; the tile of x travels while the codes are decoded
         x_parity = (uint32_t)k & 1u;
-        if (B > 1 && a.update && lane == 0) {
-            tma::store_wait_read();
-            tma::mbar_expect_tx(x_bar(warp), kOutBytes);
-            tma::load_tile_2d(out_tile, out_map, x_bar(warp), 0, tile * 32);
-        }
+        if (B > 1 && a.update && lane == 0) request_x(out_map, out_tile, tile, x_bar(warp));
         if constexpr (B > 1) {
 #pragma unroll 1
             for (int m0 = 0; m0 < M; m0 += MC, ++it) {
@@ -256,10 +432,10 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
 #pragma unroll
                 for (int j = 0; j < MC; ++j) scale[j] = nxt[j] * unit;
                 if (m0 + MC < M) {
-                    request_norms(m0 + MC, bucket, valid);
+                    request_norms(m0 + MC, bucket);
                 } else if (k + 1 < n_tiles) {
                     locate(tile + hop, nbucket, nvalid);
-                    request_norms(0, nbucket, nvalid);
+                    request_norms(0, nbucket);
                 }
                 // every lane polls the barrier itself; the verdict is made warp-uniform
                 if (!__all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), (it >> 1) & 1u, a.wait))) {
@@ -295,45 +471,7 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
             }
             if (timed_out) break;
         }
-        // (B = 1: s = 0, every value is 0, and an update by 0 leaves x as it is)
-        if (!(B == 1 && a.update)) {
-            float acc[32];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], acc[2 * q], acc[2 * q + 1]);
-            Normalise<B, 0>::run(acc);
-            if (valid < 32) {
-#pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    if (e >= valid) acc[e] = 0.0f;
-            }
-            if (a.update) {
-                // nothing is stored from a tile whose parameters did not arrive
-                if (!__all_sync(0xffffffffu, tma::mbar_wait(x_bar(warp), x_parity, a.wait))) {
-                    timed_out = true;
-                    break;
-                }
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    float4* p = reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c));
-                    const float4 x = *p;
-                    *p = make_float4(fmaf(a.neg_lr, acc[4 * c], x.x), fmaf(a.neg_lr, acc[4 * c + 1], x.y),
-                                     fmaf(a.neg_lr, acc[4 * c + 2], x.z), fmaf(a.neg_lr, acc[4 * c + 3], x.w));
-                }
-            } else {
-                if (lane == 0) tma::store_wait_read();
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c)) =
-                        make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
-            }
-            tma::fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) {
-                tma::store_tile_2d(out_map, out_tile, 0, tile * 32);          // (rows outside the layout are clipped)
-                tma::store_commit();
-            }
-        }
+        if (!finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), x_parity)) { timed_out = true; break; }
         tile += hop;
         if (B == 1 && k + 1 < n_tiles) locate(tile, nbucket, nvalid);
         bucket = nbucket;
@@ -381,7 +519,15 @@ unpack_average_kernel(const __grid_constant__ AverageArgs a, const __grid_consta
     }
 
     switch (b) {
-#define DQ_CASE(BB) case BB: average_tiles<BB>(a, &out_map, tbl_in_smem); break;
+#define DQ_CASE(BB) case BB:                                                                             \
+            if constexpr (DirectWords<BB>::value) {                                                       \
+                if (a.M >= DirectWords<BB>::min_workers) {                                                \
+                    average_tiles_direct<BB>(a, &out_map, tbl_in_smem);                                   \
+                    break;                                                                                \
+                }                                                                                         \
+            }                                                                                             \
+            average_tiles<BB>(a, &out_map, tbl_in_smem);                                                  \
+            break;
         DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
         DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
 #undef DQ_CASE
