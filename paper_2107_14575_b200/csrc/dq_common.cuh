@@ -131,20 +131,9 @@ __device__ __forceinline__ void dq_checked_store(T* p, const T& v, const void* b
 #define DQ_STORE(p, v, base, extent_bytes, status) (*(p) = (v))
 #endif
 
-// Index of the last entry of starts[0..n] (n + 1 entries, non-decreasing) that is <= x.
+// Index of the last of n entries (non-decreasing, entry 0 <= x) that is <= x, found by the warp together: 32
+// entries are looked at a step, so that 1023 tensors take two steps and not ten.  start(i) is entry i.
 // Tensors of zero size repeat a start; the last repeat is the non-empty one.
-__device__ __forceinline__ int last_not_above(const int32_t* __restrict__ starts, int n, int x)
-{
-    int lo = 0, hi = n;            // invariant: starts[lo] <= x < starts[hi]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(starts + mid) <= x) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-// The same for the warp together (x and the answer are the warp's): 32 entries are looked at a step, so
-// that 1023 tensors take two steps and not ten.  start(i) is entry i.
 template <class Start>
 __device__ __forceinline__ int last_not_above_by_warp(const int x, const int n, const Start& start)
 {
@@ -159,41 +148,6 @@ __device__ __forceinline__ int last_not_above_by_warp(const int x, const int n, 
         len = len - skip < stride ? len - skip : stride;
     } while (stride > 1);
     return lo;
-}
-
-// Bucket and number of valid elements of group g (32 padded elements).
-__device__ __forceinline__ void group_info(const LayoutView& v, int g, int& bucket, int& valid)
-{
-    int local, n, b0;
-    if (v.n_seg == 1) {
-        local = g; n = v.seg0_elems; b0 = 0;
-    } else {
-        const int i = last_not_above(v.seg_group0, v.n_seg, g);
-        local = g - __ldg(v.seg_group0 + i);
-        n = __ldg(v.seg_elems + i);
-        b0 = __ldg(v.seg_bucket0 + i);
-    }
-    bucket = b0 + local / v.groups_per_bucket;
-    const int left = n - local * 32;
-    valid = left < 32 ? left : 32;
-}
-
-// First padded element and valid length of bucket k.
-__device__ __forceinline__ void bucket_info(const LayoutView& v, int k, int64_t& start, int& len)
-{
-    int local, n, g0;
-    if (v.n_seg == 1) {
-        local = k; n = v.seg0_elems; g0 = 0;
-    } else {
-        const int i = last_not_above(v.seg_bucket0, v.n_seg, k);
-        local = k - __ldg(v.seg_bucket0 + i);
-        n = __ldg(v.seg_elems + i);
-        g0 = __ldg(v.seg_group0 + i);
-    }
-    const int bsz = v.groups_per_bucket * 32;
-    start = (int64_t)g0 * 32 + (int64_t)local * bsz;
-    const int left = n - local * bsz;
-    len = left < bsz ? left : bsz;
 }
 
 #endif  // __CUDACC__

@@ -95,15 +95,11 @@ __device__ __forceinline__ float finish(const float a)
 // entries, an overflowed square, a NaN) the bucket is reduced again: first its largest magnitude
 // (exact), then the squares of the entries scaled by the power of two that brings that magnitude
 // into [1, 2), in the same order as before, and the square root is scaled back.  The functors
-// below are the three reductions; the kernels supply the loads and the joins between threads.
+// below are those two reductions; the kernels supply the loads and the joins between threads.
 __device__ __forceinline__ bool l2_sum_in_range(const float sum)
 {
     return sum >= 0x1p-100f && sum <= 3.402823466e38f;       // false for a NaN as well
 }
-struct SumSquares {
-    __device__ __forceinline__ float take(const float acc, const float x) const { return fmaf(x, x, acc); }
-    __device__ __forceinline__ float join(const float a, const float b) const { return a + b; }
-};
 struct MaxMagnitude {
     __device__ __forceinline__ float take(const float acc, const float x) const { return max_nan(acc, fabsf(x)); }
     __device__ __forceinline__ float join(const float a, const float b) const { return max_nan(a, b); }
@@ -117,9 +113,6 @@ struct ScaledSquares {
     }
     __device__ __forceinline__ float join(const float a, const float b) const { return a + b; }
 };
-// the reduction a member of the family starts with
-template <int P> struct FamilyReduction { using type = SumSquares; };
-template <> struct FamilyReduction<DQ_NORM_LINF> { using type = MaxMagnitude; };
 // Exponent to scale by, from the bucket's largest magnitude (0 when there is nothing to scale:
 // an all-zero bucket, an infinity or a NaN, for which rescaled_l2 returns the magnitude itself).
 __device__ __forceinline__ bool magnitude_scalable(const float mx) { return mx > 0.0f && mx <= 3.402823466e38f; }
@@ -516,31 +509,13 @@ struct CodePos {
     static constexpr int k = in_place ? sh : (in_upper ? sh - 16 : 0);
 };
 
-template <int B, int E>
-__device__ __forceinline__ float decode_code(const uint32_t (&wd)[B], const uint32_t (&hi)[B], const uint32_t magic)
-{
-    using P = CodePos<B, E>;
-    constexpr uint32_t kCode = (1u << B) - 1u;
-    constexpr int s = (1 << (B - 1)) - 1;
-    uint32_t m;                                  // magic = 0x4B000000, the bits of 2^23
-    if constexpr (P::in_place) {
-        m = and_or(wd[P::w], kCode << P::k, magic);
-    } else if constexpr (P::in_upper) {
-        m = and_or(hi[P::w], kCode << P::k, magic);
-    } else if constexpr (!P::straddles) {
-        m = and_or(wd[P::w] >> P::sh, kCode, magic);
-    } else {
-        m = and_or(__funnelshift_r(wd[P::w], wd[P::w + 1], P::sh), kCode, magic);
-    }
-    return __uint_as_float(m) - (8388608.0f + (float)(s << P::k));      // sgn * level * 2^k, exact
-}
-
-// The same decoding for two neighbouring codes at once with the packed two-lane fp32 forms of
+// Two neighbouring codes are decoded at once with the packed two-lane fp32 forms of
 // sm_100 (add.f32x2, fma.f32x2 on 64-bit register pairs): one packed subtract and one packed FMA
 // replace two of each, which halves the operand traffic of the accumulation (the scalar form
 // keeps 32 accumulators, a scale and an immediate in flight per code).  Results are bit for bit
-// those of decode_code: the same exact subtract, the same single rounding in the FMA.
-// bits of the float 2^23 + code * 2^k for code E of a group (the part of decode_code before the subtract)
+// those of scalar subtracts and FMAs: the same exact subtract, the same single rounding in the FMA.
+
+// bits of the float 2^23 + code * 2^k for code E of a group (the part before the subtract)
 template <int B, int E>
 __device__ __forceinline__ uint32_t code_bits(const uint32_t (&wd)[B], const uint32_t (&hi)[B], const uint32_t magic)
 {

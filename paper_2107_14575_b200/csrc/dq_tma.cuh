@@ -63,13 +63,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
                  : "memory");
 }
 
-// Plain arrival (one of the barrier's expected arrivals), with release semantics for the
-// arriving thread's earlier shared-memory accesses.
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar_addr, uint32_t parity)
 {
     uint32_t ok;
@@ -104,15 +97,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
         if (global_timer_ns() - t0 > lim.ns) return false;
     }
 }
-// 3-D tiled tensor copy global -> shared, completion counted on `bar`.
-__device__ __forceinline__ void load_tile_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(smem_addr(dst)), "l"(map), "r"(smem_addr(bar)), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
-}
-
 // 2-D tiled tensor copy global -> shared (rows outside the tensor arrive as zeros and still
 // count towards the barrier's bytes), completion counted on `bar`.
 __device__ __forceinline__ void load_tile_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1)

@@ -7,7 +7,7 @@
 // at a time: their words of the tile are as many linear bulk copies, one per lane, into one of two
 // 4 KB stages, so that the copies of the next workers travel while these are decoded.  The norms of the
 // next workers are requested before the wait.  A code is decoded where it stands in its word (mask under
-// the exponent of 2^23, subtract 2^23 + s: see decode_code) and accumulated with one FMA; the power of two
+// the exponent of 2^23, subtract 2^23 + s: see accumulate_pair) and accumulated with one FMA; the power of two
 // its position carries is removed once per element after the last worker.  The 32 rows of sums go through a
 // swizzled 4 KB tile of the warp and leave with one bulk tensor store (straight from registers, 32 bytes a
 // lane, every store touched 32 lines: one worker, 2^25 elements, b = 4 37 us against 30).
@@ -130,7 +130,7 @@ struct AccumulateAll<B, 16> {
                                                const uint32_t) {}
 };
 
-// The upper halves of the words whose codes need them (see decode_code) come straight from shared
+// The upper halves of the words whose codes need them (see CodePos) come straight from shared
 // memory as 16-bit loads, two bytes into the word: the load pipe has room, the logic pipe, which a
 // shift would use, is the busiest one of this kernel.
 template <int B, int W>
