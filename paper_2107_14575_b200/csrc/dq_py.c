@@ -9,10 +9,26 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "dq.h"
 
 static PyObject* g_data_ptr; /* the string "data_ptr" */
+
+/* An integer argument: what int() makes of it (a number that lives in a tensor or an array among them). */
+static int to_integer(PyObject* o, uint64_t* v)
+{
+    PyObject* n;
+    if (PyLong_CheckExact(o)) {
+        *v = PyLong_AsUnsignedLongLongMask(o);
+        return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
+    }
+    n = PyNumber_Long(o);
+    if (!n) return -1;
+    *v = PyLong_AsUnsignedLongLongMask(n);
+    Py_DECREF(n);
+    return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
+}
 
 /* Integer value or device address of an argument; 0 on success. */
 static int to_u64(PyObject* o, uint64_t* v)
@@ -55,18 +71,21 @@ static int to_rule(PyObject* o, dq_rule_t* r)
 
 enum { MAX_ARGS = 18 };
 
-/* All arguments as integers, except number `rule` (a dq_rule_t) and number `real` (a float); -1: none. */
-static int convert(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, int rule, int real, uint64_t* v, dq_rule_t* r, float* f)
+/* Arguments by their kinds, a letter each: p a device address, i an integer, r the rule, f a float. */
+static int convert(PyObject* const* args, Py_ssize_t n, const char* kinds, uint64_t* v, dq_rule_t* r, float* f)
 {
+    const Py_ssize_t want = (Py_ssize_t)strlen(kinds);
     Py_ssize_t i;
     if (n != want) {
         PyErr_Format(PyExc_TypeError, "%zd arguments are wanted, got %zd", want, n);
         return -1;
     }
     for (i = 0; i < n; ++i) {
-        if (i == rule) {
+        if (kinds[i] == 'i') {
+            if (to_integer(args[i], &v[i]) != 0) return -1;
+        } else if (kinds[i] == 'r') {
             if (to_rule(args[i], r) != 0) return -1;
-        } else if (i == real) {
+        } else if (kinds[i] == 'f') {
             const double d = PyFloat_AsDouble(args[i]);
             if (d == -1.0 && PyErr_Occurred()) return -1;
             *f = (float)d;
@@ -82,7 +101,7 @@ static int convert(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, int rul
 #define I32(i) ((int32_t)v[i])
 #define U32(i) ((uint32_t)v[i])
 
-#define ENTRY(name, want, rule, real, call)                                                         \
+#define ENTRY(name, kinds, call)                                                                    \
     static __typeof__(&dq_##name) p_##name;                                                         \
     static PyObject* py_##name(PyObject* self, PyObject* const* args, Py_ssize_t n)                 \
     {                                                                                               \
@@ -91,28 +110,28 @@ static int convert(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, int rul
         float f = 0.0f;                                                                             \
         int rc;                                                                                     \
         (void)self; (void)f; (void)r;                                                               \
-        if (convert(args, n, want, rule, real, v, &r, &f) != 0) return NULL;                        \
+        if (convert(args, n, kinds, v, &r, &f) != 0) return NULL;                                   \
         Py_BEGIN_ALLOW_THREADS                                                                      \
         rc = p_##name call;                                                                         \
         Py_END_ALLOW_THREADS                                                                        \
         return PyLong_FromLong(rc);                                                                 \
     }
 
-ENTRY(bucket_norms, 7, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), P(6)))
-ENTRY(tensor_norms, 9, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), (size_t)v[6], P(7), P(8)))
-ENTRY(choose_bits, 9, 3, -1, (P(0), P(1), I32(2), &r, P(4), P(5), (size_t)v[6], P(7), P(8)))
-ENTRY(quantize_pack, 12, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), P(11)))
-ENTRY(quantize_pack_worker, 13, -1, -1,
+ENTRY(bucket_norms, "ppiippp", (P(0), P(1), I64(2), I32(3), P(4), P(5), P(6)))
+ENTRY(tensor_norms, "ppiippipp", (P(0), P(1), I64(2), I32(3), P(4), P(5), (size_t)v[6], P(7), P(8)))
+ENTRY(choose_bits, "ppirppipp", (P(0), P(1), I32(2), &r, P(4), P(5), (size_t)v[6], P(7), P(8)))
+ENTRY(quantize_pack, "ppiippiipipp", (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), P(11)))
+ENTRY(quantize_pack_worker, "ppiippiiipipp",
       (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), U32(8), P(9), I64(10), P(11), P(12)))
-ENTRY(norms_quantize_pack, 12, -1, -1, (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), P(7), P(8), I64(9), P(10), P(11)))
-ENTRY(norms_quantize_pack_worker, 13, -1, -1,
+ENTRY(norms_quantize_pack, "ppiipiippipp", (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), P(7), P(8), I64(9), P(10), P(11)))
+ENTRY(norms_quantize_pack_worker, "ppiipiiippipp",
       (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), U32(7), P(8), P(9), I64(10), P(11), P(12)))
-ENTRY(unpack_dequant_average, 9, -1, -1, (P(0), P(1), I64(2), P(3), I32(4), P(5), P(6), P(7), P(8)))
-ENTRY(unpack_average_update, 10, -1, 6, (P(0), P(1), I64(2), P(3), I32(4), P(5), f, P(7), P(8), P(9)))
-ENTRY(norms_choose_bits, 11, 5, -1, (P(0), P(1), I64(2), I32(3), P(4), &r, P(6), P(7), (size_t)v[8], P(9), P(10)))
-ENTRY(quantize_average, 15, -1, 12,
+ENTRY(unpack_dequant_average, "ppipipppp", (P(0), P(1), I64(2), P(3), I32(4), P(5), P(6), P(7), P(8)))
+ENTRY(unpack_average_update, "ppipipfppp", (P(0), P(1), I64(2), P(3), I32(4), P(5), f, P(7), P(8), P(9)))
+ENTRY(norms_choose_bits, "ppiiprppipp", (P(0), P(1), I64(2), I32(3), P(4), &r, P(6), P(7), (size_t)v[8], P(9), P(10)))
+ENTRY(quantize_average, "ppiippiipipifpp",
       (P(0), P(1), I64(2), I32(3), P(4), P(5), v[6], U32(7), P(8), I64(9), P(10), I32(11), f, P(13), P(14)))
-ENTRY(norms_quantize_average, 18, 13, 12,
+ENTRY(norms_quantize_average, "ppiipiippipifrpipp",
       (P(0), P(1), I64(2), I32(3), P(4), v[5], U32(6), P(7), P(8), I64(9), P(10), I32(11), f, &r, P(14), (size_t)v[15], P(16), P(17)))
 
 #define EACH(X)                                                                                     \

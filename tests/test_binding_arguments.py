@@ -1,0 +1,65 @@
+"""The binding's conversion of arguments, with recorders in the place of the library's calls (no GPU)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+_KINDS = {"p": C.c_void_p, "i": C.c_int32, "l": C.c_int64, "u": C.c_uint32, "q": C.c_uint64, "z": C.c_size_t, "f": C.c_float}
+_CALLS = {
+    "dq_bucket_norms": "pplippp", "dq_tensor_norms": "pplippzpp", "dq_choose_bits": "ppirppzpp",
+    "dq_quantize_pack": "pplippquplpp", "dq_quantize_pack_worker": "pplippquuplpp",
+    "dq_norms_quantize_pack": "pplipqupplpp", "dq_norms_quantize_pack_worker": "pplipquupplpp",
+    "dq_unpack_dequant_average": "pplpipppp", "dq_unpack_average_update": "pplpipfppp",
+    "dq_norms_choose_bits": "pplip" "rppzpp", "dq_quantize_average": "pplippquplpifpp",
+    "dq_norms_quantize_average": "pplipqupplpifrpzpp",
+}
+
+
+@pytest.fixture()
+def recorded(dqlib):
+    """(dq, the list of the calls made): every call of a step goes to a recorder that answers DQ_OK."""
+    from paper_2107_14575_b200 import dq
+    dq.lib()
+    made, keep, table = [], [], {}
+    for name, kinds in _CALLS.items():
+        types = [C.POINTER(dq.Rule) if k == "r" else _KINDS[k] for k in kinds]
+
+        def record(*args, _name=name, _kinds=kinds):
+            made.append((_name, [(a.contents.T, a.contents.b_max, a.contents.eps_hat) if k == "r" else a
+                                 for a, k in zip(args, _kinds)]))
+            return 0
+        f = C.CFUNCTYPE(C.c_int, *types)(record)
+        keep.append(f)
+        table[name] = C.cast(f, C.c_void_p).value
+    dq._calls.bind(table)
+    try:
+        yield dq, made
+    finally:
+        dq._calls.bind({n: C.cast(getattr(dq.lib(), n), C.c_void_p).value for n in _CALLS})
+
+
+@pytest.fixture()
+def layout(dqlib):
+    from paper_2107_14575_b200 import dq
+    return dq.Layout([100], 32)
+
+
+def _quantize(dq, layout, **other):
+    a = dict(grads=16, worker_stride_elems=128, M=1, norms=32, dev_b=48, seed=5, step=7, packed=64,
+             packed_stride_words=64, status=80, stream=0)
+    a.update(other)
+    dq.quantize_pack(layout, **a)
+
+
+def test_integers_are_taken_by_value(recorded, layout):
+    """What int() makes of an argument is its value: also of a number that lives in a tensor or an array."""
+    dq, made = recorded
+    for x in (3, np.int64(3), np.uint32(3), np.array(3), torch.tensor(3), torch.tensor([3]), True + 2, 3.0):
+        _quantize(dq, layout, M=x, seed=x, step=x, worker_stride_elems=x, packed_stride_words=x)
+        name, args = made.pop()
+        assert name == "dq_quantize_pack"
+        assert (args[2], args[3], args[6], args[7], args[9]) == (3, 3, 3, 3, 3), repr(x)
+    _quantize(dq, layout, seed=-1, step=(1 << 40) + 9)
+    _, args = made.pop()
+    assert args[6] == 2 ** 64 - 1 and args[7] == 9
