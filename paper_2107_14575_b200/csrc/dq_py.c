@@ -2,8 +2,8 @@
  *
  * Bound by host work: a round's one call has 18 arguments, which ctypes converts in 5 us and a Python
  * wrapper prepares in as much again (one core of the host), longer than a small round takes on the GPU.
- * Here an argument costs some tens of nanoseconds.  Arguments are integers, or objects with a data_ptr()
- * method (device addresses), or None (NULL); the answer is the C call's status.  No state is kept but the
+ * Here an argument costs some tens of nanoseconds.  Device addresses are objects with a data_ptr()
+ * method, integers, or None (NULL); the answer is the C call's status.  No state is kept but the
  * addresses of the library's entry points, which bind() receives from the Python side, so that any build
  * of the library can stand behind them. */
 #define PY_SSIZE_T_CLEAN
@@ -30,28 +30,30 @@ static int to_integer(PyObject* o, uint64_t* v)
     return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
 }
 
-/* Integer value or device address of an argument; 0 on success. */
-static int to_u64(PyObject* o, uint64_t* v)
+/* A device address: None (NULL), an integer, or what the object's data_ptr() says.  Nothing else is one: a number
+ * given in the place of a tensor must not reach a kernel as a pointer. */
+static int to_address(PyObject* o, uint64_t* v)
 {
     PyObject* n;
-    if (PyLong_CheckExact(o)) {
-        *v = PyLong_AsUnsignedLongLongMask(o);
-        return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
-    }
     if (o == Py_None) {
         *v = 0;
         return 0;
     }
-    n = PyObject_VectorcallMethod(g_data_ptr, &o, 1 | PY_VECTORCALL_ARGUMENTS_OFFSET, NULL);
-    if (!n) {
-        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return -1;
-        PyErr_Clear();
-        n = PyNumber_Long(o); /* numpy integers and other numbers */
-        if (!n) return -1;
+    if (PyLong_Check(o)) {
+        *v = PyLong_AsUnsignedLongLongMask(o);
+        return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
     }
-    *v = PyLong_AsUnsignedLongLongMask(n);
+    n = PyObject_VectorcallMethod(g_data_ptr, &o, 1 | PY_VECTORCALL_ARGUMENTS_OFFSET, NULL);
+    if (!n) return -1;
+    if (n == Py_None) {
+        *v = 0;
+    } else if (PyLong_Check(n)) {
+        *v = PyLong_AsUnsignedLongLongMask(n);
+    } else {
+        PyErr_SetString(PyExc_TypeError, "data_ptr() did not return an address");
+    }
     Py_DECREF(n);
-    return (*v == (uint64_t)-1 && PyErr_Occurred()) ? -1 : 0;
+    return PyErr_Occurred() ? -1 : 0;
 }
 
 /* The rule travels as a ctypes structure of dq_rule_t's layout. */
@@ -89,7 +91,7 @@ static int convert(PyObject* const* args, Py_ssize_t n, const char* kinds, uint6
             const double d = PyFloat_AsDouble(args[i]);
             if (d == -1.0 && PyErr_Occurred()) return -1;
             *f = (float)d;
-        } else if (to_u64(args[i], &v[i]) != 0) {
+        } else if (to_address(args[i], &v[i]) != 0) {
             return -1;
         }
     }
@@ -151,7 +153,7 @@ static PyObject* py_bind(PyObject* self, PyObject* dict)
     {                                                                                               \
         PyObject* o = PyDict_GetItemString(dict, "dq_" #name);                                      \
         uint64_t a = 0;                                                                             \
-        if (!o || to_u64(o, &a) != 0 || !a) {                                                       \
+        if (!o || to_address(o, &a) != 0 || !a) {                                                       \
             if (!PyErr_Occurred()) PyErr_SetString(PyExc_KeyError, "dq_" #name);                    \
             return NULL;                                                                            \
         }                                                                                           \

@@ -63,3 +63,31 @@ def test_integers_are_taken_by_value(recorded, layout):
     _quantize(dq, layout, seed=-1, step=(1 << 40) + 9)
     _, args = made.pop()
     assert args[6] == 2 ** 64 - 1 and args[7] == 9
+
+
+class _Address:
+    def __init__(self, answer):
+        self.answer = answer
+
+    def data_ptr(self):
+        if isinstance(self.answer, Exception):
+            raise self.answer
+        return self.answer
+
+
+def test_an_address_is_none_an_integer_or_what_data_ptr_says(recorded, layout):
+    dq, made = recorded
+    t = torch.zeros(4)
+    for x, want in ((None, None), (0, None), (64, 64), (t, t.data_ptr()), (_Address(128), 128), (_Address(None), None)):
+        _quantize(dq, layout, grads=x, packed=x)
+        _, args = made.pop()
+        assert (args[1], args[8]) == (want, want), repr(x)
+    for x in ("7", b"12", 3.0, np.int64(64), np.array(64), [64], _Address("64"), _Address(64.0)):
+        for name in ("grads", "norms", "dev_b", "packed", "status"):
+            with pytest.raises((TypeError, AttributeError)):
+                _quantize(dq, layout, **{name: x})
+    with pytest.raises(AttributeError, match="gone"):
+        _quantize(dq, layout, grads=_Address(AttributeError("gone")))
+    with pytest.raises(TypeError):
+        _quantize(dq, layout, M=None)
+    assert not made
