@@ -4,8 +4,8 @@
  * wrapper prepares in as much again (one core of the host), longer than a small round takes on the GPU.
  * Here an argument costs some tens of nanoseconds.  Device addresses are objects with a data_ptr()
  * method, integers, or None (NULL); the answer is the C call's status.  No state is kept but the
- * addresses of the library's entry points, which bind() receives from the Python side, so that any build
- * of the library can stand behind them. */
+ * addresses of the library's entry points and the class of the rules, which bind() receives from the Python
+ * side, so that any build of the library can stand behind them. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -14,6 +14,7 @@
 #include "dq.h"
 
 static PyObject* g_data_ptr; /* the string "data_ptr" */
+static PyObject* g_rule;     /* the class dq.Rule */
 
 /* An integer argument: what int() makes of it (a number that lives in a tensor or an array among them). */
 static int to_integer(PyObject* o, uint64_t* v)
@@ -56,18 +57,37 @@ static int to_address(PyObject* o, uint64_t* v)
     return PyErr_Occurred() ? -1 : 0;
 }
 
-/* The rule travels as a ctypes structure of dq_rule_t's layout. */
+/* The rule travels as the binding's ctypes structure of dq_rule_t's layout, and as no other object. */
 static int to_rule(PyObject* o, dq_rule_t* r)
 {
     Py_buffer b;
+    if (!PyObject_TypeCheck(o, (PyTypeObject*)g_rule)) {
+        PyErr_SetString(PyExc_TypeError, "a dq.Rule is wanted");
+        return -1;
+    }
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) return -1;
-    if (b.len != (Py_ssize_t)sizeof(dq_rule_t)) {
+    if (b.len < (Py_ssize_t)sizeof(dq_rule_t)) {
         PyBuffer_Release(&b);
         PyErr_SetString(PyExc_TypeError, "a dq.Rule is wanted");
         return -1;
     }
-    *r = *(const dq_rule_t*)b.buf;
+    memcpy(r, b.buf, sizeof(*r));
     PyBuffer_Release(&b);
+    return 0;
+}
+
+/* A float argument: what float() makes of it. */
+static int to_float(PyObject* o, float* f)
+{
+    PyObject* n;
+    if (PyFloat_CheckExact(o)) {
+        *f = (float)PyFloat_AS_DOUBLE(o);
+        return 0;
+    }
+    n = PyNumber_Float(o);
+    if (!n) return -1;
+    *f = (float)PyFloat_AS_DOUBLE(n);
+    Py_DECREF(n);
     return 0;
 }
 
@@ -88,9 +108,7 @@ static int convert(PyObject* const* args, Py_ssize_t n, const char* kinds, uint6
         } else if (kinds[i] == 'r') {
             if (to_rule(args[i], r) != 0) return -1;
         } else if (kinds[i] == 'f') {
-            const double d = PyFloat_AsDouble(args[i]);
-            if (d == -1.0 && PyErr_Occurred()) return -1;
-            *f = (float)d;
+            if (to_float(args[i], f) != 0) return -1;
         } else if (to_address(args[i], &v[i]) != 0) {
             return -1;
         }
@@ -141,14 +159,12 @@ ENTRY(norms_quantize_average, "ppiipiippipifrpipp",
     X(norms_quantize_pack) X(norms_quantize_pack_worker) X(unpack_dequant_average)                  \
     X(unpack_average_update) X(norms_choose_bits) X(quantize_average) X(norms_quantize_average)
 
-/* bind({"dq_...": address}): the entry points of the library that was loaded. */
-static PyObject* py_bind(PyObject* self, PyObject* dict)
+/* bind({"dq_...": address}, Rule): the entry points of the library that was loaded, the class of the rules. */
+static PyObject* py_bind(PyObject* self, PyObject* args)
 {
+    PyObject *dict, *rule, *old;
     (void)self;
-    if (!PyDict_Check(dict)) {
-        PyErr_SetString(PyExc_TypeError, "a dict of addresses is wanted");
-        return NULL;
-    }
+    if (!PyArg_ParseTuple(args, "O!O!", &PyDict_Type, &dict, &PyType_Type, &rule)) return NULL;
 #define X(name)                                                                                     \
     {                                                                                               \
         PyObject* o = PyDict_GetItemString(dict, "dq_" #name);                                      \
@@ -161,11 +177,15 @@ static PyObject* py_bind(PyObject* self, PyObject* dict)
     }
     EACH(X)
 #undef X
+    old = g_rule;
+    Py_INCREF(rule);
+    g_rule = rule;
+    Py_XDECREF(old);
     Py_RETURN_NONE;
 }
 
 static PyMethodDef methods[] = {
-    {"bind", py_bind, METH_O, NULL},
+    {"bind", py_bind, METH_VARARGS, NULL},
 #define X(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL},
     EACH(X)
 #undef X

@@ -141,7 +141,7 @@ def lib():
         except ImportError as e:
             raise RuntimeError("the binding's _dqcall.so is missing: build it with "
                                "`python -m paper_2107_14575_b200.build`") from e
-        _dqcall.bind({n: C.cast(getattr(L, n), vp).value for n in SYMBOLS})
+        _dqcall.bind({n: C.cast(getattr(L, n), vp).value for n in SYMBOLS}, Rule)
         _calls = _dqcall
         _lib = L
     return _lib

@@ -32,11 +32,11 @@ def recorded(dqlib):
         f = C.CFUNCTYPE(C.c_int, *types)(record)
         keep.append(f)
         table[name] = C.cast(f, C.c_void_p).value
-    dq._calls.bind(table)
+    dq._calls.bind(table, dq.Rule)
     try:
         yield dq, made
     finally:
-        dq._calls.bind({n: C.cast(getattr(dq.lib(), n), C.c_void_p).value for n in _CALLS})
+        dq._calls.bind({n: C.cast(getattr(dq.lib(), n), C.c_void_p).value for n in _CALLS}, dq.Rule)
 
 
 @pytest.fixture()
@@ -90,4 +90,25 @@ def test_an_address_is_none_an_integer_or_what_data_ptr_says(recorded, layout):
         _quantize(dq, layout, grads=_Address(AttributeError("gone")))
     with pytest.raises(TypeError):
         _quantize(dq, layout, M=None)
+    assert not made
+
+
+def test_the_rule_is_a_rule_and_the_step_size_a_float(recorded, layout):
+    dq, made = recorded
+    rule = dq.Rule.dynamic(10, 3, 0.25, 0.9, 2, 9)
+
+    class Mine(dq.Rule):
+        pass
+    for r in (rule, Mine(10, 3, 0.25, 0.9, 2, 9, 0)):
+        dq.choose_bits(layout, 16, 1, r, 32, 48, 256, 64, stream=0)
+        assert made.pop()[1][3] == (10, 9, 0.25)
+    for r in (bytes(rule), bytearray(bytes(rule)), np.zeros(5), None, 4):
+        with pytest.raises((TypeError, C.ArgumentError)):
+            dq.choose_bits(layout, 16, 1, r, 32, 48, 256, 64, stream=0)
+    for lr in (0.5, np.float32(0.5), torch.tensor(0.5), "0.5"):
+        dq.unpack_average_update(layout, 16, 4, 32, 1, 48, lr, 64, 80, stream=0)
+        assert made.pop()[1][6] == 0.5
+    for lr in (None, "x"):
+        with pytest.raises((TypeError, ValueError)):
+            dq.unpack_average_update(layout, 16, 4, 32, 1, 48, lr, 64, 80, stream=0)
     assert not made
