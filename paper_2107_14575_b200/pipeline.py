@@ -120,7 +120,7 @@ class Round:
         if events is None:
             dq.norms_quantize_average(self.layout, grads, self.stride, self.M, self.dev_b, seed, step, self.norms, self.packed,
                                       self.packed_stride, self.out if params is None else params, next_rule, self._ws,
-                                      self._ws_bytes, self.status, None if params is None else lr)
+                                      self._ws_bytes, self.status, None if params is None else float(lr))
             return self.out if params is None else params
 
         def server_step():
