@@ -271,7 +271,8 @@ int dq_choose_bits_noalloc(const dq_layout_t* layout, const float* dev_norms, in
  * Rounding toward zero keeps |x| <= s for every element with |g_j| <= norm, which
  * holds for the norms dq_bucket_norms computes (a bucket's norm dominates its
  * entries).  The codes of a bucket whose norm is smaller than one of its entries
- * are unspecified (nothing outside the packed stream is touched).
+ * are unspecified (nothing outside the packed stream is touched).  A bucket whose norm is an
+ * infinity or a NaN has the scale 0: its codes are all s, its averages NaN.
  * v = (2k + 1) / 2^17 in (0, 1) is the element's uniform draw: k is half (j & 1)
  * (0 = low 16 bits) of word ((j >> 1) & 3) of Philox4x32-10 with counter
  * (j >> 3, 0, m, step) and key (seed low word, seed high word); j is the

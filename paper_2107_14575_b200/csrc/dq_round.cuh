@@ -206,6 +206,23 @@ __device__ __noinline__ void clear_row_tail(const uint32_t row, const int valid)
     __syncwarp();
 }
 
+// A norm that is an infinity or a NaN: the scale of the codes is 0, every code is s and every term of the average
+// 0 * norm = NaN, but 0 times an entry that is not finite has no code (for b <= 4 its bits reach the codes of its
+// neighbours).  So the words of such a row are set after the encoder; the kernels with l2 norms and the average,
+// which have no register to spare for that (VGG-16 shape M = 16 with update 256 -> 264 us), set the row to zero
+// beforehand, in the call that finds such norms.  (Clearing the row everywhere: l-inf rounds 25.9 -> 27.9 us.)
+template <int MODE, bool AVG, bool LINF>
+struct ClearsRow {
+    static constexpr bool value = AVG && !LINF && MODE != kGivenNorms;
+};
+template <bool CLEAR>
+__device__ __forceinline__ void clear_nonfinite_row(const uint32_t row, const int valid, const float nrm)
+{
+    if (!CLEAR || valid == 0 || isfinite(nrm)) return;           // (valid = 0: the lane has no row of its own)
+#pragma unroll 1
+    for (int c = 0; c < 128; c += 16) *reinterpret_cast<float4*>(smem + (row ^ (uint32_t)c)) = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // The lanes of a bucket combine their v; the result is the same in all of them.
 template <int MODE, class Op>
 __device__ __forceinline__ float join_lanes(float v, const int gpb, const Op& op)
@@ -305,8 +322,9 @@ __device__ __forceinline__ float odd_bucket_sums(const uint32_t stage, const int
     return mine;
 }
 // ... and the norms of those out of range, as rare_norm has them.
+template <bool CLEAR>
 __device__ __noinline__ float rare_norm_odd(const uint32_t stage, const int row, const int len, const int gpb, const int R, const int r,
-                                            const float sum, const float nrm)
+                                            const float sum, const float nrm, const uint32_t own, const int valid)
 {
     const int lane = threadIdx.x & 31, lanes = gpb >= 4 ? 32 : 16;
     float mine = nrm;
@@ -324,6 +342,7 @@ __device__ __noinline__ float rare_norm_odd(const uint32_t stage, const int row,
         for (int o = 16; o > 0; o >>= 1) ss = sq.join(ss, __shfl_xor_sync(0xffffffffu, ss, o));
         if (r == k && !l2_sum_in_range(sum)) mine = rescaled_l2(mx, ss, e);
     }
+    clear_nonfinite_row<CLEAR>(own, valid, mine);
     return mine;
 }
 
@@ -332,7 +351,7 @@ __device__ __noinline__ float rare_norm_odd(const uint32_t stage, const int row,
 // on the sum); zero buckets are settled by their largest magnitude, the others are reduced again with
 // their entries scaled, and lanes whose own bucket was in range keep `nrm`.  Always two exchanges of a
 // team.  Out of line: it is rare, and the common case does not pay for its registers.
-template <int MODE>
+template <int MODE, bool CLEAR>
 __device__ __noinline__ float rare_norm(const uint32_t row, const int valid, const int gpb, float2* slots, const int T_shift,
                                         uint32_t exchanges, const float sum, const float nrm)
 {
@@ -354,7 +373,9 @@ __device__ __noinline__ float rare_norm(const uint32_t row, const int valid, con
         scaled = valid == 32 ? (a0 + a1) + (a2 + a3) : (valid > 0 ? chain : 0.0f);
         scaled = join_team<MODE>(join_lanes<MODE>(scaled, gpb, AddOp{}), slots, T_shift, exchanges, true, lost, AddOp{});
     }
-    return again ? (magnitude_scalable(mx) ? rescaled_l2(mx, scaled, e) : mx) : nrm;
+    const float norm = again ? (magnitude_scalable(mx) ? rescaled_l2(mx, scaled, e) : mx) : nrm;
+    clear_nonfinite_row<CLEAR>(row, valid, norm);
+    return norm;
 }
 
 template <int B, int MODE, bool AVG, bool LINF>
@@ -371,6 +392,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     const int M = a.M;
     const int nb = a.v.nb;
     const int G = a.v.total_groups;
+    constexpr bool kClears = ClearsRow<MODE, AVG, LINF>::value;
     constexpr bool ODD = MODE == kOddBuckets;
     constexpr bool TILES = MODE == kWarpBuckets || ODD;               // tiles of whole buckets
     const int gpb = ODD ? a.v.groups_per_bucket : 1 << a.gpb_shift;
@@ -621,9 +643,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             if (!plain) {
                 if constexpr (!LINF) {
                     if constexpr (ODD) {
-                        nrm = rare_norm_odd(row - own, t.row, t.len, gpb, R, r, v, nrm);
+                        nrm = rare_norm_odd<kClears>(row - own, t.row, t.len, gpb, R, r, v, nrm, row, t.valid);
                     } else {
-                        nrm = rare_norm<MODE>(row, t.valid, gpb, slots, T_shift, exchanges, v, nrm);
+                        nrm = rare_norm<MODE, kClears>(row, t.valid, gpb, slots, T_shift, exchanges, v, nrm);
                         exchanges += 2;
                     }
                 }
@@ -683,6 +705,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 } else {
                     encode_row<B, AVG>([row](int c) { return row_quad(row, c); }, inv2, scale2, acc2, words, q0,
                                        (uint32_t)mm + a.worker0, a.step, a.keys);
+                    if constexpr (!kClears) {
+                        if (!isfinite(nrm)) zero_group_words<B>(words);
+                    }
                 }
 
                 // ---- words out, the stage refilled.  The fence orders the warp's accesses to the stage before the copy's
