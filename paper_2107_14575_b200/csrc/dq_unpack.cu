@@ -162,16 +162,29 @@ struct Normalise<B, 32> {
     static __device__ __forceinline__ void run(float (&)[32]) {}
 };
 
+// Whether a lane's 32 sums are finite: 0 times each of them adds up to 0.
+__device__ __forceinline__ bool sums_finite(const uint64_t (&acc2)[16])
+{
+    uint64_t t = 0ull;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) t = fma_pair(acc2[q], 0ull, t);
+    float lo, hi;
+    unpack_pair(t, lo, hi);
+    return lo + hi == 0.0f;
+}
+
 // The end of a tile: the powers of two removed, padding zeroed, the rows through the warp's output tile.
-// False if the tile of x did not arrive.
+// kOutOfRange (nothing stored): a sum is not finite.  kLost: the tile of x did not arrive.
+enum TileEnd { kDone, kOutOfRange, kLost };
 template <int B>
-__device__ __forceinline__ bool finish_tile(const AverageArgs& a, const CUtensorMap* out_map, unsigned char* out_tile,
+__device__ __forceinline__ TileEnd finish_tile(const AverageArgs& a, const CUtensorMap* out_map, unsigned char* out_tile,
                                             const uint64_t (&acc2)[16], const int tile, const int valid, uint64_t* xbar,
                                             const uint32_t x_parity)
 {
     const int lane = threadIdx.x & 31;
     // (B = 1: s = 0, every value is 0, and an update by 0 leaves x as it is)
     if (!(B == 1 && a.update)) {
+        if (B > 1 && __any_sync(0xffffffffu, valid > 0 && !sums_finite(acc2))) return kOutOfRange;
         float acc[32];
 #pragma unroll
         for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], acc[2 * q], acc[2 * q + 1]);
@@ -183,7 +196,7 @@ __device__ __forceinline__ bool finish_tile(const AverageArgs& a, const CUtensor
         }
         if (a.update) {
             // nothing is stored from a tile whose parameters did not arrive
-            if (!__all_sync(0xffffffffu, tma::mbar_wait(xbar, x_parity, a.wait))) return false;
+            if (!__all_sync(0xffffffffu, tma::mbar_wait(xbar, x_parity, a.wait))) return kLost;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 float4* p = reinterpret_cast<float4*>(out_tile + tma::swizzle128(lane, c));
@@ -206,7 +219,7 @@ __device__ __forceinline__ bool finish_tile(const AverageArgs& a, const CUtensor
             tma::store_commit();
         }
     }
-    return true;
+    return kDone;
 }
 // The start of a tile of the update: the tile before must have left the warp's output tile; the tile of x
 // travels while the codes are decoded.
@@ -238,6 +251,43 @@ __device__ __forceinline__ void locate_group(const AverageArgs& a, const bool tb
     bucket = b0 + (int)div_gpb(a, (uint32_t)local);
     const int left = n - local * 32;
     valid = left < 32 ? left : 32;
+}
+
+// Tiles `tile`, `tile` + `hop`, ... (n of them) with every code shifted down and without the power of two of its
+// position, which takes sums of 2^106 and more out of the fp32 range: the same values, order and roundings as in
+// the one-pass kernels.  The warp ends here with the first tile that has such norms (or an infinity or a NaN); what
+// it has in flight has landed by then.  Out of line, with plain loads and stores: the others pay 16 packed FMAs.
+__device__ __noinline__ void average_tiles_plain(const AverageArgs& a, const bool tbl_in_smem, const int B, int tile, const int hop, int n)
+{
+    const int lane = threadIdx.x & 31;
+    const int s = (1 << (B - 1)) - 1;
+    const float unit = __fdiv_rn(1.0f, (float)s * (float)a.M);
+    for (; n > 0; --n, tile += hop) {
+        int bucket, valid;
+        locate_group(a, tbl_in_smem, tile, bucket, valid);
+        if (valid == 0) continue;
+        const int group = tile * 32 + lane;
+        const uint32_t* words = a.packed + (int64_t)group * B;
+        const float* norm = a.norms + bucket;
+        float sums[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) sums[e] = 0.0f;
+#pragma unroll 1
+        for (int m = 0; m < a.M; ++m, words += a.packed_stride, norm += a.v.nb) {
+            const float scale = __ldg(norm) * unit;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                const int i = e * B >> 5, sh = e * B & 31;
+                const uint32_t lo = __ldg(words + i), hi = sh + B > 32 ? __ldg(words + i + 1) : 0u;
+                const int code = (int)(__funnelshift_r(lo, hi, sh) & ((1u << B) - 1u));
+                sums[e] = fmaf((float)(code - s), scale, sums[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 32; ++e)
+            if (e >= valid) sums[e] = 0.0f;
+        store_row(a.out + (int64_t)group * 32, sums, a.update != 0, a.neg_lr, false, a.out, (int64_t)a.v.total_groups * 128, a.status);
+    }
 }
 
 // ---- b = 2, 3, 4 and 20 workers or more: words straight into registers --------------------------
@@ -344,12 +394,16 @@ __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const
                 }
             }
         }
-        if (!finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), (uint32_t)k & 1u)) {
+        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), (uint32_t)k & 1u);
+        if (end != kDone) {
             if (lane == 0) {
-                atomicOr(a.status, DQ_STAT_WAIT);
+                if (end == kLost) atomicOr(a.status, DQ_STAT_WAIT);
                 tma::store_wait_read();
             }
-            (void)tma::mbar_wait(x_bar(warp), (uint32_t)k & 1u, a.wait);       // the copy must not outlive the shared memory
+            // (the copy must not outlive the shared memory)
+            if (a.update && !__all_sync(0xffffffffu, tma::mbar_wait(x_bar(warp), (uint32_t)k & 1u, a.wait)) && lane == 0)
+                atomicOr(a.status, DQ_STAT_WAIT);
+            if (end == kOutOfRange) average_tiles_plain(a, tbl_in_smem, B, tile, hop, n_tiles - k);
             return;
         }
         tile += hop;
@@ -414,6 +468,7 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
     unsigned char* out_tile = smem + warp * kOutBytes;
     uint32_t it = 0;
     bool timed_out = false;
+    int plain_left = 0;                           // tiles left to average_tiles_plain
     uint32_t x_parity = 0;                        // of the tile of x at hand
     // (test hook: the warp's first wait counts as lost, and the warp goes straight to what follows a time-out)
     const bool skip_all = a.wait.lose_first != 0u && items > 0;
@@ -471,20 +526,25 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
             }
             if (timed_out) break;
         }
-        if (!finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), x_parity)) { timed_out = true; break; }
+        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), x_parity);
+        if (end == kOutOfRange) { plain_left = n_tiles - k; break; }
+        if (end == kLost) { timed_out = true; break; }
         tile += hop;
         if (B == 1 && k + 1 < n_tiles) locate(tile, nbucket, nvalid);
         bucket = nbucket;
         valid = nvalid;
     }
     if (lane == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
-    if (timed_out || skip_all) {
-        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
+    if (timed_out || skip_all || plain_left > 0) {
         // every copy the warp has issued and not seen land, the one whose wait ran out included, gets the
         // full limit before the CTA's shared memory is released
+        bool landed = plain_left > 0;
         for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
-            (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
-        if (B > 1 && a.update && !skip_all) (void)tma::mbar_wait(x_bar(warp), x_parity, a.wait);
+            landed &= tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
+        if (B > 1 && a.update && !skip_all) landed &= tma::mbar_wait(x_bar(warp), x_parity, a.wait);
+        landed = __all_sync(0xffffffffu, landed);
+        if (lane == 0 && !landed) atomicOr(a.status, DQ_STAT_WAIT);
+        if (plain_left > 0) average_tiles_plain(a, tbl_in_smem, B, tile, hop, plain_left);
     }
 }
 

@@ -194,3 +194,40 @@ def test_linf_and_tensor_norms_over_the_range(G, p):
         for k, (o, n) in enumerate(zip(ref.offsets, segs)):
             assert np.all(np.abs(g[:, o: o + n]).max(axis=1) <= got[:, k])
     assert r.read_status() == 0 and r.guards_intact()
+
+
+@pytest.mark.parametrize("M", [1, 4, 24])
+@pytest.mark.parametrize("b", [2, 3, 4, 5, 8, 12, 16])
+def test_average_of_norms_up_to_the_top_of_the_range(G, b, M):
+    """Entries of 2^-90 to 2^120: the average from the words is finite and the one of the one-pass kernel bit for
+    bit, beside buckets of ordinary size, and so are the updated parameters."""
+    dq = G.dq
+    bucket, segs = 64, [7000, 33, 64 * 40]
+    ref = oracle.Layout(segs, bucket)
+    rng = np.random.default_rng(31 * b + M)
+    g = np.zeros((M, ref.D32), np.float32)
+    for k in range(ref.nb):
+        s, n = int(ref.bucket_start[k]), int(ref.bucket_len[k])
+        e = (0, 90, 104, 108, 111, 116, 120, -90)[k % 8]
+        g[:, s: s + n] = np.ldexp(rng.uniform(-1, 1, (M, n)), e).astype(np.float32)
+    r = G.GpuRound(segs, bucket, M)
+    r.set_grads(g)
+    r.set_b(b)
+    norms, packed = r.norms_quantize(SEED, 4)
+    norms, packed = norms.copy(), packed.copy()
+    want = oracle.unpack_dequant_average(ref, packed[:, : ref.packed_words(b)], norms, b)
+    out = r.average(fill=1e30).copy()
+    assert np.isfinite(want).all() and np.isfinite(out).all()
+    # per bucket: the 1e-6 of the ordinary averages, relative to the bucket's own size
+    for k in range(ref.nb):
+        s, n = int(ref.bucket_start[k]), int(ref.bucket_len[k])
+        scale = np.float64(norms[:, k].max())
+        assert G.rel_l2(out[s: s + n] / scale, want[s: s + n] / scale) <= 1e-6
+    x0 = np.linspace(-1, 1, ref.D32, dtype=np.float32)
+    upd = r.update(0.25, x0).copy()
+    for lr, w in ((None, out), (0.25, upd)):
+        r.g_out.view.copy_(torch.from_numpy(x0))
+        dq.quantize_average(r.lay, r.grads, r.stride, M, r.g_norms.view, r.g_b.view, SEED, 4, r.g_packed.view, r.pstride,
+                            r.g_out.view, r.status, lr=lr)
+        np.testing.assert_array_equal(r.g_out.view.cpu().numpy(), w)
+    assert r.read_status() == 0 and r.guards_intact()
