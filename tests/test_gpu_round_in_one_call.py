@@ -204,3 +204,35 @@ def test_norms_and_rule_in_one_call(G, segs, bucket, M):
         np.testing.assert_array_equal(r.g_norms.view.cpu().numpy().reshape(M, -1), norms)
         assert tuple(r.g_b.view.cpu().tolist()) == want
     assert r.read_status() == 0 and r.guards_intact()
+
+
+@pytest.mark.parametrize("bucket", [32, 96, 160, 480, 512, 992])
+def test_zero_buckets_take_no_longer_than_full_ones(G, bucket):
+    """Buckets of zeros, which sparse gradients are full of, need no draws and no second reduction: a round and the
+    codes alone take no longer on zeros than on normal values, for bucket lengths that are no power of two as well.
+    (Best of five trains of 10 calls: 0.79 to 1.10 of the dense time; 2.7 times and more where tiles of zeros took the
+    general way.)"""
+    dq = G.dq
+    from paper_2107_14575_b200.pipeline import Round
+    M, d, b = 4, 1 << 23, 4
+    rnd = Round([d], bucket, M)
+    rule = dq.Rule.fixed(b)
+    dense = torch.randn((M, d), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    times = {}
+    for name, g in (("dense", dense), ("zeros", torch.zeros_like(dense))):
+        rnd.norms_(g)
+        rnd.bits_(rule)
+        for call in (lambda: rnd.step_fused(g, rule, SEED, 0), lambda: rnd.norms_quantize_(g, SEED, 0)):
+            best = []
+            for _ in range(6):
+                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                e0.record()
+                for _ in range(10):
+                    call()
+                e1.record()
+                torch.cuda.synchronize()
+                best.append(e0.elapsed_time(e1))
+            times.setdefault(name, []).append(min(best[1:]))
+    assert rnd.read_status() == 0
+    for zeros, full in zip(times["zeros"], times["dense"]):
+        assert zeros <= 1.25 * full, times
