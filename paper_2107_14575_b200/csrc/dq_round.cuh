@@ -218,9 +218,11 @@ struct ClearsRow {
 template <bool CLEAR>
 __device__ __forceinline__ void clear_nonfinite_row(const uint32_t row, const int valid, const float nrm)
 {
-    if (!CLEAR || valid == 0 || isfinite(nrm)) return;           // (valid = 0: the lane has no row of its own)
+    if constexpr (CLEAR) {
+        if (valid == 0 || isfinite(nrm)) return;                 // (valid = 0: the lane has no row of its own)
 #pragma unroll 1
-    for (int c = 0; c < 128; c += 16) *reinterpret_cast<float4*>(smem + (row ^ (uint32_t)c)) = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < 128; c += 16) *reinterpret_cast<float4*>(smem + (row ^ (uint32_t)c)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 // The lanes of a bucket combine their v; the result is the same in all of them.
@@ -889,7 +891,10 @@ int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, R
 {
     size_t smem_need = (size_t)SmemMap::table;
     if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
+    // (the limit of the largest table, whatever this one's size: with each call's own, another thread's call for a
+    // smaller layout can narrow it again before this launch, which then fails)
+    constexpr int kLargest = SmemMap::table + 3 * (kMaxSmemSegs + 1) * 4;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLargest) != cudaSuccess) {
         (void)cudaGetLastError();
         return DQ_ERR_CUDA;
     }

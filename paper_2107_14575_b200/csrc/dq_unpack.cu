@@ -643,7 +643,10 @@ int launch_average(const dq_layout_t* L, const uint32_t* dev_packed, int64_t pac
 
     size_t smem_need = (size_t)kTblOffset;
     if (L->n_seg > 1 && L->n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (L->n_seg + 1) * 4;
-    if (cudaFuncSetAttribute(unpack_average_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_need) != cudaSuccess) {
+    // (the limit of the largest table, whatever this one's size: with each call's own, another thread's call for a
+    // smaller layout can narrow it again before this launch, which then fails)
+    constexpr int kLargest = kTblOffset + 3 * (kMaxSmemSegs + 1) * 4;
+    if (cudaFuncSetAttribute(unpack_average_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLargest) != cudaSuccess) {
         (void)cudaGetLastError();
         return DQ_ERR_CUDA;
     }
