@@ -13,8 +13,8 @@
 // lane, every store touched 32 lines: one worker, 2^25 elements, b = 4 37 us against 30).
 // HBM traffic per output element: M*b/8 bytes read, 4 written.  Bound by the logic pipe for small b
 // (one half-rate operation per code) and the issue of about 100 instructions per lane, worker and group,
-// by HBM from b = 8 on.  For many workers and b <= 4 the words go straight into registers (below).  Measured, d = 8.4M, M = 16: b = 4 23.8 us (4.2 TB/s), b = 8 30.2 us (5.6), b = 16
-// 51.7 us (5.8); one worker, 2^25 elements, b = 4 26.9 us (5.6).  (Codes taken two at a time as fp16 pairs,
+// by HBM from b = 8 on.  Measured, d = 8.4M, M = 16: b = 4 21.0 us (4.8 TB/s), b = 8 29.6 us (5.7), b = 16 51.7 us (5.8);
+// one worker, 2^25 elements, b = 4 28.2 us (5.3).  (Codes taken two at a time as fp16 pairs,
 // for half the logic operations, and widened by mixed-precision adds: 9 % slower at b = 4.)
 //
 // dq_unpack_average_update ends with the parameter update of Algorithm 1 instead, x <- x - eta * average;
@@ -162,29 +162,18 @@ struct Normalise<B, 32> {
     static __device__ __forceinline__ void run(float (&)[32]) {}
 };
 
-// Whether a lane's 32 sums are finite: 0 times each of them adds up to 0.
-__device__ __forceinline__ bool sums_finite(const uint64_t (&acc2)[16])
-{
-    uint64_t t = 0ull;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) t = fma_pair(acc2[q], 0ull, t);
-    float lo, hi;
-    unpack_pair(t, lo, hi);
-    return lo + hi == 0.0f;
-}
-
 // The end of a tile: the powers of two removed, padding zeroed, the rows through the warp's output tile.
-// kOutOfRange (nothing stored): a sum is not finite.  kLost: the tile of x did not arrive.
+// kOutOfRange (nothing stored): some lane says so of its sums.  kLost: the tile of x did not arrive.
 enum TileEnd { kDone, kOutOfRange, kLost };
 template <int B>
 __device__ __forceinline__ TileEnd finish_tile(const AverageArgs& a, const CUtensorMap* out_map, unsigned char* out_tile,
-                                            const uint64_t (&acc2)[16], const int tile, const int valid, uint64_t* xbar,
-                                            const uint32_t x_parity)
+                                            const uint64_t (&acc2)[16], const int tile, const int valid, const bool out_of_range,
+                                            uint64_t* xbar, const uint32_t x_parity)
 {
     const int lane = threadIdx.x & 31;
     // (B = 1: s = 0, every value is 0, and an update by 0 leaves x as it is)
     if (!(B == 1 && a.update)) {
-        if (B > 1 && __any_sync(0xffffffffu, valid > 0 && !sums_finite(acc2))) return kOutOfRange;
+        if (B > 1 && __any_sync(0xffffffffu, out_of_range)) return kOutOfRange;
         float acc[32];
 #pragma unroll
         for (int q = 0; q < 16; ++q) unpack_pair(acc2[q], acc[2 * q], acc[2 * q + 1]);
@@ -255,8 +244,8 @@ __device__ __forceinline__ void locate_group(const AverageArgs& a, const bool tb
 
 // Tiles `tile`, `tile` + `hop`, ... (n of them) with every code shifted down and without the power of two of its
 // position, which takes sums of 2^106 and more out of the fp32 range: the same values, order and roundings as in
-// the one-pass kernels.  The warp ends here with the first tile that has such norms (or an infinity or a NaN); what
-// it has in flight has landed by then.  Out of line, with plain loads and stores: the others pay 16 packed FMAs.
+// the one-pass kernels.  The warp ends here with the first tile that has such norms (an infinity or a NaN among them); what
+// it has in flight has landed by then.  Out of line, with plain loads and stores.
 __device__ __noinline__ void average_tiles_plain(const AverageArgs& a, const bool tbl_in_smem, const int B, int tile, const int hop, int n)
 {
     const int lane = threadIdx.x & 31;
@@ -290,18 +279,18 @@ __device__ __noinline__ void average_tiles_plain(const AverageArgs& a, const boo
     }
 }
 
-// ---- b = 2, 3, 4 and 20 workers or more: words straight into registers --------------------------
-// A lane's words of a worker are one to three loads that neighbouring lanes coalesce.  Up to eight workers'
-// words and norms wait in registers; as soon as one has been decoded, its registers are the target of
-// the load for the worker eight further on (of the next tile, when this one's are through), so nothing is
-// moved, staged or waited for.  Pays where tiles are long: staged / direct (us), 2^24 elements M = 32 b = 2
-// 73.7 / 65.4, b = 3 78.3 / 72.0, b = 4 78.5 / 75.8, VGG-16 shape M = 24 b = 4 55.8 / 55.2; d = 8.4M M = 16
-// b = 4 23.9 / 24.4, 2^24 elements M = 4 19.6 / 22.3.
+// ---- b = 2, 3 and workers in whole eights: words straight into registers --------------------------
+// A lane's words of a worker are one to three loads that neighbouring lanes coalesce.  Eight workers' words and
+// norms wait in registers; as soon as one has been decoded, its registers are the target of the load for the worker
+// eight further on (of the next tile, when this one's are through), so nothing is moved, staged or waited for.
+// Measured, by asynchronous copies / direct (us): 2^25 elements M = 8 b = 2 45.0 / 41.2, b = 3 49.2 / 46.6, M = 16 72.2 /
+// 69.5 and 77.2 / 74.1; 2^24 elements M = 24 52.3 / 51.8 and 55.9 / 54.1, M = 64 123.4 / 124.9 and 131.7 / 129.9; d = 4.2M M = 8
+// 7.8 / 8.2 and 8.3 / 8.8.  A last group of fewer than eight costs more than it saves: 2^24 elements M = 20 47.4 / 51.4 and
+// 50.7 / 55.2; and at b = 4 so do the wider loads: M = 32 68.9 / 73.7.
 template <int B>
 struct DirectWords {
-    static constexpr bool value = B >= 2 && B <= 4;
+    static constexpr bool value = B == 2 || B == 3;
     static constexpr int workers = 8;
-    static constexpr int min_workers = 20;
 };
 template <int B>
 __device__ __forceinline__ void request_words(const uint32_t* p, uint32_t (&w)[B])
@@ -314,6 +303,16 @@ __device__ __forceinline__ void request_words(const uint32_t* p, uint32_t (&w)[B
 #pragma unroll
         for (int i = 0; i < B; ++i) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[i]) : "l"(p + i));
     }
+}
+// Whether a lane's 32 sums are finite: 0 times each of them adds up to 0.
+__device__ __forceinline__ bool sums_finite(const uint64_t (&acc2)[16])
+{
+    uint64_t t = 0ull;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) t = fma_pair(acc2[q], 0ull, t);
+    float lo, hi;
+    unpack_pair(t, lo, hi);
+    return lo + hi == 0.0f;
 }
 template <int B>
 __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const CUtensorMap* out_map, const bool tbl_in_smem)
@@ -348,10 +347,8 @@ __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const
         const float* q = a.norms + bucket;
 #pragma unroll
         for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
-            if (j < M) {
-                request_words<B>(p, wd[j]);
-                nrm[j] = load_norm_early(q);
-            }
+            request_words<B>(p, wd[j]);
+            nrm[j] = load_norm_early(q);
         }
     }
     auto decode = [&](uint64_t (&acc2)[16], const uint32_t (&w)[B], const float norm) {
@@ -369,13 +366,15 @@ __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const
         if (a.update && lane == 0) request_x(out_map, out_tile, tile, x_bar(warp));
 #pragma unroll 1
         for (int m0 = 0; m0 < M; m0 += MC) {
-            // the workers eight further on: of this tile, or the first ones of the next
+            // the workers eight further on: of this tile, or the first ones of the next, if there is one.  (The second
+            // loop keeps its bounds, although groups are whole here: without them the compiler orders the first
+            // one's loads worse, 2^26 elements M = 32 b = 3 262.5 -> 268.8 us.)
             const bool same = m0 + MC < M;
             if (!same && k + 1 < n_tiles) locate_group(a, tbl_in_smem, tile + hop, nbucket, nvalid);
             const int first = same ? m0 + MC : 0;
-            const int more = same ? M - first : (k + 1 < n_tiles ? M : 0);        // workers that are there to be requested
             const uint32_t* p = words_of(same ? tile : tile + hop, first);
             const float* q = a.norms + (int64_t)first * nb + (same ? bucket : nbucket);
+            const int more = same ? M - first : (k + 1 < n_tiles ? M : 0);
             if (m0 + MC <= M && more >= MC) {
 #pragma unroll
                 for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
@@ -385,16 +384,18 @@ __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const
                 }
             } else {
 #pragma unroll
-                for (int j = 0; j < MC; ++j, p += a.packed_stride, q += nb) {
+                for (int j = 0; j < MC; ++j) {
                     if (m0 + j < M) decode(acc2, wd[j], nrm[j]);
                     if (j < more) {
                         request_words<B>(p, wd[j]);
                         nrm[j] = load_norm_early(q);
                     }
+                    p += a.packed_stride; q += nb;
                 }
             }
         }
-        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), (uint32_t)k & 1u);
+        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, valid > 0 && !sums_finite(acc2), x_bar(warp),
+                                           (uint32_t)k & 1u);
         if (end != kDone) {
             if (lane == 0) {
                 if (end == kLost) atomicOr(a.status, DQ_STAT_WAIT);
@@ -413,7 +414,37 @@ __device__ __forceinline__ void average_tiles_direct(const AverageArgs& a, const
     if (lane == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
 }
 
+// ---- how the words come into a stage --------------------------------------------------------------
+// ASYNC = false: one bulk copy of 128 * b bytes per worker.  ASYNC = true: 16 bytes per lane and instruction, straight
+// to shared memory.  The bulk copies are so small that their rate is the limit where there are many workers (2^25
+// elements, M = 12, b = 2: one copy of 256 bytes every 15 cycles of an SM); with few, a stage is a few copies, which cost
+// the warp less than its own.  Measured, bulk / async (us): 2^25 elements M = 12 b = 2 66.7 / 62.5, b = 4 68.4 / 65.7,
+// b = 5 71.7 / 74.2; M = 8 b = 2 46.9 / 45.6, b = 4 49.3 / 49.7, b = 5 57.7 / 59.9, b = 7 60.1 / 62.5; M = 4 b = 2 34.5 / 35.8,
+// b = 5 38.3 / 43.2; d = 8.4M M = 16 b = 4 22.9 / 21.0, b = 6 29.1 / 29.1, b = 7 30.4 / 30.1; 2^24 elements M = 32 b = 5
+// 89.2 / 88.2, b = 6 91.5 / 87.9, b = 7 99.4 / 95.0, b = 8 94.3 / 93.2 (M = 16 29.6 / 29.8).
 template <int B>
+struct AsyncCopies {
+    static constexpr bool value = B >= 2 && B <= 7;
+    static constexpr int min_workers = B <= 4 ? 8 : 16;
+};
+// The codes of N workers of a stage, added to the sums; moves on to the workers behind them.
+template <int B, int N, int MC>
+__device__ __forceinline__ void add_workers(uint64_t (&acc2)[16], const uint32_t*& base, float (&scale)[MC], const uint32_t magic)
+{
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        uint32_t wd[B], hi[B];
+        load_words<B>(base + j * (32 * B), wd);
+        UpperHalves<B, 0>::run(base + j * (32 * B), hi);
+        const uint32_t sc = __float_as_uint(scale[j]);
+        AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
+    }
+    base += N * (32 * B);
+#pragma unroll
+    for (int j = 0; j + N < MC; ++j) scale[j] = scale[j + N];
+}
+
+template <int B, bool ASYNC>
 __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtensorMap* out_map, const bool tbl_in_smem)
 {
     constexpr int s = (1 << (B - 1)) - 1;
@@ -435,17 +466,36 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
     // ---- producer side: item = (tile, chunk of workers), fetched two ahead of the consumer
     int p_tile = (int)id, p_m0 = 0, p_left = items;
     auto fetch = [&](int st) {
-        if (p_left <= 0) return;
-        --p_left;
-        const int rows = (G - p_tile * 32) < 32 ? (G - p_tile * 32) : 32;
-        const uint32_t bytes = ((uint32_t)(rows * B * 4) + 15u) & ~15u;      // the stream's stride is a multiple of 16 bytes
-        const int mc = (M - p_m0) < MC ? (M - p_m0) : MC;
-        if (lane == 0) tma::mbar_expect_tx(stage_bar(warp, st), bytes * (uint32_t)mc);
-        if (lane < mc)
-            tma::load_bulk(stage_words(warp, st) + lane * (32 * B),
-                           a.packed + (int64_t)(p_m0 + lane) * a.packed_stride + (int64_t)p_tile * (32 * B), bytes, stage_bar(warp, st));
-        p_m0 += MC;
-        if (p_m0 >= M) { p_m0 = 0; p_tile += hop; }
+        if (p_left > 0) {
+            --p_left;
+            const int rows = (G - p_tile * 32) < 32 ? (G - p_tile * 32) : 32;
+            const uint32_t bytes = ((uint32_t)(rows * B * 4) + 15u) & ~15u;      // the stream's stride is a multiple of 16 bytes
+            if constexpr (ASYNC) {
+                const uint32_t dst = tma::smem_addr(stage_words(warp, st)) + lane * 16;
+                const uint32_t* src = a.packed + (int64_t)p_m0 * a.packed_stride + (int64_t)p_tile * (32 * B) + lane * 4;
+#pragma unroll
+                for (int j = 0; j < MC; ++j, src += a.packed_stride) {
+                    if (p_m0 + j < M) {
+#pragma unroll
+                        for (int u = 0; u < 128 * B; u += 512)
+                            if ((uint32_t)(lane * 16 + u) < bytes)
+                                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + j * (128 * B) + u), "l"(src + u / 4)
+                                             : "memory");
+                    }
+                }
+            } else {
+                const int mc = (M - p_m0) < MC ? (M - p_m0) : MC;
+                if (lane == 0) tma::mbar_expect_tx(stage_bar(warp, st), bytes * (uint32_t)mc);
+                if (lane < mc)
+                    tma::load_bulk(stage_words(warp, st) + lane * (32 * B),
+                                   a.packed + (int64_t)(p_m0 + lane) * a.packed_stride + (int64_t)p_tile * (32 * B), bytes,
+                                   stage_bar(warp, st));
+            }
+            p_m0 += MC;
+            if (p_m0 >= M) { p_m0 = 0; p_tile += hop; }
+        }
+        // (an empty group where nothing is left to copy: the wait counts groups)
+        if constexpr (ASYNC) asm volatile("cp.async.commit_group;" ::: "memory");
     };
 #pragma unroll
     for (int st = 0; st < kStages; ++st) fetch(st);
@@ -476,6 +526,7 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
         uint64_t acc2[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) acc2[q] = 0ull;
+        float largest = 0.0f;
         int nbucket = bucket, nvalid = valid;
         x_parity = (uint32_t)k & 1u;
         if (B > 1 && a.update && lane == 0) request_x(out_map, out_tile, tile, x_bar(warp));
@@ -485,48 +536,47 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
                 const int st = (int)(it & 1u);
                 // the norms of the chunk after this one travel during the wait and the decoding
 #pragma unroll
-                for (int j = 0; j < MC; ++j) scale[j] = nxt[j] * unit;
+                for (int j = 0; j < MC; ++j) {
+                    scale[j] = nxt[j] * unit;
+                    if (j & 1 || j + 1 == MC) largest = max_magnitude(largest, nxt[j], nxt[j > 0 ? j - 1 : 0]);
+                }
                 if (m0 + MC < M) {
                     request_norms(m0 + MC, bucket);
                 } else if (k + 1 < n_tiles) {
                     locate(tile + hop, nbucket, nvalid);
                     request_norms(0, nbucket);
                 }
-                // every lane polls the barrier itself; the verdict is made warp-uniform
-                if (!__all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), (it >> 1) & 1u, a.wait))) {
+                if constexpr (ASYNC) {
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");           // all but the stage after this one
+                    __syncwarp();
+                } else if (!__all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, st), (it >> 1) & 1u, a.wait))) {
+                    // (every lane polls the barrier itself; the verdict is made warp-uniform)
                     timed_out = true;
                     break;
                 }
                 const uint32_t* base = stage_words(warp, st) + lane * B;
-                if (m0 + MC <= M) {              // a full stage: no loop
-#pragma unroll
-                    for (int j = 0; j < MC; ++j) {
-                        uint32_t wd[B], hi[B];
-                        load_words<B>(base + j * (32 * B), wd);
-                        UpperHalves<B, 0>::run(base + j * (32 * B), hi);
-                        const uint32_t sc = __float_as_uint(scale[j]);
-                        AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
-                    }
+                if (m0 + MC <= M) {              // a full stage, or what is left in blocks of 4, 2 and 1: no loop
+                    add_workers<B, MC>(acc2, base, scale, magic);
                 } else {
-#pragma unroll
-                    for (int j = 0; j < MC - 1; ++j) {
-                        if (m0 + j >= M) break;
-                        uint32_t wd[B], hi[B];
-                        load_words<B>(base + j * (32 * B), wd);
-                        UpperHalves<B, 0>::run(base + j * (32 * B), hi);
-                        const uint32_t sc = __float_as_uint(scale[j]);
-                        AccumulateAll<B, 0>::run(acc2, wd, hi, pack_pair(sc, sc), magic);
+                    const int left = M - m0;
+                    if constexpr (MC > 4) {
+                        if (left & 4) add_workers<B, 4>(acc2, base, scale, magic);
                     }
+                    if constexpr (MC > 2) {
+                        if (left & 2) add_workers<B, 2>(acc2, base, scale, magic);
+                    }
+                    if (left & 1) add_workers<B, 1>(acc2, base, scale, magic);
                 }
-                // the warp's reads of the stage come before the copies that refill it (another proxy)
-                tma::fence_proxy_async();
+                // the warp's reads of the stage come before the copies that refill it (another proxy, if they are bulk copies)
+                if constexpr (!ASYNC) tma::fence_proxy_async();
                 __syncwarp();
                 fetch(st);
                 __syncwarp();
             }
             if (timed_out) break;
         }
-        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, x_bar(warp), x_parity);
+        // (decoded values carry up to 2^21: sums of norms below 2^104 stay in the fp32 range)
+        const TileEnd end = finish_tile<B>(a, out_map, out_tile, acc2, tile, valid, !(largest < 0x1p104f), x_bar(warp), x_parity);
         if (end == kOutOfRange) { plain_left = n_tiles - k; break; }
         if (end == kLost) { timed_out = true; break; }
         tile += hop;
@@ -535,11 +585,12 @@ __device__ __forceinline__ void average_tiles(const AverageArgs& a, const CUtens
         valid = nvalid;
     }
     if (lane == 0) tma::store_wait_read();         // shared memory must outlive the last store's reads
+    if constexpr (ASYNC) asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (timed_out || skip_all || plain_left > 0) {
         // every copy the warp has issued and not seen land, the one whose wait ran out included, gets the
         // full limit before the CTA's shared memory is released
         bool landed = plain_left > 0;
-        for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
+        for (uint32_t i = it; !ASYNC && i < (uint32_t)(items - p_left); ++i)
             landed &= tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
         if (B > 1 && a.update && !skip_all) landed &= tma::mbar_wait(x_bar(warp), x_parity, a.wait);
         landed = __all_sync(0xffffffffu, landed);
@@ -581,12 +632,18 @@ unpack_average_kernel(const __grid_constant__ AverageArgs a, const __grid_consta
     switch (b) {
 #define DQ_CASE(BB) case BB:                                                                             \
             if constexpr (DirectWords<BB>::value) {                                                       \
-                if (a.M >= DirectWords<BB>::min_workers) {                                                \
+                if (a.M % DirectWords<BB>::workers == 0) {                                                \
                     average_tiles_direct<BB>(a, &out_map, tbl_in_smem);                                   \
                     break;                                                                                \
                 }                                                                                         \
             }                                                                                             \
-            average_tiles<BB>(a, &out_map, tbl_in_smem);                                                  \
+            if constexpr (AsyncCopies<BB>::value) {                                                       \
+                if (a.M >= AsyncCopies<BB>::min_workers) {                                                \
+                    average_tiles<BB, true>(a, &out_map, tbl_in_smem);                                    \
+                    break;                                                                                \
+                }                                                                                         \
+            }                                                                                             \
+            average_tiles<BB, false>(a, &out_map, tbl_in_smem);                                           \
             break;
         DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
         DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)

@@ -31,8 +31,8 @@ def G(dqlib):
 
 
 @pytest.mark.parametrize("huge", [False, True])
-@pytest.mark.parametrize("M,b,bucket", [(20, 2, 512), (24, 3, 512), (33, 4, 512), (20, 4, 480), (24, 2, 4096), (33, 3, 0), (7, 4, 512),
-                                        (20, 5, 96), (12, 8, 512), (5, 16, 128)])
+@pytest.mark.parametrize("M,b,bucket", [(20, 2, 512), (24, 3, 512), (33, 4, 512), (20, 4, 480), (24, 2, 4096), (32, 3, 512), (33, 3, 0), (7, 4, 512),
+                                        (20, 5, 96), (17, 6, 512), (21, 7, 512), (11, 7, 512), (12, 8, 512), (5, 16, 128)])
 def test_every_element_of_every_tile(G, M, b, bucket, huge):
     dq = G.dq
     ref = oracle.Layout(SEGS, bucket if bucket else oracle.whole_tensor_bucket(SEGS))
