@@ -10,6 +10,7 @@
 // before its gradients are: a bucket that sits in registers can be measured, coded and added to the
 // average at once, and every gradient byte is read from HBM a single time.
 #include "dq_round.cuh"
+#include "dq_route.h"
 
 namespace {
 
@@ -61,25 +62,16 @@ int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, boo
                   : dq_launch_round<kTeamBuckets, AVG, false>(a, map, L->n_seg, entries, st);
 }
 
-// One pass for codes and average, or codes (all workers' tiles side by side) and then the average from
-// the words?  In one pass a warp takes a position through all M workers, one after the other: P positions
-// on U warps are `full` turns of M tiles and a last turn in which only a fraction f of the warps has work.
-// Two kernels spread the M * P tiles evenly, but cost a launch and read the words back.  Per worker, a
-// turn's tile takes 1.8 us when the SMs are nearly empty (1.2 with given norms) and 0.9 more when they are
-// full; two kernels take 2.6 us times the turns' share, and 7.5 us for the second launch; a full turn is
-// 0.4 us cheaper in one pass (0.7 with given norms).  So the last turn decides.  Measured on one B200, b = 5, bucket 512, one
-// pass / two kernels (us): 70k elements M = 4 14.5 / 13.2, M = 32 80 / 20; 600k M = 4 12.6 / 14.2, M = 8
-// 20.4 / 19.2, M = 32 66 / 35; 1.5M M = 8 24.9 / 26.0, M = 32 82 / 64; 3M M = 8 36.5 / 39.3, M = 32
-// 123 / 114; 6M M = 32 210 / 217; bucket 480: 600k M = 8 21.6 / 22.9, M = 32 66 / 55.
 bool one_pass(const RoundArgs& a, bool given)
 {
-    int64_t units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
-    if (!given && a.div_shift >= 0 && a.gpb_shift > 5) units >>= a.gpb_shift - 5;
-    const int64_t p = dq_tile_positions(a, given);
-    const int64_t full = p / units;
-    const double f = (double)(p - full * units) / (double)units;
-    if (a.M == 1 || f == 0.0) return true;                       // no worker to wait for, or no idle warp
-    return a.M * ((given ? 1.2 : 1.8) - 1.7 * f - (given ? 0.7 : 0.4) * (double)full) <= 7.5;
+    RouteQuery q = {};
+    q.positions = dq_tile_positions(a, given);
+    q.units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
+    if (!given && a.div_shift >= 0 && a.gpb_shift > 5) q.units >>= a.gpb_shift - 5;
+    q.M = a.M;
+    q.given = given ? 1 : 0;
+    q.odd_buckets = !given && a.div_shift < 0 ? 32 / a.v.groups_per_bucket : 0;
+    return dq_one_pass(q);
 }
 
 }  // namespace
