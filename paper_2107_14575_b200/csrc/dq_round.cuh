@@ -208,12 +208,13 @@ __device__ __noinline__ void clear_row_tail(const uint32_t row, const int valid)
 
 // A norm that is an infinity or a NaN: the scale of the codes is 0, every code is s and every term of the average
 // 0 * norm = NaN, but 0 times an entry that is not finite has no code (for b <= 4 its bits reach the codes of its
-// neighbours).  So the words of such a row are set after the encoder; the kernels with l2 norms and the average,
-// which have no register to spare for that (VGG-16 shape M = 16 with update 256 -> 264 us), set the row to zero
-// beforehand, in the call that finds such norms.  (Clearing the row everywhere: l-inf rounds 25.9 -> 27.9 us.)
-template <int MODE, bool AVG, bool LINF>
+// neighbours).  Kernels with l2 norms set the row of such a bucket to zero beforehand, in the call that finds the norm,
+// which costs the others nothing; the ones that have no such call set the words after the encoder.  (That in all of
+// them: VGG-16 shape M = 16 with update 256 -> 264 us, codes of 1.6M elements M = 4 8.9 -> 9.3; clearing the row beside the
+// encoder: l-inf rounds 25.9 -> 27.9.)
+template <int MODE, bool LINF>
 struct ClearsRow {
-    static constexpr bool value = AVG && !LINF && MODE != kGivenNorms;
+    static constexpr bool value = !LINF && MODE != kGivenNorms;
 };
 template <bool CLEAR>
 __device__ __forceinline__ void clear_nonfinite_row(const uint32_t row, const int valid, const float nrm)
@@ -411,7 +412,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     const int M = a.M;
     const int nb = a.v.nb;
     const int G = a.v.total_groups;
-    constexpr bool kClears = ClearsRow<MODE, AVG, LINF>::value;
+    constexpr bool kClears = B != 0 && ClearsRow<MODE, LINF>::value;
     constexpr bool ODD = MODE == kOddBuckets;
     constexpr bool TILES = MODE == kWarpBuckets || ODD;               // tiles of whole buckets
     const int gpb = ODD ? a.v.groups_per_bucket : 1 << a.gpb_shift;
