@@ -12,9 +12,8 @@
 
 namespace {
 
-// Both kernels are small on purpose (128 threads, well under 100 registers): in the order of
-// Algorithm 1 they run on a second stream beside the average, whose persistent CTAs leave
-// about a fifth of an SM's registers free, and CTAs of this size fit into that room.
+// Both kernels are small (128 threads, well under 100 registers), so that their CTAs fit beside the persistent ones of
+// an average that a caller runs on another stream.  A round in one call applies the rule at the end of its own kernel.
 constexpr int kThreads = 128;       // threads of the second kernel
 constexpr int kChunk = 8192;        // norms per CTA of the first kernel
 constexpr int kSumThreads = 128;    // threads of the first kernel: 64 norms each, all loads in flight at once

@@ -18,7 +18,7 @@
 // HBM traffic: 4 + b/8 bytes per element and worker, plus 4 (8 with the update) per output element.
 // What bounds it: per tile of a worker a warp issues some 530 instructions at b = 4 (290 of them the codes,
 // their draws and the sums; 65 are the wide multiplies of the generator, four cycles of the multiplier
-// each), 65 % of the issue slots' and 70 % of the multiplier's time, beside loads that alone take 0.9 of
+// each), 60 % of the issue slots' and 67 % of the multiplier's time, beside loads that alone take 0.9 of
 // the measured copy bandwidth.  Measured: 2^26 elements M = 32 b = 4 1.89 ms (5.2 TB/s; separate
 // quantizer and average 2.29), ResNet-18 shape M = 8 92 us (4.9), VGG-16 shape M = 16 b = 5 with update 260 us.
 #pragma once
@@ -68,13 +68,9 @@ int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64
 // CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower); 102 without them
 // (codes of 2^24 elements, b = 6: 17.4 us with five CTAs, 18.1 with six of 80 registers, 18.7 with four; buckets of
 // 4096, M = 16, b = 5: 251, 256 and 254 us).
-#ifndef DQ_ROUND_CTAS_AVG
-#define DQ_ROUND_CTAS_AVG 4
-#define DQ_ROUND_CTAS_ENC 5
-#endif
 template <bool AVG>
 struct RoundShape {
-    static constexpr int ctas_per_sm = AVG ? DQ_ROUND_CTAS_AVG : DQ_ROUND_CTAS_ENC;
+    static constexpr int ctas_per_sm = AVG ? 4 : 5;
 };
 
 constexpr int kRoundThreads = 128;
@@ -872,12 +868,8 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
     double square_sum = 0.0;
     switch (b) {
 #define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG, LINF>(a, &map, tbl_in_smem, square_sum); break;
-#ifdef DQ_ONLY_B
-        DQ_CASE(DQ_ONLY_B)
-#else
         DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
         DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
-#endif
 #undef DQ_CASE
         default: break;
     }

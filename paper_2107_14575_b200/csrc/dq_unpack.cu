@@ -295,9 +295,7 @@ struct DirectWords {
 template <int B>
 __device__ __forceinline__ void request_words(const uint32_t* p, uint32_t (&w)[B])
 {
-    if constexpr (B == 4) {
-        asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
-    } else if constexpr (B == 2) {
+    if constexpr (B == 2) {
         asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
     } else {
 #pragma unroll
