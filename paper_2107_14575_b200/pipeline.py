@@ -27,8 +27,8 @@ class Round:
         self.norms = torch.empty((M, L.nb), dtype=torch.float32, device=self.device)
         self.packed = torch.empty((M, self.packed_stride), dtype=torch.int32, device=self.device)
         self.out = torch.empty(L.D32, dtype=torch.float32, device=self.device)
-        # two (b, s) slots of 16 bytes: the rounds of ``step_fused`` alternate between them, so that
-        # the next b can be written while the average still reads the current one
+        # two (b, s) slots of 16 bytes: where ``step_fused`` puts the bit rule on a second stream (``events``), the
+        # next b goes to the other one while the average still reads this one; one-call rounds stay in their slot
         self._b = torch.zeros((2, 4), dtype=torch.int32, device=self.device)
         self._cur = 0
         self._side = None
@@ -111,7 +111,7 @@ class Round:
         separate calls instead, with the events recorded around them (e* on the current stream, s*
         around the bit rule): ``overlap`` then puts the bit rule on a second stream next to the average
         (it needs only the norms, and writes the other (b, s) slot); ``overlap=None`` decides by size,
-        ``OVERLAP_MIN_NORMS``.
+        ``OVERLAP_MIN_NORMS``.  The one call takes no notice of ``overlap``: its rule is part of its last kernel.
 
         With ``params`` (fp32 [D32] in the padded layout) the server step also applies the
         update of Eq. 2, ``params <- params - lr * average``, in the same kernel; ``out`` is
