@@ -2,9 +2,9 @@
 """Benchmark of the DQ-SGD quantizer hot path on B200.
 
 One step = one communication round of Algorithm 1 on one batch of synthetic
-gradients, all through the C-ABI library: bucket norms and quantize+pack in one
-pass with the bit width chosen after the previous round, unpack+dequantize+average,
-and the bit rule for the next round beside the average.
+gradients, all through the C-ABI library: bucket norms, quantize+pack with the bit
+width chosen after the previous round, the average, and the bit rule for the next
+round, in one kernel.
 
 The workload is the largest single-GPU point of the bandwidth sweep: one flat
 N(0,1) fp32 gradient of d = 2^26 elements per worker, M = 32 workers (8 GiB of
@@ -21,7 +21,8 @@ are timed as secondary figures.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Prints ONE JSON line.  ``value`` is GB/s of fp32 gradient processed
+Prints ONE JSON line on stdout (and the full record, with the tables named above, as
+one line on stderr).  ``value`` is GB/s of fp32 gradient processed
 (4 * M * d bytes per step over the step time), inputs resident in HBM;
 ``e2e`` is the same with pinned host buffers and the copies timed.
 ``--impl reference`` times the CPU checker on the host cores instead.
@@ -264,8 +265,10 @@ class Timer:
         return s.elapsed_time(e) / n
 
     def single(self, fn, n: int) -> float:
-        """mean ms of `n` calls each bracketed by its own pair of events (sees the launch latency too)."""
+        """mean ms of `n` calls each bracketed by its own pair of events (sees the launch latency too), after one
+        untimed call: a kernel's first launch also loads its code."""
         torch = self.torch
+        fn(0)
         ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(n)]
         torch.cuda.synchronize()
         for i, (s, e) in enumerate(ev):
@@ -475,7 +478,7 @@ def run_cuda(args) -> dict:
     # ---- headline: K steps in the order of Algorithm 1 at b = 4
     set_b(HEADLINE_B)
     for i in range(W):
-        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
+        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i)
     torch.cuda.synchronize()
     assert rnd.read_status() == 0, "device status %d" % rnd.read_status()
     start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -486,7 +489,7 @@ def run_cuda(args) -> dict:
     start.record()
     h0 = time.perf_counter()
     for i in range(K):
-        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
+        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i)
     end.record()
     host_submit_ms = (time.perf_counter() - h0) * 1e3 / K
     torch.cuda.synchronize()
@@ -499,7 +502,7 @@ def run_cuda(args) -> dict:
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(n_ev)]
     for i, (e0, e1) in enumerate(ev):
         e0.record()
-        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i, overlap=(False if args.no_overlap else None))
+        rnd.step_fused(grads, rule_b(HEADLINE_B, i + 1), SEED, i)
         e1.record()
     torch.cuda.synchronize()
     step_ms = {"round": sum(e0.elapsed_time(e1) for e0, e1 in ev) / n_ev}
@@ -587,7 +590,7 @@ def run_cuda(args) -> dict:
             r["single_launch_frac_of_measured"] = round(alg_bytes[name](b) / (t_single * 1e-3) / 1e9 / peak, 4)
             r["gradient_gbs"] = round(4.0 * M * d / (t_train * 1e-3) / 1e9, 1)
             rec[name] = r
-        step = timer.train(lambda i: rnd.step_fused(grads, rule_b(b, i + 1), SEED, i, overlap=(False if args.no_overlap else None)), K)
+        step = timer.train(lambda i: rnd.step_fused(grads, rule_b(b, i + 1), SEED, i), K)
         rec["step_ms"] = round(step, 5)
         rec["step_gradient_gbs"] = round(4.0 * M * d / (step * 1e-3) / 1e9, 1)
         per_b[str(b)] = rec
@@ -682,6 +685,9 @@ def _cpu_baseline(torch, gen, dev) -> dict:
                       "of all %d workers (1 GiB of gradients per round), %.1f s" % (steps, b, MAIN_M, dt)}
 
 
+TABLES = ("per_b", "bucket_norms", "size_sweep", "model_workloads")     # of the full record, on stderr only
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -693,8 +699,6 @@ def main():
     ap.add_argument("--no-sweep", action="store_true", help="skip the M = 1 sizes and the other bucket lengths of the bandwidth sweep")
     ap.add_argument("--no-models", action="store_true", help="skip the secondary timing of the model-shaped workloads")
     ap.add_argument("--no-per-b", action="store_true", help="skip the per-b table (profiling runs)")
-    ap.add_argument("--no-overlap", action="store_true",
-                    help="run the bit rule after the average on the same stream instead of beside it")
     ap.add_argument("--source-digests", action="store_true",
                     help="print the digest of each kernel's sources (stored beside a counter capture) and exit")
     args = ap.parse_args()
@@ -708,7 +712,9 @@ def main():
         return
     out = run_cuda(args)
     if out:
-        print(json.dumps(out))
+        # the line on stdout is kept short enough to be read whole from a log's end; the tables go to stderr with it
+        print(json.dumps(out), file=sys.stderr)
+        print(json.dumps({k: v for k, v in out.items() if k not in TABLES}))
 
 
 if __name__ == "__main__":

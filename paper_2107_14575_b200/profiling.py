@@ -9,7 +9,7 @@ counters kept under ``profiles/``.
     python -m paper_2107_14575_b200.profiling summarize capture.csv --kernel unpack_dequant_average \
         --log2d 24 --M 32 --b 4 --command "<the full ncu command>" [--update-counters]
 
-    # the per-b table of a bench line as markdown
+    # the per-b table of the bench's full record (bench.py's line on stderr: python bench.py 2> bench_line.json) as markdown
     python -m paper_2107_14575_b200.profiling table bench_line.json > profiles/bench_per_b.md
 
     # per kernel launches / time / share from an `ncu --metrics gpu__time_duration.sum --csv --log-file` run
