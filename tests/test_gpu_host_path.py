@@ -64,7 +64,7 @@ def test_a_round_can_be_captured_in_a_cuda_graph(dqlib):
     rule = dq.Rule.dynamic(T, 30, T * alpha ** (T - 1) * G2 / 36.0, alpha)
     rnd.bits_(dq.Rule.fixed(4))
     cur0 = rnd._cur
-    want = rnd.step_fused(g, rule, 3, 12).clone()          # eager; also creates the side stream and its events
+    want = rnd.step_fused(g, rule, 3, 12).clone()          # eager
     want_packed, want_norms, want_b = rnd.packed.clone(), rnd.norms.clone(), rnd._b.clone()
     torch.cuda.synchronize()
 
@@ -82,5 +82,29 @@ def test_a_round_can_be_captured_in_a_cuda_graph(dqlib):
     nw = rnd.layout.packed_words(4)                        # words beyond the stream are never written
     assert torch.equal(rnd.out, want) and torch.equal(rnd.norms, want_norms)
     assert torch.equal(rnd.packed[:, :nw], want_packed[:, :nw])
-    assert torch.equal(rnd._b[1 - cur0], want_b[1 - cur0])  # the next b came out of the captured bit rule
+    assert torch.equal(rnd._b, want_b)                     # the next b came out of the captured bit rule
     assert rnd.read_status() == 0
+
+
+@pytest.mark.parametrize("update", [False, True])
+@pytest.mark.parametrize("overlap", [False, True])
+def test_separate_calls_with_events_write_what_the_one_call_writes(dqlib, overlap, update):
+    """``step_fused(events=...)``: norms + codes, average and bit rule as calls of their own, the rule on a second stream or
+    behind the average.  Three rounds in a row, so that the slots of b alternate."""
+    from paper_2107_14575_b200 import workloads as W
+    from paper_2107_14575_b200.pipeline import Round
+    dq = dqlib
+    w = W.scaled_down(W.config_resnet18(M=3), 16)
+    a, b = (Round(w.segments, w.bucket, w.M) for _ in range(2))
+    gen = torch.Generator().manual_seed(11)
+    g = torch.randn((w.M, a.layout.D32), generator=gen).mul_(0.02).cuda()
+    x = [torch.ones(a.layout.D32, device="cuda") if update else None for _ in range(2)]
+    for r in (a, b):
+        r.bits_(dq.Rule.fixed(4))
+    for i, nxt in enumerate((6, 3, 5)):
+        events = [torch.cuda.Event(enable_timing=True) for _ in range(5)]
+        want = a.step_fused(g, dq.Rule.fixed(nxt), 3, i, params=x[0], lr=0.5)
+        got = b.step_fused(g, dq.Rule.fixed(nxt), 3, i, overlap=overlap, events=events, params=x[1], lr=0.5)
+        assert torch.equal(got, want) and torch.equal(b.norms, a.norms) and torch.equal(b.dev_b[:2], a.dev_b[:2])
+        assert b.bits() == nxt and events[0].elapsed_time(events[2]) > 0 and events[3].elapsed_time(events[4]) >= 0
+    assert a.read_status() == 0 and b.read_status() == 0
