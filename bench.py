@@ -59,7 +59,7 @@ def _peaks():
     if os.path.exists(path):
         with open(path) as fh:
             return float(json.load(fh)["hbm_gbs"]), "measured (MEASURED_PEAKS.json hbm_gbs); of measured"
-    return 6650.0, "fallback (earlier measurement on this pool); of fallback"
+    return 6650.0, "fallback (an earlier B200 measurement); of fallback"
 
 
 # Sources whose text decides what each timed call moves through DRAM and how many instructions
