@@ -30,7 +30,9 @@ SOURCES = ["dq_layout.cu", "dq_tma.cu", "dq_norms.cu", "dq_bits.cu", "dq_quantiz
            "dq_round_team_average.cu", "dq_round_team_average_linf.cu", "dq_round_given_encode.cu",
            "dq_round_given_average.cu", "dq_round_norms.cu",
            "dq_round_odd_encode.cu", "dq_round_odd_encode_linf.cu",
-           "dq_round_odd_average.cu", "dq_round_odd_average_linf.cu"]
+           "dq_round_odd_average.cu", "dq_round_odd_average_linf.cu",
+           "dq_round_warp_tile.cu", "dq_round_warp_tile_linf.cu", "dq_round_team_tile.cu", "dq_round_team_tile_linf.cu",
+           "dq_round_odd_tile.cu", "dq_round_odd_tile_linf.cu", "dq_round_given_tile.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 

@@ -33,23 +33,47 @@ inline PhiloxKeys make_philox_keys(uint64_t seed)
 
 #ifdef __CUDACC__
 
-// One Philox4x32-10 block (Salmon et al., SC'11): ten rounds of two 32x32->64
-// multiplies and a three-way xor with the counter words and the round key.
-__device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                              const PhiloxKeys& K, uint32_t (&out)[4])
+// Philox4x32-10 blocks (Salmon et al., SC'11): ten rounds of two 32x32->64 multiplies and a three-way
+// xor with the counter words and the round key.  N blocks side by side, in place; FIRST: rounds already done.
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+template <int FIRST, int N>
+__device__ __forceinline__ void philox_rounds(uint32_t (&c)[N][4], const PhiloxKeys& K)
 {
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
-        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
-        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ K.k0[r];
-        const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ K.k1[r];
-        c1 = (uint32_t)p1;
-        c3 = (uint32_t)p0;
-        c0 = n0;
-        c2 = n2;
+    for (int r = FIRST; r < 10; ++r) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const uint64_t p0 = (uint64_t)kPhiloxM0 * c[n][0];
+            const uint64_t p1 = (uint64_t)kPhiloxM1 * c[n][2];
+            c[n][0] = (uint32_t)(p1 >> 32) ^ c[n][1] ^ K.k0[r];
+            c[n][2] = (uint32_t)(p0 >> 32) ^ c[n][3] ^ K.k1[r];
+            c[n][1] = (uint32_t)p1;
+            c[n][3] = (uint32_t)p0;
+        }
     }
-    out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
+}
+
+// The first two rounds of the block with the counter (octet, 0, worker, step): of their four multiplies two
+// depend on the octet alone and two on the worker alone.  What is left of them is an xor for two of the words.
+struct OctetRounds { uint32_t a, b, c; };
+__device__ __forceinline__ OctetRounds octet_rounds(const uint32_t octet, const uint32_t step, const PhiloxKeys& K)
+{
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * octet;
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ step ^ K.k1[0]);
+    return {(uint32_t)(p1 >> 32), (uint32_t)p0, (uint32_t)p1};
+}
+__device__ __forceinline__ uint4 worker_rounds(const uint32_t worker, const PhiloxKeys& K)        // (w: not used)
+{
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * worker;
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ K.k0[0]);
+    return make_uint4((uint32_t)p1 ^ K.k0[1], (uint32_t)(p0 >> 32) ^ K.k1[1], (uint32_t)p0, 0u);
+}
+__device__ __forceinline__ void third_round(uint32_t (&c)[4], const OctetRounds& o, const uint4& w)
+{
+    c[0] = o.a ^ w.x;
+    c[1] = o.c;
+    c[2] = o.b ^ w.y;
+    c[3] = w.z;
 }
 
 // The three places where the members of the l_p family differ.  P = DQ_NORM_L2: sum of
@@ -341,17 +365,14 @@ __device__ __forceinline__ void pack_eight(uint32_t (&words)[B], uint32_t& cur, 
     }
 }
 
-// Elements 8C .. 8C + 7 (one Philox block); with AVG, level * scale is added to their sums.
-template <int B, int C, bool AVG>
-__device__ __forceinline__ void encode_eight(const ulonglong2 lo, const ulonglong2 hi, const uint64_t inv2, const uint64_t scale2,
-                                             uint64_t (&acc2)[16], uint32_t (&words)[B], uint32_t& cur, const uint32_t q,
-                                             const uint32_t worker, const uint32_t step, const PhiloxKeys& keys)
+// Eight elements and the four words drawn for them: t, u as pack_eight takes them; with AVG, level * scale is added
+// to their sums.
+template <int B, bool AVG>
+__device__ __forceinline__ void octet_codes(const ulonglong2 lo, const ulonglong2 hi, const uint64_t inv2, const uint64_t scale2,
+                                            uint64_t* sums, const uint32_t (&w)[4], uint32_t (&t)[8], uint32_t (&u)[8])
 {
     constexpr uint32_t s = (1u << (B - 1)) - 1u;
-    uint32_t w[4];
-    philox4x32_10(q, 0u, worker, step, keys, w);
     const uint64_t x[4] = {lo.x, lo.y, hi.x, hi.y};
-    uint32_t t[8], u[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const uint64_t pos = mul_pair_rz(x[i], inv2);
@@ -366,10 +387,21 @@ __device__ __forceinline__ void encode_eight(const ulonglong2 lo, const ulonglon
             split_pair(u2, u[2 * i], u[2 * i + 1]);
             if constexpr (AVG) {
                 const uint64_t level = add_pair(u2, both(0xCB400000u + s));
-                acc2[4 * C + i] = fma_pair(level, scale2, acc2[4 * C + i]);
+                sums[i] = fma_pair(level, scale2, sums[i]);
             }
         }
     }
+}
+
+// Elements 8C .. 8C + 7 of a group (one Philox block).
+template <int B, int C, bool AVG>
+__device__ __forceinline__ void encode_eight(const ulonglong2 lo, const ulonglong2 hi, const uint64_t inv2, const uint64_t scale2,
+                                             uint64_t (&acc2)[16], uint32_t (&words)[B], uint32_t& cur, const uint32_t q,
+                                             const uint32_t worker, const uint32_t step, const PhiloxKeys& keys)
+{
+    uint32_t w[1][4] = {{q, 0u, worker, step}}, t[8], u[8];
+    philox_rounds<0>(w, keys);
+    octet_codes<B, AVG>(lo, hi, inv2, scale2, acc2 + 4 * C, w[0], t, u);
     pack_eight<B, C>(words, cur, t, u);
 }
 
@@ -484,6 +516,112 @@ __device__ __forceinline__ void store_words(uint32_t* dst, const uint32_t (&w)[B
         for (int i = 0; i < B / 4; ++i)
             DQ_STORE(reinterpret_cast<uint4*>(dst) + i, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]), base, extent,
                      status);
+    }
+}
+
+// ---- eight codes of a lane ------------------------------------------------------------------
+// The 8 * B bits of an octet, from bit 0 on; what stands above them in the last word is zero.
+template <int B>
+struct OctetWords {
+    static constexpr int n = (8 * B + 31) / 32;
+};
+template <int B, int E, int N>
+__device__ __forceinline__ void push_codes(uint32_t (&w)[N], uint32_t& cur, const uint32_t (&u)[8])
+{
+    if constexpr (E < 8) {
+        push_bits<E * B, B>(w, cur, u[E]);
+        push_codes<B, E + 1>(w, cur, u);
+    }
+}
+template <int B>
+__device__ __forceinline__ void pack_octet(uint32_t (&w)[OctetWords<B>::n], const uint32_t (&t)[8], const uint32_t (&u)[8])
+{
+    if constexpr (B == 1) {
+        w[0] = 0u;
+    } else if constexpr (B <= 4) {
+        // halves of q: the codes of elements 0..3 and of 4..7, 4 * B bits each
+        const uint32_t q = (((code_halves(t[3], t[7]) << B) + code_halves(t[2], t[6]) << B) + code_halves(t[1], t[5]) << B) +
+                           code_halves(t[0], t[4]);
+        if constexpr (B == 4) w[0] = q;
+        else if constexpr (B == 3) w[0] = (q & 0xFFFu) | ((q >> 4) & 0xFFF000u);
+        else w[0] = __byte_perm(q, 0u, 0x4420);
+    } else if constexpr (B == 8) {
+        w[0] = __byte_perm(__byte_perm(u[0], u[1], 0x0040), __byte_perm(u[2], u[3], 0x0040), 0x5410);
+        w[1] = __byte_perm(__byte_perm(u[4], u[5], 0x0040), __byte_perm(u[6], u[7], 0x0040), 0x5410);
+    } else if constexpr (B == 16) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = __byte_perm(u[2 * i], u[2 * i + 1], 0x5410);
+    } else {
+        uint32_t cur = 0;
+        push_codes<B, 0>(w, cur, u);
+        if constexpr (8 * B % 32 != 0) w[OctetWords<B>::n - 1] = cur >> (32 - 8 * B % 32);
+    }
+}
+// ... of eight codes that all equal s
+template <int B>
+__device__ __forceinline__ void zero_octet_words(uint32_t (&w)[OctetWords<B>::n])
+{
+    constexpr uint32_t s = (1u << (B - 1)) - 1u;
+    uint32_t cur = 0;
+    const uint32_t u[8] = {s, s, s, s, s, s, s, s};
+    push_codes<B, 0>(w, cur, u);
+    if constexpr (8 * B % 32 != 0) w[OctetWords<B>::n - 1] = cur >> (32 - 8 * B % 32);
+}
+// Octets of 1, 2, 4, 8 or 16 bytes leave straight from registers, neighbouring lanes side by side; the others are
+// brought into the order of memory in the warp's own part of a consumed stage and leave a word per lane.
+template <int B>
+struct OctetDirect {
+    static constexpr bool value = (B & (B - 1)) == 0;
+};
+template <int B>
+__device__ __forceinline__ void store_octet(unsigned char* dst, const uint32_t (&w)[OctetWords<B>::n], const void* base,
+                                            const int64_t extent, int32_t* status)
+{
+    if constexpr (B == 1) DQ_STORE(dst, (unsigned char)w[0], base, extent, status);
+    else if constexpr (B == 2) DQ_STORE(reinterpret_cast<uint16_t*>(dst), (uint16_t)w[0], base, extent, status);
+    else if constexpr (B == 4) DQ_STORE(reinterpret_cast<uint32_t*>(dst), w[0], base, extent, status);
+    else if constexpr (B == 8) DQ_STORE(reinterpret_cast<uint2*>(dst), make_uint2(w[0], w[1]), base, extent, status);
+    else DQ_STORE(reinterpret_cast<uint4*>(dst), make_uint4(w[0], w[1], w[2], w[3]), base, extent, status);
+}
+template <int B>
+__device__ __forceinline__ void stage_octet(unsigned char* dst, const uint32_t (&w)[OctetWords<B>::n])
+{
+    if constexpr (B % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < B / 4; ++i) reinterpret_cast<uint32_t*>(dst)[i] = w[i];
+    } else if constexpr (B % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < B / 2; ++i) reinterpret_cast<uint16_t*>(dst)[i] = (uint16_t)(w[i / 2] >> (16 * (i % 2)));
+    } else {
+#pragma unroll
+        for (int i = 0; i < B; ++i) dst[i] = (unsigned char)(w[i / 4] >> (8 * (i % 4)));
+    }
+}
+// Eight sums (or the update of the parameters there).
+__device__ __forceinline__ void store_sums(float* dst, const float (&r)[8], const bool update, const float neg_lr, const bool wide,
+                                           const void* base, const int64_t extent, int32_t* status)
+{
+    float y[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) y[e] = r[e];
+    if (wide) {
+        if (update) {
+            float p[8];
+            load_wide(dst, p);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[e] = fmaf(neg_lr, y[e], p[e]);
+        }
+        store_wide(dst, y, base, extent, status);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float4 z = make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
+            if (update) {
+                const float4 p = *reinterpret_cast<const float4*>(dst + 4 * i);
+                z = make_float4(fmaf(neg_lr, z.x, p.x), fmaf(neg_lr, z.y, p.y), fmaf(neg_lr, z.z, p.z), fmaf(neg_lr, z.w, p.w));
+            }
+            DQ_STORE(reinterpret_cast<float4*>(dst + 4 * i), z, base, extent, status);
+        }
     }
 }
 

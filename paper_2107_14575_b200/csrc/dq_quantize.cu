@@ -62,16 +62,32 @@ int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, boo
                   : dq_launch_round<kTeamBuckets, AVG, false>(a, map, L->n_seg, entries, st);
 }
 
-bool one_pass(const RoundArgs& a, bool given)
+// The round by CTAs.
+int launch_tiles(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, bool given, cudaStream_t st)
 {
+    const int64_t entries = dq_tile_positions(a, given);
+    if (given) return dq_launch_tile_round<kGivenNorms, false>(a, map, L->n_seg, entries, st);
+    if (a.div_shift < 0)
+        return a.linf ? dq_launch_tile_round<kOddBuckets, true>(a, map, L->n_seg, entries, st)
+                      : dq_launch_tile_round<kOddBuckets, false>(a, map, L->n_seg, entries, st);
+    if (a.gpb_shift <= 5)
+        return a.linf ? dq_launch_tile_round<kWarpBuckets, true>(a, map, L->n_seg, entries, st)
+                      : dq_launch_tile_round<kWarpBuckets, false>(a, map, L->n_seg, entries, st);
+    return a.linf ? dq_launch_tile_round<kTeamBuckets, true>(a, map, L->n_seg, entries, st)
+                  : dq_launch_tile_round<kTeamBuckets, false>(a, map, L->n_seg, entries, st);
+}
+
+RoundRoute route_of(const RoundArgs& a, bool given)
+{
+    const bool teams = !given && a.div_shift >= 0 && a.gpb_shift > 5;
     RouteQuery q = {};
     q.positions = dq_tile_positions(a, given);
     q.units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
-    if (!given && a.div_shift >= 0 && a.gpb_shift > 5) q.units >>= a.gpb_shift - 5;
+    if (teams) q.units >>= a.gpb_shift - 5;
     q.M = a.M;
     q.given = given ? 1 : 0;
     q.odd_buckets = !given && a.div_shift < 0 ? 32 / a.v.groups_per_bucket : 0;
-    return dq_one_pass(q);
+    return dq_round_route(q, !teams || a.gpb_shift == 6, teams);
 }
 
 }  // namespace
@@ -224,12 +240,14 @@ extern "C" int dq_quantize_average(const dq_layout_t* L, const float* dev_grads,
     if (!fill_args(a, map, L, dev_grads, worker_stride_elems, M, dev_norms, dev_b, seed, step, 0u, dev_packed,
                    packed_stride_words, dev_status))
         return DQ_ERR_CUDA;
-    if (!one_pass(a, true)) {
+    const RoundRoute route = route_of(a, true);
+    if (route == kTwoKernels) {
         rc = launch<false>(a, map, L, true, static_cast<cudaStream_t>(stream));
         if (rc != DQ_OK) return rc;
         return average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, dev_out, update, lr, dev_status, stream);
     }
     fill_average(a, dev_out, update, lr);
+    if (route == kCtaTiles) return launch_tiles(a, map, L, true, static_cast<cudaStream_t>(stream));
     return launch<true>(a, map, L, true, static_cast<cudaStream_t>(stream));
 }
 
@@ -274,7 +292,8 @@ extern "C" int dq_norms_quantize_average(const dq_layout_t* L, const float* dev_
                    packed_stride_words, dev_status))
         return DQ_ERR_CUDA;
     attach_rule(a, next_rule, M, ws);
-    if (!one_pass(a, given)) {
+    const RoundRoute route = route_of(a, given);
+    if (route == kTwoKernels) {
         // the next b is chosen at the end of the first kernel, which leaves its own for the second
         a.rule.this_b = reinterpret_cast<int32_t*>(ws + kThisBOffset);
         rc = launch<false>(a, map, L, given, static_cast<cudaStream_t>(stream));
@@ -282,5 +301,6 @@ extern "C" int dq_norms_quantize_average(const dq_layout_t* L, const float* dev_
         return average(L, dev_packed, packed_stride_words, dev_norms, M, a.rule.this_b, dev_out, update, lr, dev_status, stream);
     }
     fill_average(a, dev_out, update, lr);
+    if (route == kCtaTiles) return launch_tiles(a, map, L, given, static_cast<cudaStream_t>(stream));
     return launch<true>(a, map, L, given, static_cast<cudaStream_t>(stream));
 }

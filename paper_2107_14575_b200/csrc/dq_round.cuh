@@ -28,6 +28,8 @@
 #include "dq_rule.cuh"
 #include "dq_tma.cuh"
 
+#include <type_traits>
+
 enum RoundMode { kWarpBuckets = 0, kTeamBuckets = 1, kGivenNorms = 2, kOddBuckets = 3 };
 
 struct RoundArgs {
@@ -64,6 +66,9 @@ template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 template <int MODE, bool AVG, bool LINF>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
+// The round in which a CTA takes its tiles through the workers (buckets of 2048, of the teams').
+template <int MODE, bool LINF>
+int dq_launch_tile_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 
 // CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower); 102 without them
 // (codes of 2^24 elements, b = 6: 17.4 us with five CTAs, 18.1 with six of 80 registers, 18.7 with four; buckets of
@@ -108,6 +113,7 @@ struct SmemMap {
     static constexpr int slots = bars + kRoundWarps * kStages * 8;
     static constexpr int sums = slots + 2 * kRoundWarps * 8;
     static constexpr int table = sums + kRoundWarps * 8 + 16;
+    static constexpr int lost = 0;                 // (none)
 };
 
 __device__ __forceinline__ uint64_t* stage_bar(int warp, int st)
@@ -419,64 +425,62 @@ __device__ __noinline__ float rare_norm(const uint32_t row, const int valid, con
     return norm;
 }
 
-template <int B, int MODE, bool AVG, bool LINF>
-__device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
-{
-    using Join = typename JoinOp<LINF>::type;
-    const int32_t* tbl_s = reinterpret_cast<const int32_t*>(smem + SmemMap::table);
-    float2* slots = reinterpret_cast<float2*>(smem + SmemMap::slots);
-    auto tbl = [&](int i) -> int { return tbl_in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); };
-    constexpr int s = B > 0 ? (1 << (B > 0 ? B - 1 : 0)) - 1 : 0;
-    const float sf = (float)s;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n1 = a.v.n_seg + 1;
-    const int M = a.M;
-    const int nb = a.v.nb;
-    const int G = a.v.total_groups;
-    constexpr bool kClears = B != 0 && ClearsRow<MODE, LINF>::value;
-    constexpr bool ODD = MODE == kOddBuckets;
-    constexpr bool TILES = MODE == kWarpBuckets || ODD;               // tiles of whole buckets
-    const int gpb = ODD ? a.v.groups_per_bucket : 1 << a.gpb_shift;
-    // warps of the CTA that share a bucket, and this warp's place among them
-    const int T_shift = MODE == kTeamBuckets ? a.gpb_shift - 5 : 0;
-    const int T = 1 << T_shift;
-    const int sub = warp & (T - 1);
-    const int R = ODD ? 32 / gpb : (MODE == kWarpBuckets ? 32 >> a.gpb_shift : 1);       // buckets per warp tile
-    // of a regular tile: the lane's bucket and its group in there (kOddBuckets: the last lanes may have none, r >= R)
-    const int r = ODD ? lane / gpb : lane >> a.gpb_shift, l = lane - (ODD ? r * gpb : r << a.gpb_shift);
+constexpr uint32_t kNoTile = 0x7fffffffu;
 
+// Where the tiles of a worker lie.  table: byte offset of the tensor table in shared memory.
+template <int MODE>
+struct TileMap {
+    static constexpr bool ODD = MODE == kOddBuckets;
+    static constexpr bool TILES = MODE == kWarpBuckets || ODD;        // tiles of whole buckets
+    const RoundArgs& a;
+    const bool in_smem;
+    const int32_t* const tbl_s;
+    const int lane, n1, gpb;
+    const int T_shift, sub;          // log2 of the warps that share a bucket, and this warp's place among them
+    const int R;                     // buckets per warp tile
+    const int r, l;                  // of a regular tile: the lane's bucket and its group in there (kOddBuckets: the last lanes may have none, r >= R)
+    // the tensor looked at last: first bucket, first group, elements, end (in buckets), full buckets
+    int c_b0, c_g0, c_n, c_end, c_full;
+
+    __device__ __forceinline__ TileMap(const RoundArgs& args, const bool tbl_in_smem, const int table, const int warp_of_team)
+        : a(args), in_smem(tbl_in_smem), tbl_s(reinterpret_cast<const int32_t*>(smem + table)), lane(threadIdx.x & 31),
+          n1(args.v.n_seg + 1), gpb(ODD ? args.v.groups_per_bucket : 1 << args.gpb_shift),
+          T_shift(MODE == kTeamBuckets ? args.gpb_shift - 5 : 0), sub(warp_of_team),
+          R(ODD ? 32 / gpb : (MODE == kWarpBuckets ? 32 >> args.gpb_shift : 1)),
+          r(ODD ? lane / gpb : lane >> args.gpb_shift), l(lane - (ODD ? r * gpb : r << args.gpb_shift))
+    {
+        c_b0 = 0;
+        c_g0 = 0;
+        c_n = a.v.seg0_elems;
+        c_end = a.v.n_seg == 1 ? 0x7fffffff : 0;
+        c_full = full_buckets(c_n);
+    }
+    __device__ __forceinline__ int full_buckets(const int n) const
+    {
+        return ODD ? (int)div_gpb(a, (uint32_t)n >> 5) : n >> (a.gpb_shift + 5);
+    }
+    __device__ __forceinline__ int tbl(const int i) const { return in_smem ? tbl_s[i] : __ldg(a.v.seg_group0 + i); }
     // Tile positions of one worker; a team takes bucket `pos`, each of its warps 1024 elements of it.
-    const int positions = TILES ? (nb + R - 1) / R : (MODE == kTeamBuckets ? nb : (G + 31) / 32);
-    // The list of work: positions (AVG: every position goes through all workers), or the worker-major
-    // list of all tiles.  Each unit -- a warp, or a team -- takes every hop-th entry, `each` of them, the
-    // first `extra` units one more: dense and sparse stretches of a gradient then fall to all units alike
-    // (text shape, 97 % of the embedding's rows zero: 154 -> 145 us against contiguous ranges).
-    const uint32_t unit = (blockIdx.x * kRoundWarps + warp) >> T_shift;
-    const int n_pos = (int)(a.each + (unit < a.extra ? 1u : 0u));
-    const int64_t begin = unit;
-    const int hop = (int)((gridDim.x * kRoundWarps) >> T_shift);
-    const int m_first = (AVG || M == 1) ? 0 : (int)(begin / positions);
-    int pos = (int)(begin - (int64_t)m_first * positions);
-    const int items = AVG ? n_pos * M : n_pos;
-
-    // ---- where tiles lie.  Codes alone: a position is worked out once, when the producer moves there, and the
-    //      consumer finds the answer in a queue.  AVG: twice, the second time from the cached tensor as a rule.
+    __device__ __forceinline__ int positions() const
+    {
+        return TILES ? (a.v.nb + R - 1) / R : (MODE == kTeamBuckets ? a.v.nb : (a.v.total_groups + 31) / 32);
+    }
     // last tensor whose first bucket (column 1) or group (column 0) is <= x
-    auto find_seg = [&](int column, int x) -> int {
+    __device__ __forceinline__ int find_seg(const int column, const int x) const
+    {
         return last_not_above_by_warp(x, a.v.n_seg, [&](int i) { return tbl(column * n1 + i); });
-    };
+    }
     // the same for an x of each lane's own, from tensor `from` on
-    auto walk_seg = [&](int column, int from, int x) -> int {
+    __device__ __forceinline__ int walk_seg(const int column, int from, const int x) const
+    {
         while (x >= tbl(column * n1 + from + 1)) ++from;
         return from;
-    };
-    constexpr uint32_t kNoTile = 0x7fffffffu;
+    }
     // kWarpBuckets, kTeamBuckets: first group of the warp's tile at position p, bit 31 set if every lane owns
     // a full row of it; kNoTile if a team's bucket ends before this warp's share.  kGivenNorms: the tensor of
-    // the tile's first group.  c_*: the tensor looked at last.
-    int c_b0 = 0, c_g0 = 0, c_n = a.v.seg0_elems, c_end = a.v.n_seg == 1 ? 0x7fffffff : 0;
-    int c_full = ODD ? (int)div_gpb(a, (uint32_t)c_n >> 5) : c_n >> (a.gpb_shift + 5);        // its full buckets
-    auto describe = [&](int p) -> uint32_t {
+    // the tile's first group. 
+    __device__ __forceinline__ uint32_t describe(const int p)
+    {
         const int k0 = MODE == kGivenNorms ? p * 32 : p * R;
         if constexpr (MODE == kGivenNorms) {
             return a.v.n_seg == 1 ? 0u : (uint32_t)find_seg(0, k0);
@@ -487,7 +491,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 c_end = tbl(n1 + i + 1);
                 c_g0 = tbl(i);
                 c_n = tbl(2 * n1 + i);
-                c_full = ODD ? (int)div_gpb(a, (uint32_t)c_n >> 5) : c_n >> (a.gpb_shift + 5);
+                c_full = full_buckets(c_n);
             }
             const int local = k0 - c_b0;
             if constexpr (TILES) {
@@ -499,8 +503,10 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 return (uint32_t)(c_g0 + share * 32) | (left >= 1024 ? 0x80000000u : 0u);
             }
         }
-    };
-    auto locate = [&](int p, uint32_t desc) -> TilePos {
+    }
+    __device__ __forceinline__ TilePos locate(const int p, const uint32_t desc) const
+    {
+        const int nb = a.v.nb, G = a.v.total_groups;
         TilePos t;
         t.row = lane; t.valid = 32; t.span = 32; t.bucket = p; t.writes = false;
         t.row0 = MODE == kGivenNorms ? p * 32 : (int)(desc & 0x7fffffffu);
@@ -576,7 +582,42 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             t.span = (G - t.row0) < 32 ? (G - t.row0) : 32;
         }
         return t;
-    };
+    }
+};
+
+template <int B, int MODE, bool AVG, bool LINF>
+__device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
+{
+    using Join = typename JoinOp<LINF>::type;
+    float2* slots = reinterpret_cast<float2*>(smem + SmemMap::slots);
+    constexpr int s = B > 0 ? (1 << (B > 0 ? B - 1 : 0)) - 1 : 0;
+    const float sf = (float)s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int M = a.M;
+    const int nb = a.v.nb;
+    const int G = a.v.total_groups;
+    constexpr bool kClears = B != 0 && ClearsRow<MODE, LINF>::value;
+    constexpr bool ODD = MODE == kOddBuckets;
+    const int T_shift = MODE == kTeamBuckets ? a.gpb_shift - 5 : 0;    // warps of the CTA that share a bucket
+    TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp & ((1 << T_shift) - 1));
+    const int gpb = tiles.gpb, R = tiles.R, r = tiles.r;
+    const int positions = tiles.positions();
+    // The list of work: positions (AVG: every position goes through all workers), or the worker-major
+    // list of all tiles.  Each unit -- a warp, or a team -- takes every hop-th entry, `each` of them, the
+    // first `extra` units one more: dense and sparse stretches of a gradient then fall to all units alike
+    // (text shape, 97 % of the embedding's rows zero: 154 -> 145 us against contiguous ranges).
+    const uint32_t unit = (blockIdx.x * kRoundWarps + warp) >> T_shift;
+    const int n_pos = (int)(a.each + (unit < a.extra ? 1u : 0u));
+    const int64_t begin = unit;
+    const int hop = (int)((gridDim.x * kRoundWarps) >> T_shift);
+    const int m_first = (AVG || M == 1) ? 0 : (int)(begin / positions);
+    int pos = (int)(begin - (int64_t)m_first * positions);
+    const int items = AVG ? n_pos * M : n_pos;
+
+    // ---- where tiles lie.  Codes alone: a position is worked out once, when the producer moves there, and the
+    //      consumer finds the answer in a queue.  AVG: twice, the second time from the cached tensor as a rule.
+    auto describe = [&](int p) -> uint32_t { return tiles.describe(p); };
+    auto locate = [&](int p, uint32_t desc) -> TilePos { return tiles.locate(p, desc); };
 
     // ---- producer side: tiles are fetched in the order they are consumed, two ahead
     int p_pos = pos, p_m = 0, p_left = items;
@@ -839,18 +880,20 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
 }
 
 // Barriers, tensor table (true if it is in shared memory), and the wait for the kernel before.
+template <class Map>
 __device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& map)
 {
     // (nothing up to the wait touches memory that an earlier kernel may still be writing)
     if (threadIdx.x == 0) {
         tma::prefetch_tensor_map(&map);
-        for (int i = 0; i < kRoundWarps * kStages; ++i) tma::mbar_init(stage_bar(0, i), 1);
+        for (int i = 0; i < kRoundWarps * kStages; ++i) tma::mbar_init(reinterpret_cast<uint64_t*>(smem + Map::bars) + i, 1);
+        if constexpr (Map::lost != 0) *reinterpret_cast<uint32_t*>(smem + Map::lost) = 0u;
         tma::fence_barrier_init();
     }
     grid_dependency_wait();
     const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
     if (tbl_in_smem) {
-        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + SmemMap::table);
+        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + Map::table);
         for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
     }
     __syncthreads();
@@ -865,7 +908,7 @@ template <int MODE, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, kNormCtasPerSm)
 norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
-    const bool tbl_in_smem = set_up(a, map);
+    const bool tbl_in_smem = set_up<SmemMap>(a, map);
     if (tma::smem_addr(smem) & 1023u) {          // the swizzled tiles need a 1024-byte aligned base
         if (threadIdx.x == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
         return;
@@ -880,7 +923,7 @@ template <int MODE, bool AVG, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
 round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
-    const bool tbl_in_smem = set_up(a, map);
+    const bool tbl_in_smem = set_up<SmemMap>(a, map);
     const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
     uint32_t trouble = 0;
     if (tma::smem_addr(smem) & 1023u) trouble = DQ_STAT_INTERNAL;          // the swizzled tiles need a 1024-byte aligned base
@@ -908,21 +951,401 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 }
 
 
-template <int MODE>
-int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, RoundArgs a, const CUtensorMap& map, int n_seg,
-                      int64_t entries, cudaStream_t st)
+// ---- rounds with few tiles: the CTA takes a tile through the workers together --------------------------
+// A chunk is a tile position of up to four workers, a warp's stage each (with buckets of 2048, whose two tiles are two
+// warps', the bucket of up to two workers).  First every warp takes the norm of its own tile, a lane a row (group), and
+// leaves the scales of every row in shared memory.  Behind a barrier the CTA goes through the workers of the chunk, a
+// thread an octet (eight elements, one Philox block) of the tile, two workers side by side, and keeps the octet's sums
+// in registers from a position's first worker to its last.
+// What bounds it: with a position per SM the chain of a chunk (20 tiles, M = 32, cycles: wait 310, norm 770, codes of four
+// workers 1400 one after the other, 1000 side by side, copies 400, two barriers 280), with many the instructions: some 650
+// per tile and worker at b = 4 against 530 in a warp's own way, 37 more per octet for the scales, the notes and the
+// addresses.  Where the line between the two lies, and what both measured: dq_route.h.
+// Five CTAs per SM (96 registers): with six (80) 600k elements M = 8 b = 5 10.9 us, 10.5 so, with four 10.1; 4.2M M = 8 b = 4
+// 40.6, 40.0, 42.0; buckets of 2048, 1.5M M = 16 35.8 with five, 41.4 with four.
+constexpr int kTileCtasPerSm = 5;
+constexpr int kSets = 2;                            // chunks in shared memory: the one at hand and one on its way
+struct TileSmem {
+    static constexpr int bars = kSets * kRoundWarps * kTileBytes;
+    static constexpr int notes = bars + kSets * kRoundWarps * 8;              // uint4[4]: worker_rounds, and whether all norms of the tile are plain
+    static constexpr int scales = notes + kRoundWarps * 16;                   // float4[4][32]: scale of the codes, scale of the sums, twice each
+    static constexpr int valid = scales + kRoundWarps * 512;                  // bytes[32], of an irregular tile
+    static constexpr int slots = valid + 32;                                  // the teams' exchange slots
+    static constexpr int sums = slots + 2 * kRoundWarps * 8;
+    static constexpr int lost = sums + kRoundWarps * 8 + 8;
+    static constexpr int table = lost + 8;
+};
+
+// A row's scales, as they stand there: that of its codes is 0 and that of its sums finite.
+__device__ __forceinline__ bool adds_zero(const ulonglong2 sc)
 {
-    size_t smem_need = (size_t)SmemMap::table;
+    return (uint32_t)sc.x == 0u && isfinite(__uint_as_float((uint32_t)sc.y));
+}
+
+// The warp's copies: its tile of every position and worker of the CTA, a chunk at a time.
+template <int MODE, int T>
+struct TileFetch {
+    static constexpr bool TEAM = MODE == kTeamBuckets;
+    static constexpr int kWorkers = kRoundWarps / T;       // of a chunk
+    TileMap<MODE>& tiles;
+    const CUtensorMap* map;
+    int pos, m, left;                // next position and worker, positions not fetched yet
+    uint32_t first;                  // where that position's tile lies
+    uint32_t parities, flying;       // a bit per set: parity of its next copy, a copy on its way
+
+    __device__ __forceinline__ TileFetch(TileMap<MODE>& where, const CUtensorMap* tensor_map, const int n_pos)
+        : tiles(where), map(tensor_map), pos((int)blockIdx.x), m((int)(threadIdx.x >> 5) / T), left(n_pos),
+          first(n_pos > 0 ? where.describe((int)blockIdx.x) : kNoTile), parities(0), flying(0)
+    {
+    }
+    __device__ __forceinline__ static uint64_t* bar(const int set)
+    {
+        return reinterpret_cast<uint64_t*>(smem + TileSmem::bars) + set * kRoundWarps + (threadIdx.x >> 5);
+    }
+    __device__ __forceinline__ void next(const int set)
+    {
+        if (left <= 0) return;
+        const RoundArgs& a = tiles.a;
+        if (m < a.M && (!TEAM || first != kNoTile)) {
+            flying |= 1u << set;
+            // (L2 policy: see round_tiles)
+            if ((threadIdx.x & 31) == 0)
+                tma::fetch_tile(tma::smem_addr(smem) + (set * kRoundWarps + (threadIdx.x >> 5)) * kTileBytes, map, tma::smem_addr(bar(set)),
+                                kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu), a.map_has_worker_dim ? m : 0,
+                                tma::policy_evict_normal());
+        }
+        m += kWorkers;
+        const int mine = (int)(threadIdx.x >> 5) / T;
+        if (m - mine >= a.M) {
+            m = mine;
+            pos += (int)gridDim.x;
+            if (--left > 0) first = tiles.describe(pos);
+        }
+    }
+    // (every lane polls the barrier itself; the verdict is made warp-uniform)
+    __device__ __forceinline__ bool wait(const int set)
+    {
+        const uint32_t par = (parities >> set) & 1u;
+        const bool landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar(set), par)) ||
+                            __all_sync(0xffffffffu, tma::mbar_wait(bar(set), par, tiles.a.wait));
+        if (landed) { parities ^= 1u << set; flying &= ~(1u << set); }
+        return landed;
+    }
+    // Every copy the warp has issued and not seen land, one whose wait ran out included, gets the full limit before
+    // the CTA's shared memory is released.
+    __device__ __forceinline__ void drain() const
+    {
+        for (int i = 0; i < kSets; ++i)
+            if ((flying >> i) & 1u) (void)tma::mbar_wait(bar(i), (parities >> i) & 1u, tiles.a.wait);
+    }
+};
+
+template <int B, int MODE, bool LINF, int T>
+__device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& tiles, TileFetch<MODE, T>& copies, const int n_pos,
+                                            double& square_sum)
+{
+    using Join = typename JoinOp<LINF>::type;
+    constexpr bool ODD = MODE == kOddBuckets, TEAM = MODE == kTeamBuckets;
+    constexpr int T_shift = T - 1;                  // (T is 1 or 2)
+    constexpr int kWorkers = kRoundWarps / T;       // of a chunk
+    constexpr int s = (1 << (B - 1)) - 1;
+    const float sf = (float)s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int M = a.M, nb = a.v.nb;
+    const int sub = warp & (T - 1), mine = warp / T;
+    float2* slots = reinterpret_cast<float2*>(smem + TileSmem::slots);
+    uint4* notes = reinterpret_cast<uint4*>(smem + TileSmem::notes);
+    float4* scales = reinterpret_cast<float4*>(smem + TileSmem::scales);
+    unsigned char* valids = smem + TileSmem::valid;
+    volatile uint32_t* lost_word = reinterpret_cast<volatile uint32_t*>(smem + TileSmem::lost);
+    const int hop = (int)gridDim.x;
+
+    const float to_unit = (B <= 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
+    bool bad = false;
+    bool timed_out = a.wait.lose_first != 0u && n_pos > 0;               // (test hook: the first wait counts as lost)
+    uint32_t exchanges = 0;
+
+    // the thread's octet of a tile: row, place in the row, and where its two 16-byte pieces stand in a stage
+    const int orow = threadIdx.x >> 2, oq = threadIdx.x & 3;
+    const uint32_t opiece = (uint32_t)(orow * 128) + ((uint32_t)((2 * oq) ^ (orow & 7)) << 4);
+    const int64_t extent = (int64_t)M * a.packed_stride * 4;
+
+    uint32_t it = 0;
+    int pos = (int)blockIdx.x;
+    for (int ip = 0; ip < n_pos && !timed_out; ++ip, pos += hop) {
+        // ---- the position: this lane's row of it, and the thread's octets
+        TilePos t;
+        int row0, span;                              // of the whole position
+        {
+            const uint32_t desc = tiles.describe(pos);
+            if constexpr (TEAM) {
+                const int local = pos - tiles.c_b0;
+                row0 = tiles.c_g0 + (local << (T_shift + 5));
+                const int rest = tiles.c_n - (local << (T_shift + 10));
+                const int len = rest < T * 1024 ? rest : T * 1024;
+                span = (len + 31) >> 5;
+                const int v = len - sub * 1024 - lane * 32;
+                t.row = lane; t.bucket = pos; t.writes = sub == 0 && lane == 0; t.len = len;
+                t.valid = v < 0 ? 0 : (v > 32 ? 32 : v);
+                t.row0 = desc == kNoTile ? -1 : row0 + 32 * sub;
+                t.regular = (desc >> 31) != 0;
+                t.span = 0;
+            } else {
+                t = tiles.locate(pos, desc);
+                row0 = t.row0;
+                span = t.span;
+                if (!t.regular && t.valid > 0) valids[t.row] = (unsigned char)t.valid;       // (all warps write the same)
+            }
+        }
+        const bool has_tile = !TEAM || t.row0 >= 0;
+        const uint32_t own = (uint32_t)(t.row * 128 + ((t.row & 7) << 4));
+        float* norm_ptr = a.norms + (int64_t)mine * nb + t.bucket;
+        float given = 0.0f;
+        if constexpr (MODE == kGivenNorms) {
+            if (mine < M && t.valid > 0) given = load_norm_early(norm_ptr);
+        }
+        unsigned char* words = reinterpret_cast<unsigned char*>(a.packed + (int64_t)row0 * B) +
+                               (OctetDirect<B>::value ? (int)threadIdx.x * B : (warp * 8 * B + lane) * 4);
+        OctetRounds oct[T];
+        uint64_t sums[T][4];
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+            oct[k] = octet_rounds((uint32_t)(row0 + 32 * k) * 4u + threadIdx.x, a.step, a.keys);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sums[k][q] = 0ull;
+        }
+
+#pragma unroll 1
+        for (int m0 = 0; m0 < M; m0 += kWorkers, ++it) {
+            const int set = (int)(it & 1u);
+            // ---- the norm of the warp's own tile
+            if (m0 + mine < M) {
+                const uint32_t row = (uint32_t)((set * kRoundWarps + warp) * kTileBytes) + own;
+                bool landed = true;
+                if (has_tile) {
+                    landed = copies.wait(set);
+                    if (!landed && lane == 0) *lost_word = 1u;
+                }
+                float nrm = 0.0f, inv = 0.0f;
+                bool plain = false;
+                if constexpr (MODE == kGivenNorms || ODD) {
+                    if (!t.regular && landed) (void)end_row<LINF>(row, t.valid);
+                }
+                if constexpr (MODE == kGivenNorms) {
+                    nrm = given;
+                    inv = inv_scale_normal(sf, nrm);
+                    plain = !__any_sync(0xffffffffu, t.valid > 0 && !norm_is_plain(nrm));
+                    if (!plain) {
+                        inv = inv_scale(sf, nrm);
+                        if (landed) clear_nonfinite_row<true>(row, t.valid, nrm);
+                    }
+                    if (t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
+                    if (m0 + mine + kWorkers < M && t.valid > 0) given = load_norm_early(norm_ptr + (int64_t)kWorkers * nb);
+                } else {
+                    bool lost = false;
+                    float v;
+                    if constexpr (ODD) {
+                        v = odd_bucket_sums<LINF>(row - own, t.row, t.len, tiles.gpb, tiles.R, tiles.r);
+                    } else {
+                        v = LINF ? row_max(row) : row_sum_squares(row);
+                        if (!t.regular) {
+                            const float end = has_tile && landed ? end_row<LINF>(row, t.valid) : 0.0f;
+                            if (t.valid != 32) v = end;
+                        }
+                        v = join_team<MODE>(join_lanes<MODE>(v, tiles.gpb, Join{}), slots, T_shift, exchanges, landed, lost, Join{});
+                    }
+                    if (landed && !lost) {
+                        nrm = LINF ? v : sqrt_normal(v);
+                        inv = inv_scale_normal(sf, nrm);
+                        plain = !__any_sync(0xffffffffu, has_say<MODE>(t) && (LINF ? !norm_is_plain(v) : !l2_sum_in_range(v)));
+                        if (!plain) {
+                            if constexpr (LINF) {
+                                clear_nonfinite_row<true>(row, t.valid, nrm);
+                            } else if constexpr (ODD) {
+                                nrm = rare_norm_odd<true>(row - own, t.row, t.len, tiles.gpb, tiles.R, tiles.r, v, nrm, row, t.valid);
+                            } else {
+                                nrm = rare_norm<MODE, true>(row, t.valid, tiles.gpb, slots, T_shift, exchanges, v, nrm);
+                                exchanges += 2;
+                            }
+                            inv = inv_scale(sf, nrm);
+                            bad |= t.writes && !isfinite(nrm);
+                        }
+                        if (t.writes) {
+                            DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
+                            square_sum = fma((double)nrm, (double)nrm, square_sum);
+                        }
+                    }
+                }
+                norm_ptr += (int64_t)kWorkers * nb;
+                if (t.valid > 0) scales[warp * 32 + t.row] = make_float4(inv, inv, nrm * to_unit, nrm * to_unit);
+                uint4 note = worker_rounds((uint32_t)(m0 + mine) + a.worker0, a.keys);
+                note.w = plain ? 1u : 0u;
+                if (lane == 0) notes[warp] = note;
+            }
+            __syncthreads();
+            if (*lost_word != 0u) { timed_out = true; break; }
+
+            // ---- the codes of the chunk, a thread an octet of each tile
+            const int slots_used = (M - m0 < kWorkers ? M - m0 : kWorkers) * T;
+            auto emit = [&](const int slot, const int k, const uint32_t (&w)[OctetWords<B>::n], unsigned char* to) {
+                if constexpr (OctetDirect<B>::value) {
+                    if (32 * k + orow < span) store_octet<B>(to, w, a.packed, extent, a.status);
+                } else {
+                    // through the warp's eight rows of the stage, which it has read
+                    unsigned char* staged = smem + (set * kRoundWarps + slot) * kTileBytes + warp * 1024;
+                    __syncwarp();
+                    stage_octet<B>(staged + lane * B, w);
+                    __syncwarp();
+                    const int rows = span - 32 * k - warp * 8;
+                    const int n = (rows > 8 ? 8 : rows) * B;
+#pragma unroll
+                    for (int q = 0; q < (8 * B + 31) / 32; ++q)
+                        if (lane + 32 * q < n)
+                            DQ_STORE(reinterpret_cast<uint32_t*>(to) + 32 * q, reinterpret_cast<const uint32_t*>(staged)[lane + 32 * q],
+                                     a.packed, extent, a.status);
+                }
+            };
+            // N tiles side by side: two workers', or both tiles of a worker's bucket
+            auto encode = [&](const int j, const int k0, const auto& note, auto count) {
+                constexpr int N = decltype(count)::value;
+                uint32_t draws[N][4];
+                ulonglong2 lo[N], hi[N], sc[N];
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                    const unsigned char* stage = smem + (set * kRoundWarps + j + n) * kTileBytes;
+                    sc[n] = *reinterpret_cast<const ulonglong2*>(scales + (j + n) * 32 + orow);
+                    lo[n] = *reinterpret_cast<const ulonglong2*>(stage + opiece);
+                    hi[n] = *reinterpret_cast<const ulonglong2*>(stage + (opiece ^ 16u));
+                    third_round(draws[n], oct[T == 1 ? 0 : k0 + n], note[n]);
+                }
+                philox_rounds<2>(draws, a.keys);
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                    uint32_t ft[8], fu[8], w[OctetWords<B>::n];
+                    const int k = T == 1 ? 0 : k0 + n;
+                    octet_codes<B, true>(lo[n], hi[n], sc[n].x, sc[n].y, sums[k], draws[n], ft, fu);
+                    pack_octet<B>(w, ft, fu);
+                    emit(j + n, k, w, words + (T == 1 ? n * (a.packed_stride * 4) : k * (128 * B)));
+                }
+            };
+            if constexpr (B == 1) {
+                const uint32_t w[1] = {0u};
+                for (int j = 0; j < slots_used; j += T, words += a.packed_stride * 4)
+                    for (int k = 0; k < T; ++k)
+                        if (32 * k < span) emit(j + k, k, w, words + k * (128 * B));
+            } else {
+                int j = 0;
+#pragma unroll 1
+                while (j < slots_used) {
+                    const uint4 note[2] = {notes[j], notes[j + 1 < kRoundWarps ? j + 1 : j]};
+                    if (j + 1 < slots_used && (T == 1 || span > 32) && (note[0].w & note[1].w) != 0u) {
+                        encode(j, 0, note, std::integral_constant<int, 2>{});
+                        j += 2;
+                        words += (2 / T) * (a.packed_stride * 4);
+                        continue;
+                    }
+#pragma unroll
+                    for (int k = 0; k < T; ++k) {
+                        if (T > 1 && 32 * k >= span) break;
+                        const ulonglong2 sc = *reinterpret_cast<const ulonglong2*>(scales + (j + k) * 32 + orow);
+                        if (note[k].w == 0u && __all_sync(0xffffffffu, adds_zero(sc) || 32 * k + orow >= span)) {
+                            // zero buckets (sparse gradients are full of them): every code is s, whatever the draw, and adds 0
+                            uint32_t w[OctetWords<B>::n];
+                            zero_octet_words<B>(w);
+                            emit(j + k, k, w, words + k * (128 * B));
+                        } else {
+                            const uint4 one[1] = {note[k]};
+                            encode(j + k, k, one, std::integral_constant<int, 1>{});
+                        }
+                    }
+                    j += T;
+                    words += a.packed_stride * 4;
+                }
+            }
+            if (m0 + kWorkers >= M && !(B == 1 && a.update)) {
+                // ---- the position's sums
+#pragma unroll
+                for (int k = 0; k < T; ++k) {
+                    const int at = 32 * k + orow;
+                    if (at < span) {
+                        float r[8];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) unpack_pair(sums[k][q], r[2 * q], r[2 * q + 1]);
+                        const int valid = (TEAM ? t.len - at * 32 : (t.regular ? 32 : (int)valids[orow])) - 8 * oq;
+                        if (valid < 8) {
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                if (q >= valid) r[q] = 0.0f;
+                        }
+                        store_sums(a.out + ((int64_t)row0 + at) * 32 + 8 * oq, r, a.update != 0, a.neg_lr, a.wide_out != 0, a.out,
+                                   (int64_t)a.v.total_groups * 128, a.status);
+                    }
+                }
+            }
+            // the CTA's accesses to the set come before the copies that refill it (they go through different proxies)
+            tma::fence_proxy_async();
+            __syncthreads();
+            copies.next(set);
+        }
+    }
+    if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
+    if (timed_out) {
+        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
+        copies.drain();
+    }
+}
+
+template <int MODE, bool LINF, int T>
+__global__ void __launch_bounds__(kRoundThreads, kTileCtasPerSm)
+tile_round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+{
+    const bool tbl_in_smem = set_up<TileSmem>(a, map);
+    const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
+    double* part = reinterpret_cast<double*>(smem + TileSmem::sums);
+    uint32_t trouble = (tma::smem_addr(smem) & 1023u) ? DQ_STAT_INTERNAL : 0u;        // the swizzled tiles need a 1024-byte aligned base
+    // The first copies are on their way before b is here and its code is fetched.
+    // Every CTA takes every hop-th position, `each` of them, the first `extra` CTAs one more.
+    const int n_pos = trouble ? 0 : (int)(a.each + (blockIdx.x < a.extra ? 1u : 0u));
+    TileMap<MODE> tiles(a, tbl_in_smem, TileSmem::table, (int)(threadIdx.x >> 5) & (T - 1));
+    TileFetch<MODE, T> copies(tiles, &map, n_pos);
+    copies.next(0);
+    copies.next(1);
+    if (!trouble) {
+        if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
+        else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
+    }
+    if (trouble) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
+        copies.drain();
+        // nothing is written but the next b, which follows from the norms that are there
+        if (a.with_rule) rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, part, a.dev_b, b, a.status);
+        return;
+    }
+    double square_sum = 0.0;
+    switch (b) {
+#define DQ_CASE(BB) case BB: tile_rounds<BB, MODE, LINF, T>(a, tiles, copies, n_pos, square_sum); break;
+        DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
+        DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
+#undef DQ_CASE
+        default: break;
+    }
+    if (a.with_rule) rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, part, a.dev_b, b, a.status);
+}
+
+// units: of work per CTA: warps, teams, or the CTA itself
+template <class Map>
+int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, int units, RoundArgs a, const CUtensorMap& map,
+                      int n_seg, int64_t entries, cudaStream_t st)
+{
+    size_t smem_need = (size_t)Map::table;
     if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
     // (the limit of the largest table, whatever this one's size: with each call's own, another thread's call for a
     // smaller layout can narrow it again before this launch, which then fails)
-    constexpr int kLargest = SmemMap::table + 3 * (kMaxSmemSegs + 1) * 4;
+    constexpr int kLargest = Map::table + 3 * (kMaxSmemSegs + 1) * 4;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLargest) != cudaSuccess) {
         (void)cudaGetLastError();
         return DQ_ERR_CUDA;
     }
-    // units of work per CTA: warps, or teams
-    const int units = MODE == kTeamBuckets ? kRoundWarps >> (a.gpb_shift - 5) : kRoundWarps;
     int64_t blocks = (int64_t)dq_sm_count() * ctas_per_sm;
     if (blocks * units > entries) blocks = (entries + units - 1) / units;
     a.each = (uint32_t)(entries / (blocks * units));
@@ -931,18 +1354,30 @@ int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, R
     return cudaGetLastError() == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
+template <int MODE>
+int units_per_cta(const RoundArgs& a)
+{
+    return MODE == kTeamBuckets ? kRoundWarps >> (a.gpb_shift - 5) : kRoundWarps;
+}
+
 }  // namespace
 
 template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<MODE>(norms_kernel<MODE, LINF>, kNormCtasPerSm, a, map, n_seg, entries, st);
+    return launch_persistent<SmemMap>(norms_kernel<MODE, LINF>, kNormCtasPerSm, units_per_cta<MODE>(a), a, map, n_seg, entries, st);
 }
 template <int MODE, bool AVG, bool LINF>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<MODE>(round_kernel<MODE, AVG, LINF>, RoundShape<AVG>::ctas_per_sm, a, map,
-                                                               n_seg, entries, st);
+    return launch_persistent<SmemMap>(round_kernel<MODE, AVG, LINF>, RoundShape<AVG>::ctas_per_sm, units_per_cta<MODE>(a), a, map,
+                                      n_seg, entries, st);
+}
+template <int MODE, bool LINF>
+int dq_launch_tile_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+{
+    constexpr int T = MODE == kTeamBuckets ? 2 : 1;
+    return launch_persistent<TileSmem>(tile_round_kernel<MODE, LINF, T>, kTileCtasPerSm, 1, a, map, n_seg, entries, st);
 }
 
 #endif  // DQ_ROUND_KERNELS
