@@ -61,7 +61,7 @@ struct RoundArgs {
 };
 
 // Launch of one of the kernels (each in a translation unit of its own): norms alone, or codes with or
-// without the average.  `entries`: length of the list of work (see round_tiles).
+// without the average.  `entries`: length of the list of work (see WarpFetch).
 template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 template <int MODE, bool AVG, bool LINF>
@@ -585,8 +585,80 @@ struct TileMap {
     }
 };
 
+// A warp's list of work and its copies: tiles are fetched in the order they are consumed, two ahead.  The list: positions
+// (AVG: every position goes through all workers), or the worker-major list of all tiles.  Each unit -- a warp, or a
+// team -- takes every hop-th entry, `each` of them, the first `extra` units one more: dense and sparse stretches of a
+// gradient then fall to all units alike (text shape, 97 % of the embedding's rows zero: 154 -> 145 us against contiguous
+// ranges).
+template <int MODE, bool AVG>
+struct WarpFetch {
+    static constexpr bool TEAM = MODE == kTeamBuckets;
+    TileMap<MODE>& tiles;
+    const CUtensorMap* map;
+    const int n_pos, hop, positions;
+    const int m_first, pos0;         // the first entry: worker (codes alone) and position
+    int pos, m, left;                // AVG: position and worker of the next copy; copies to come
+    int worker;                      // !AVG: worker of the next copy, as a coordinate
+    uint32_t first;                  // what describe() says of its position
+    // A team's warp has no tile of some buckets, so it keeps the parity of each stage's next copy and which
+    // copies are on their way, a bit each; the others find the parity by counting.
+    uint32_t parities, flying;
+    // !AVG: descriptions of the positions fetched and not done with, the consumer's and at most two more
+    uint32_t queue0, queue1, queue2;
+    int queued;
+
+    __device__ __forceinline__ static uint32_t unit_of(const RoundArgs& a)
+    {
+        return (blockIdx.x * kRoundWarps + (threadIdx.x >> 5)) >> (TEAM ? a.gpb_shift - 5 : 0);
+    }
+    __device__ __forceinline__ WarpFetch(TileMap<MODE>& where, const CUtensorMap* tensor_map)
+        : tiles(where), map(tensor_map), n_pos((int)(where.a.each + (unit_of(where.a) < where.a.extra ? 1u : 0u))),
+          hop((int)((gridDim.x * kRoundWarps) >> where.T_shift)), positions(where.positions()),
+          m_first((AVG || where.a.M == 1) ? 0 : (int)((int64_t)unit_of(where.a) / positions)),
+          pos0((int)((int64_t)unit_of(where.a) - (int64_t)m_first * positions)), pos(pos0), m(0),
+          left(AVG ? n_pos * where.a.M : n_pos), worker(m_first * (where.a.map_has_worker_dim ? 1 : 0)), first(kNoTile),
+          parities(0), flying(0), queue0(0), queue1(0), queue2(0), queued(0)
+    {
+        if (left > 0) first = tiles.describe(pos);
+    }
+    __device__ __forceinline__ int items() const { return AVG ? n_pos * tiles.a.M : n_pos; }
+    __device__ __forceinline__ void next(const int st)
+    {
+        if (left <= 0) return;
+        --left;
+        const RoundArgs& a = tiles.a;
+        if (!AVG) {
+            if (queued == 0) queue0 = first;
+            else if (queued == 1) queue1 = first;
+            else queue2 = first;
+            ++queued;
+        }
+        if (TEAM && first != kNoTile) flying |= 1u << st;
+        // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
+        // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
+        // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
+        // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
+        // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).
+        if ((threadIdx.x & 31) == 0 && (!TEAM || first != kNoTile))
+            tma::fetch_tile(tma::smem_addr(stage_ptr(threadIdx.x >> 5, st)), map, tma::smem_addr(stage_bar(threadIdx.x >> 5, st)),
+                            kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu),
+                            AVG ? (a.map_has_worker_dim ? m : 0) : worker,
+                            (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal());
+        if (AVG) {
+            if (++m == a.M) {
+                m = 0; pos += hop;
+                if (left > 0) first = tiles.describe(pos);
+            }
+        } else {
+            pos += hop;
+            while (pos >= positions) { pos -= positions; worker += a.map_has_worker_dim ? 1 : 0; }
+            if (left > 0) first = tiles.describe(pos);
+        }
+    }
+};
+
 template <int B, int MODE, bool AVG, bool LINF>
-__device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMap* map, const bool tbl_in_smem, double& square_sum)
+__device__ __forceinline__ void round_tiles(const RoundArgs& a, TileMap<MODE>& tiles, WarpFetch<MODE, AVG>& copies, double& square_sum)
 {
     using Join = typename JoinOp<LINF>::type;
     float2* slots = reinterpret_cast<float2*>(smem + SmemMap::slots);
@@ -598,76 +670,11 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     const int G = a.v.total_groups;
     constexpr bool kClears = B != 0 && ClearsRow<MODE, LINF>::value;
     constexpr bool ODD = MODE == kOddBuckets;
-    const int T_shift = MODE == kTeamBuckets ? a.gpb_shift - 5 : 0;    // warps of the CTA that share a bucket
-    TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp & ((1 << T_shift) - 1));
+    const int T_shift = tiles.T_shift;
     const int gpb = tiles.gpb, R = tiles.R, r = tiles.r;
-    const int positions = tiles.positions();
-    // The list of work: positions (AVG: every position goes through all workers), or the worker-major
-    // list of all tiles.  Each unit -- a warp, or a team -- takes every hop-th entry, `each` of them, the
-    // first `extra` units one more: dense and sparse stretches of a gradient then fall to all units alike
-    // (text shape, 97 % of the embedding's rows zero: 154 -> 145 us against contiguous ranges).
-    const uint32_t unit = (blockIdx.x * kRoundWarps + warp) >> T_shift;
-    const int n_pos = (int)(a.each + (unit < a.extra ? 1u : 0u));
-    const int64_t begin = unit;
-    const int hop = (int)((gridDim.x * kRoundWarps) >> T_shift);
-    const int m_first = (AVG || M == 1) ? 0 : (int)(begin / positions);
-    int pos = (int)(begin - (int64_t)m_first * positions);
-    const int items = AVG ? n_pos * M : n_pos;
-
-    // ---- where tiles lie.  Codes alone: a position is worked out once, when the producer moves there, and the
-    //      consumer finds the answer in a queue.  AVG: twice, the second time from the cached tensor as a rule.
-    auto describe = [&](int p) -> uint32_t { return tiles.describe(p); };
-    auto locate = [&](int p, uint32_t desc) -> TilePos { return tiles.locate(p, desc); };
-
-    // ---- producer side: tiles are fetched in the order they are consumed, two ahead
-    int p_pos = pos, p_m = 0, p_left = items;
-    uint32_t p_first = items > 0 ? describe(p_pos) : kNoTile;
-    // !AVG: descriptions of the positions fetched and not done with, the consumer's and at most two more
-    uint32_t queue0 = 0, queue1 = 0, queue2 = 0;
-    int queued = 0;
-    // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
-    // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
-    // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
-    // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
-    // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).
-    const uint64_t policy = (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal();
-    const int p_step = a.map_has_worker_dim ? 1 : 0;
-    int p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu), p_worker = m_first * p_step;         // coordinates of the next copy
-    const uint32_t stage0 = tma::smem_addr(smem) + warp * (kStages * kTileBytes);
+    const int n_pos = copies.n_pos, hop = copies.hop, items = copies.items();
+    int pos = copies.pos0;
     const uint32_t bar0 = tma::smem_addr(stage_bar(warp, 0));
-    // A team's warp has no tile of some buckets, so it keeps the parity of each stage's next copy and which
-    // copies are on their way, a bit each; the others find the parity by counting.
-    uint32_t parities = 0, flying = 0;
-    auto move_producer = [&]() {
-        p_first = describe(p_pos);
-        p_row = MODE == kGivenNorms ? p_pos * 32 : (int)(p_first & 0x7fffffffu);
-    };
-    auto fetch = [&](int st) {
-        if (p_left <= 0) return;
-        --p_left;
-        if (!AVG) {
-            if (queued == 0) queue0 = p_first;
-            else if (queued == 1) queue1 = p_first;
-            else queue2 = p_first;
-            ++queued;
-        }
-        if (MODE == kTeamBuckets && p_first != kNoTile) flying |= 1u << st;
-        if (lane == 0 && (MODE != kTeamBuckets || p_first != kNoTile))
-            tma::fetch_tile(stage0 + st * kTileBytes, map, bar0 + st * 8, kTileBytes, p_row, p_worker, policy);
-        if (AVG) {
-            p_worker += p_step;
-            if (++p_m == M) {
-                p_m = 0; p_worker = 0; p_pos += hop;
-                if (p_left > 0) move_producer();
-            }
-        } else {
-            p_pos += hop;
-            while (p_pos >= positions) { p_pos -= positions; p_worker += p_step; }
-            if (p_left > 0) move_producer();
-        }
-    };
-#pragma unroll
-    for (int st = 0; st < kStages; ++st) fetch(st);
 
     const float to_unit = (B <= 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
     uint32_t it = 0;                              // items consumed; item i travels through stage i & 1
@@ -675,19 +682,21 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
     bool timed_out = false, bad = false;
     // (test hook: the warp's first wait counts as lost, and the warp goes straight to what follows a time-out)
     const bool skip_all = a.wait.lose_first != 0u && items > 0;
-    int m = m_first;
+    int m = copies.m_first;
     // Every lane polls the barrier itself; the verdict is made warp-uniform so that the warp-level
     // synchronisations are always reached by all lanes or by none.
     auto wait_for = [&](int stage) -> bool {
-        const uint32_t par = MODE == kTeamBuckets ? (parities >> stage) & 1u : (it >> 1) & 1u;
+        const uint32_t par = MODE == kTeamBuckets ? (copies.parities >> stage) & 1u : (it >> 1) & 1u;
         const bool landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar0 + stage * 8, par)) ||
                             __all_sync(0xffffffffu, tma::mbar_wait(stage_bar(warp, stage), par, a.wait));
-        if (MODE == kTeamBuckets && landed) { parities ^= 1u << stage; flying &= ~(1u << stage); }
+        if (MODE == kTeamBuckets && landed) { copies.parities ^= 1u << stage; copies.flying &= ~(1u << stage); }
         return landed;
     };
 
     for (int ip = 0; ip < n_pos && !skip_all; ++ip) {
-        const TilePos t = locate(pos, AVG ? describe(pos) : queue0);
+        // (where the tile lies -- codes alone: worked out once, when the copies move there; AVG: twice, the second time from
+        // the tensor looked at last as a rule)
+        const TilePos t = tiles.locate(pos, AVG ? tiles.describe(pos) : copies.queue0);
         const bool has_tile = MODE != kTeamBuckets || t.row0 >= 0;
         // byte offset of the lane's row inside a stage, swizzle phase folded in: chunk c sits at own ^ (c << 4)
         const uint32_t own = (uint32_t)(t.row * 128 + ((t.row & 7) << 4));
@@ -773,11 +782,11 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 settle(v, row, norm_ptr);
             }
             if (!has_tile) {
-                fetch(st);
+                copies.next(st);
             } else if constexpr (B == 0) {       // norms alone: the row has been read (see the refill below)
                 tma::fence_proxy_async();
                 __syncwarp();
-                fetch(st);
+                copies.next(st);
             } else {
                 // ---- codes of the row against that norm, and the lane's share of the average
                 uint32_t words[B];
@@ -804,7 +813,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                 if constexpr (StoresDirectly<B>::value) {
                     tma::fence_proxy_async();
                     __syncwarp();
-                    fetch(st);
+                    copies.next(st);
                     if (t.valid > 0) store_words<B>(tile_words + t.row * B, words, a.wide_words != 0, a.packed, extent, a.status);
                 } else {
                     __syncwarp();                // the warp has read all of its rows
@@ -836,7 +845,7 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
                     }
                     tma::fence_proxy_async();
                     __syncwarp();
-                    fetch(st);
+                    copies.next(st);
                 }
                 __syncwarp();
             }
@@ -860,8 +869,8 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
             pos += hop;
         } else {
             pos += hop;
-            while (pos >= positions) { pos -= positions; ++m; }
-            queue0 = queue1; queue1 = queue2; --queued;
+            while (pos >= copies.positions) { pos -= copies.positions; ++m; }
+            copies.queue0 = copies.queue1; copies.queue1 = copies.queue2; --copies.queued;
         }
     }
     if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
@@ -871,9 +880,9 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, const CUtensorMa
         // full limit before the CTA's shared memory is released
         if constexpr (MODE == kTeamBuckets) {
             for (int i = 0; i < kStages; ++i)
-                if ((flying >> i) & 1u) (void)tma::mbar_wait(stage_bar(warp, i), (parities >> i) & 1u, a.wait);
+                if ((copies.flying >> i) & 1u) (void)tma::mbar_wait(stage_bar(warp, i), (copies.parities >> i) & 1u, a.wait);
         } else {
-            for (uint32_t i = it; i < (uint32_t)(items - p_left); ++i)
+            for (uint32_t i = it; i < (uint32_t)(items - copies.left); ++i)
                 (void)tma::mbar_wait(stage_bar(warp, (int)(i & 1u)), (i >> 1) & 1u, a.wait);
         }
     }
@@ -900,6 +909,22 @@ __device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& ma
     return tbl_in_smem;
 }
 
+template <int MODE>
+__device__ __forceinline__ int warp_of_team(const RoundArgs& a)
+{
+    return MODE == kTeamBuckets ? (int)(threadIdx.x >> 5) & ((1 << (a.gpb_shift - 5)) - 1) : 0;
+}
+// The first two copies of a warp that will not look at them: the CTA's shared memory outlives them.
+template <int MODE, bool AVG>
+__device__ __forceinline__ void drain_first(const WarpFetch<MODE, AVG>& copies)
+{
+    const int issued = copies.items() - copies.left;
+#pragma unroll
+    for (int st = 0; st < kStages; ++st)
+        if (MODE == kTeamBuckets ? ((copies.flying >> st) & 1u) != 0u : st < issued)
+            (void)tma::mbar_wait(stage_bar(threadIdx.x >> 5, st), 0u, copies.tiles.a.wait);
+}
+
 // Norms alone.  Bound by HBM, 4 bytes read per element.  Against a CTA-wide ring of 16 KB tiles with a barrier
 // per tile (three CTAs of 128 threads per SM): ResNet-18 shape M = 8 72 -> 57 us (6.3 TB/s), VGG-16 shape M = 16,
 // bucket 2048, 191 -> 150, text shape with its zero rows 407 -> 103, pieces of whole tensors 84 -> 60.
@@ -914,7 +939,11 @@ norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         return;
     }
     double square_sum = 0.0;
-    round_tiles<0, MODE, false, LINF>(a, &map, tbl_in_smem, square_sum);
+    TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp_of_team<MODE>(a));
+    WarpFetch<MODE, false> copies(tiles, &map);
+    copies.next(0);
+    copies.next(1);
+    round_tiles<0, MODE, false, LINF>(a, tiles, copies, square_sum);
     if (a.with_rule)
         rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + SmemMap::sums), a.dev_b, 0, a.status);
 }
@@ -927,24 +956,49 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
     const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
     uint32_t trouble = 0;
     if (tma::smem_addr(smem) & 1023u) trouble = DQ_STAT_INTERNAL;          // the swizzled tiles need a 1024-byte aligned base
-    else if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
-    else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
-    if (trouble) {
+    auto look_at_b = [&] {
+        if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
+        else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
+    };
+    auto give_up = [&] {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
         // nothing is written but the next b, which follows from the norms that are there
         if (a.with_rule)
             rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, reinterpret_cast<double*>(smem + SmemMap::sums),
                                        a.dev_b, b, a.status);
-        return;
-    }
-
+    };
     double square_sum = 0.0;
-    switch (b) {
-#define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG, LINF>(a, &map, tbl_in_smem, square_sum); break;
-        DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
-        DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
+    if constexpr (AVG && (MODE == kWarpBuckets || MODE == kTeamBuckets)) {
+        if (!trouble) look_at_b();
+        if (trouble) return give_up();
+        switch (b) {
+#define DQ_CASE(BB) case BB: {                                                                                               TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp_of_team<MODE>(a));                                  WarpFetch<MODE, AVG> copies(tiles, &map);                                                                    copies.next(0);                                                                                              copies.next(1);                                                                                              round_tiles<BB, MODE, AVG, LINF>(a, tiles, copies, square_sum);                                              break;                                                                                                   }
+            DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
+            DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
 #undef DQ_CASE
-        default: break;
+            default: break;
+        }
+    } else {
+        // The first copies are on their way before b is here and its code is fetched; a call that cannot run waits for
+        // them.  Codes, b = 6, one worker (us): 16.8M elements 17.1 -> 15.6, 1M 3.7 -> 3.4.  (With the sums of the two modes
+        // above there are no registers for what that keeps alive: ResNet-18 shape M = 8 78.0 us, 83.8 so.)
+        if (trouble) return give_up();
+        TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp_of_team<MODE>(a));
+        WarpFetch<MODE, AVG> copies(tiles, &map);
+        copies.next(0);
+        copies.next(1);
+        look_at_b();
+        if (trouble) {
+            drain_first(copies);
+            return give_up();
+        }
+        switch (b) {
+#define DQ_CASE(BB) case BB: round_tiles<BB, MODE, AVG, LINF>(a, tiles, copies, square_sum); break;
+            DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
+            DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
+#undef DQ_CASE
+            default: break;
+        }
     }
     if (a.with_rule)
         rule_at_end<kRoundThreads>(a.rule, square_sum, nullptr, 0, reinterpret_cast<double*>(smem + SmemMap::sums), a.dev_b, b, a.status);
@@ -1008,7 +1062,7 @@ struct TileFetch {
         const RoundArgs& a = tiles.a;
         if (m < a.M && (!TEAM || first != kNoTile)) {
             flying |= 1u << set;
-            // (L2 policy: see round_tiles)
+            // (L2 policy: see WarpFetch)
             if ((threadIdx.x & 31) == 0)
                 tma::fetch_tile(tma::smem_addr(smem) + (set * kRoundWarps + (threadIdx.x >> 5)) * kTileBytes, map, tma::smem_addr(bar(set)),
                                 kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu), a.map_has_worker_dim ? m : 0,
