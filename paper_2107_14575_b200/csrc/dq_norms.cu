@@ -43,6 +43,8 @@ bool dq_fill_round(RoundArgs& a, CUtensorMap& map, const dq_layout_t* L, const L
 {
     a = RoundArgs{};
     a.v = v;
+    a.grads = dev_grads;
+    a.grad_stride = M > 1 ? worker_stride_elems : 0;
     a.status = dev_status;
     a.M = M;
     a.linf = L->norm == DQ_NORM_LINF ? 1 : 0;

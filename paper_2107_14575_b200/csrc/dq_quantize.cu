@@ -63,18 +63,18 @@ int launch(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, boo
 }
 
 // The round by CTAs.
-int launch_tiles(const RoundArgs& a, const CUtensorMap& map, const dq_layout_t* L, bool given, cudaStream_t st)
+int launch_tiles(const RoundArgs& a, const dq_layout_t* L, bool given, cudaStream_t st)
 {
     const int64_t entries = dq_tile_positions(a, given);
-    if (given) return dq_launch_tile_round<kGivenNorms, false>(a, map, L->n_seg, entries, st);
+    if (given) return dq_launch_tile_round<kGivenNorms, false>(a, L->n_seg, entries, st);
     if (a.div_shift < 0)
-        return a.linf ? dq_launch_tile_round<kOddBuckets, true>(a, map, L->n_seg, entries, st)
-                      : dq_launch_tile_round<kOddBuckets, false>(a, map, L->n_seg, entries, st);
+        return a.linf ? dq_launch_tile_round<kOddBuckets, true>(a, L->n_seg, entries, st)
+                      : dq_launch_tile_round<kOddBuckets, false>(a, L->n_seg, entries, st);
     if (a.gpb_shift <= 5)
-        return a.linf ? dq_launch_tile_round<kWarpBuckets, true>(a, map, L->n_seg, entries, st)
-                      : dq_launch_tile_round<kWarpBuckets, false>(a, map, L->n_seg, entries, st);
-    return a.linf ? dq_launch_tile_round<kTeamBuckets, true>(a, map, L->n_seg, entries, st)
-                  : dq_launch_tile_round<kTeamBuckets, false>(a, map, L->n_seg, entries, st);
+        return a.linf ? dq_launch_tile_round<kWarpBuckets, true>(a, L->n_seg, entries, st)
+                      : dq_launch_tile_round<kWarpBuckets, false>(a, L->n_seg, entries, st);
+    return a.linf ? dq_launch_tile_round<kTeamBuckets, true>(a, L->n_seg, entries, st)
+                  : dq_launch_tile_round<kTeamBuckets, false>(a, L->n_seg, entries, st);
 }
 
 RoundRoute route_of(const RoundArgs& a, bool given)
@@ -247,7 +247,7 @@ extern "C" int dq_quantize_average(const dq_layout_t* L, const float* dev_grads,
         return average(L, dev_packed, packed_stride_words, dev_norms, M, dev_b, dev_out, update, lr, dev_status, stream);
     }
     fill_average(a, dev_out, update, lr);
-    if (route == kCtaTiles) return launch_tiles(a, map, L, true, static_cast<cudaStream_t>(stream));
+    if (route == kCtaTiles) return launch_tiles(a, L, true, static_cast<cudaStream_t>(stream));
     return launch<true>(a, map, L, true, static_cast<cudaStream_t>(stream));
 }
 
@@ -301,6 +301,6 @@ extern "C" int dq_norms_quantize_average(const dq_layout_t* L, const float* dev_
         return average(L, dev_packed, packed_stride_words, dev_norms, M, a.rule.this_b, dev_out, update, lr, dev_status, stream);
     }
     fill_average(a, dev_out, update, lr);
-    if (route == kCtaTiles) return launch_tiles(a, map, L, given, static_cast<cudaStream_t>(stream));
+    if (route == kCtaTiles) return launch_tiles(a, L, given, static_cast<cudaStream_t>(stream));
     return launch<true>(a, map, L, given, static_cast<cudaStream_t>(stream));
 }

@@ -34,6 +34,8 @@ enum RoundMode { kWarpBuckets = 0, kTeamBuckets = 1, kGivenNorms = 2, kOddBucket
 
 struct RoundArgs {
     LayoutView v;
+    const float* grads;
+    int64_t grad_stride;          // elements from a worker's gradient to the next
     float* norms;                 // written, or read (kGivenNorms)
     int32_t* dev_b;               // b of this call; with the rule attached, the next b when the kernel ends
     uint32_t* packed;
@@ -68,7 +70,7 @@ template <int MODE, bool AVG, bool LINF>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
 // The round in which a CTA takes its tiles through the workers (buckets of 2048, of the teams').
 template <int MODE, bool LINF>
-int dq_launch_tile_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st);
+int dq_launch_tile_round(const RoundArgs& a, int n_seg, int64_t entries, cudaStream_t st);
 
 // CTAs per SM, i.e. registers per thread: 128 with the 32 sums (96 spill and run 4-6 % slower); 102 without them
 // (codes of 2^24 elements, b = 6: 17.4 us with five CTAs, 18.1 with six of 80 registers, 18.7 with four; buckets of
@@ -113,7 +115,6 @@ struct SmemMap {
     static constexpr int slots = bars + kRoundWarps * kStages * 8;
     static constexpr int sums = slots + 2 * kRoundWarps * 8;
     static constexpr int table = sums + kRoundWarps * 8 + 16;
-    static constexpr int lost = 0;                 // (none)
 };
 
 __device__ __forceinline__ uint64_t* stage_bar(int warp, int st)
@@ -888,25 +889,28 @@ __device__ __forceinline__ void round_tiles(const RoundArgs& a, TileMap<MODE>& t
     }
 }
 
-// Barriers, tensor table (true if it is in shared memory), and the wait for the kernel before.
-template <class Map>
+// The tensor table (true if it is in shared memory); behind it the CTA is in step.
+__device__ __forceinline__ bool copy_table(const RoundArgs& a, const int table)
+{
+    const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
+    if (tbl_in_smem) {
+        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + table);
+        for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
+    }
+    __syncthreads();
+    return tbl_in_smem;
+}
+// Barriers, tensor table, and the wait for the kernel before.
 __device__ __forceinline__ bool set_up(const RoundArgs& a, const CUtensorMap& map)
 {
     // (nothing up to the wait touches memory that an earlier kernel may still be writing)
     if (threadIdx.x == 0) {
         tma::prefetch_tensor_map(&map);
-        for (int i = 0; i < kRoundWarps * kStages; ++i) tma::mbar_init(reinterpret_cast<uint64_t*>(smem + Map::bars) + i, 1);
-        if constexpr (Map::lost != 0) *reinterpret_cast<uint32_t*>(smem + Map::lost) = 0u;
+        for (int i = 0; i < kRoundWarps * kStages; ++i) tma::mbar_init(stage_bar(0, i), 1);
         tma::fence_barrier_init();
     }
     grid_dependency_wait();
-    const bool tbl_in_smem = a.v.n_seg > 1 && a.v.n_seg <= kMaxSmemSegs;
-    if (tbl_in_smem) {
-        int32_t* tbl_s = reinterpret_cast<int32_t*>(smem + Map::table);
-        for (int i = threadIdx.x; i < 3 * (a.v.n_seg + 1); i += kRoundThreads) tbl_s[i] = __ldg(a.v.seg_group0 + i);
-    }
-    __syncthreads();
-    return tbl_in_smem;
+    return copy_table(a, SmemMap::table);
 }
 
 template <int MODE>
@@ -933,7 +937,7 @@ template <int MODE, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, kNormCtasPerSm)
 norms_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
-    const bool tbl_in_smem = set_up<SmemMap>(a, map);
+    const bool tbl_in_smem = set_up(a, map);
     if (tma::smem_addr(smem) & 1023u) {          // the swizzled tiles need a 1024-byte aligned base
         if (threadIdx.x == 0) atomicOr(a.status, DQ_STAT_INTERNAL);
         return;
@@ -952,7 +956,7 @@ template <int MODE, bool AVG, bool LINF>
 __global__ void __launch_bounds__(kRoundThreads, RoundShape<AVG>::ctas_per_sm)
 round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
 {
-    const bool tbl_in_smem = set_up<SmemMap>(a, map);
+    const bool tbl_in_smem = set_up(a, map);
     const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
     uint32_t trouble = 0;
     if (tma::smem_addr(smem) & 1023u) trouble = DQ_STAT_INTERNAL;          // the swizzled tiles need a 1024-byte aligned base
@@ -1020,14 +1024,12 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 constexpr int kTileCtasPerSm = 5;
 constexpr int kSets = 2;                            // chunks in shared memory: the one at hand and one on its way
 struct TileSmem {
-    static constexpr int bars = kSets * kRoundWarps * kTileBytes;
-    static constexpr int notes = bars + kSets * kRoundWarps * 8;              // uint4[4]: worker_rounds, and whether all norms of the tile are plain
+    static constexpr int notes = kSets * kRoundWarps * kTileBytes;            // uint4[4]: worker_rounds, and whether all norms of the tile are plain
     static constexpr int scales = notes + kRoundWarps * 16;                   // float4[4][32]: scale of the codes, scale of the sums, twice each
     static constexpr int valid = scales + kRoundWarps * 512;                  // bytes[32], of an irregular tile
     static constexpr int slots = valid + 32;                                  // the teams' exchange slots
     static constexpr int sums = slots + 2 * kRoundWarps * 8;
-    static constexpr int lost = sums + kRoundWarps * 8 + 8;
-    static constexpr int table = lost + 8;
+    static constexpr int table = sums + kRoundWarps * 8 + 16;
 };
 
 // A row's scales, as they stand there: that of its codes is 0 and that of its sums finite.
@@ -1036,62 +1038,59 @@ __device__ __forceinline__ bool adds_zero(const ulonglong2 sc)
     return (uint32_t)sc.x == 0u && isfinite(__uint_as_float((uint32_t)sc.y));
 }
 
-// The warp's copies: its tile of every position and worker of the CTA, a chunk at a time.
+// The warp's copies: its tile of every position and worker of the CTA, a chunk at a time, 16 bytes per lane and instruction
+// straight to where a swizzled tensor copy would put them.  With one position per SM a chunk's chain is what counts, and
+// a tensor copy costs that chain some 250 cycles to issue, 250 to find landed and 100 for the fence before its stage is refilled.
 template <int MODE, int T>
 struct TileFetch {
     static constexpr bool TEAM = MODE == kTeamBuckets;
     static constexpr int kWorkers = kRoundWarps / T;       // of a chunk
     TileMap<MODE>& tiles;
-    const CUtensorMap* map;
     int pos, m, left;                // next position and worker, positions not fetched yet
     uint32_t first;                  // where that position's tile lies
-    uint32_t parities, flying;       // a bit per set: parity of its next copy, a copy on its way
 
-    __device__ __forceinline__ TileFetch(TileMap<MODE>& where, const CUtensorMap* tensor_map, const int n_pos)
-        : tiles(where), map(tensor_map), pos((int)blockIdx.x), m((int)(threadIdx.x >> 5) / T), left(n_pos),
-          first(n_pos > 0 ? where.describe((int)blockIdx.x) : kNoTile), parities(0), flying(0)
+    __device__ __forceinline__ TileFetch(TileMap<MODE>& where, const int n_pos)
+        : tiles(where), pos((int)blockIdx.x), m((int)(threadIdx.x >> 5) / T), left(n_pos),
+          first(n_pos > 0 ? where.describe((int)blockIdx.x) : kNoTile)
     {
-    }
-    __device__ __forceinline__ static uint64_t* bar(const int set)
-    {
-        return reinterpret_cast<uint64_t*>(smem + TileSmem::bars) + set * kRoundWarps + (threadIdx.x >> 5);
     }
     __device__ __forceinline__ void next(const int set)
     {
-        if (left <= 0) return;
-        const RoundArgs& a = tiles.a;
-        if (m < a.M && (!TEAM || first != kNoTile)) {
-            flying |= 1u << set;
-            // (L2 policy: see WarpFetch)
-            if ((threadIdx.x & 31) == 0)
-                tma::fetch_tile(tma::smem_addr(smem) + (set * kRoundWarps + (threadIdx.x >> 5)) * kTileBytes, map, tma::smem_addr(bar(set)),
-                                kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu), a.map_has_worker_dim ? m : 0,
-                                tma::policy_evict_normal());
+        if (left > 0) {
+            const RoundArgs& a = tiles.a;
+            if (m < a.M && (!TEAM || first != kNoTile)) {
+                const int lane = threadIdx.x & 31, at = lane >> 3;                      // row of the first four, piece lane & 7
+                const int row0 = MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu);
+                const float* src = a.grads + (int64_t)m * a.grad_stride + (int64_t)(row0 + at) * 32 + (lane & 7) * 4;
+                const uint32_t dst = tma::smem_addr(smem) + (set * kRoundWarps + (threadIdx.x >> 5)) * kTileBytes + at * 128;
+                const uint32_t even = (uint32_t)((lane & 7) ^ at) << 4, odd = even ^ 64u;       // swizzled piece
+                const int rows = a.v.total_groups - row0 - at;                          // (rows behind the last arrive as zeros)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int bytes = 4 * i < rows ? 16 : 0;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + i * 512 + (i % 2 ? odd : even)),
+                                 "l"(bytes ? src + i * 128 : a.grads), "r"(bytes)
+                                 : "memory");
+                }
+            }
+            m += kWorkers;
+            const int mine = (int)(threadIdx.x >> 5) / T;
+            if (m - mine >= a.M) {
+                m = mine;
+                pos += (int)gridDim.x;
+                if (--left > 0) first = tiles.describe(pos);
+            }
         }
-        m += kWorkers;
-        const int mine = (int)(threadIdx.x >> 5) / T;
-        if (m - mine >= a.M) {
-            m = mine;
-            pos += (int)gridDim.x;
-            if (--left > 0) first = tiles.describe(pos);
-        }
+        // (an empty group where nothing is left to copy: the wait counts groups)
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // (every lane polls the barrier itself; the verdict is made warp-uniform)
-    __device__ __forceinline__ bool wait(const int set)
+    // The chunk before the last one requested is there.
+    __device__ __forceinline__ void wait() const
     {
-        const uint32_t par = (parities >> set) & 1u;
-        const bool landed = __all_sync(0xffffffffu, tma::mbar_try_wait(bar(set), par)) ||
-                            __all_sync(0xffffffffu, tma::mbar_wait(bar(set), par, tiles.a.wait));
-        if (landed) { parities ^= 1u << set; flying &= ~(1u << set); }
-        return landed;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
     }
-    // Every copy the warp has issued and not seen land, one whose wait ran out included, gets the full limit before
-    // the CTA's shared memory is released.
-    __device__ __forceinline__ void drain() const
-    {
-        for (int i = 0; i < kSets; ++i)
-            if ((flying >> i) & 1u) (void)tma::mbar_wait(bar(i), (parities >> i) & 1u, tiles.a.wait);
-    }
+    __device__ __forceinline__ void drain() const { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 };
 
 template <int B, int MODE, bool LINF, int T>
@@ -1111,12 +1110,10 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
     uint4* notes = reinterpret_cast<uint4*>(smem + TileSmem::notes);
     float4* scales = reinterpret_cast<float4*>(smem + TileSmem::scales);
     unsigned char* valids = smem + TileSmem::valid;
-    volatile uint32_t* lost_word = reinterpret_cast<volatile uint32_t*>(smem + TileSmem::lost);
     const int hop = (int)gridDim.x;
 
     const float to_unit = (B <= 1) ? 0.0f : __fdiv_rn(1.0f, (float)s * (float)M);          // 1 / (s * M)
     bool bad = false;
-    bool timed_out = a.wait.lose_first != 0u && n_pos > 0;               // (test hook: the first wait counts as lost)
     uint32_t exchanges = 0;
 
     // the thread's octet of a tile: row, place in the row, and where its two 16-byte pieces stand in a stage
@@ -1126,7 +1123,7 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
 
     uint32_t it = 0;
     int pos = (int)blockIdx.x;
-    for (int ip = 0; ip < n_pos && !timed_out; ++ip, pos += hop) {
+    for (int ip = 0; ip < n_pos; ++ip, pos += hop) {
         // ---- the position: this lane's row of it, and the thread's octets
         TilePos t;
         int row0, span;                              // of the whole position
@@ -1173,17 +1170,13 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
         for (int m0 = 0; m0 < M; m0 += kWorkers, ++it) {
             const int set = (int)(it & 1u);
             // ---- the norm of the warp's own tile
+            copies.wait();
             if (m0 + mine < M) {
                 const uint32_t row = (uint32_t)((set * kRoundWarps + warp) * kTileBytes) + own;
-                bool landed = true;
-                if (has_tile) {
-                    landed = copies.wait(set);
-                    if (!landed && lane == 0) *lost_word = 1u;
-                }
                 float nrm = 0.0f, inv = 0.0f;
                 bool plain = false;
                 if constexpr (MODE == kGivenNorms || ODD) {
-                    if (!t.regular && landed) (void)end_row<LINF>(row, t.valid);
+                    if (!t.regular) (void)end_row<LINF>(row, t.valid);
                 }
                 if constexpr (MODE == kGivenNorms) {
                     nrm = given;
@@ -1191,43 +1184,41 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
                     plain = !__any_sync(0xffffffffu, t.valid > 0 && !norm_is_plain(nrm));
                     if (!plain) {
                         inv = inv_scale(sf, nrm);
-                        if (landed) clear_nonfinite_row<true>(row, t.valid, nrm);
+                        clear_nonfinite_row<true>(row, t.valid, nrm);
                     }
                     if (t.writes) square_sum = fma((double)nrm, (double)nrm, square_sum);
                     if (m0 + mine + kWorkers < M && t.valid > 0) given = load_norm_early(norm_ptr + (int64_t)kWorkers * nb);
                 } else {
-                    bool lost = false;
+                    bool lost = false;           // (of teams; not here)
                     float v;
                     if constexpr (ODD) {
                         v = odd_bucket_sums<LINF>(row - own, t.row, t.len, tiles.gpb, tiles.R, tiles.r);
                     } else {
                         v = LINF ? row_max(row) : row_sum_squares(row);
                         if (!t.regular) {
-                            const float end = has_tile && landed ? end_row<LINF>(row, t.valid) : 0.0f;
+                            const float end = has_tile ? end_row<LINF>(row, t.valid) : 0.0f;
                             if (t.valid != 32) v = end;
                         }
-                        v = join_team<MODE>(join_lanes<MODE>(v, tiles.gpb, Join{}), slots, T_shift, exchanges, landed, lost, Join{});
+                        v = join_team<MODE>(join_lanes<MODE>(v, tiles.gpb, Join{}), slots, T_shift, exchanges, true, lost, Join{});
                     }
-                    if (landed && !lost) {
-                        nrm = LINF ? v : sqrt_normal(v);
-                        inv = inv_scale_normal(sf, nrm);
-                        plain = !__any_sync(0xffffffffu, has_say<MODE>(t) && (LINF ? !norm_is_plain(v) : !l2_sum_in_range(v)));
-                        if (!plain) {
-                            if constexpr (LINF) {
-                                clear_nonfinite_row<true>(row, t.valid, nrm);
-                            } else if constexpr (ODD) {
-                                nrm = rare_norm_odd<true>(row - own, t.row, t.len, tiles.gpb, tiles.R, tiles.r, v, nrm, row, t.valid);
-                            } else {
-                                nrm = rare_norm<MODE, true>(row, t.valid, tiles.gpb, slots, T_shift, exchanges, v, nrm);
-                                exchanges += 2;
-                            }
-                            inv = inv_scale(sf, nrm);
-                            bad |= t.writes && !isfinite(nrm);
+                    nrm = LINF ? v : sqrt_normal(v);
+                    inv = inv_scale_normal(sf, nrm);
+                    plain = !__any_sync(0xffffffffu, has_say<MODE>(t) && (LINF ? !norm_is_plain(v) : !l2_sum_in_range(v)));
+                    if (!plain) {
+                        if constexpr (LINF) {
+                            clear_nonfinite_row<true>(row, t.valid, nrm);
+                        } else if constexpr (ODD) {
+                            nrm = rare_norm_odd<true>(row - own, t.row, t.len, tiles.gpb, tiles.R, tiles.r, v, nrm, row, t.valid);
+                        } else {
+                            nrm = rare_norm<MODE, true>(row, t.valid, tiles.gpb, slots, T_shift, exchanges, v, nrm);
+                            exchanges += 2;
                         }
-                        if (t.writes) {
-                            DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
-                            square_sum = fma((double)nrm, (double)nrm, square_sum);
-                        }
+                        inv = inv_scale(sf, nrm);
+                        bad |= t.writes && !isfinite(nrm);
+                    }
+                    if (t.writes) {
+                        DQ_STORE(norm_ptr, nrm, a.norms, (int64_t)M * nb * 4, a.status);
+                        square_sum = fma((double)nrm, (double)nrm, square_sum);
                     }
                 }
                 norm_ptr += (int64_t)kWorkers * nb;
@@ -1237,7 +1228,6 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
                 if (lane == 0) notes[warp] = note;
             }
             __syncthreads();
-            if (*lost_word != 0u) { timed_out = true; break; }
 
             // ---- the codes of the chunk, a thread an octet of each tile
             const int slots_used = (M - m0 < kWorkers ? M - m0 : kWorkers) * T;
@@ -1336,38 +1326,33 @@ __device__ __forceinline__ void tile_rounds(const RoundArgs& a, TileMap<MODE>& t
                     }
                 }
             }
-            // the CTA's accesses to the set come before the copies that refill it (they go through different proxies)
-            tma::fence_proxy_async();
             __syncthreads();
             copies.next(set);
         }
     }
+    copies.drain();
     if (bad) atomicOr(a.status, DQ_STAT_NONFINITE);
-    if (timed_out) {
-        if (lane == 0) atomicOr(a.status, DQ_STAT_WAIT);
-        copies.drain();
-    }
 }
 
 template <int MODE, bool LINF, int T>
 __global__ void __launch_bounds__(kRoundThreads, kTileCtasPerSm)
-tile_round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtensorMap map)
+tile_round_kernel(const __grid_constant__ RoundArgs a)
 {
-    const bool tbl_in_smem = set_up<TileSmem>(a, map);
+    grid_dependency_wait();
     const int b = *reinterpret_cast<const volatile int32_t*>(a.dev_b);
+    const bool tbl_in_smem = copy_table(a, TileSmem::table);
     double* part = reinterpret_cast<double*>(smem + TileSmem::sums);
-    uint32_t trouble = (tma::smem_addr(smem) & 1023u) ? DQ_STAT_INTERNAL : 0u;        // the swizzled tiles need a 1024-byte aligned base
-    // The first copies are on their way before b is here and its code is fetched.
+    // The first copies are on their way before b is here and its code is fetched; a call that cannot run waits for them.
     // Every CTA takes every hop-th position, `each` of them, the first `extra` CTAs one more.
-    const int n_pos = trouble ? 0 : (int)(a.each + (blockIdx.x < a.extra ? 1u : 0u));
+    // (test hook: with lose_first all that is done is to say that a wait was lost; no wait here has a limit to run out of)
+    const int n_pos = a.wait.lose_first != 0u ? 0 : (int)(a.each + (blockIdx.x < a.extra ? 1u : 0u));
     TileMap<MODE> tiles(a, tbl_in_smem, TileSmem::table, (int)(threadIdx.x >> 5) & (T - 1));
-    TileFetch<MODE, T> copies(tiles, &map, n_pos);
+    TileFetch<MODE, T> copies(tiles, n_pos);
     copies.next(0);
     copies.next(1);
-    if (!trouble) {
-        if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
-        else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
-    }
+    uint32_t trouble = 0;
+    if (b < 1 || b > DQ_MAX_BITS) trouble = DQ_STAT_BAD_BITS;
+    else if ((int64_t)b * a.v.total_groups > a.packed_stride) trouble = DQ_STAT_CAPACITY;
     if (trouble) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, (int)trouble);
         copies.drain();
@@ -1375,6 +1360,7 @@ tile_round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ C
         if (a.with_rule) rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, part, a.dev_b, b, a.status);
         return;
     }
+    if (a.wait.lose_first != 0u && (threadIdx.x & 31) == 0) atomicOr(a.status, DQ_STAT_WAIT);
     double square_sum = 0.0;
     switch (b) {
 #define DQ_CASE(BB) case BB: tile_rounds<BB, MODE, LINF, T>(a, tiles, copies, n_pos, square_sum); break;
@@ -1387,9 +1373,9 @@ tile_round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ C
 }
 
 // units: of work per CTA: warps, teams, or the CTA itself
-template <class Map>
-int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, int units, RoundArgs a, const CUtensorMap& map,
-                      int n_seg, int64_t entries, cudaStream_t st)
+template <class Map, class... Maps>
+int launch_persistent(void (*kernel)(RoundArgs, Maps...), int ctas_per_sm, int units, RoundArgs a, int n_seg, int64_t entries,
+                      cudaStream_t st, const Maps&... maps)
 {
     size_t smem_need = (size_t)Map::table;
     if (n_seg > 1 && n_seg <= kMaxSmemSegs) smem_need += (size_t)3 * (n_seg + 1) * 4;
@@ -1404,7 +1390,7 @@ int launch_persistent(void (*kernel)(RoundArgs, CUtensorMap), int ctas_per_sm, i
     if (blocks * units > entries) blocks = (entries + units - 1) / units;
     a.each = (uint32_t)(entries / (blocks * units));
     a.extra = (uint32_t)(entries - (int64_t)a.each * blocks * units);
-    dq_launch(kernel, dim3((unsigned)blocks), dim3(kRoundThreads), smem_need, st, a, map);
+    dq_launch(kernel, dim3((unsigned)blocks), dim3(kRoundThreads), smem_need, st, a, maps...);
     return cudaGetLastError() == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
@@ -1419,19 +1405,19 @@ int units_per_cta(const RoundArgs& a)
 template <int MODE, bool LINF>
 int dq_launch_norms(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<SmemMap>(norms_kernel<MODE, LINF>, kNormCtasPerSm, units_per_cta<MODE>(a), a, map, n_seg, entries, st);
+    return launch_persistent<SmemMap>(norms_kernel<MODE, LINF>, kNormCtasPerSm, units_per_cta<MODE>(a), a, n_seg, entries, st, map);
 }
 template <int MODE, bool AVG, bool LINF>
 int dq_launch_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
 {
-    return launch_persistent<SmemMap>(round_kernel<MODE, AVG, LINF>, RoundShape<AVG>::ctas_per_sm, units_per_cta<MODE>(a), a, map,
-                                      n_seg, entries, st);
+    return launch_persistent<SmemMap>(round_kernel<MODE, AVG, LINF>, RoundShape<AVG>::ctas_per_sm, units_per_cta<MODE>(a), a,
+                                      n_seg, entries, st, map);
 }
 template <int MODE, bool LINF>
-int dq_launch_tile_round(const RoundArgs& a, const CUtensorMap& map, int n_seg, int64_t entries, cudaStream_t st)
+int dq_launch_tile_round(const RoundArgs& a, int n_seg, int64_t entries, cudaStream_t st)
 {
     constexpr int T = MODE == kTeamBuckets ? 2 : 1;
-    return launch_persistent<TileSmem>(tile_round_kernel<MODE, LINF, T>, kTileCtasPerSm, 1, a, map, n_seg, entries, st);
+    return launch_persistent<TileSmem>(tile_round_kernel<MODE, LINF, T>, kTileCtasPerSm, 1, a, n_seg, entries, st);
 }
 
 #endif  // DQ_ROUND_KERNELS

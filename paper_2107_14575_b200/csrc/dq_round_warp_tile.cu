@@ -2,4 +2,4 @@
 #define DQ_ROUND_KERNELS
 #include "dq_round.cuh"
 
-template int dq_launch_tile_round<kWarpBuckets, false>(const RoundArgs&, const CUtensorMap&, int, int64_t, cudaStream_t);
+template int dq_launch_tile_round<kWarpBuckets, false>(const RoundArgs&, int, int64_t, cudaStream_t);
