@@ -43,9 +43,9 @@ norm_square_partials(const float* __restrict__ norms, const int64_t n, double* _
         }
     }
     const double s = block_sum<kSumThreads>(a0 + a1, sh);
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x >= 32) return;
     if (gridDim.x == 1) write_next_bits(r, s, dev_b, status);
-    else partial[blockIdx.x] = s;       // one entry per CTA of the grid: in bounds by construction
+    else if (threadIdx.x == 0) partial[blockIdx.x] = s;       // one entry per CTA of the grid: in bounds by construction
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -56,7 +56,7 @@ apply_rule(const RuleArgs r, const int npartial, int32_t* __restrict__ dev_b, in
     double acc = 0.0;
     for (int i = threadIdx.x; i < npartial; i += kThreads) acc += r.partial[i];
     const double sum = block_sum<kThreads>(acc, sh);
-    if (threadIdx.x == 0) write_next_bits(r, sum, dev_b, status);
+    if (threadIdx.x < 32) write_next_bits(r, sum, dev_b, status);
 }
 
 inline int64_t num_chunks(int64_t n) { return (n + kChunk - 1) / kChunk; }

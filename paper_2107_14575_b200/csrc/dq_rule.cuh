@@ -43,25 +43,31 @@ __device__ __forceinline__ double block_sum(double v, double* sh)
     return total;
 }
 
-// One thread: b from the sum of squared norms, into dev_b[0] and its s into dev_b[1].
-__device__ __forceinline__ void write_next_bits(const RuleArgs& r, const double sum, int32_t* dev_b, int32_t* status)
+// One warp, all of it (lane 0 has the sum of squared norms): b into dev_b[0] and its s into dev_b[1].  The sixteen
+// thresholds are looked at by a lane each: one after the other, with a conversion to fp64 in every step, they took up to
+// 400 cycles of the tail of a round.
+__device__ __forceinline__ void write_next_bits(const RuleArgs& r, double sum, int32_t* dev_b, int32_t* status)
 {
+    const int lane = threadIdx.x & 31;
     int b;
     if (r.fixed_b != 0) {
         b = r.fixed_b;
     } else {
+        sum = __shfl_sync(0xffffffffu, sum, 0);
         const double x = r.coef * sqrt(sum / (double)r.M);
+        const int c = lane + 1;
+        const uint32_t enough = __ballot_sync(0xffffffffu, c >= r.b_min && c <= r.b_max && (double)((1 << lane) - 1) >= x);
         b = r.b_max;
         if (isfinite(x)) {
-            for (int c = r.b_min; c <= r.b_max; ++c) {
-                if ((double)((1 << (c - 1)) - 1) >= x) { b = c; break; }
-            }
-        } else {
+            if (enough) b = __ffs(enough);
+        } else if (lane == 0) {
             atomicOr(status, DQ_STAT_NONFINITE);
         }
     }
-    dev_b[0] = b;
-    dev_b[1] = (1 << (b - 1)) - 1;
+    if (lane == 0) {
+        dev_b[0] = b;
+        dev_b[1] = (1 << (b - 1)) - 1;
+    }
 }
 
 // End of a kernel whose CTAs all come here: `v` is a thread's share of the sum of squared norms.
@@ -91,7 +97,14 @@ __device__ __forceinline__ void rule_at_end(const RuleArgs& r, const double v, c
     double acc = 0.0;
     if (sums) {
         __threadfence();
-        for (uint32_t i = threadIdx.x; i < gridDim.x; i += NT) acc += __ldcg(r.partial + i);
+        // (eight at a time: a load behind the other's addition costs the round its latency each time)
+        for (uint32_t first = threadIdx.x; first < gridDim.x; first += 8 * NT) {
+            double x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = first + k * NT < gridDim.x ? __ldcg(r.partial + first + k * NT) : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc += x[k];
+        }
     } else if (r.fixed_b == 0) {
         for (int64_t i = threadIdx.x; i < n; i += NT) {
             const double x = (double)norms[i];
@@ -99,8 +112,8 @@ __device__ __forceinline__ void rule_at_end(const RuleArgs& r, const double v, c
         }
     }
     const double sum = block_sum<NT>(acc, sh);
-    if (threadIdx.x == 0) {
-        if (r.this_b) *r.this_b = b;
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0 && r.this_b) *r.this_b = b;
         write_next_bits(r, sum, dev_b, status);
     }
 }
