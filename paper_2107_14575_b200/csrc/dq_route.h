@@ -47,24 +47,27 @@ enum RoundRoute { kWarpTiles, kCtaTiles, kTwoKernels };
 
 // A CTA's four warps are through with a tile in a quarter of a warp's time, so with few tiles the round is as much shorter;
 // with many, the barriers and the eight elements that a thread goes through at a time (a warp's lane: 32) cost more than the
-// unused part of a last turn.  The line lies at 0.6 tiles a warp of the chip (0.45 for teams' buckets, 0.2 with one worker),
-// and beyond it wherever one pass by warps would lose to two kernels.  On 952 triples of times on one B200 (buckets of 32, 96, 480,
-// 512, 2048 and whole tensors, b = 4 to 8, M = 1 to 32, 3k to 24M elements) the fastest of the three is missed by 0.4 to
-// 1.1 % on average, by 24 % at worst; with the lines at 0.3 or at 1.0 by 0.5 to 1.3 %.  Some of them, by warps / two kernels / by CTAs
-// (us), bucket 512, b = 4: 20k elements M = 4 9 / 11 / 5, M = 16 26 / 12 / 10, M = 32 48 / 14 / 17; 600k M = 4 10 / 12 / 6, M = 16 28 / 23 / 16,
-// M = 32 52 / 30 / 28; 1M M = 4 10 / 14 / 8, M = 8 17 / 21 / 15; 1.7M M = 4 13 / 20 / 14, M = 16 35 / 37 / 32; 8M M = 8 61 / 78 / 72; bucket
-// 2048, b = 5: 20k M = 4 9 / 13 / 7, M = 16 28 / 15 / 19; 600k M = 8 16 / 19 / 13; 1.7M M = 8 22 / 33 / 27; bucket 96: 20k M = 4 13 / 14 / 6;
-// 600k M = 8 26 / 20 / 13; 5M M = 8 73 / 74 / 67; whole tensors: 20k M = 4 12 / 15 / 9, 600k M = 8 20 / 21 / 15.
+// unused part of a last turn.  The line lies at 1.2 tiles a warp of the chip (0.6 for the teams of buckets of 2048, 0.25 with one
+// worker), and beyond it wherever one pass by warps would lose to two kernels (teams: nowhere).  On 1183 triples of times on one
+// B200 (buckets of 32, 96, 480, 512, 2048 and whole tensors, b = 4 to 8, M = 1 to 32, 3k to 13M elements, the rule attached) the
+// fastest of the three is missed by 0.3 % on average and 15 % at worst; with a line of 0.6 by 0.7 %, of 2.2 by 0.7 %.  Some of them, by warps /
+// two kernels / by CTAs (us), bucket 512, b = 4: 16k M = 4 10 / 12 / 6; 16k M = 16 27 / 13 / 11; 16k M = 32 49 / 15 /
+// 17; 456k M = 4 11 / 13 / 7; 456k M = 16 28 / 20 / 14; 797k M = 4 11 / 14 / 9; 797k M = 8 18 / 18 / 13; 1.4M M = 4 13 /
+// 17 / 11; 1.4M M = 16 36 / 32 / 30; 2.4M M = 16 54 / 48 / 42; 7.4M M = 8 57 / 71 / 64; bucket 2048, b = 5: 16k M = 4 11
+// / 12 / 8; 16k M = 16 30 / 16 / 20; 456k M = 8 17 / 18 / 14; 1.4M M = 8 23 / 29 / 21; bucket 96, b = 4: 16k M = 4 15 /
+// 15 / 7; 456k M = 8 24 / 19 / 12; 4.3M M = 8 60 / 66 / 58; whole tensors: 16k M = 4 13 / 16 / 10; 456k M = 8 20 / 21 /
+// 14; 2.4M M = 8 47 / 47 / 44.
 //
 // Only where a few tiles have a great many workers does the CTA, which takes them in turn after all, lose to
-// two kernels that spread them: per worker 0.42 us against 0.1 (0.97 and 0.18 with buckets of 2048, two workers a
-// turn), 4.3 and 11.2 us besides (3.9 and 11.6), and the two kernels slow down with the number of tiles first.
+// two kernels that spread them over the chip and slow down with the number of tiles first.
 inline RoundRoute dq_round_route(const RouteQuery& q, const bool cta_tiles, const bool pairs)
 {
     const bool one = dq_one_pass(q);
     const double m = (double)q.M, tiles = (double)q.positions;
-    const double line = q.M == 1 ? 0.2 : (pairs ? 0.45 : 0.6);
-    if (!cta_tiles || !(tiles <= line * (double)q.units || !one)) return one ? kWarpTiles : kTwoKernels;
-    const bool spread = pairs ? 0.79 * m - 7.7 > 0.0011 * tiles * m : 0.32 * m - 6.9 > 0.0005 * tiles * m;
-    return spread ? kTwoKernels : kCtaTiles;
+    const double line = q.M == 1 ? 0.25 : (pairs ? 0.6 : 1.2);
+    if (!cta_tiles) return one ? kWarpTiles : kTwoKernels;
+    if (tiles > line * (double)q.units && (one || pairs)) return kWarpTiles;
+    // what two kernels save per worker, and what they cost besides
+    const double per_worker = pairs ? 0.5 : (q.odd_buckets > 0 ? 0.32 : 0.24), besides = pairs ? 5.5 : (q.odd_buckets > 0 ? 6.9 : 6.2);
+    return per_worker * m - besides > 0.0005 * tiles * m ? kTwoKernels : kCtaTiles;
 }

@@ -3,7 +3,7 @@
 Sizes around the edges of that kernel: one row, a tile and its neighbours, two tiles of a bucket of 2048, more
 positions than CTAs, chunks of four (two) workers with and without a remainder, every width of a code (those that leave
 from registers and those that go through shared memory), strides, an output that is only 16-byte aligned, buckets
-that are zero, tiny or not finite.  The layouts of two million elements have too many tiles for it: the same comparison
+that are zero, tiny or not finite.  The layouts of 3.3 million elements have too many tiles for it: the same comparison
 for the kernel that takes those.
 """
 import numpy as np
@@ -29,11 +29,11 @@ def G(dqlib):
 CASES = [([d], bucket, M, b) for d, bucket, M, b in (
     (1, 32, 2, 4), (31, 512, 5, 8), (33, 1024, 4, 2), (1024, 512, 3, 16), (1025, 1024, 8, 4), (2047, 2048, 3, 5), (2048, 2048, 2, 4),
     (2080, 2048, 9, 6), (8193, 128, 17, 3), (70001, 512, 4, 8), (70001, 96, 6, 4), (70001, 0, 5, 4), (70001, 2048, 7, 8),
-    (760001, 512, 3, 4), (1300001, 480, 2, 5), (1000001, 0, 2, 6), (1050001, 2048, 4, 4))]
+    (760001, 512, 3, 4), (2700001, 512, 2, 4), (1300001, 480, 2, 5), (1000001, 0, 2, 6), (1050001, 2048, 4, 4))]
 CASES += [(RAGGED, bucket, 6, b) for bucket, b in ((32, 6), (96, 5), (480, 8), (512, 9), (2048, 7), (0, 11))]
 CASES += [(RAGGED, 512, 5, b) for b in range(1, 17)] + [(RAGGED, 2048, 5, b) for b in range(1, 17)]
-CASES += [(RAGGED + [2000000], bucket, 3, b) for bucket, b in ((32, 4), (96, 4), (480, 6), (512, 8), (2048, 4), (0, 3))]
-CASES += [(RAGGED + [2000000], 4096, 3, 5), ([40] * 1100, 64, 5, 7)]
+CASES += [(RAGGED + [3300000], bucket, 3, b) for bucket, b in ((32, 4), (96, 4), (480, 6), (512, 8), (2048, 4), (0, 3))]
+CASES += [(RAGGED + [3300000], 4096, 3, 5), ([40] * 1100, 64, 5, 7)]
 CASES = [c + (False,) for c in CASES] + [c + (True,) for c in CASES if c[3] in (4, 5, 8)]
 
 
