@@ -16,11 +16,12 @@
 // bucket combine by shuffles, then the lane encodes its row against that norm; the words leave from
 // registers or through the consumed stage, which is refilled.
 // HBM traffic: 4 + b/8 bytes per element and worker, plus 4 (8 with the update) per output element.
-// What bounds it: per tile of a worker a warp issues some 530 instructions at b = 4 (290 of them the codes,
+// What bounds it: per tile of a worker a warp issues some 515 instructions at b = 4 (290 of them the codes,
 // their draws and the sums; 65 are the wide multiplies of the generator, four cycles of the multiplier
 // each), 60 % of the issue slots' and 67 % of the multiplier's time, beside loads that alone take 0.9 of
-// the measured copy bandwidth.  Measured: 2^26 elements M = 32 b = 4 1.89 ms (5.2 TB/s; separate
-// quantizer and average 2.29), ResNet-18 shape M = 8 92 us (4.9), VGG-16 shape M = 16 b = 5 with update 260 us.
+// the measured copy bandwidth.  Measured: 2^26 elements M = 32 b = 4 1.87 ms (5.3 TB/s; separate
+// quantizer and average 2.29), ResNet-18 shape M = 8 88 us (5.1), VGG-16 shape M = 16 b = 5 with update 252 us.
+// Rounds with few tiles: see tile_rounds.
 #pragma once
 
 #include "dq_common.cuh"
@@ -1015,12 +1016,13 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 // leaves the scales of every row in shared memory.  Behind a barrier the CTA goes through the workers of the chunk, a
 // thread an octet (eight elements, one Philox block) of the tile, two workers side by side, and keeps the octet's sums
 // in registers from a position's first worker to its last.
-// What bounds it: with a position per SM the chain of a chunk (20 tiles, M = 32, cycles: wait 310, norm 770, codes of four
-// workers 1400 one after the other, 1000 side by side, copies 400, two barriers 280), with many the instructions: some 650
-// per tile and worker at b = 4 against 530 in a warp's own way, 37 more per octet for the scales, the notes and the
-// addresses.  Where the line between the two lies, and what both measured: dq_route.h.
-// Five CTAs per SM (96 registers): with six (80) 600k elements M = 8 b = 5 10.9 us, 10.5 so, with four 10.1; 4.2M M = 8 b = 4
-// 40.6, 40.0, 42.0; buckets of 2048, 1.5M M = 16 35.8 with five, 41.4 with four.
+// What bounds it: with a position per SM the chain of a chunk (20 tiles, M = 16, cycles: norm 710, codes of four workers 1090
+// two by two, 1400 one after the other, two barriers 180; the rest copies and addresses), with many the instructions,
+// some 700 per tile and worker at b = 4, 515 in a warp's own way: scales, notes and addresses come once per eight elements.  Where
+// the line between the two lies, and what both measured: dq_route.h.
+// Five CTAs per SM (96 registers).  By five / four / six of them (us): bucket 512, 600k elements M = 8 b = 5 10.4 / 10.2 / 12.2
+// (six spill); 610k, one turn of five, two of four, M = 8 b = 4 9.4 / 11.3; 1.3M M = 8 17.4 / 17.1 / 23.2; bucket 2048, 1.2M
+// M = 16 31.4 / 29.6 / 38.1, 1.3M M = 8 21.6 / 23.0.
 constexpr int kTileCtasPerSm = 5;
 constexpr int kSets = 2;                            // chunks in shared memory: the one at hand and one on its way
 struct TileSmem {
