@@ -79,15 +79,8 @@ int launch_tiles(const RoundArgs& a, const dq_layout_t* L, bool given, cudaStrea
 
 RoundRoute route_of(const RoundArgs& a, bool given)
 {
-    const bool teams = !given && a.div_shift >= 0 && a.gpb_shift > 5;
-    RouteQuery q = {};
-    q.positions = dq_tile_positions(a, given);
-    q.units = (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps;
-    if (teams) q.units >>= a.gpb_shift - 5;
-    q.M = a.M;
-    q.given = given ? 1 : 0;
-    q.odd_buckets = !given && a.div_shift < 0 ? 32 / a.v.groups_per_bucket : 0;
-    return dq_round_route(q, !teams || a.gpb_shift == 6, teams);
+    return dq_route_of(dq_tile_positions(a, given), (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps,
+                       a.v.groups_per_bucket, a.M, given);
 }
 
 }  // namespace

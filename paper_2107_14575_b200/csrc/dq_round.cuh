@@ -1419,6 +1419,7 @@ template <int MODE, bool LINF>
 int dq_launch_tile_round(const RoundArgs& a, int n_seg, int64_t entries, cudaStream_t st)
 {
     constexpr int T = MODE == kTeamBuckets ? 2 : 1;
+    if (MODE == kTeamBuckets && a.gpb_shift != 6) return DQ_ERR_RANGE;          // (the kernel's teams are pairs; see dq_cta_form)
     return launch_persistent<TileSmem>(tile_round_kernel<MODE, LINF, T>, kTileCtasPerSm, 1, a, n_seg, entries, st);
 }
 

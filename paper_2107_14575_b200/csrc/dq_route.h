@@ -71,3 +71,20 @@ inline RoundRoute dq_round_route(const RouteQuery& q, const bool cta_tiles, cons
     const double per_worker = pairs ? 0.5 : (q.odd_buckets > 0 ? 0.32 : 0.24), besides = pairs ? 5.5 : (q.odd_buckets > 0 ? 6.9 : 6.2);
     return per_worker * m - besides > 0.0005 * tiles * m ? kTwoKernels : kCtaTiles;
 }
+
+// What a CTA has a form for: given norms, and buckets of up to 1024 elements or of 2048, which are a pair of its warps'.
+inline bool dq_cta_form(int32_t groups_per_bucket, bool given) { return given || groups_per_bucket <= 64; }
+
+// The route of a call: tile positions of a worker, warps of a launch by warps, and the layout's bucket (32-element groups; where
+// the norms are not given a power of two or less than 32).
+inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_per_bucket, int32_t M, bool given)
+{
+    const bool teams = !given && groups_per_bucket > 32;
+    RouteQuery q = {};
+    q.positions = positions;
+    q.units = teams ? warps / (groups_per_bucket / 32) : warps;
+    q.M = M;
+    q.given = given ? 1 : 0;
+    q.odd_buckets = !given && (groups_per_bucket & (groups_per_bucket - 1)) != 0 ? 32 / groups_per_bucket : 0;
+    return dq_round_route(q, dq_cta_form(groups_per_bucket, given), teams);
+}

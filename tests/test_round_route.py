@@ -53,3 +53,17 @@ def test_buckets_of_4096_never_take_the_kernel_they_have_no_form_of(route):
     for d in (1, 70001, 1 << 20, 1 << 24):
         for M in (1, 2, 8, 32):
             assert route(_query(4096, d, M), 0, 0) != 1
+
+
+def test_which_buckets_a_cta_has_a_form_for(tmp_path):
+    """Teams are pairs of warps there: buckets of 4096 go by warps or by two kernels whatever their size, the others, given
+    norms of any bucket among them, by CTAs where they are small."""
+    import route_util
+    route = route_util.compile_route(tmp_path)
+    for d in (1, 70001, 1 << 20, 1 << 24):
+        groups = -(-d // 32)
+        for M in (1, 2, 8, 32):
+            assert route(groups, -(-d // 4096), 4096, M) != route_util.CTAS
+    for bucket in (32, 64, 96, 480, 512, 992, 1024, 2048, 1056, 4064, 0):
+        nb = -(-70001 // bucket) if bucket else 1
+        assert route(-(-70001 // 32), nb, bucket, 4) == route_util.CTAS
