@@ -389,13 +389,17 @@ int dq_unpack_average_update(const dq_layout_t* layout, const uint32_t* dev_pack
 const char* dq_status_string(int code);
 
 /* Test hook for the bounded waits (no counterpart in the paper).  Every wait of a
- * kernel for one of its own asynchronous copies is bounded by `limit_ns` of the GPU's
- * global timer (default 2e9; 0 restores the default).  With `lose_first_wait` != 0 the
+ * kernel on a barrier that one of its own asynchronous copies completes is bounded by
+ * `limit_ns` of the GPU's global timer (default 2e9; 0 restores the default).  Copies
+ * that complete in the issuing lane's own order, as loads do, have no such barrier:
+ * rounds with few tiles and the average of many workers' words wait for those.  With `lose_first_wait` != 0 the
  * first such wait of every warp or CTA that consumes copies is declared lost at once,
  * although its copy is valid and lands a moment later: this exercises what a kernel does
  * after a time-out -- raise DQ_STAT_WAIT, stop producing output, wait (with limit_ns)
  * for every copy it has issued, return -- without anything being lost, faulting or
- * hanging.  Host state of the library, read when a call is made; not for production use
+ * hanging.  Rounds that would take the kernel without such a wait take those that have
+ * one while it is set; the average of such words raises the status without a wait lost.
+ * Host state of the library, read when a call is made; not for production use
  * (the outputs of a call made under it are incomplete). */
 void dq_debug_set_wait_limits(uint64_t limit_ns, int32_t lose_first_wait);
 

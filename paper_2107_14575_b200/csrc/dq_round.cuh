@@ -1041,7 +1041,8 @@ __device__ __forceinline__ bool adds_zero(const ulonglong2 sc)
 }
 
 // The warp's copies: its tile of every position and worker of the CTA, a chunk at a time, 16 bytes per lane and instruction
-// straight to where a swizzled tensor copy would put them.  With one position per SM a chunk's chain is what counts, and
+// straight to where a swizzled tensor copy would put them.  They complete as loads do: there is no barrier to poll, and
+// WaitLimits does not apply (under its test hook a round is never sent here).  With one position per SM a chunk's chain is what counts, and
 // a tensor copy costs that chain some 250 cycles to issue, 250 to find landed and 100 for the fence before its stage is refilled.
 template <int MODE, int T>
 struct TileFetch {
@@ -1346,8 +1347,7 @@ tile_round_kernel(const __grid_constant__ RoundArgs a)
     double* part = reinterpret_cast<double*>(smem + TileSmem::sums);
     // The first copies are on their way before b is here and its code is fetched; a call that cannot run waits for them.
     // Every CTA takes every hop-th position, `each` of them, the first `extra` CTAs one more.
-    // (test hook: with lose_first all that is done is to say that a wait was lost; no wait here has a limit to run out of)
-    const int n_pos = a.wait.lose_first != 0u ? 0 : (int)(a.each + (blockIdx.x < a.extra ? 1u : 0u));
+    const int n_pos = (int)(a.each + (blockIdx.x < a.extra ? 1u : 0u));
     TileMap<MODE> tiles(a, tbl_in_smem, TileSmem::table, (int)(threadIdx.x >> 5) & (T - 1));
     TileFetch<MODE, T> copies(tiles, n_pos);
     copies.next(0);
@@ -1362,7 +1362,6 @@ tile_round_kernel(const __grid_constant__ RoundArgs a)
         if (a.with_rule) rule_at_end<kRoundThreads>(a.rule, 0.0, a.norms, (int64_t)a.M * a.v.nb, part, a.dev_b, b, a.status);
         return;
     }
-    if (a.wait.lose_first != 0u && (threadIdx.x & 31) == 0) atomicOr(a.status, DQ_STAT_WAIT);
     double square_sum = 0.0;
     switch (b) {
 #define DQ_CASE(BB) case BB: tile_rounds<BB, MODE, LINF, T>(a, tiles, copies, n_pos, square_sum); break;

@@ -76,8 +76,9 @@ inline RoundRoute dq_round_route(const RouteQuery& q, const bool cta_tiles, cons
 inline bool dq_cta_form(int32_t groups_per_bucket, bool given) { return given || groups_per_bucket <= 64; }
 
 // The route of a call: tile positions of a worker, warps of a launch by warps, and the layout's bucket (32-element groups; where
-// the norms are not given a power of two or less than 32).
-inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_per_bucket, int32_t M, bool given)
+// the norms are not given a power of two or less than 32).  lose_first: the test hook of the waits is set; a round by CTAs has no
+// wait to lose, so the call takes the kernels that have.
+inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_per_bucket, int32_t M, bool given, bool lose_first)
 {
     const bool teams = !given && groups_per_bucket > 32;
     RouteQuery q = {};
@@ -86,5 +87,5 @@ inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_p
     q.M = M;
     q.given = given ? 1 : 0;
     q.odd_buckets = !given && (groups_per_bucket & (groups_per_bucket - 1)) != 0 ? 32 / groups_per_bucket : 0;
-    return dq_round_route(q, dq_cta_form(groups_per_bucket, given), teams);
+    return dq_round_route(q, dq_cta_form(groups_per_bucket, given) && !lose_first, teams);
 }

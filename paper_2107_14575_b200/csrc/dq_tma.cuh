@@ -15,9 +15,10 @@ bool dq_encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, uint32_t r
                           const uint64_t* dims, const uint64_t* strides_bytes /*rank-1*/, const uint32_t* box,
                           CUtensorMapSwizzle swizzle);
 
-// Limits of the waits for asynchronous copies; every kernel that waits receives them as part of
-// its (constant-bank) arguments.  `ns` bounds every wait, in nanoseconds of the global timer (2 s
-// unless dq_debug_set_wait_limits changed it).  `lose_first` is the test hook: when set, the FIRST
+// Limits of the waits on a barrier for asynchronous copies; every kernel that waits receives them as part of
+// its (constant-bank) arguments.  `ns` bounds every such wait, in nanoseconds of the global timer (2 s
+// unless dq_debug_set_wait_limits changed it).  (Asynchronous copies of a lane's own, cp.async, complete in its
+// own order as loads do: nothing polls for them and no limit applies.)  `lose_first` is the test hook: when set, the FIRST
 // wait of every consumer (a warp or a CTA, as the kernel is organised) is declared lost without a
 // look at its barrier, while its copy is valid and lands a moment later -- the path taken after a
 // time-out then runs with nothing actually lost.  The kernels look at the hook outside their tile

@@ -67,3 +67,17 @@ def test_which_buckets_a_cta_has_a_form_for(tmp_path):
     for bucket in (32, 64, 96, 480, 512, 992, 1024, 2048, 1056, 4064, 0):
         nb = -(-70001 // bucket) if bucket else 1
         assert route(-(-70001 // 32), nb, bucket, 4) == route_util.CTAS
+
+
+@pytest.mark.parametrize("bucket", [32, 96, 480, 512, 1024, 2048, 4096, 1056, 0])
+def test_under_the_hook_of_the_waits_a_round_takes_kernels_that_have_one_to_lose(tmp_path, bucket):
+    """... the ones the same size would take if there were no kernel by CTAs."""
+    import route_util
+    route = route_util.compile_route(tmp_path)
+    for d in (1, 3001, 70001, 600001, 1 << 20, 3300001, 1 << 24):
+        groups, nb = -(-d // 32), -(-d // bucket) if bucket else 1
+        for M in (1, 2, 3, 8, 40):
+            lost = route(groups, nb, bucket, M, lost=True)
+            assert lost != route_util.CTAS
+            if route(groups, nb, bucket, M) == route_util.WARPS and bucket != 2048:
+                assert lost == route_util.WARPS
