@@ -919,15 +919,22 @@ __device__ __forceinline__ int warp_of_team(const RoundArgs& a)
 {
     return MODE == kTeamBuckets ? (int)(threadIdx.x >> 5) & ((1 << (a.gpb_shift - 5)) - 1) : 0;
 }
-// The first two copies of a warp that will not look at them: the CTA's shared memory outlives them.
+// The first two copies of a warp that will not look at them: the CTA's shared memory outlives them, or the call says that a
+// wait ran out (beside what else is wrong with it).
 template <int MODE, bool AVG>
 __device__ __forceinline__ void drain_first(const WarpFetch<MODE, AVG>& copies)
 {
+    const RoundArgs& a = copies.tiles.a;
     const int issued = copies.items() - copies.left;
+    bool lost = false;
 #pragma unroll
-    for (int st = 0; st < kStages; ++st)
-        if (MODE == kTeamBuckets ? ((copies.flying >> st) & 1u) != 0u : st < issued)
-            (void)tma::mbar_wait(stage_bar(threadIdx.x >> 5, st), 0u, copies.tiles.a.wait);
+    for (int st = 0; st < kStages; ++st) {
+        if (MODE == kTeamBuckets ? ((copies.flying >> st) & 1u) != 0u : st < issued) {
+            lost |= a.wait.lose_first != 0u;         // (test hook: the wait counts as lost, and the copy is waited for all the same)
+            lost |= !tma::mbar_wait(stage_bar(threadIdx.x >> 5, st), 0u, a.wait);
+        }
+    }
+    if (__any_sync(0xffffffffu, lost) && (threadIdx.x & 31) == 0) atomicOr(a.status, DQ_STAT_WAIT);
 }
 
 // Norms alone.  Bound by HBM, 4 bytes read per element.  Against a CTA-wide ring of 16 KB tiles with a barrier

@@ -147,3 +147,33 @@ def test_limits_are_restored(G):
     norms, packed = r.norms_quantize(SEED, 0)
     r.average()
     assert r.read_status() == 0 and r.guards_intact()
+
+
+@pytest.mark.parametrize("bucket", [64, 512, 2048, 4096, 480])
+def test_a_call_that_cannot_run_waits_for_the_copies_it_has_issued(G, bucket):
+    """The codes' first copies leave before b is known to be usable.  A b of 17 and a stream too short for b are what the
+    status says, nothing is written, and a wait for those copies that runs out is said as well."""
+    ref = oracle.Layout(SEGS, bucket)
+    M = 3
+    r = G.GpuRound(SEGS, bucket, M, packed_stride=(ref.packed_words(6) + 3) // 4 * 4)
+    r.set_grads(_grads(ref, M, bucket))
+    r.set_norms(oracle.bucket_norms(ref, _grads(ref, M, bucket)))
+    for b, why in ((17, G.dq.STAT_BAD_BITS), (0, G.dq.STAT_BAD_BITS), (9, G.dq.STAT_CAPACITY)):
+        for call in (r.norms_quantize, r.quantize):
+            for lost in (False, True):
+                r.set_b(b)
+                r.clear_status()
+                G.dq.debug_set_wait_limits(LIMIT_NS, lost)
+                try:
+                    call(SEED, 1, fill=-7)
+                    torch.cuda.synchronize()
+                finally:
+                    G.dq.debug_set_wait_limits()
+                assert r.read_status() == why | (G.dq.STAT_WAIT if lost else 0)
+                assert bool((r.g_packed.view == -7).all()) and r.guards_intact()
+    r.set_b(5)
+    r.clear_status()
+    norms, packed = r.norms_quantize(SEED, 1)
+    want = oracle.quantize_pack(ref, _grads(ref, M, bucket), norms, 5, SEED, 1)
+    np.testing.assert_array_equal(packed[:, : want.shape[1]], want)
+    assert r.read_status() == 0 and r.guards_intact()
