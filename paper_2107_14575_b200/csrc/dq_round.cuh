@@ -608,6 +608,14 @@ struct WarpFetch {
     // !AVG: descriptions of the positions fetched and not done with, the consumer's and at most two more
     uint32_t queue0, queue1, queue2;
     int queued;
+    // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
+    // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
+    // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
+    // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
+    // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal), and made once:
+    // made at every copy it cost codes of 33.5M elements, M = 4, b = 4, given norms 102.4 us against 98.9, norms found 105.0
+    // against 102.5.  (AVG has no registers to keep it.)
+    uint64_t policy;
 
     __device__ __forceinline__ static uint32_t unit_of(const RoundArgs& a)
     {
@@ -619,7 +627,8 @@ struct WarpFetch {
           m_first((AVG || where.a.M == 1) ? 0 : (int)((int64_t)unit_of(where.a) / positions)),
           pos0((int)((int64_t)unit_of(where.a) - (int64_t)m_first * positions)), pos(pos0), m(0),
           left(AVG ? n_pos * where.a.M : n_pos), worker(m_first * (where.a.map_has_worker_dim ? 1 : 0)), first(kNoTile),
-          parities(0), flying(0), queue0(0), queue1(0), queue2(0), queued(0)
+          parities(0), flying(0), queue0(0), queue1(0), queue2(0), queued(0),
+          policy(AVG ? 0 : (where.a.stream_reads ? tma::policy_evict_first() : tma::policy_evict_normal()))
     {
         if (left > 0) first = tiles.describe(pos);
     }
@@ -636,16 +645,11 @@ struct WarpFetch {
             ++queued;
         }
         if (TEAM && first != kNoTile) flying |= 1u << st;
-        // L2 policy of the reads.  AVG: evict-normal.  The words are not read again by the call, and gradients
-        // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
-        // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
-        // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
-        // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).
         if ((threadIdx.x & 31) == 0 && (!TEAM || first != kNoTile))
             tma::fetch_tile(tma::smem_addr(stage_ptr(threadIdx.x >> 5, st)), map, tma::smem_addr(stage_bar(threadIdx.x >> 5, st)),
                             kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu),
                             AVG ? (a.map_has_worker_dim ? m : 0) : worker,
-                            (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal());
+                            AVG ? tma::policy_evict_normal() : policy);
         if (AVG) {
             if (++m == a.M) {
                 m = 0; pos += hop;
