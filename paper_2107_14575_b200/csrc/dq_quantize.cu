@@ -80,7 +80,7 @@ int launch_tiles(const RoundArgs& a, const dq_layout_t* L, bool given, cudaStrea
 RoundRoute route_of(const RoundArgs& a, bool given)
 {
     return dq_route_of(dq_tile_positions(a, given), (int64_t)dq_sm_count() * RoundShape<true>::ctas_per_sm * kRoundWarps,
-                       a.v.groups_per_bucket, a.M, given, a.wait.lose_first != 0u);
+                       a.v.groups_per_bucket, a.M, given, a.linf != 0, a.wait.lose_first != 0u);
 }
 
 }  // namespace

@@ -45,28 +45,47 @@ inline bool dq_one_pass(const RouteQuery& q)
 //   kTwoKernels  codes, then the average from the words
 enum RoundRoute { kWarpTiles, kCtaTiles, kTwoKernels };
 
-// A CTA's four warps are through with a tile in a quarter of a warp's time, so with few tiles the round is as much shorter;
-// with many, the barriers and the eight elements that a thread goes through at a time (a warp's lane: 32) cost more than the
-// unused part of a last turn.  The line lies at 1.2 tiles a warp of the chip (0.6 for the teams of buckets of 2048, 0.25 with one
-// worker), and beyond it wherever one pass by warps would lose to two kernels (teams: nowhere).  On 1183 triples of times on one
-// B200 (buckets of 32, 96, 480, 512, 2048 and whole tensors, b = 4 to 8, M = 1 to 32, 3k to 13M elements, the rule attached) the
-// fastest of the three is missed by 0.3 % on average and 15 % at worst; with a line of 0.6 by 0.7 %, of 2.2 by 0.7 %.  Some of them, by warps /
-// two kernels / by CTAs (us), bucket 512, b = 4: 16k M = 4 10 / 12 / 6; 16k M = 16 27 / 13 / 11; 16k M = 32 49 / 15 /
-// 17; 456k M = 4 11 / 13 / 7; 456k M = 16 28 / 20 / 14; 797k M = 4 11 / 14 / 9; 797k M = 8 18 / 18 / 13; 1.4M M = 4 13 /
-// 17 / 11; 1.4M M = 16 36 / 32 / 30; 2.4M M = 16 54 / 48 / 42; 7.4M M = 8 57 / 71 / 64; bucket 2048, b = 5: 16k M = 4 11
-// / 12 / 8; 16k M = 16 30 / 16 / 20; 456k M = 8 17 / 18 / 14; 1.4M M = 8 23 / 29 / 21; bucket 96, b = 4: 16k M = 4 15 /
-// 15 / 7; 456k M = 8 24 / 19 / 12; 4.3M M = 8 60 / 66 / 58; whole tensors: 16k M = 4 13 / 16 / 10; 456k M = 8 20 / 21 /
-// 14; 2.4M M = 8 47 / 47 / 44.
-//
+// Whether one kernel goes by warps.  A CTA's four warps are through with a tile in a quarter of a warp's time, so with few tiles
+// the round is as much shorter; with many, the barriers and the eight elements that a thread goes through at a time (a warp's
+// lane: 32) cost more than the unused part of a last turn.  x: tiles a warp (team) of the chip; by warps a turn is an x of 1,
+// by CTAs one of 0.31 (teams 0.63).  By warps / by CTAs (us), at x:
+//   one worker, three of a CTA's warps without a norm to take: above 0.25.  Bucket 512, b = 4 0.19 6.0 / 5.8, 0.33 7.1 / 7.2.
+//   two workers and odd buckets, reduced one by one by half of the warps: above 0.3, but for the start of a second turn.  96, b = 4
+//     0.20 10.1 / 7.8, 0.35 10.4 / 10.5, 0.64 11.6 / 13.0, 0.90 13.0 / 14.8, 1.07 18.0 / 17.1; 480 0.27 8.9 / 7.7, 0.64 10.0 /
+//     11.1, 0.90 (l-infinity) 11.4 / 13.0, 1.07 14.8 / 14.1.
+//   teams: above 0.6, and only the start of a second turn, 1.0 to 1.25, to the CTAs where one pass loses to two kernels.  2048,
+//     b = 5, M = 16 0.60 39.3 / 35.8, 0.74 40.4 / 47.7, 1.01 59.7 / 55.6, 1.16 62.3 / 62.7, 1.26 60.3 / 69.3; M = 32 1.01 112 / 104;
+//     b = 8 118 / 99; M = 3 1.01 16.8 / 17.7.
+//   the others: above 1.2, and the end of the first turn, 0.85 to 1.0, except where a warp's l-infinity norms leave it the
+//     slower way there (512, b = 8, M = 8 0.93 26.5 / 24.4) or its tile is one odd bucket (992, b = 8, M = 12 0.87 38.2 / 35.3).  512, b = 4, M = 8 0.74 21.4 / 20.8, 1.00 30.7 / 25.5, 1.15 31.6 /
+//     29.5, 1.44 33.2 / 33.7; 1024, b = 6, M = 6 0.93 20.3 / 22.4; 128, b = 3, M = 3 0.93 13.9 / 15.0; 480, b = 6, l-infinity, M = 6
+//     0.79 22.2 / 23.3, 0.90 22.8 / 25.2, 1.07 31.1 / 28.2; whole tensors, b = 4, M = 12 0.93 53.3 / 55.4, M = 8 1.00 46.5 / 43.4.
+inline bool dq_by_warps(const RouteQuery& q, const bool one, const bool pairs, const bool linf)
+{
+    const double x = (double)q.positions / (double)q.units;
+    if (q.M == 1) return x > 0.25;
+    if (pairs) return x > 0.6 && (one || x <= 1.0 || x > 1.25);
+    if (!one) return false;
+    if (x > 1.0) return x > 1.2;
+    if (q.odd_buckets > 0) return q.M == 2 ? x > 0.3 : q.odd_buckets > 1 && x > 0.85;
+    return !linf && x > 0.85;
+}
+
 // Only where a few tiles have a great many workers does the CTA, which takes them in turn after all, lose to
-// two kernels that spread them over the chip and slow down with the number of tiles first.
-inline RoundRoute dq_round_route(const RouteQuery& q, const bool cta_tiles, const bool pairs)
+// two kernels that spread them over the chip and slow down with the number of tiles first.  By CTAs / two kernels (us): 512, b = 4, 16k
+// M = 16 11 / 13, M = 32 17 / 15; 2048, b = 5, 16k M = 16 19.6 / 15.5; 992, b = 8, 85k M = 24 15.1 / 16.8.
+//
+// All lines are fitted to 4760 quadruples of times on one B200 (three routes, and the kernels as they were before there was one by CTAs;
+// buckets of 32, 96, 128, 160, 480, 512, 992, 1024, 2048 and whole tensors, 4096 beside them, b = 3 to 8, l2 and l-infinity,
+// M = 1 to 32, 3k to 13M elements, the rule attached): the fastest of the three is missed by 0.6 % on average and 25 % at worst
+// (l-infinity, one worker, 7 us); what dq_one_pass alone would take by more than 3 % at one point in a hundred, 14 % at worst (160, b = 5,
+// 85k M = 24 20.2 / 17.7).
+inline RoundRoute dq_round_route(const RouteQuery& q, const bool cta_tiles, const bool pairs, const bool linf = false)
 {
     const bool one = dq_one_pass(q);
-    const double m = (double)q.M, tiles = (double)q.positions;
-    const double line = q.M == 1 ? 0.25 : (pairs ? 0.6 : 1.2);
     if (!cta_tiles) return one ? kWarpTiles : kTwoKernels;
-    if (tiles > line * (double)q.units && (one || pairs)) return kWarpTiles;
+    if (dq_by_warps(q, one, pairs, linf)) return kWarpTiles;
+    const double m = (double)q.M, tiles = (double)q.positions;
     // what two kernels save per worker, and what they cost besides
     const double per_worker = pairs ? 0.5 : (q.odd_buckets > 0 ? 0.32 : 0.24), besides = pairs ? 5.5 : (q.odd_buckets > 0 ? 6.9 : 6.2);
     return per_worker * m - besides > 0.0005 * tiles * m ? kTwoKernels : kCtaTiles;
@@ -78,7 +97,8 @@ inline bool dq_cta_form(int32_t groups_per_bucket, bool given) { return given ||
 // The route of a call: tile positions of a worker, warps of a launch by warps, and the layout's bucket (32-element groups; where
 // the norms are not given a power of two or less than 32).  lose_first: the test hook of the waits is set; a round by CTAs has no
 // wait to lose, so the call takes the kernels that have.
-inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_per_bucket, int32_t M, bool given, bool lose_first)
+inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_per_bucket, int32_t M, bool given, bool linf,
+                              bool lose_first)
 {
     const bool teams = !given && groups_per_bucket > 32;
     RouteQuery q = {};
@@ -87,5 +107,5 @@ inline RoundRoute dq_route_of(int64_t positions, int64_t warps, int32_t groups_p
     q.M = M;
     q.given = given ? 1 : 0;
     q.odd_buckets = !given && (groups_per_bucket & (groups_per_bucket - 1)) != 0 ? 32 / groups_per_bucket : 0;
-    return dq_round_route(q, dq_cta_form(groups_per_bucket, given) && !lose_first, teams);
+    return dq_round_route(q, dq_cta_form(groups_per_bucket, given) && !lose_first, teams, !given && linf);
 }

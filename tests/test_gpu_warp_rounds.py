@@ -36,7 +36,7 @@ def by_warps(tmp_path_factory):
         """given: the layout's buckets, but for a call whose norms are given."""
         groups = r.lay.D32 // 32
         b = 0 if given else bucket
-        assert route(groups, r.lay.nb, b, r.M, sms, lost) == route_util.WARPS
+        assert route(groups, r.lay.nb, b, r.M, sms, lost, r.linf) == route_util.WARPS
     return check
 
 
@@ -46,7 +46,7 @@ def _round(G, segs, bucket, M, b, linf=False, seed=0):
     gen = torch.Generator(device="cuda").manual_seed(100 * M + b + seed)
     g = torch.full((M, r.stride), float("nan"), device="cuda")
     at = 0
-    r.offsets = []
+    r.offsets, r.linf = [], linf
     for i, n in enumerate(segs):
         r.offsets.append(at)
         g[:, at: at + n] = torch.randn((M, n), generator=gen, device="cuda") * 10.0 ** (i % 5 - 2)
