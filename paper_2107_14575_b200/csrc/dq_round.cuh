@@ -612,11 +612,17 @@ struct WarpFetch {
     // that leave the L2 ahead of them leave a cache full of dirty words: writing 1 GB beside 8.6 GB of reads
     // then costs twice its bytes (copy loop without the encoder, d = 2^26, M = 32, b = 4: 1706 us with
     // evict-first, 1585 normal; text shape 145 -> 134 us, whole-tensor norms 160 -> 155 us at b = 4).  Codes
-    // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal), and made once:
-    // made at every copy it cost codes of 33.5M elements, M = 4, b = 4, given norms 102.4 us against 98.9, norms found 105.0
-    // against 102.5.  (AVG has no registers to keep it.)
+    // alone: evict-first above 64 MB, the average reads them next (2^24 elements: 16.6 us, 17.3 normal).  For given norms it
+    // is made once, before the loop: at every copy / once (us) 33.5M elements M = 4 b = 4 102.4 / 98.9, M = 8 b = 2 199.0 / 192.8.  Where
+    // the norms are found as well it makes 1 or 2 % either way: 33.5M M = 4 b = 4 104.2 / 102.9, 16.8M M = 4 b = 8 l-infinity 59.7 / 61.0,
+    // M = 1 b = 6 16.4 / 16.5; and AVG has no registers to keep it.
+    static constexpr bool kKeepsPolicy = MODE == kGivenNorms && !AVG;
     uint64_t policy;
 
+    __device__ __forceinline__ static uint64_t policy_of(const RoundArgs& a)
+    {
+        return (!AVG && a.stream_reads) ? tma::policy_evict_first() : tma::policy_evict_normal();
+    }
     __device__ __forceinline__ static uint32_t unit_of(const RoundArgs& a)
     {
         return (blockIdx.x * kRoundWarps + (threadIdx.x >> 5)) >> (TEAM ? a.gpb_shift - 5 : 0);
@@ -628,7 +634,7 @@ struct WarpFetch {
           pos0((int)((int64_t)unit_of(where.a) - (int64_t)m_first * positions)), pos(pos0), m(0),
           left(AVG ? n_pos * where.a.M : n_pos), worker(m_first * (where.a.map_has_worker_dim ? 1 : 0)), first(kNoTile),
           parities(0), flying(0), queue0(0), queue1(0), queue2(0), queued(0),
-          policy(AVG ? 0 : (where.a.stream_reads ? tma::policy_evict_first() : tma::policy_evict_normal()))
+          policy(kKeepsPolicy ? policy_of(where.a) : 0)
     {
         if (left > 0) first = tiles.describe(pos);
     }
@@ -649,7 +655,7 @@ struct WarpFetch {
             tma::fetch_tile(tma::smem_addr(stage_ptr(threadIdx.x >> 5, st)), map, tma::smem_addr(stage_bar(threadIdx.x >> 5, st)),
                             kTileBytes, MODE == kGivenNorms ? pos * 32 : (int)(first & 0x7fffffffu),
                             AVG ? (a.map_has_worker_dim ? m : 0) : worker,
-                            AVG ? tma::policy_evict_normal() : policy);
+                            kKeepsPolicy ? policy : policy_of(a));
         if (AVG) {
             if (++m == a.M) {
                 m = 0; pos += hop;
