@@ -994,7 +994,15 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
         if (!trouble) look_at_b();
         if (trouble) return give_up();
         switch (b) {
-#define DQ_CASE(BB) case BB: {                                                                                               TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp_of_team<MODE>(a));                                  WarpFetch<MODE, AVG> copies(tiles, &map);                                                                    copies.next(0);                                                                                              copies.next(1);                                                                                              round_tiles<BB, MODE, AVG, LINF>(a, tiles, copies, square_sum);                                              break;                                                                                                   }
+#define DQ_CASE(BB)                                                                          \
+        case BB: {                                                                               \
+            TileMap<MODE> tiles(a, tbl_in_smem, SmemMap::table, warp_of_team<MODE>(a));          \
+            WarpFetch<MODE, AVG> copies(tiles, &map);                                            \
+            copies.next(0);                                                                      \
+            copies.next(1);                                                                      \
+            round_tiles<BB, MODE, AVG, LINF>(a, tiles, copies, square_sum);                      \
+            break;                                                                               \
+        }
             DQ_CASE(1) DQ_CASE(2) DQ_CASE(3) DQ_CASE(4) DQ_CASE(5) DQ_CASE(6) DQ_CASE(7) DQ_CASE(8)
             DQ_CASE(9) DQ_CASE(10) DQ_CASE(11) DQ_CASE(12) DQ_CASE(13) DQ_CASE(14) DQ_CASE(15) DQ_CASE(16)
 #undef DQ_CASE
@@ -1035,11 +1043,14 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 // in registers from a position's first worker to its last.
 // What bounds it: with a position per SM the chain of a chunk (20 tiles, M = 16, cycles: norm 710, codes of four workers 1090
 // two by two, 1400 one after the other, two barriers 180; the rest copies and addresses), with many the instructions,
-// some 700 per tile and worker at b = 4, 515 in a warp's own way: scales, notes and addresses come once per eight elements.  Where
-// the line between the two lies, and what both measured: dq_route.h.
-// Five CTAs per SM (96 registers).  By five / four / six of them (us): bucket 512, 600k elements M = 8 b = 5 10.4 / 10.2 / 12.2
+// 820 per tile and worker at b = 4 (2^19 elements, M = 8, set-up and the rule's end among them), 515 in a warp's own way:
+// scales, notes and addresses come once per eight elements.  A capture, whose caches are cold, has waiting for instructions as its
+// largest stall (2.9 of some 9 per issue, 0.25 by warps); with warm ones it is not measured.  Where the line between the two lies,
+// and what both measured: dq_route.h.
+// Five CTAs per SM (96 registers; buckets of 2048, l2, spill 632 bytes, the others next to nothing).  By five / four / six of them (us): bucket 512, 600k elements M = 8 b = 5 10.4 / 10.2 / 12.2
 // (six spill); 610k, one turn of five, two of four, M = 8 b = 4 9.4 / 11.3; 1.3M M = 8 17.4 / 17.1 / 23.2; bucket 2048, 1.2M
-// M = 16 31.4 / 29.6 / 38.1, 1.3M M = 8 21.6 / 23.0.
+// M = 16 31.4 / 29.6 / 38.1, 1.3M M = 8 21.6 / 23.0.  (Four for buckets of 2048 alone: 6 to 15 % less where the positions fill
+// as many turns, 2 to 14 % more where they need another, 0.6M and 1.25M.)
 constexpr int kTileCtasPerSm = 5;
 constexpr int kSets = 2;                            // chunks in shared memory: the one at hand and one on its way
 struct TileSmem {

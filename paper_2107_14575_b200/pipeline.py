@@ -30,7 +30,7 @@ class Round:
         # two (b, s) slots of 16 bytes: where ``step_fused`` puts the bit rule on a second stream (``events``), the
         # next b goes to the other one while the average still reads this one; one-call rounds stay in their slot
         self._b = torch.zeros((2, 4), dtype=torch.int32, device=self.device)
-        # (taking a slot out of the tensor costs a call 1.1 us of the host's time: 70,001 elements M = 4 7.7 us of the host a round, now 5.2)
+        # (taking a slot out of the tensor costs a call 1.1 us of the host's time)
         self._slots = (self._b[0], self._b[1])
         self._cur = 0
         self._side = None
