@@ -1043,7 +1043,7 @@ round_kernel(const __grid_constant__ RoundArgs a, const __grid_constant__ CUtens
 // in registers from a position's first worker to its last.
 // What bounds it: with a position per SM the chain of a chunk (20 tiles, M = 16, cycles: norm 710, codes of four workers 1090
 // two by two, 1400 one after the other, two barriers 180; the rest copies and addresses), with many the instructions,
-// 820 per tile and worker at b = 4 (2^19 elements, M = 8, set-up and the rule's end among them), 515 in a warp's own way:
+// 830 per tile and worker at b = 4 (2^19 elements, M = 8, set-up and the rule's end among them), 515 in a warp's own way:
 // scales, notes and addresses come once per eight elements.  A capture, whose caches are cold, has waiting for instructions as its
 // largest stall (2.9 of some 9 per issue, 0.25 by warps); with warm ones it is not measured.  Where the line between the two lies,
 // and what both measured: dq_route.h.
